@@ -1,132 +1,148 @@
 // Adjoint of the forward scatter: a conflict-free gather over observers.
 //
-// The forward adds, for panel p, observer o and source sample k,
-//   a g + cc m  to bin k - i0   and   b g + dd m  to bin k - i0 - 1,
-// with g = c . F[k], m = c . M[k].  Its transpose, for the gradient G of the
-// loss with respect to p_out (zero outside the valid bins 0 <= j < N_o), is
-//   gF = a G[k - i0] + b G[k - i0 - 1],   gM = cc G[k - i0] + dd G[k - i0 - 1]
-//   Xbar[p][k][s]     = sum_o c_s gF,     Xbar[p][k][8 + s] = sum_o c_s gM,
+// The forward adds, for panel p, observer o and sample s (row s + 1 of X),
+// w_t G_s to the bin of interval s + 1 - t, t = 0 .. 3, with G_s = c . X[s].
+// Its transpose, for the gradient g of the loss with respect to p_out (zero
+// outside the valid bins 0 <= j < N_o), is
+//   q = w3 g[s-2-i0] + w2 g[s-1-i0] + w1 g[s-i0] + w0 g[s+1-i0]
+//   Xbar[p][s][v] = sum_o c_v q,
 // so each (panel, sample) output is owned by one lane and summed over the
-// observers in registers, 20 FMA per (panel, sample, observer).  Two forms:
-// k_adjoint_set (FP32) gathers per panel set from a window of G staged in
+// observers in registers, 12 multiply-adds per (panel, sample, observer).
+// The ghost rows beta_{-1} = 2 beta_0 - beta_1 and beta_nt = 2 beta_{nt-1} -
+// beta_{nt-2} hand their gradients to the two samples next to them: q of those
+// samples takes the ghost's q times 2 and -1 (edge chunks only).  Two forms:
+// k_adjoint_set (FP32) gathers per panel set from a window of g staged in
 // shared memory, with atomics only to add the partial sums of several
-// 36-observer groups; k_adjoint (FP64, and FP32 shapes with 256-sample
-// chunks) is one CTA per panel reading G from L2, without atomics.
-// Nothing from the forward pass is stored: only the per-(p, o) records
-// (geometry, computed once per observer set), the plan and G are read.
+// 36-observer groups; k_adjoint (FP64) is one CTA per panel reading g from
+// L2, without atomics.  Nothing from the forward pass is stored: only the
+// per-(p, o) records (geometry, computed once per observer set), the plan and
+// g are read.
 #include "fwh_internal.cuh"
 
 namespace fwh {
 
 namespace {
 
-template <typename T> __device__ __forceinline__ int i0_of(T v);
-template <> __device__ __forceinline__ int i0_of<float>(float v) { return __float_as_int(v); }
-template <> __device__ __forceinline__ int i0_of<double>(double v) { return (int)v; }
-
-// G converted to T with zeros outside [0, N_o): Gt[o][j], j < ntp.
+// g converted to T with zeros outside [0, N_o): Gt[o][j], j < g_ld.
 template <typename T>
 __global__ void k_grad_pad(const double *grad_p, const int *n_valid, T *Gt, int O, int nt,
-                           int ntp) {
+                           int g_ld) {
   for (int o = blockIdx.y; o < O; o += gridDim.y) {  // grid y is capped at 65535
     const int nv = n_valid[o];
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < ntp; j += gridDim.x * blockDim.x)
-      Gt[(size_t)o * ntp + j] = (j < nv && j < nt) ? (T)grad_p[(size_t)o * nt + j] : T(0);
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < g_ld; j += gridDim.x * blockDim.x)
+      Gt[(size_t)o * g_ld + j] = (j < nv && j < nt) ? (T)grad_p[(size_t)o * nt + j] : T(0);
   }
 }
 
-// One CTA per (panel, group of 8 chunks), one warp per chunk.  The panel's
-// records are staged in shared memory in tiles of kObsTile observers (read
-// back as broadcasts), and each lane loads the two gradient bins of the next
-// observer while it accumulates the current one.
+// q of a sample from g at the intervals s - 2 .. s + 1.
+template <typename T>
+__device__ __forceinline__ T gather_q(const T *w, T gm2, T gm1, T g0, T g1) {
+  return fma(w[0], g1, fma(w[1], g0, fma(w[2], gm1, w[3] * gm2)));
+}
+// The ghost rows' share of sample s (see above).
+template <typename T>
+__device__ __forceinline__ T ghost_q(int s, int nt, const T *w, T gm2, T gm1, T g0, T g1) {
+  T v = T(0);
+  if (s == 0) v += T(2) * (w[0] * g0);
+  if (s == 1) v -= w[0] * gm1;
+  if (s == nt - 1) v += T(2) * (w[3] * gm1 + w[2] * g0);
+  if (s == nt - 2) v -= w[3] * g0 + w[2] * g1;
+  return v;
+}
+
+// FP64: one CTA per (panel, group of 8 chunks of 64 samples), one warp per
+// chunk.  The panel's records are staged in shared memory in tiles of
+// kObsTile observers (read back as broadcasts), and each lane loads the
+// gradient bins of the next observer while it accumulates the current one.
 constexpr int kObsTile = 128;
 
-template <typename T, int TK>
-__global__ void __launch_bounds__(256) k_adjoint(const T *coef, const T *Gt, T *Xbar, int P,
-                                                 int O, int ntp) {
-  constexpr int CH = 32 * TK;
-  __shared__ __align__(16) T srec[kObsTile * kRec];
+__global__ void __launch_bounds__(256) k_adjoint(AdjArgs<double> a) {
+  constexpr int TK = 2, CH = 32 * TK;
+  __shared__ __align__(16) double srec[kObsTile * kRec];
   const int lane = threadIdx.x & 31;
   const int w = threadIdx.x >> 5;
-  const int nch = ntp / CH;
+  const int nch = (a.nt + CH - 1) / CH;
   const int ngrp = (nch + 7) / 8;
   const int p = blockIdx.x / ngrp;
   const int ch = (blockIdx.x % ngrp) * 8 + w;
   const bool live = ch < nch;  // warps past the last chunk only help staging
   const int k0 = ch * CH;
-  T acc[TK][kRec];
+  const bool edge = k0 == 0 || k0 + CH >= a.nt - 1;
+  double acc[TK][kSer];
 #pragma unroll
   for (int j = 0; j < TK; ++j)
 #pragma unroll
-    for (int s = 0; s < kRec; ++s) acc[j][s] = T(0);
-  const T *rec0 = coef + (size_t)p * O * kRec;
-  for (int ob = 0; ob < O; ob += kObsTile) {
-    const int no = min(kObsTile, O - ob);
+    for (int s = 0; s < kSer; ++s) acc[j][s] = 0.0;
+  const double *rec0 = a.coef + (size_t)p * a.O * kRec;
+  for (int ob = 0; ob < a.O; ob += kObsTile) {
+    const int no = min(kObsTile, a.O - ob);
     __syncthreads();
     for (int idx = threadIdx.x; idx < no * kRec; idx += blockDim.x)
       srec[idx] = rec0[(size_t)ob * kRec + idx];
     __syncthreads();
     if (!live) continue;
-    auto bins = [&](int o, T (&g0)[TK], T (&g1)[TK]) {
-      const int i0 = i0_of<T>(srec[o * kRec + slot::i0]);
-      const T *G = Gt + (size_t)(ob + o) * ntp;
+    auto bins = [&](int o, double (&g)[TK][4]) {
+      const int i0 = (int)srec[o * kRec + slot::i0];
+      const double *G = a.Gt + (size_t)(ob + o) * a.g_ld;
 #pragma unroll
-      for (int j = 0; j < TK; ++j) {
-        const int jb = k0 + lane + 32 * j - i0;  // bin fed by the left spline node
-        g0[j] = jb >= 0 ? __ldg(G + jb) : T(0);
-        g1[j] = jb >= 1 ? __ldg(G + jb - 1) : T(0);
-      }
-    };
-    T g0[TK], g1[TK];
-    bins(0, g0, g1);
-    for (int o = 0; o < no; ++o) {
-      T n0[TK], n1[TK];
-      if (o + 1 < no) bins(o + 1, n0, n1);
-      const T *r = srec + o * kRec;
-      T c[12];
+      for (int j = 0; j < TK; ++j)
 #pragma unroll
-      for (int s = 0; s < 12; ++s) c[s] = r[s];  // c0..c7, then the four weights
-#pragma unroll
-      for (int j = 0; j < TK; ++j) {
-        const T gF = c[slot::a] * g0[j] + c[slot::b] * g1[j];
-        const T gM = c[slot::cc] * g0[j] + c[slot::dd] * g1[j];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-          acc[j][s] = fma(c[slot::c + s], gF, acc[j][s]);
-          acc[j][8 + s] = fma(c[slot::c + s], gM, acc[j][8 + s]);
+        for (int t = 0; t < 4; ++t) {
+          const int jb = k0 + lane + 32 * j - 2 + t - i0;  // bin of interval s - 2 + t
+          g[j][t] = jb >= 0 && jb < a.g_ld ? __ldg(G + jb) : 0.0;
         }
+    };
+    double g[TK][4];
+    bins(0, g);
+    for (int o = 0; o < no; ++o) {
+      double gn[TK][4];
+      if (o + 1 < no) bins(o + 1, gn);
+      double c[12];
+#pragma unroll
+      for (int s = 0; s < 12; ++s) c[s] = srec[o * kRec + s];
+#pragma unroll
+      for (int j = 0; j < TK; ++j) {
+        double q = gather_q(c + slot::w, g[j][0], g[j][1], g[j][2], g[j][3]);
+        if (edge)
+          q += ghost_q(k0 + lane + 32 * j, a.nt, c + slot::w, g[j][0], g[j][1], g[j][2], g[j][3]);
+#pragma unroll
+        for (int s = 0; s < kSer; ++s) acc[j][s] = fma(c[s], q, acc[j][s]);
       }
       if (o + 1 < no) {
 #pragma unroll
-        for (int j = 0; j < TK; ++j) {
-          g0[j] = n0[j];
-          g1[j] = n1[j];
-        }
+        for (int j = 0; j < TK; ++j)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) g[j][t] = gn[j][t];
       }
     }
   }
   if (!live) return;
-  T *out = Xbar + ((size_t)p * ntp + k0 + lane) * kRec;
+  double *out = a.Xbar + ((size_t)p * a.xb_ld + k0 + lane) * kSer;
 #pragma unroll
   for (int j = 0; j < TK; ++j)
 #pragma unroll
-    for (int s = 0; s < kRec; ++s) out[(size_t)j * 32 * kRec + s] = acc[j][s];
+    for (int s = 0; s < kSer; s += 4)
+      stg256(out + (size_t)j * 32 * kSer + s, __double_as_longlong(acc[j][s]),
+             __double_as_longlong(acc[j][s + 1]), __double_as_longlong(acc[j][s + 2]),
+             __double_as_longlong(acc[j][s + 3]));
 }
 
 // Set form (FP32).  Work item = (panel set, observer group, 128-sample
 // chunk), numbered observer group fastest, then chunk, then the sets in
 // descending size.  The gradient bins every (panel, observer) of the set can
-// touch in the chunk, G[k0 - i0max(o) - 1 + t] for t < win + 1 (the planner
-// bounds each record's offset i0max - i0 by the window slack), are staged in
-// shared memory once per item; each warp then takes panels of the set in
-// turn and, for every observer of the group, reads the two bins of each of
-// its samples from that window (conflict-free, consecutive lanes at
-// consecutive slots) and accumulates the 16 components of Xbar in registers.
-// Each warp stages the group's records of its next panel in shared memory
-// (cp.async, a double buffer per warp) while it works on the current one, so
-// the inner loop reads every record as a shared-memory broadcast instead of
-// waiting on L2.  One observer group writes Xbar directly; several add their
-// partial sums with vector atomics into a zeroed Xbar.
+// touch in the chunk are staged in shared memory once per item, quarter-split
+// as the forward's windows (slot Y, the bin of interval k0 - 2 + Y at the
+// set's largest shift, in quarter Y & 3 at word Y >> 2), so the records'
+// byte offsets serve here too.  Each warp then takes panels of the set in
+// turn; a lane holds four consecutive samples, reads the seven bins they
+// touch per observer (conflict-free) and accumulates the eight components of
+// its Xbar rows as register pairs with packed FMAs.  Each warp stages the
+// group's records of its next panel in shared memory (cp.async, a double
+// buffer per warp) while it works on the current one, so the inner loop reads
+// every record as a shared-memory broadcast instead of waiting on L2.  One
+// observer group writes Xbar directly, 32 bytes a lane and store; several add
+// their partial sums with vector atomics into a zeroed Xbar.
+// @ADJ@
 constexpr int kAdjGroup = 36;    // observers per item
 constexpr int kAdjWarps = 4;
 constexpr int kAdjTK = 4;        // samples per lane (chunk 128)
@@ -158,41 +174,43 @@ __device__ __forceinline__ void red_add_v4(float *addr, float4 v) {
 template <bool kAtomic>
 __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a) {
   constexpr int CH = 32 * kAdjTK;
-  extern __shared__ __align__(16) float gw[];  // [kAdjGroup][wstride], then the record buffers
-  const int wstride = (a.win + 1 + 3) & ~3;
+  extern __shared__ __align__(16) float gw[];  // [kAdjGroup][win], then the record buffers
+  const int win = a.win, H = win >> 2;
   const int lane = threadIdx.x & 31;
   const int w = threadIdx.x >> 5;
   const int ng = (a.O + kAdjGroup - 1) / kAdjGroup;
-  const int nch = a.ntp / CH;
+  const int nch = (a.nt + CH - 1) / CH;
   const int item = blockIdx.x;
   const int g = item % ng;
   const int rest = item / ng;
   const int ch = rest % nch;
   const int sidx = a.set_order[rest / nch];
   const int k0 = ch * CH;
+  const bool edge = k0 == 0 || k0 + CH >= a.nt - 1;
   const int o0 = g * kAdjGroup;
   const int no = min(kAdjGroup, a.O - o0);
   const int p_begin = a.set_begin[sidx], p_end = a.set_begin[sidx + 1];
   // stage the window of each observer of the group (cp.async: every copy in
   // flight at once; zero outside the record)
   for (int o = 0; o < no; ++o) {
-    const int base = k0 - a.i0max_tab[(size_t)sidx * a.O + o0 + o] - 1;
-    const float *G = a.Gt + (size_t)(o0 + o) * a.ntp;
-    for (int t = threadIdx.x; t <= a.win; t += blockDim.x) {
+    const int base = k0 - 2 - a.i0max_tab[(size_t)sidx * a.O + o0 + o];
+    const float *G = a.Gt + (size_t)(o0 + o) * a.g_ld;
+    for (int t = threadIdx.x; t < win; t += blockDim.x) {
       const int j = base + t;
-      const bool ok = j >= 0 && j < a.ntp;
-      cp_async4_zf(gw + o * wstride + t, G + (ok ? j : 0), ok);
+      const bool ok = j >= 0 && j < a.g_ld;
+      cp_async4_zf(gw + o * win + (t & 3) * H + (t >> 2), G + (ok ? j : 0), ok);
     }
   }
   cp_async_commit();
   // this warp's record double buffer: [2][kAdjGroup][kRec]
-  float *rb = gw + (size_t)kAdjGroup * wstride + (size_t)w * 2 * kAdjGroup * kRec;
+  float *rb = gw + (size_t)kAdjGroup * win + (size_t)w * 2 * kAdjGroup * kRec;
   auto stage = [&](int p, int buf) {  // the group's records of panel p, 16 bytes a copy
     const float *src = a.coef + ((size_t)p * a.O + o0) * kRec;
     float *dst = rb + (size_t)buf * kAdjGroup * kRec;
     for (int c = lane; c < no * (kRec / 4); c += 32) cp_async16(dst + 4 * c, src + 4 * c);
     cp_async_commit();
   };
+  const int shift = a.slot_shift;  // the records' offsets are in slots of 2^shift bytes
   int buf = 0;
   if (p_begin + w < p_end) stage(p_begin + w, 0);
   cp_async_wait<0>();  // the window (and this warp's first records)
@@ -206,46 +224,51 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
       cp_async_wait<0>();
     }
     __syncwarp();
-    float acc[kAdjTK][kRec];
+    f32x2 acc[kAdjTK][kSer / 2];
 #pragma unroll
     for (int j = 0; j < kAdjTK; ++j)
 #pragma unroll
-      for (int s = 0; s < kRec; ++s) acc[j][s] = 0.f;
-    const float4 *rec = reinterpret_cast<const float4 *>(rb + (size_t)buf * kAdjGroup * kRec);
+      for (int s = 0; s < kSer / 2; ++s) acc[j][s] = 0ull;
+    const float *rec = rb + (size_t)buf * kAdjGroup * kRec;
 #pragma unroll 2
     for (int o = 0; o < no; ++o) {
-      const float4 r0 = rec[4 * o], r1 = rec[4 * o + 1], r2 = rec[4 * o + 2],
-                   r3 = rec[4 * o + 3];
-      const float c[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-      const float wa = r2.x, wb = r2.y, wcc = r2.z, wdd = r2.w;  // slots a, b, cc, dd
-      const int off = __float_as_int(r3.y);                       // slot off = i0max - i0
-      // G[k - i0] at window slot (k - k0) + off + 1, G[k - i0 - 1] one below
-      const float *gp = gw + o * wstride + off + lane;
+      const ulonglong2 c01 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec);
+      const ulonglong2 c23 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec + 4);
+      const float4 wv = *reinterpret_cast<const float4 *>(rec + o * kRec + slot::w);
+      const uint4 qo = *reinterpret_cast<const uint4 *>(rec + o * kRec + slot::q0);
+      const f32x2 c[4] = {c01.x, c01.y, c23.x, c23.y};
+      const float wt[4] = {wv.x, wv.y, wv.z, wv.w};
+      const float *gp = gw + o * win + lane;
+      const float *A[4] = {gp + (qo.x >> shift), gp + (qo.y >> shift), gp + (qo.z >> shift),
+                           gp + (qo.w >> shift)};
+      float gv[7];  // bins of intervals s - 2 .. s + 4 of the lane's first sample s
+#pragma unroll
+      for (int i = 0; i < 7; ++i) gv[i] = A[i & 3][i >> 2];
 #pragma unroll
       for (int j = 0; j < kAdjTK; ++j) {
-        const float g1 = gp[32 * j], g0 = gp[32 * j + 1];
-        const float gF = wa * g0 + wb * g1;
-        const float gM = wcc * g0 + wdd * g1;
+        float q = gather_q(wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
+        if (edge)
+          q += ghost_q(k0 + 4 * lane + j, a.nt, wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
+        const f32x2 q2 = f2_dup(q);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
-          acc[j][s] = fmaf(c[s], gF, acc[j][s]);
-          acc[j][8 + s] = fmaf(c[s], gM, acc[j][8 + s]);
-        }
+        for (int s = 0; s < kSer / 2; ++s) acc[j][s] = f2_fma(c[s], q2, acc[j][s]);
       }
     }
-    float *out = a.Xbar + ((size_t)p * a.ntp + k0 + lane) * kRec;
+    float *out = a.Xbar + ((size_t)p * a.xb_ld + k0 + 4 * lane) * kSer;
 #pragma unroll
-    for (int j = 0; j < kAdjTK; ++j)
+    for (int j = 0; j < kAdjTK; ++j) {
+      if (kAtomic) {
 #pragma unroll
-      for (int q = 0; q < kRec / 4; ++q) {
-        const float4 v = make_float4(acc[j][4 * q], acc[j][4 * q + 1], acc[j][4 * q + 2],
-                                     acc[j][4 * q + 3]);
-        float *dst = out + (size_t)j * 32 * kRec + 4 * q;
-        if (kAtomic)
-          red_add_v4(dst, v);
-        else
-          *reinterpret_cast<float4 *>(dst) = v;
+        for (int h = 0; h < 2; ++h) {
+          float4 v;
+          f2_split(acc[j][2 * h], v.x, v.y);
+          f2_split(acc[j][2 * h + 1], v.z, v.w);
+          red_add_v4(out + j * kSer + 4 * h, v);
+        }
+      } else {
+        stg256(out + j * kSer, acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
       }
+    }
     __syncwarp();  // every lane is done with this buffer before it is refilled
     buf ^= 1;
   }
@@ -255,44 +278,32 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
 
 template <typename T>
 cudaError_t launch_adjoint(const AdjArgs<T> &a, cudaStream_t s) {
-  constexpr int TK = sizeof(T) == 4 ? 4 : 2;
-  constexpr int CH = 32 * TK;
-  T *Gt = a.Gt;
-  dim3 gg((a.ntp + 255) / 256, a.O < 65535 ? a.O : 65535);
-  k_grad_pad<T><<<gg, 256, 0, s>>>(a.grad_p, a.n_valid, Gt, a.O, a.nt, a.ntp);
+  dim3 gg((a.g_ld + 255) / 256, a.O < 65535 ? a.O : 65535);
+  k_grad_pad<T><<<gg, 256, 0, s>>>(a.grad_p, a.n_valid, a.Gt, a.O, a.nt, a.g_ld);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if constexpr (sizeof(T) == 4) {
-    if (a.win > 0) {
-      constexpr int SCH = 32 * kAdjTK;
-      if (a.ntp % SCH != 0) return cudaErrorInvalidValue;
-      const int ng = (a.O + kAdjGroup - 1) / kAdjGroup;
-      const long items = (long)a.nsets * ng * (a.ntp / SCH);
-      if (items <= 0) return cudaSuccess;
-      if (items > INT32_MAX) return cudaErrorInvalidValue;
-      const size_t smem = ((size_t)kAdjGroup * ((a.win + 1 + 3) & ~3) +
-                           (size_t)kAdjWarps * 2 * kAdjGroup * kRec) * sizeof(float);
-      if (ng > 1) {
-        e = cudaMemsetAsync(a.Xbar, 0, (size_t)a.P * a.ntp * kRec * sizeof(float), s);
-        if (e != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_adjoint_set<true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-          return e;
-        k_adjoint_set<true><<<(unsigned)items, kAdjWarps * 32, smem, s>>>(a);
-      } else {
-        if ((e = cudaFuncSetAttribute(k_adjoint_set<false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-          return e;
-        k_adjoint_set<false><<<(unsigned)items, kAdjWarps * 32, smem, s>>>(a);
-      }
-      return cudaGetLastError();
+    constexpr int CH = 32 * kAdjTK;
+    const int ng = (a.O + kAdjGroup - 1) / kAdjGroup;
+    const long items = (long)a.nsets * ng * ((a.nt + CH - 1) / CH);
+    if (items <= 0) return cudaSuccess;
+    if (items > INT32_MAX) return cudaErrorInvalidValue;
+    const size_t smem = ((size_t)kAdjGroup * a.win + (size_t)kAdjWarps * 2 * kAdjGroup * kRec) *
+                        sizeof(float);
+    auto kern = ng > 1 ? k_adjoint_set<true> : k_adjoint_set<false>;
+    if (ng > 1) {
+      e = cudaMemsetAsync(a.Xbar, 0, (size_t)a.P * a.xb_ld * kSer * sizeof(float), s);
+      if (e != cudaSuccess) return e;
     }
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)items, kAdjWarps * 32, smem, s>>>(a);
+  } else {
+    const long blocks = (long)a.P * (((a.nt + 63) / 64 + 7) / 8);
+    if (blocks <= 0) return cudaSuccess;
+    if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+    k_adjoint<<<(unsigned)blocks, 256, 0, s>>>(a);
   }
-  const long blocks = (long)a.P * ((a.ntp / CH + 7) / 8);
-  if (blocks <= 0) return cudaSuccess;
-  k_adjoint<T, TK><<<(unsigned)blocks, 256, 0, s>>>(a.coef, Gt, a.Xbar, a.P, a.O, a.ntp);
   return cudaGetLastError();
 }
 

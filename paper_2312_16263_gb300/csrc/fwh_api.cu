@@ -29,6 +29,7 @@ using namespace fwh;
 namespace {
 
 constexpr int kMaxSet = 64;
+constexpr int kWantItems = 152 * 6;  // work items a forward launch should have
 
 struct Buf {
   void *p = nullptr;
@@ -48,7 +49,7 @@ struct BatchPlan {
   std::vector<BatchParams<float>> pf;   // [nr] launch parameters (FP32 surfaces)
   std::vector<BatchParams<double>> pd;  // [nr] launch parameters (FP64 surfaces)
   std::vector<int> total;      // work items of each round's scatter launch
-  std::vector<int> x_ld;       // X rows per panel of each surface (ring or whole record)
+  std::vector<int> x_ld;       // X rows per panel of each surface (one round or whole record)
   std::vector<int> nseg;       // time segments of each surface
   int nq = 0;                  // time segments of the longest record
   int R = 0;                   // segments per round (nq: the whole record in one round)
@@ -71,8 +72,8 @@ struct fwh_ctx {
   // device state
   double *d_y = nullptr, *d_n = nullptr, *d_dS = nullptr, *d_x = nullptr;
   double *d_Rmax = nullptr, *d_Rmin = nullptr;
-  int *d_perm = nullptr, *d_err = nullptr;
-  Buf coef, X, G, nvalid, sets, sord, stage_in, stage_out, stage_grad, imax;
+  int *d_place = nullptr, *d_err = nullptr;  // caller index -> library position; error flag
+  Buf coef, i0, X, G, nvalid, sets, sord, stage_in, stage_out, stage_grad, imax;
   // X tensor map (passed to single launches as a kernel parameter; batched
   // calls keep device copies in their plans)
   alignas(64) unsigned char tmap_host[128] = {};
@@ -92,11 +93,10 @@ struct fwh_ctx {
   bool err_pending = false;
   // per-nt
   int64_t nt = -1;
-  int ntp = 0;
   std::vector<int> h_nvalid;
   std::vector<double> h_tstart;
   // planner
-  int plan_win = -1, plan_ch = -1, plan_sb = -1;
+  int plan_win = -1, plan_slack = -1, plan_sb = -1;
   std::vector<int> set_begin;
   int cfg = -1;  // forced/tuned forward config (-1 default)
   bool timing = false;
@@ -225,10 +225,13 @@ int default_cfg(const fwh_ctx *h) {
   return 0;
 }
 
-// Observer tiling for a config: observers per warp and groups.
+// Observer tiling for a config: the fewest groups that hold all observers,
+// and observers per warp as even as they go over those (37 observers: two
+// groups of 20 and 17, not 36 and 1).
 void obs_tiling(const fwh_ctx *h, const FwdConfig &c, int *obs_per_cta, int *groups) {
-  int opw = (int)std::min<int64_t>(c.obs_per_warp, (h->O + c.warps - 1) / c.warps);
-  if (opw < 1) opw = 1;
+  const int64_t most = (int64_t)c.obs_per_warp * c.warps;
+  const int64_t ng = (h->O + most - 1) / most;
+  const int opw = (int)std::max<int64_t>(1, (h->O + ng * c.warps - 1) / (ng * c.warps));
   *obs_per_cta = opw * c.warps;
   *groups = (int)((h->O + *obs_per_cta - 1) / *obs_per_cta);
 }
@@ -236,10 +239,10 @@ void obs_tiling(const fwh_ctx *h, const FwdConfig &c, int *obs_per_cta, int *gro
 // Panel sets for a config, and the plan kernel's per-(set, observer) shift
 // table and per-record window offsets, enqueued on `s`.
 fwh_status plan(fwh_handle h, const FwdConfig &c, cudaStream_t s) {
-  const int ch = 32 * c.tk;
+  const bool fp64 = h->precision == FWH_FP64;
+  const int smax = fwd_slack(fp64, c);
   const int sb = c.acc == 5 ? 8 : 4;  // bytes per FP32 window slot (sum, or sum + compensation)
-  if (h->plan_win == c.win && h->plan_ch == ch && h->plan_sb == sb) return FWH_OK;
-  const int smax = c.win - ch - 1;
+  if (h->plan_win == c.win && h->plan_slack == smax && h->plan_sb == sb) return FWH_OK;
   h->set_begin = build_sets(h->y, h->P, h->mach, h->dt, smax);
   const size_t bytes = h->set_begin.size() * sizeof(int);
   const int nsets = (int)h->set_begin.size() - 1;
@@ -255,23 +258,22 @@ fwh_status plan(fwh_handle h, const FwdConfig &c, cudaStream_t s) {
     CK(h, cudaMemcpy(h->sord.p, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice));
   }
   CK(h, ensure(h->imax, (size_t)nsets * h->O * sizeof(int)));
-  if (h->precision == FWH_FP64)
-    CK(h, launch_plan<double>(reinterpret_cast<double *>(h->coef.p),
-                              reinterpret_cast<const int *>(h->sets.p), nsets, (int)h->O, smax,
-                              0, 0, reinterpret_cast<int *>(h->imax.p), h->d_err, s));
+  const int *i0 = reinterpret_cast<const int *>(h->i0.p);
+  const int *sets = reinterpret_cast<const int *>(h->sets.p);
+  int *imax = reinterpret_cast<int *>(h->imax.p);
+  if (fp64)
+    CK(h, launch_plan<double>(reinterpret_cast<double *>(h->coef.p), i0, sets, nsets, (int)h->O,
+                              smax, c.win, sb, imax, h->d_err, s));
   else
-    CK(h, launch_plan<float>(reinterpret_cast<float *>(h->coef.p),
-                             reinterpret_cast<const int *>(h->sets.p), nsets, (int)h->O, smax,
-                             (c.win / 2) * sb, sb,
-                             reinterpret_cast<int *>(h->imax.p), h->d_err, s));
+    CK(h, launch_plan<float>(reinterpret_cast<float *>(h->coef.p), i0, sets, nsets, (int)h->O,
+                             smax, c.win, sb, imax, h->d_err, s));
   h->plan_win = c.win;
-  h->plan_ch = ch;
+  h->plan_slack = smax;
   h->plan_sb = sb;
   return FWH_OK;
 }
 
-// Per-nt window and workspace.  ntp is a multiple of 256, hence of every
-// forward chunk (32 x TK samples) and prep chunk.
+// Per-nt window and workspace.
 constexpr int64_t kMaxNt = (int64_t)1 << 28;
 
 fwh_status prepare_window(fwh_handle h, int64_t nt) {
@@ -294,33 +296,95 @@ fwh_status prepare_window(fwh_handle h, int64_t nt) {
     CK(h, ensure(h->nvalid, h->O * sizeof(int)));
     CK(h, cudaMemcpy(h->nvalid.p, h->h_nvalid.data(), h->O * sizeof(int),
                      cudaMemcpyHostToDevice));
-    const int64_t ntp = (nt + 255) / 256 * 256;  // a multiple of every chunk length
     h->nt = nt;
-    h->ntp = (int)ntp;
   }
   return FWH_OK;
 }
 
-// Window and the whole-record series buffer X.
+// Xbar rows per panel of the backward pass: whole 128-sample chunks.
+int64_t xbar_rows(int64_t nt) { return (nt + 127) / 128 * 128; }
+
+// Window and the whole-record buffer: X of a forward pass, Xbar of a backward.
 fwh_status prepare_nt(fwh_handle h, int64_t nt) {
   fwh_status st = prepare_window(h, nt);
   if (st != FWH_OK) return st;
-  const size_t ts = tsize(h->precision);
-  CK(h, ensure(h->X, (size_t)h->P * h->ntp * kRec * ts));
+  CK(h, ensure(h->X, (size_t)h->P * std::max(x_rows(nt), xbar_rows(nt)) * kSer *
+                             tsize(h->precision) + kXPad));
   return FWH_OK;
 }
 
-// Config actually used: TMA configs address X rows with 32-bit coordinates
-// (FP64 falls back to a direct-load shape; every FP32 shape is a TMA shape,
-// its rows are sample pairs, and prepare_nt bounds P x ntp below 2^32).
-int effective_cfg(const fwh_ctx *h, int64_t ntp) {
+// Config actually used: FP64 TMA configs address X lines with 32-bit
+// coordinates and fall back to a direct-load shape (every FP32 shape is a TMA
+// shape; prepare_window bounds its rows).
+int effective_cfg(const fwh_ctx *h, int64_t nt) {
   const bool fp64 = h->precision == FWH_FP64;
   int cfg = h->cfg >= 0 ? h->cfg : default_cfg(h);
-  if (fwd_config(fp64, cfg).pipe != 0 && h->P * ntp >= ((int64_t)1 << 31)) {
+  if (fp64 && fwd_config(fp64, cfg).pipe != 0 && h->P * x_rows(nt) >= ((int64_t)1 << 31)) {
     for (int i = 0; i < fwd_num_configs(fp64); ++i)
       if (fwd_config(fp64, i).pipe == 0) return i;
   }
   return cfg;
+}
+
+// Work items a panel set is cut into, from sizes of the whole problem only
+// (every launch form of it then forms the same partial sums): enough items to
+// give each SM several CTAs, at least eight panels an item.
+int set_subs(const fwh_ctx *h, int groups, int n_segs) {
+  const int64_t nsets = (int64_t)h->set_begin.size() - 1;
+  const int64_t items = nsets * groups * n_segs;
+  const int64_t want = (kWantItems + items - 1) / items;
+  const int64_t most = std::max<int64_t>(1, h->P / nsets / 8);
+  return (int)std::min(want, most);
+}
+
+// The forward arguments of a whole record; X rows from row 0.
+template <typename T>
+FwdArgs<T> forward_args(fwh_ctx *h, const FwdConfig &c, int64_t nt, const T *X, int x_ld,
+                        const int *n_valid, double *p_out) {
+  constexpr bool fp64 = sizeof(T) == 8;
+  FwdArgs<T> fa{};
+  fa.wait_cycles = h->wait_limit;
+  fa.withhold = h->withhold;
+  fa.X = X;
+  fa.x_ld = x_ld;
+  fa.row0 = 0;
+  fa.coef = reinterpret_cast<const T *>(h->coef.p);
+  fa.p_out = p_out;
+  fa.n_valid = n_valid;
+  fa.set_begin = reinterpret_cast<const int *>(h->sets.p);
+  fa.set_order = reinterpret_cast<const int *>(h->sord.p);
+  fa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
+  fa.err = h->d_err;
+  fa.nsets = (int)h->set_begin.size() - 1;
+  fa.O = (int)h->O;
+  fa.nt = (int)nt;
+  fa.k_top = (int)(fp64 ? nt + 2 : nt);
+  obs_tiling(h, c, &fa.obs_per_cta, &fa.n_obs_groups);
+  fa.seg_len = c.seg_chunks * fwd_chunk(fp64, c);
+  fa.n_segs = (fa.k_top + fa.seg_len - 1) / fa.seg_len;
+  fa.subs = set_subs(h, fa.n_obs_groups, fa.n_segs);
+  fa.seg_lo = 0;
+  fa.seg_cnt = fa.n_segs;
+  fa.win = c.win;
+  fa.wfl = c.win * (c.acc == 5 ? 2 : 1);
+  return fa;
+}
+
+template <typename T>
+PrepArgs<T> prep_args(const fwh_ctx *h, const T *fields, int64_t nt, T *X, int x_ld) {
+  PrepArgs<T> pa{};
+  pa.fields = fields;
+  pa.place = h->identity ? nullptr : h->d_place;
+  pa.n = h->d_n;
+  pa.X = X;
+  pa.P = (int)h->P;
+  pa.nt = (int)nt;
+  pa.x_ld = x_ld;
+  pa.row0 = 0;
+  pa.ca = h->ca;
+  pa.sa = h->sa;
+  pa.dt = h->dt;
+  return pa;
 }
 
 // Panel-set plan of the handle's configured tile shape, made at set-up
@@ -336,8 +400,8 @@ fwh_status plan_default(fwh_handle h) {
 
 // TMA descriptor of the handle's X buffer, kept on the host (re-encoded when
 // the buffer, its row count or the box changes).
-fwh_status ensure_tmap(fwh_handle h, int box_rows, int x_ld = 0) {
-  const long long rows = (long long)h->P * (x_ld > 0 ? x_ld : h->ntp);
+fwh_status ensure_tmap(fwh_handle h, int box_rows) {
+  const long long rows = (long long)h->P * x_rows(h->nt);
   if (h->tmap_X == h->X.p && h->tmap_rows == rows && h->tmap_box == box_rows) return FWH_OK;
   if (!encode_x_tensor_map(h->tmap_host, h->X.p, (unsigned long long)rows,
                            h->precision == FWH_FP64, box_rows))
@@ -379,8 +443,9 @@ template <typename T>
 fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStream_t s,
                        const T *host_fields = nullptr) {
   const bool fp64 = sizeof(T) == 8;
-  const int cfg = effective_cfg(h, h->ntp);
+  const int cfg = effective_cfg(h, h->nt);
   const FwdConfig c = fwd_config(fp64, cfg);
+  const int x_ld = (int)x_rows(h->nt), n_rb = x_ld / kRowBlk;
   if (c.pipe != 0) {
     fwh_status st0 = ensure_tmap(h, 32 * c.tk);
     if (st0 != FWH_OK) return st0;
@@ -401,42 +466,15 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     CK(h, cudaEventRecord(tev[0], s));
   }
   CK(h, cudaMemsetAsync(d_pout, 0, (size_t)h->O * h->nt * sizeof(double), s));
-  PrepArgs<T> pa{};
-  pa.fields = d_fields;
-  pa.perm = h->identity ? nullptr : h->d_perm;
-  pa.n = h->d_n;
-  pa.X = reinterpret_cast<T *>(h->X.p);
-  pa.P = (int)h->P;
-  pa.nt = (int)h->nt;
-  pa.ntp = h->ntp;
-  pa.ca = h->ca;
-  pa.sa = h->sa;
-  pa.dt = h->dt;
-  pa.x_ld = h->ntp;
-  FwdArgs<T> fa{};
-  fa.tmX = nullptr;
-  fa.wait_cycles = h->wait_limit;
-  fa.withhold = h->withhold;
-  fa.x_ld = h->ntp;
-  fa.X = pa.X;
-  fa.coef = reinterpret_cast<const T *>(h->coef.p);
-  fa.p_out = d_pout;
-  fa.n_valid = reinterpret_cast<const int *>(h->nvalid.p);
-  fa.set_begin = reinterpret_cast<const int *>(h->sets.p);
-  fa.set_order = reinterpret_cast<const int *>(h->sord.p);
-  fa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
-  fa.err = h->d_err;
-  fa.nsets = (int)h->set_begin.size() - 1;
-  fa.O = (int)h->O;
-  fa.ntp = h->ntp;
-  fa.nt = (int)h->nt;
-  obs_tiling(h, c, &fa.obs_per_cta, &fa.n_obs_groups);
-  fa.seg_len = c.seg_chunks * 32 * c.tk;
-  fa.n_segs = (h->ntp + fa.seg_len - 1) / fa.seg_len;
-  fa.seg_lo = 0;
-  fa.seg_cnt = fa.n_segs;
-  fa.win = c.win;
-  fa.wfl = c.win * (c.acc == 5 ? 2 : 1);
+  T *X = reinterpret_cast<T *>(h->X.p);
+  PrepArgs<T> pa = prep_args<T>(h, d_fields, h->nt, X, x_ld);
+  FwdArgs<T> fa = forward_args<T>(h, c, h->nt, X, x_ld, reinterpret_cast<const int *>(h->nvalid.p),
+                                  d_pout);
+  // prep blocks whose rows segment q's chunks read
+  auto blocks_upto = [&](int q) -> int {
+    const int64_t top = std::min<int64_t>(fa.k_top, (int64_t)(q + 1) * fa.seg_len) + 3;
+    return q + 1 >= fa.n_segs ? n_rb : (int)std::min<int64_t>(n_rb, (top + kRowBlk - 1) / kRowBlk);
+  };
   if (host_fields == nullptr && (!h->pipeline || fa.n_segs < 2)) {
     CK(h, launch_prep<T>(pa, s));
     if (tev) CK(h, cudaEventRecord(tev[1], s));
@@ -454,11 +492,10 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     cudaEvent_t *ev_x = h->slab_ev.data(), ev_go = ev_x[fa.n_segs];
     CK(h, cudaEventRecord(ev_go, s));
     CK(h, cudaStreamWaitEvent(h->pstream, ev_go, 0));
-    const int cps = fa.seg_len / 64;  // 64-sample prep chunks per segment
     for (int q = 0; q < fa.n_segs; ++q) {
-      pa.c_lo = q * cps;
-      pa.c_hi = std::min(h->ntp / 64, (q + 1) * cps);
-      CK(h, launch_prep<T>(pa, h->pstream));
+      pa.c_lo = q == 0 ? 0 : pa.c_hi;
+      pa.c_hi = blocks_upto(q);
+      if (pa.c_hi > pa.c_lo) CK(h, launch_prep<T>(pa, h->pstream));
       CK(h, cudaEventRecord(ev_x[q], h->pstream));
     }
     for (int q = 0; q < fa.n_segs; ++q) {
@@ -471,8 +508,8 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
   } else {
     // Three streams: `copy` moves the slabs, `prep` (high priority, so that
     // its blocks get onto SMs between the scatter's) prepares slab q - 1 once
-    // slab q is in (the filters reach 83 frames past a slab), and `s` scatters
-    // each two-chunk time segment once all its rows are prepared.
+    // slab q is in (the filters reach 19 frames past a slab's rows), and `s`
+    // scatters each 250-odd-interval time segment once its rows are prepared.
     // The copy stream first waits for the work already on `s` (the previous
     // call's scatter reads X and its prep the staging buffer), so every later
     // step of this call is ordered after it.
@@ -481,19 +518,19 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     if (!h->copy) CK(h, cudaStreamCreateWithFlags(&h->copy, cudaStreamNonBlocking));
     fwh_status st1 = ensure_pstream(h);
     if (st1 != FWH_OK) return st1;
-    fa.seg_len = 2 * 32 * c.tk;
-    fa.n_segs = (h->ntp + fa.seg_len - 1) / fa.seg_len;
+    fa.seg_len = (c.tk > 4 ? 1 : 2) * fwd_chunk(fp64, c);
+    fa.n_segs = (fa.k_top + fa.seg_len - 1) / fa.seg_len;
     st1 = ensure_events(h, 2 * nslab + 1);
     if (st1 != FWH_OK) return st1;
     cudaEvent_t *ev_in = h->slab_ev.data(), *ev_x = ev_in + nslab, ev_go = ev_in[2 * nslab];
     CK(h, cudaEventRecord(ev_go, s));
     CK(h, cudaStreamWaitEvent(h->copy, ev_go, 0));
-    constexpr int cps = kSlab / 64;  // 64-sample prep chunks per slab
-    static_assert(kSlab % 64 == 0 && 256 % kSlab == 0, "slabs tile the padded record");
+    constexpr int cps = kSlab / kRowBlk;  // prep blocks per slab
+    static_assert(kSlab % kRowBlk == 0, "slabs are whole prep blocks");
     int seg_done = 0;
     // scatter the segments whose rows lie below rows_ready (prepared by slab j)
     auto scatter_upto = [&](int rows_ready, int j) -> fwh_status {
-      const int ready = rows_ready >= h->ntp ? fa.n_segs : rows_ready / fa.seg_len;
+      const int ready = rows_ready >= x_ld ? fa.n_segs : (rows_ready - 3) / fa.seg_len;
       if (ready <= seg_done) return FWH_OK;
       CK(h, cudaStreamWaitEvent(s, ev_x[j], 0));
       if (tev && seg_done == 0) CK(h, cudaEventRecord(tev[1], s));
@@ -515,14 +552,58 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
       const int j = q - 1;  // slab to prepare
       CK(h, cudaStreamWaitEvent(h->pstream, ev_in[std::min(q, nslab - 1)], 0));
       pa.c_lo = j * cps;
-      pa.c_hi = q < nslab ? q * cps : h->ntp / 64;
+      pa.c_hi = q < nslab ? std::min(n_rb, q * cps) : n_rb;
       CK(h, launch_prep<T>(pa, h->pstream));
       CK(h, cudaEventRecord(ev_x[j], h->pstream));
-      const fwh_status st2 = scatter_upto(pa.c_hi * 64, j);
+      const fwh_status st2 = scatter_upto(pa.c_hi * kRowBlk, j);
       if (st2 != FWH_OK) return st2;
     }
   }
   if (tev) CK(h, cudaEventRecord(tev[2], s));
+  return FWH_OK;
+}
+
+template <typename T>
+fwh_status run_backward(fwh_handle h, const T *fields, const double *grad_p, T *grad_fields,
+                        int g_ld, cudaStream_t s) {
+  const int nt = (int)h->nt, xb_ld = (int)xbar_rows(nt);
+  AdjArgs<T> aa{};
+  aa.coef = reinterpret_cast<const T *>(h->coef.p);
+  aa.Gt = reinterpret_cast<T *>(h->G.p);
+  aa.grad_p = grad_p;
+  aa.n_valid = reinterpret_cast<const int *>(h->nvalid.p);
+  aa.Xbar = reinterpret_cast<T *>(h->X.p);
+  aa.P = (int)h->P;
+  aa.O = (int)h->O;
+  aa.nt = nt;
+  aa.g_ld = g_ld;
+  aa.xb_ld = xb_ld;
+  if (sizeof(T) == 4) {
+    // gathers with the forward's plan (panel sets and each record's offsets)
+    const FwdConfig c = fwd_config(false, effective_cfg(h, nt));
+    const fwh_status st = plan(h, c, s);
+    if (st != FWH_OK) return st;
+    aa.set_begin = reinterpret_cast<const int *>(h->sets.p);
+    aa.set_order = reinterpret_cast<const int *>(h->sord.p);
+    aa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
+    aa.nsets = (int)h->set_begin.size() - 1;
+    aa.win = c.win;
+    aa.slot_shift = c.acc == 5 ? 3 : 2;
+  }
+  CK(h, launch_adjoint<T>(aa, s));
+  PrepAdjArgs<T> pa{};
+  pa.fields = fields;
+  pa.place = h->identity ? nullptr : h->d_place;
+  pa.n = h->d_n;
+  pa.Xbar = aa.Xbar;
+  pa.grad_fields = grad_fields;
+  pa.P = aa.P;
+  pa.nt = nt;
+  pa.xb_ld = xb_ld;
+  pa.ca = h->ca;
+  pa.sa = h->sa;
+  pa.dt = h->dt;
+  CK(h, launch_prep_adjoint<T>(pa, s));
   return FWH_OK;
 }
 
@@ -669,7 +750,7 @@ fwh_status fwh_create(fwh_handle *out, int64_t P, const double *centroids,
   // planner order: the caller's order unless a Morton order packs the
   // arrival spreads much better (decided with the default window).
   const FwdConfig c0cfg = fwd_config(precision == FWH_FP64, 0);
-  const int smax = c0cfg.win - 32 * c0cfg.tk - 1;
+  const int smax = fwd_slack(precision == FWH_FP64, c0cfg);
   std::vector<int> sets_id = build_sets(y, P, mach, dt, smax);
   const double avg_id = (double)P / (double)(sets_id.size() - 1);
   std::vector<int> order(P);
@@ -700,6 +781,8 @@ fwh_status fwh_create(fwh_handle *out, int64_t P, const double *centroids,
   h->perm = order;
   h->identity = true;
   for (int64_t p = 0; p < P; ++p) h->identity = h->identity && order[p] == p;
+  std::vector<int> place(P);
+  for (int64_t p = 0; p < P; ++p) place[order[p]] = (int)p;
   h->y.resize(3 * P);
   h->n.resize(3 * P);
   h->dS.resize(P);
@@ -714,7 +797,7 @@ fwh_status fwh_create(fwh_handle *out, int64_t P, const double *centroids,
   if ((e = cudaMalloc(&h->d_y, 3 * P * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_n, 3 * P * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_dS, P * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_perm, P * sizeof(int))) != cudaSuccess ||
+      (e = cudaMalloc(&h->d_place, P * sizeof(int))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_err, sizeof(int))) != cudaSuccess ||
       (e = cudaMemcpy(h->d_y, h->y.data(), 3 * P * sizeof(double), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
@@ -722,10 +805,9 @@ fwh_status fwh_create(fwh_handle *out, int64_t P, const double *centroids,
           cudaSuccess ||
       (e = cudaMemcpy(h->d_dS, h->dS.data(), P * sizeof(double), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
-      (e = cudaMemcpy(h->d_perm, h->perm.data(), P * sizeof(int), cudaMemcpyHostToDevice)) !=
+      (e = cudaMemcpy(h->d_place, place.data(), P * sizeof(int), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
-      (e = cudaMemset(h->d_err, 0, sizeof(int))) != cudaSuccess ||
-      (e = upload_pivots(0)) != cudaSuccess) {
+      (e = cudaMemset(h->d_err, 0, sizeof(int))) != cudaSuccess) {
     fwh_destroy(h);
     return cuda_fail(nullptr, e, "fwh_create device setup");
   }
@@ -768,6 +850,7 @@ fwh_status fwh_set_observers(fwh_handle h, int64_t O, const double *xyz) {
   CK(h, cudaMemcpy(h->d_x, x.data(), 3 * O * sizeof(double), cudaMemcpyHostToDevice));
   const size_t ts = tsize(h->precision);
   CK(h, ensure(h->coef, (size_t)h->P * O * kRec * ts));
+  if (h->precision == FWH_MIXED) CK(h, ensure(h->i0, (size_t)h->P * O * sizeof(int)));
   GeomArgs g{};
   g.y = h->d_y;
   g.n = h->d_n;
@@ -783,9 +866,10 @@ fwh_status fwh_set_observers(fwh_handle h, int64_t O, const double *xyz) {
   g.Rmin = h->d_Rmin;
   CK(h, launch_window(g, 0));
   if (h->precision == FWH_FP64)
-    CK(h, launch_coef<double>(g, reinterpret_cast<double *>(h->coef.p), 0));
+    CK(h, launch_coef<double>(g, reinterpret_cast<double *>(h->coef.p), nullptr, 0));
   else
-    CK(h, launch_coef<float>(g, reinterpret_cast<float *>(h->coef.p), 0));
+    CK(h, launch_coef<float>(g, reinterpret_cast<float *>(h->coef.p),
+                             reinterpret_cast<int *>(h->i0.p), 0));
   h->Rmax.resize(O);
   h->Rmin.resize(O);
   CK(h, cudaMemcpy(h->Rmax.data(), h->d_Rmax, O * sizeof(double), cudaMemcpyDeviceToHost));
@@ -842,9 +926,10 @@ fwh_status fwh_set_observer_extremes(fwh_handle h, const double *r_max, const do
   g.Rmin = h->d_Rmin;
   // records: shifts and spline weights relative to the new t_start (Eq. t_start)
   if (h->precision == FWH_FP64)
-    CK(h, launch_coef<double>(g, reinterpret_cast<double *>(h->coef.p), 0));
+    CK(h, launch_coef<double>(g, reinterpret_cast<double *>(h->coef.p), nullptr, 0));
   else
-    CK(h, launch_coef<float>(g, reinterpret_cast<float *>(h->coef.p), 0));
+    CK(h, launch_coef<float>(g, reinterpret_cast<float *>(h->coef.p),
+                             reinterpret_cast<int *>(h->i0.p), 0));
   h->Rmax = mx;
   h->Rmin = mn;
   h->nt = -1;
@@ -937,45 +1022,14 @@ fwh_status fwh_backward(fwh_handle h, const void *fields, int64_t nt, const doub
     CK(h, ensure(h->stage_grad, fbytes));
     dgf = h->stage_grad.p;
   }
-  CK(h, ensure(h->G, (size_t)h->O * h->ntp * ts));
-  if (h->precision == FWH_FP64) {
-    AdjArgs<double> aa{reinterpret_cast<const double *>(h->coef.p),
-                       reinterpret_cast<double *>(h->G.p), dg,
-                       reinterpret_cast<const int *>(h->nvalid.p),
-                       reinterpret_cast<double *>(h->X.p), (int)h->P, (int)h->O, h->ntp,
-                       (int)nt};
-    CK(h, launch_adjoint<double>(aa, s));
-    PrepAdjArgs<double> pa{reinterpret_cast<const double *>(df),
-                           h->identity ? nullptr : h->d_perm, h->d_n,
-                           reinterpret_cast<const double *>(h->X.p),
-                           reinterpret_cast<double *>(dgf), (int)h->P, (int)nt, h->ntp, 0,
-                           h->ca, h->sa, h->dt};
-    CK(h, launch_prep_adjoint<double>(pa, s));
-  } else {
-    AdjArgs<float> aa{reinterpret_cast<const float *>(h->coef.p),
-                      reinterpret_cast<float *>(h->G.p), dg,
-                      reinterpret_cast<const int *>(h->nvalid.p),
-                      reinterpret_cast<float *>(h->X.p), (int)h->P, (int)h->O, h->ntp, (int)nt};
-    // the set form gathers with the forward's plan (panel sets and each
-    // record's window offset) of a 128-sample-chunk tile shape
-    const FwdConfig c = fwd_config(false, effective_cfg(h, h->ntp));
-    if (32 * c.tk == 128) {
-      st = plan(h, c, s);
-      if (st != FWH_OK) return st;
-      aa.set_begin = reinterpret_cast<const int *>(h->sets.p);
-      aa.set_order = reinterpret_cast<const int *>(h->sord.p);
-      aa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
-      aa.nsets = (int)h->set_begin.size() - 1;
-      aa.win = c.win;
-    }
-    CK(h, launch_adjoint<float>(aa, s));
-    PrepAdjArgs<float> pa{reinterpret_cast<const float *>(df),
-                          h->identity ? nullptr : h->d_perm, h->d_n,
-                          reinterpret_cast<const float *>(h->X.p),
-                          reinterpret_cast<float *>(dgf), (int)h->P, (int)nt, h->ntp, 0,
-                          h->ca, h->sa, h->dt};
-    CK(h, launch_prep_adjoint<float>(pa, s));
-  }
+  const int64_t g_ld = (nt + 255) / 256 * 256;
+  CK(h, ensure(h->G, (size_t)h->O * g_ld * ts));
+  st = h->precision == FWH_FP64
+           ? run_backward<double>(h, reinterpret_cast<const double *>(df), dg,
+                                  reinterpret_cast<double *>(dgf), (int)g_ld, s)
+           : run_backward<float>(h, reinterpret_cast<const float *>(df), dg,
+                                 reinterpret_cast<float *>(dgf), (int)g_ld, s);
+  if (st != FWH_OK) return st;
   if (!dout) {
     CK(h, cudaMemcpyAsync(grad_fields, dgf, fbytes, cudaMemcpyDeviceToHost, s));
     return check_device_flag(h, s);
@@ -1109,9 +1163,9 @@ void fwh_destroy(fwh_handle h) {
   for (auto &kv : h->bplans) release(kv.second.counter);
   for (double *p : {h->d_y, h->d_n, h->d_dS, h->d_x, h->d_Rmax, h->d_Rmin})
     if (p) cudaFree(p);
-  if (h->d_perm) cudaFree(h->d_perm);
+  if (h->d_place) cudaFree(h->d_place);
   if (h->d_err) cudaFree(h->d_err);
-  for (Buf *b : {&h->coef, &h->X, &h->G, &h->nvalid, &h->sets, &h->sord, &h->stage_in,
+  for (Buf *b : {&h->coef, &h->i0, &h->X, &h->G, &h->nvalid, &h->sets, &h->sord, &h->stage_in,
                  &h->stage_out,
                  &h->stage_grad, &h->imax})
     release(*b);
@@ -1155,7 +1209,7 @@ int batch_cfg(int n, const fwh_handle *hs, fwh_handle h0) {
   const bool fp64 = h0->precision == FWH_FP64;
   int cfg = h0->cfg >= 0 ? h0->cfg : default_cfg(h0);
   for (int i = 0; i < n; ++i) {
-    const int ci = effective_cfg(hs[i], hs[i]->ntp);
+    const int ci = effective_cfg(hs[i], hs[i]->nt);
     if (fwd_config(fp64, ci).pipe != fwd_config(fp64, cfg).pipe) cfg = ci;
   }
   return cfg;
@@ -1168,15 +1222,29 @@ template <typename T> const std::vector<BatchParams<T>> &batch_params(const Batc
   return batch_params<T>(const_cast<BatchPlan &>(bp));
 }
 
-// Segments per round of a batched call led by h0 (0: the whole record).
-int batch_round_segs(const fwh_ctx *h0, int seg) {
+// Intervals per time segment of a config.
+int seg_len_of(bool fp64, const FwdConfig &c) { return c.seg_chunks * fwd_chunk(fp64, c); }
+
+// Segments per round of a batched call led by h0 (0: the whole record).  Ring
+// lengths count segments of 512 samples; a segment is that or slightly less.
+int batch_round_segs(const fwh_ctx *h0, const FwdConfig &c) {
+  const int seg = c.seg_chunks * 32 * c.tk;
   return h0->batch_ring > 0 ? (int)std::max<int64_t>(1, h0->batch_ring / seg) : 0;
 }
 
-// X rows per panel of a surface in a batched call: the whole record, or a
-// ring of R time segments when the record spans more than R of them.
+// X rows per panel of a surface in a batched call: the whole record, or the
+// rows of one round (R time segments from a block boundary, and the three rows
+// the last intervals reach past them) when the record spans more.
 int batch_x_ld(const fwh_ctx *h, int seg, int R) {
-  return R > 0 && (h->ntp + seg - 1) / seg > R ? R * seg : h->ntp;
+  const int64_t whole = x_rows(h->nt);
+  return (int)(R > 0 ? std::min<int64_t>(
+                           whole, ((int64_t)R * seg + 2 * kRowBlk + 2) / kRowBlk * kRowBlk)
+                     : whole);
+}
+
+// First record row in X of round r.
+int batch_row0(const BatchPlan &bp, int i, int64_t nt, int r) {
+  return bp.x_ld[i] == x_rows(nt) ? 0 : (int)((int64_t)r * bp.R * bp.seg / kRowBlk * kRowBlk);
 }
 
 template <typename T>
@@ -1185,8 +1253,8 @@ fwh_status batch_build(int n, const fwh_handle *hs, double *const *p_out, fwh_ha
   const bool fp64 = sizeof(T) == 8;
   const int cfg = batch_cfg(n, hs, h0);
   const FwdConfig c = fwd_config(fp64, cfg);
-  const int seg = c.seg_chunks * 32 * c.tk;
-  const int R0 = batch_round_segs(h0, seg);
+  const int seg = seg_len_of(fp64, c);
+  const int R0 = batch_round_segs(h0, c);
   std::vector<FwdArgs<T>> base(n);
   std::vector<TmapBytes> maps(n);
   bp.x_ld.assign(n, 0);
@@ -1197,42 +1265,26 @@ fwh_status batch_build(int n, const fwh_handle *hs, double *const *p_out, fwh_ha
     fwh_status st = plan(h, c, h0->side);
     if (st != FWH_OK) return fail(h0, st, h->err);
     CK(h0, cudaStreamSynchronize(h0->side));
-    bp.nseg[i] = (h->ntp + seg - 1) / seg;
     bp.x_ld[i] = batch_x_ld(h, seg, R0);
-    bp.nq = std::max(bp.nq, bp.nseg[i]);
-    if (h->X.bytes < (size_t)h->P * bp.x_ld[i] * kRec * sizeof(T))
+    if (h->X.bytes < (size_t)h->P * bp.x_ld[i] * kSer * sizeof(T) + kXPad)
       return fail(h0, FWH_ERR_STATE, "series buffer of a batched surface is too small");
     std::memset(maps[i].b, 0, sizeof maps[i].b);
     if (c.pipe != 0 &&
         !encode_x_tensor_map(maps[i].b, h->X.p, (unsigned long long)h->P * bp.x_ld[i], fp64,
                              32 * c.tk))
       return fail(h0, FWH_ERR_CUDA, "cuTensorMapEncodeTiled refused the series layout");
-    FwdArgs<T> &fa = base[i];
-    fa.tmX = nullptr;  // the launch passes the descriptors in its parameter block
-    fa.wait_cycles = h0->wait_limit;
-    fa.withhold = h0->withhold;
-    fa.X = reinterpret_cast<const T *>(h->X.p);
-    fa.x_ld = bp.x_ld[i];
-    fa.coef = reinterpret_cast<const T *>(h->coef.p);
-    fa.p_out = p_out[i];
-    fa.n_valid = reinterpret_cast<const int *>(h->nvalid.p);
-    fa.set_begin = reinterpret_cast<const int *>(h->sets.p);
-    fa.set_order = reinterpret_cast<const int *>(h->sord.p);
-    fa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
-    fa.err = h0->d_err;
-    fa.nsets = (int)h->set_begin.size() - 1;
-    fa.O = (int)h->O;
-    fa.ntp = h->ntp;
-    fa.nt = (int)h->nt;
-    obs_tiling(h, c, &fa.obs_per_cta, &fa.n_obs_groups);
-    fa.seg_len = seg;
-    fa.n_segs = bp.nseg[i];
-    fa.win = c.win;
-    fa.wfl = c.win * (c.acc == 5 ? 2 : 1);
+    base[i] = forward_args<T>(h, c, h->nt, reinterpret_cast<const T *>(h->X.p), bp.x_ld[i],
+                              reinterpret_cast<const int *>(h->nvalid.p), p_out[i]);
+    base[i].wait_cycles = h0->wait_limit;
+    base[i].withhold = h0->withhold;
+    base[i].err = h0->d_err;
+    bp.nseg[i] = base[i].n_segs;
+    bp.nq = std::max(bp.nq, bp.nseg[i]);
   }
   // one scatter launch per round over every surface's items of it
   bp.R = R0 > 0 ? std::min(R0, bp.nq) : bp.nq;
   bp.nr = (bp.nq + bp.R - 1) / bp.R;
+  bp.seg = seg;
   std::vector<BatchParams<T>> &prm = batch_params<T>(bp);
   prm.assign(bp.nr, BatchParams<T>{});
   bp.total.assign(bp.nr, 0);
@@ -1246,14 +1298,14 @@ fwh_status batch_build(int n, const fwh_handle *hs, double *const *p_out, fwh_ha
       const bool has = cnt > 0;
       fa.seg_lo = has ? r * bp.R : 0;
       fa.seg_cnt = has ? cnt : 1;
+      fa.row0 = has ? batch_row0(bp, i, hs[i]->nt, r) : 0;
       P.a[i] = fa;
       P.tm[i] = maps[i];
-      P.prefix[i + 1] = P.prefix[i] + (has ? fa.nsets * fa.n_obs_groups * cnt : 0);
+      P.prefix[i + 1] = P.prefix[i] + (has ? fa.nsets * fa.subs * fa.n_obs_groups * cnt : 0);
     }
     P.total = P.prefix[n];
     bp.total[r] = P.total;
   }
-  bp.seg = seg;
   bp.cfg = cfg;
   bp.form = h0->batch_form;
   CK(h0, ensure(bp.counter, (size_t)bp.nr * sizeof(int)));
@@ -1279,21 +1331,14 @@ fwh_status batch_build(int n, const fwh_handle *hs, double *const *p_out, fwh_ha
 template <typename T>
 fwh_status batch_prep(const fwh_handle h, const void *field, const BatchPlan &bp, int i, int r,
                       fwh_handle h0, cudaStream_t s) {
-  const int cps = bp.seg / 64;
-  PrepArgs<T> pa{};
-  pa.fields = reinterpret_cast<const T *>(field);
-  pa.perm = h->identity ? nullptr : h->d_perm;
-  pa.n = h->d_n;
-  pa.X = reinterpret_cast<T *>(h->X.p);
-  pa.P = (int)h->P;
-  pa.nt = (int)h->nt;
-  pa.ntp = h->ntp;
-  pa.x_ld = bp.x_ld[i];
-  pa.ca = h->ca;
-  pa.sa = h->sa;
-  pa.dt = h->dt;
-  pa.c_lo = r * bp.R * cps;
-  pa.c_hi = std::min(h->ntp / 64, (r + 1) * bp.R * cps);
+  PrepArgs<T> pa = prep_args<T>(h, reinterpret_cast<const T *>(field), h->nt,
+                                reinterpret_cast<T *>(h->X.p), bp.x_ld[i]);
+  // the blocks of round r's rows (consecutive rounds of a ring share some)
+  const int64_t n_rb = x_rows(h->nt) / kRowBlk, top = ((int64_t)r + 1) * bp.R * bp.seg + 3;
+  pa.row0 = batch_row0(bp, i, h->nt, r);
+  pa.c_lo = pa.row0 / kRowBlk;
+  pa.c_hi = (int)(pa.x_ld == x_rows(h->nt) ? n_rb : std::min(n_rb, (top + kRowBlk - 1) / kRowBlk));
+  if (pa.x_ld == x_rows(h->nt) && r > 0) return FWH_OK;  // prepared whole in round 0
   CK(h0, launch_prep<T>(pa, s));
   return FWH_OK;
 }
@@ -1337,7 +1382,7 @@ fwh_status batch_enqueue(int n, const fwh_handle *hs, const void *const *fields,
   std::vector<int> order(n);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    return hs[x]->P * (int64_t)hs[x]->ntp < hs[y]->P * (int64_t)hs[y]->ntp;
+    return hs[x]->P * hs[x]->nt < hs[y]->P * hs[y]->nt;
   });
   cudaStream_t lane[2] = {s, h0->bstream};
   int k = 0;
@@ -1393,11 +1438,11 @@ extern "C" fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void 
   }
   {  // series buffers (the whole record, or a ring of time segments) before the key
     const FwdConfig c = fwd_config(h0->precision == FWH_FP64, batch_cfg(n, hs, h0));
-    const int seg = c.seg_chunks * 32 * c.tk;
-    const int R = batch_round_segs(h0, seg);
+    const int seg = seg_len_of(h0->precision == FWH_FP64, c);
+    const int R = batch_round_segs(h0, c);
     for (int i = 0; i < n; ++i)
-      CK(h0, ensure(hs[i]->X, (size_t)hs[i]->P * batch_x_ld(hs[i], seg, R) * kRec *
-                                  tsize(h0->precision)));
+      CK(h0, ensure(hs[i]->X, (size_t)hs[i]->P * batch_x_ld(hs[i], seg, R) * kSer *
+                                      tsize(h0->precision) + kXPad));
   }
   std::vector<uintptr_t> key;
   for (int i = 0; i < n; ++i) {
@@ -1475,17 +1520,20 @@ template <typename T>
 fwh_status forward_into_scratch_t(fwh_handle h, const T *d_fields, int64_t nt, double *d_pout,
                                   cudaStream_t s, unsigned char *scratch, size_t cap) {
   const bool fp64 = sizeof(T) == 8;
-  const int ntp = (int)((nt + 255) / 256 * 256);  // same padding as prepare_nt
-  const int cfg = effective_cfg(h, ntp);
+  const int cfg = effective_cfg(h, nt);
   const FwdConfig c = fwd_config(fp64, cfg);
+  const int x_ld = (int)x_rows(nt);
   const size_t off_x = ((size_t)h->O * sizeof(int) + 1023) / 1024 * 1024;
-  const size_t need = off_x + (size_t)h->P * ntp * kRec * sizeof(T);
+  // the stated limit (16 values per panel and padded step), and what is used
+  const size_t need = std::max(off_x + (size_t)h->P * ((nt + 255) / 256 * 256) * 16 * sizeof(T),
+                               off_x + (size_t)h->P * x_ld * kSer * sizeof(T) + kXPad);
   if (need > cap)
     return fail(h, FWH_ERR_ARG,
                 "problem needs " + std::to_string(need) + " bytes of scratch (panels x nt rounded "
                 "up to 256 x 16 values + windows); the static scratch holds " +
                     std::to_string(cap) + " bytes");
-  if (h->plan_win != c.win || h->plan_ch != 32 * c.tk || h->plan_sb != (c.acc == 5 ? 8 : 4))
+  if (h->plan_win != c.win || h->plan_slack != fwd_slack(fp64, c) ||
+      h->plan_sb != (c.acc == 5 ? 8 : 4))
     return fail(h, FWH_ERR_STATE,
                 "the handle's panel-set plan belongs to another tile shape; call "
                 "fwh_set_tile_config (which plans without a forward pass) first");
@@ -1495,46 +1543,11 @@ fwh_status forward_into_scratch_t(fwh_handle h, const T *d_fields, int64_t nt, d
   CK(h, launch_nvalid(h->d_Rmax, h->d_Rmin, (int)h->O, h->mach, h->dt, (int)nt, d_nv, s));
   alignas(64) unsigned char desc[128];
   if (c.pipe != 0 &&
-      !encode_x_tensor_map(desc, d_X, (unsigned long long)h->P * ntp, fp64, 32 * c.tk))
+      !encode_x_tensor_map(desc, d_X, (unsigned long long)h->P * x_ld, fp64, 32 * c.tk))
     return fail(h, FWH_ERR_CUDA, "cuTensorMapEncodeTiled refused the series layout");
   CK(h, cudaMemsetAsync(d_pout, 0, (size_t)h->O * nt * sizeof(double), s));
-  PrepArgs<T> pa{};
-  pa.fields = d_fields;
-  pa.perm = h->identity ? nullptr : h->d_perm;
-  pa.n = h->d_n;
-  pa.X = d_X;
-  pa.P = (int)h->P;
-  pa.nt = (int)nt;
-  pa.ntp = ntp;
-  pa.x_ld = ntp;
-  pa.ca = h->ca;
-  pa.sa = h->sa;
-  pa.dt = h->dt;
-  CK(h, launch_prep<T>(pa, s));
-  FwdArgs<T> fa{};
-  fa.tmX = nullptr;
-  fa.wait_cycles = h->wait_limit;
-  fa.withhold = h->withhold;
-  fa.x_ld = ntp;
-  fa.X = d_X;
-  fa.coef = reinterpret_cast<const T *>(h->coef.p);
-  fa.p_out = d_pout;
-  fa.n_valid = d_nv;
-  fa.set_begin = reinterpret_cast<const int *>(h->sets.p);
-  fa.set_order = reinterpret_cast<const int *>(h->sord.p);
-  fa.i0max_tab = reinterpret_cast<const int *>(h->imax.p);
-  fa.err = h->d_err;
-  fa.nsets = (int)h->set_begin.size() - 1;
-  fa.O = (int)h->O;
-  fa.ntp = ntp;
-  fa.nt = (int)nt;
-  obs_tiling(h, c, &fa.obs_per_cta, &fa.n_obs_groups);
-  fa.seg_len = c.seg_chunks * 32 * c.tk;
-  fa.n_segs = (ntp + fa.seg_len - 1) / fa.seg_len;
-  fa.seg_lo = 0;
-  fa.seg_cnt = fa.n_segs;
-  fa.win = c.win;
-  fa.wfl = c.win * (c.acc == 5 ? 2 : 1);
+  CK(h, launch_prep<T>(prep_args<T>(h, d_fields, nt, d_X, x_ld), s));
+  const FwdArgs<T> fa = forward_args<T>(h, c, nt, d_X, x_ld, d_nv, d_pout);
   CK(h, launch_forward<T>(fa, c.pipe ? desc : nullptr, cfg, s));
   return defer_check(h, s);
 }

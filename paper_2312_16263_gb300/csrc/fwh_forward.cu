@@ -2,48 +2,54 @@
 // ("compute Noise" + "interp pressure signal" + surface integration,
 // Sec. III B/C; integrand of Eqs. pT_WT_nd + pL_WT_nd).
 //
-// For panel p, observer o and source sample k, with the observer-independent
-// row X[p][k] (8 series F and their spline moments M) and the per-(p, o)
-// record (coefficients c, shift i0, weights a, b, cc, dd):
-//   g = c . F[k],   m = c . M[k]                     (source pressure, moment)
-//   bin k - i0     += a g + cc m                     (spline, left node)
-//   bin k - i0 - 1 += b g + dd m                     (spline, right node)
-// which is the natural-spline value at tau = t_j - M0 R for every observer
-// bin j (Eq. tau2), summed over panels.  20 FMA per (panel, sample, observer).
+// For panel p, observer o and the observer-independent rows X[p][r] (B-spline
+// coefficients of the 8 series, row r = sample r - 1), with the per-(p, o)
+// record (coefficients c, weights w0..w3, shift i0):
+//   G[r] = c . X[r]
+//   bin k - i0 += w0 G[k] + w1 G[k+1] + w2 G[k+2] + w3 G[k+3]
+// for every spline interval k = 0 .. nt - 1, which is the natural-spline value
+// at tau = t_j - M0 R for every observer bin j (Eq. tau2), summed over panels:
+// 12 multiply-adds per (panel, sample, observer).
 //
-// Work item = (panel set, observer group, time segment).  A CTA holds NW
-// compute warps; warp w owns observers o_begin + w + NW m (m < obs_per_warp)
-// of the group and keeps, per observer, a window of `win` bins in shared
-// memory.  Lanes map to source samples (k = k0 + lane + 32 j, j < TK), so each
-// X row is loaded once per warp and reused for all of the warp's observers,
-// the coefficient record is a warp-uniform broadcast, and the window updates
-// are conflict-free (consecutive lanes, consecutive bins).  The per-(p, o)
-// shift only moves the window offset, never the lane pattern.  After each
-// chunk of 32 TK samples the oldest 32 TK bins of every window are complete
-// for this panel set: they are flushed to p_out with FP64 atomics (one per bin
-// per panel set, not per panel) and the window slides.
+// Work item = (panel set or a part of it, observer group, time segment).  A
+// CTA holds NW compute warps; warp w owns observers o_begin + w + NW m (m <
+// obs_per_warp) of the group and keeps, per observer, a window of `win` bins
+// in shared memory.  Lanes map to rows, so each X row is loaded once per warp
+// and reused for all of the warp's observers, the record is a warp-uniform
+// broadcast, and the window updates are conflict-free.  The per-(p, o) shift
+// only moves the window offset, never the lane pattern.  After each chunk the
+// oldest bins of every window are complete for this item: they are flushed to
+// p_out with FP64 atomics (one per bin per item, not per panel) and the
+// window slides.
+//
+// FP32 gathers: a lane holds four consecutive rows of each 128-row block,
+// forms G of its rows, takes the next three values from the lane above (the
+// last lane of a block from lane 0 of the next block) and adds four complete
+// bin values to the window, one read-modify-write per sample.  FP64 scatters:
+// a lane holds rows 32 apart and adds each G to its four bins in turn (the
+// FP64 pipe, not the window traffic, bounds that form).
 //
 // Two ways to feed the compute warps:
 //  * direct: every warp loads its X rows and coefficient records from global
 //    memory (L1/L2) itself;
 //  * TMA pipeline: one producer warp streams, per (chunk, panel) step, the X
-//    rows (a 2D tensor-map load, 128B swizzled so the per-lane row reads are
-//    bank-conflict-free) and the group's coefficient records (a 1D bulk
-//    copy) into a ring of shared-memory stages; full/empty mbarriers hand the
-//    stages over.  Every wait is bounded by a clock limit: on expiry the
-//    kernel raises kErrTimeout, stops issuing copies, waits (bounded) for the
-//    copies already in flight and leaves.
+//    rows (a 2D tensor-map load of 128-byte lines, 128B swizzled so the
+//    per-lane reads are bank-conflict-free) and the group's coefficient
+//    records (a 1D bulk copy) into a ring of shared-memory stages; full/empty
+//    mbarriers hand the stages over.  Every wait is bounded by a clock limit:
+//    on expiry the kernel raises kErrTimeout, stops issuing copies, waits
+//    (bounded) for the copies already in flight and leaves.
 //
 // Window bound: a panel set's shifts for one observer span S = i0max - i0min;
-// slots touched in a chunk are [0, CH + S], so S <= win - CH - 1 is required.
-// The host planner bounds S from the set's extent; the plan kernel records,
-// per (set, observer), i0max and, per (panel, observer) record, the window
-// offset i0max - i0 clamped to [0, win - CH - 1], raising kErrWindow if the
-// bound is exceeded; the hot loop adds that offset and can never leave the
-// window.
+// fwd_slack() is the largest S whose slots stay inside the window.  The host
+// planner bounds S from the set's extent; the plan kernel records, per (set,
+// observer), i0max and, per (panel, observer) record, the window offset
+// i0max - i0 clamped to [0, slack], raising kErrWindow if the bound is
+// exceeded; the hot loop adds that offset and can never leave the window.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 
@@ -57,79 +63,40 @@ constexpr int kMaxObsPerWarp = 16;
 constexpr int kMaxObsPerWarpF32 = 9;  // the FP32 consumer unrolls its observer loop to this
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 
-template <typename T> struct Vec;
-template <> struct Vec<float> {
-  using V = float4;
-  static constexpr int per = 4;
-};
-template <> struct Vec<double> {
-  using V = double2;
-  static constexpr int per = 2;
-};
-
-template <typename T> __device__ __forceinline__ int rec_i0_of(T v);
-template <> __device__ __forceinline__ int rec_i0_of<float>(float v) {
-  return __float_as_int(v);
-}
-template <> __device__ __forceinline__ int rec_i0_of<double>(double v) { return (int)v; }
-
-template <typename T>
-__device__ __forceinline__ void load16(const T *src, T (&dst)[kRec]) {
-  using V = typename Vec<T>::V;
-  constexpr int per = Vec<T>::per;
-  const V *s = reinterpret_cast<const V *>(src);
+// 16-byte loads of N doubles.
+template <int N>
+__device__ __forceinline__ void ldg_f64(const double *src, double (&dst)[N]) {
+  const double2 *s = reinterpret_cast<const double2 *>(src);
 #pragma unroll
-  for (int q = 0; q < kRec / per; ++q) {
-    V v = __ldg(s + q);
-    if constexpr (per == 4) {
-      dst[4 * q] = v.x; dst[4 * q + 1] = v.y; dst[4 * q + 2] = v.z; dst[4 * q + 3] = v.w;
-    } else {
-      dst[2 * q] = v.x; dst[2 * q + 1] = v.y;
-    }
+  for (int q = 0; q < N / 2; ++q) {
+    const double2 v = __ldg(s + q);
+    dst[2 * q] = v.x;
+    dst[2 * q + 1] = v.y;
+  }
+}
+template <int N>
+__device__ __forceinline__ void lds_f64(const double *src, double (&dst)[N]) {
+  const double2 *s = reinterpret_cast<const double2 *>(src);
+#pragma unroll
+  for (int q = 0; q < N / 2; ++q) {
+    const double2 v = s[q];
+    dst[2 * q] = v.x;
+    dst[2 * q + 1] = v.y;
   }
 }
 
-// Shared-memory broadcast read of a 16-value record.
-template <typename T>
-__device__ __forceinline__ void lds16(const T *src, T (&dst)[kRec]) {
-  using V = typename Vec<T>::V;
-  constexpr int per = Vec<T>::per;
-  const V *s = reinterpret_cast<const V *>(src);
+// One FP64 X row (64 bytes, two per 128-byte line) from a TMA stage written
+// with SWIZZLE_128B, which XORs the 16-byte chunk index (address bits 4..6)
+// with address bits 7..9: chunk q of row r is chunk (((r & 1) << 2) | q) ^
+// ((r >> 1) & 7) of line r >> 1, so 8 consecutive lanes hit 8 distinct
+// 16-byte bank groups.
+__device__ __forceinline__ void lds_row_f64(const unsigned char *stg, int r, double (&dst)[kSer]) {
 #pragma unroll
-  for (int q = 0; q < kRec / per; ++q) {
-    V v = s[q];
-    if constexpr (per == 4) {
-      dst[4 * q] = v.x; dst[4 * q + 1] = v.y; dst[4 * q + 2] = v.z; dst[4 * q + 3] = v.w;
-    } else {
-      dst[2 * q] = v.x; dst[2 * q + 1] = v.y;
-    }
-  }
-}
-
-// One X row from a TMA stage written with SWIZZLE_128B.  The swizzle XORs the
-// 16-byte chunk index (address bits 4..6) with address bits 7..9.  FP64 rows
-// are 128 B, so chunk q of row r sits at chunk q ^ (r & 7) of that row; FP32
-// rows are 64 B, two per 128-byte line, so chunk q of row r is chunk
-// (((r & 1) << 2) | q) ^ ((r >> 1) & 7) of line r >> 1.  Consecutive rows read
-// by 8 consecutive lanes then hit 8 distinct 16-byte bank groups.
-template <typename T>
-__device__ __forceinline__ void lds_row_swz(const unsigned char *stg, int r, T (&dst)[kRec]) {
-  using V = typename Vec<T>::V;
-  constexpr int per = Vec<T>::per;
-#pragma unroll
-  for (int q = 0; q < kRec / per; ++q) {
-    const unsigned char *addr;
-    if constexpr (sizeof(T) == 4) {
-      addr = stg + (size_t)(r >> 1) * 128 + (((((r & 1) << 2) | q) ^ ((r >> 1) & 7)) << 4);
-    } else {
-      addr = stg + (size_t)r * 128 + ((q ^ (r & 7)) << 4);
-    }
-    const V v = *reinterpret_cast<const V *>(addr);
-    if constexpr (per == 4) {
-      dst[4 * q] = v.x; dst[4 * q + 1] = v.y; dst[4 * q + 2] = v.z; dst[4 * q + 3] = v.w;
-    } else {
-      dst[2 * q] = v.x; dst[2 * q + 1] = v.y;
-    }
+  for (int q = 0; q < kSer / 2; ++q) {
+    const double2 v = *reinterpret_cast<const double2 *>(
+        stg + (size_t)(r >> 1) * 128 + (((((r & 1) << 2) | q) ^ ((r >> 1) & 7)) << 4));
+    dst[2 * q] = v.x;
+    dst[2 * q + 1] = v.y;
   }
 }
 
@@ -237,20 +204,21 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned b
 
 __device__ __forceinline__ void atomic_add_f64(double *addr, double v) { atomicAdd(addr, v); }
 
-template <typename T> __device__ __forceinline__ T int_as_rec(int v);
-template <> __device__ __forceinline__ float int_as_rec<float>(int v) { return __int_as_float(v); }
-template <> __device__ __forceinline__ double int_as_rec<double>(int v) { return (double)v; }
-
 template <typename T>
-__global__ void __launch_bounds__(128) k_plan(T *coef, const int *set_begin, int O, int slack,
-                                              int half_bytes, int slot_bytes, int *i0max_tab,
-                                              int *err) {
+__global__ void __launch_bounds__(128) k_plan(T *coef, const int *i0_tab, const int *set_begin,
+                                              int O, int slack, int win, int slot_bytes,
+                                              int *i0max_tab, int *err) {
   const int sidx = blockIdx.x;
   const int pb = set_begin[sidx], pe = set_begin[sidx + 1];
   for (int o = threadIdx.x; o < O; o += blockDim.x) {
+    auto i0_at = [&](int p) -> int {
+      const size_t e = (size_t)p * O + o;
+      if constexpr (sizeof(T) == 4) return i0_tab[e];
+      return (int)coef[e * kRec + slot::i0];
+    };
     int lo = 0x7fffffff, hi = -0x7fffffff;
     for (int p = pb; p < pe; ++p) {
-      const int i0 = rec_i0_of<T>(coef[((size_t)p * O + o) * kRec + slot::i0]);
+      const int i0 = i0_at(p);
       lo = min(lo, i0);
       hi = max(hi, i0);
     }
@@ -258,12 +226,17 @@ __global__ void __launch_bounds__(128) k_plan(T *coef, const int *set_begin, int
     i0max_tab[(size_t)sidx * O + o] = hi;
     for (int p = pb; p < pe; ++p) {
       T *rec = coef + ((size_t)p * O + o) * kRec;
-      const int off = min(hi - rec_i0_of<T>(rec[slot::i0]), slack);
-      rec[slot::off] = int_as_rec<T>(off);
-      if (sizeof(T) == 4) {  // split window: slot x in half x & 1, word x >> 1
-        const int x = off + 1, r = x & 1, q = x >> 1;
-        rec[slot::w0] = int_as_rec<T>(r * half_bytes + slot_bytes * q);
-        rec[slot::w1] = int_as_rec<T>((1 - r) * half_bytes + slot_bytes * (q + r));
+      const int off = min(hi - i0_at(p), slack);
+      if constexpr (sizeof(T) == 4) {  // quarter-split window: slot x in quarter x & 3
+        const int H = win / 4;
+        int4 a;
+        a.x = ((off & 3) * H + (off >> 2)) * slot_bytes;
+        a.y = (((off + 1) & 3) * H + ((off + 1) >> 2)) * slot_bytes;
+        a.z = (((off + 2) & 3) * H + ((off + 2) >> 2)) * slot_bytes;
+        a.w = (((off + 3) & 3) * H + ((off + 3) >> 2)) * slot_bytes;
+        *reinterpret_cast<int4 *>(rec + slot::q0) = a;
+      } else {
+        rec[slot::off] = (T)off;
       }
     }
   }
@@ -276,24 +249,28 @@ struct Item {
   __device__ __forceinline__ Item(const FwdArgs<T> &a, int item, int w) {
     const int ng = a.n_obs_groups;
     // observer group fastest (groups share the set's X rows in L2), then the
-    // time segments of one set, then the sets, largest first so that the
-    // last CTAs to start are the shortest
+    // time segments of one set, then its parts, then the sets, largest first
+    // so that the last CTAs to start are the shortest
     const int g = item % ng;
     const int rest = item / ng;
     const int q = a.seg_lo + rest % a.seg_cnt;
     const int r2 = rest / a.seg_cnt;
-    sidx = a.set_order ? a.set_order[r2] : r2;
-    p_begin = a.set_begin[sidx];
-    p_end = a.set_begin[sidx + 1];
+    const int sub = r2 % a.subs, r3 = r2 / a.subs;
+    sidx = a.set_order ? a.set_order[r3] : r3;
+    const int pb = a.set_begin[sidx], np = a.set_begin[sidx + 1] - pb;
+    p_begin = pb + np * sub / a.subs;
+    p_end = pb + np * (sub + 1) / a.subs;
     opw = a.obs_per_cta / NW;
     o_begin = g * a.obs_per_cta;
     o_end = min(a.O, o_begin + a.obs_per_cta);
     k_begin = q * a.seg_len;
-    k_end = min(a.ntp, k_begin + a.seg_len);
+    k_end = min(a.k_top, k_begin + a.seg_len);
     nobs = 0;
     for (int m = 0; m < opw; ++m)
       if (o_begin + w + NW * m < o_end) nobs = m + 1;
   }
+  // chunks of `ch` rows or intervals
+  __device__ __forceinline__ int chunks(int ch) const { return (k_end - k_begin + ch - 1) / ch; }
 };
 
 // Per-observer largest shift of the panel set (from the plan); zero windows.
@@ -307,118 +284,112 @@ __device__ __forceinline__ void item_prologue(const FwdArgs<T> &a, const Item<T,
   __syncwarp();
 }
 
-// Signal, moment and the two spline-node updates of one (panel, observer),
-// one sample per lane per block: read-modify-write of the window; the two
-// node updates of neighbouring lanes meet in one bin, so they are separated
-// by __syncwarp.
-template <typename T, int TK>
-__device__ __forceinline__ void accumulate(const T (&x)[TK][kRec], const T (&c)[kRec], T *wm) {
-  T gv[TK], mv[TK];
+// FP64, one (panel, observer): lane rows k0 + lane + 32 j (j < nj).  Row r
+// enters the bins of intervals r - 3 .. r with weights w3 .. w0; wm is the
+// window slot of interval r - 3 of the lane's first row.  Neighbouring lanes'
+// updates meet in one bin, so the four steps are separated by __syncwarp.
+template <int TK>
+__device__ __forceinline__ void accumulate(const double (&x)[TK][kSer], const double (&c)[12],
+                                           double *wm, int nj) {
+  double g[TK];
 #pragma unroll
   for (int j = 0; j < TK; ++j) {
-    T g0 = c[0] * x[j][0], m0 = c[0] * x[j][8];
+    if (j >= nj) break;
+    double v = c[0] * x[j][0];
 #pragma unroll
-    for (int s = 1; s < 8; ++s) {
-      g0 = fma(c[s], x[j][s], g0);
-      m0 = fma(c[s], x[j][8 + s], m0);
+    for (int s = 1; s < kSer; ++s) v = fma(c[s], x[j][s], v);
+    g[j] = v;
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+#pragma unroll
+    for (int j = 0; j < TK; ++j) {
+      if (j >= nj) break;
+      wm[32 * j + t] = fma(c[slot::w + 3 - t], g[j], wm[32 * j + t]);
     }
-    gv[j] = g0;
-    mv[j] = m0;
+    __syncwarp();
   }
-#pragma unroll
-  for (int j = 0; j < TK; ++j) {
-    T v = wm[32 * j];
-    v = fma(c[8], gv[j], v);
-    v = fma(c[10], mv[j], v);
-    wm[32 * j] = v;
-  }
-  __syncwarp();
-#pragma unroll
-  for (int j = 0; j < TK; ++j) {
-    T v = wm[32 * j - 1];
-    v = fma(c[9], gv[j], v);
-    v = fma(c[11], mv[j], v);
-    wm[32 * j - 1] = v;
-  }
-  __syncwarp();
 }
 
-// Flush the first CH (complete) bins of every window to p_out and slide.
-template <typename T, int CH, int NW>
-__device__ __forceinline__ void flush_slide(const FwdArgs<T> &a, const Item<T, NW> &it, int w,
-                                            T *wwin, const int *s_i0max, int k0) {
+// FP64: flush the first CH (complete) bins of every window to p_out and slide.
+// Window slot 0 is the bin of interval k0 - 3 at the set's largest shift.
+template <int CH, int NW>
+__device__ __forceinline__ void flush_slide(const FwdArgs<double> &a, const Item<double, NW> &it,
+                                            int w, double *wwin, const int *s_i0max, int k0) {
   const int lane = threadIdx.x & 31;
   const int win = a.win;
   for (int m = 0; m < it.nobs; ++m) {
     const int o = it.o_begin + w + NW * m;
-    T *wm = wwin + (size_t)m * win;
-    const int wbase = k0 - s_i0max[m] - 1;
+    double *wm = wwin + (size_t)m * win;
+    const int wbase = k0 - s_i0max[m] - 3;
     const int nvalid = a.n_valid[o];
     double *po = a.p_out + (size_t)o * a.nt;
     for (int t = lane; t < CH; t += 32) {
       const int bin = wbase + t;
-      const T v = wm[t];
-      if (bin >= 0 && bin < nvalid && v != T(0)) atomic_add_f64(po + bin, (double)v);
+      const double v = wm[t];
+      if (bin >= 0 && bin < nvalid && v != 0.0) atomic_add_f64(po + bin, v);
     }
     __syncwarp();
     for (int t = lane; t < win - CH; t += 32) wm[t] = wm[CH + t];  // win - CH <= CH
     __syncwarp();
-    for (int t = win - CH + lane; t < win; t += 32) wm[t] = T(0);
+    for (int t = win - CH + lane; t < win; t += 32) wm[t] = 0.0;
     __syncwarp();
   }
 }
 
-// Segment end: the remaining window holds partial bins of the next segment.
-template <typename T, int CH, int NW>
-__device__ __forceinline__ void flush_tail(const FwdArgs<T> &a, const Item<T, NW> &it, int w,
-                                           T *wwin, const int *s_i0max) {
+// Segment end (k0: the row after the last chunk): the remaining window holds
+// partial bins of the next segment.
+template <int CH, int NW>
+__device__ __forceinline__ void flush_tail(const FwdArgs<double> &a, const Item<double, NW> &it,
+                                           int w, double *wwin, const int *s_i0max, int k0) {
   const int lane = threadIdx.x & 31;
   const int win = a.win;
   for (int m = 0; m < it.nobs; ++m) {
     const int o = it.o_begin + w + NW * m;
-    T *wm = wwin + (size_t)m * win;
-    const int wbase = it.k_end - s_i0max[m] - 1;
+    double *wm = wwin + (size_t)m * win;
+    const int wbase = k0 - s_i0max[m] - 3;
     const int nvalid = a.n_valid[o];
     double *po = a.p_out + (size_t)o * a.nt;
     for (int t = lane; t < win - CH; t += 32) {
       const int bin = wbase + t;
-      const T v = wm[t];
-      if (bin >= 0 && bin < nvalid && v != T(0)) atomic_add_f64(po + bin, (double)v);
+      const double v = wm[t];
+      if (bin >= 0 && bin < nvalid && v != 0.0) atomic_add_f64(po + bin, v);
     }
   }
   __syncwarp();
 }
 
-// ---- direct-load pipeline --------------------------------------------------
-template <typename T, int TK, int NW>
-__device__ __forceinline__ void process_item_direct(const FwdArgs<T> &a, int item, T *smem,
-                                                    int *st) {
-  static_assert(sizeof(T) == 8, "scalar consumers read the 16-value FP64 record");
+// ---- direct-load pipeline (FP64) -------------------------------------------
+template <int TK, int NW>
+__device__ __forceinline__ void process_item_direct(const FwdArgs<double> &a, int item,
+                                                    double *smem, int *st) {
   constexpr int CH = 32 * TK;
   const int lane = threadIdx.x & 31;
   const int w = threadIdx.x >> 5;
-  const Item<T, NW> it(a, item, w);
-  T *wwin = smem + (size_t)w * it.opw * a.wfl;
+  const Item<double, NW> it(a, item, w);
+  double *wwin = smem + (size_t)w * it.opw * a.wfl;
   int *s_i0max = st + w * kMaxObsPerWarp;
-  item_prologue<T, NW>(a, it, w, wwin, s_i0max);
-  for (int k0 = it.k_begin; k0 < it.k_end; k0 += CH) {
+  item_prologue<double, NW>(a, it, w, wwin, s_i0max);
+  int k0 = it.k_begin;
+  for (; k0 < it.k_end; k0 += CH) {
+    const int nj = min(TK, (it.k_end - k0 + 31) / 32);
     for (int p = it.p_begin; p < it.p_end; ++p) {
-      T x[TK][kRec];
-      const T *Xp = a.X + ((size_t)p * a.x_ld + k0 % a.x_ld + lane) * kRec;
+      double x[TK][kSer];
+      const double *Xp = a.X + ((size_t)p * a.x_ld + (k0 - a.row0) + lane) * kSer;
 #pragma unroll
-      for (int j = 0; j < TK; ++j) load16<T>(Xp + (size_t)j * 32 * kRec, x[j]);
-      const T *rec0 = a.coef + (size_t)p * a.O * kRec;
+      for (int j = 0; j < TK; ++j)
+        if (j < nj) ldg_f64(Xp + (size_t)j * 32 * kSer, x[j]);
+      const double *rec0 = a.coef + (size_t)p * a.O * kRec;
       for (int m = 0; m < it.nobs; ++m) {
-        const int o = it.o_begin + w + NW * m;
-        T c[kRec];
-        load16<T>(rec0 + (size_t)o * kRec, c);
-        T *wm = wwin + (m * a.win + 1 + lane + rec_i0_of<T>(c[slot::off]));
-        accumulate<T, TK>(x, c, wm);
+        const double *rec = rec0 + (size_t)(it.o_begin + w + NW * m) * kRec;
+        double c[12];
+        ldg_f64(rec, c);
+        accumulate<TK>(x, c, wwin + (m * a.win + lane + (int)__ldg(rec + slot::off)), nj);
       }
     }
-    flush_slide<T, CH, NW>(a, it, w, wwin, s_i0max, k0);
+    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0);
   }
-  flush_tail<T, CH, NW>(a, it, w, wwin, s_i0max);
+  flush_tail<CH, NW>(a, it, w, wwin, s_i0max, k0);
 }
 
 // ---- TMA pipeline ------------------------------------------------------------
@@ -428,35 +399,18 @@ struct PipeState {
   unsigned stage_bytes, x_bytes;
   int nst;
   volatile int *abort;
-  int *released;  // in-line producer: per-stage count of warps done with it
-  int *issued;    // in-line producer: steps issued so far (for the drain)
   const void *tmap;  // tensor map of the X rows being streamed
   int *err;          // device error flag and the bound of each wait (SM clocks):
   long long wait_cycles;  // the same for every surface of a launch
 };
 
-// Threads per CTA: compute warps, plus the producer warp of the TMA pipeline
-// (pipe 1); the in-line producer (pipe 2) has none.
+// Threads per CTA: compute warps, plus the producer warp of the TMA pipeline.
 template <int NW, int PIPE>
 constexpr int cta_threads() { return (NW + (PIPE == 1 ? 1 : 0)) * 32; }
 
-// In-line producer: load step j (in-item index) of `it` into stage `slot`.
-// Step j covers panel p_begin + j % np and chunk k_begin + (j / np) CH.
-template <typename T, int TK, int NW>
-__device__ __forceinline__ void issue_step(const FwdArgs<T> &a, const Item<T, NW> &it,
-                                           const PipeState &ps, int j, unsigned slot) {
-  constexpr int CH = 32 * TK;
-  const int np = it.p_end - it.p_begin;
-  const int p = it.p_begin + j % np;
-  const int k0 = it.k_begin + (j / np) * CH;
-  const unsigned cbytes = (unsigned)((it.o_end - it.o_begin) * kRec * sizeof(T));
-  uint64_t *bar = &ps.full[slot];
-  unsigned char *dst = ps.stage0 + (size_t)slot * ps.stage_bytes;
-  mbar_expect_tx(bar, ps.x_bytes + cbytes);
-  const int row = p * a.x_ld + k0 % a.x_ld;  // tensor rows are 128 bytes
-  tma_load_2d(dst, ps.tmap, 0, sizeof(T) == 4 ? row >> 1 : row, bar);
-  bulk_load(dst + ps.x_bytes, a.coef + ((size_t)p * a.O + it.o_begin) * kRec, cbytes, bar);
-}
+// Rows or intervals a chunk completes.
+template <typename T, int TK>
+constexpr int chunk_of() { return 32 * TK - (sizeof(T) == 4 ? 4 : 0); }
 
 // Producer (one lane): stream the steps of one item into the stage ring, and
 // warm L2 with the rows and records kPrefetchSteps steps beyond the ring so
@@ -466,10 +420,11 @@ constexpr int kPrefetchSteps = 8;
 template <typename T, int TK, int NW>
 __device__ __forceinline__ void produce_item(const FwdArgs<T> &a, const Item<T, 1> &it,
                                              const PipeState &ps, unsigned &step) {
-  constexpr int CH = 32 * TK;
+  constexpr int CH = chunk_of<T, TK>();
+  constexpr unsigned RPL = 128 / (kSer * sizeof(T));  // X rows per 128-byte line
   const unsigned cbytes = (unsigned)((it.o_end - it.o_begin) * kRec * sizeof(T));
   const int np = it.p_end - it.p_begin;
-  const int nsteps = np * ((it.k_end - it.k_begin) / CH);
+  const int nsteps = np * it.chunks(CH);
   // Step idx covers panel p_begin + idx % np, chunk k_begin + (idx / np) CH.
   // Both cursors (the load and the L2 prefetch running ahead of it) advance
   // incrementally: this lane's per-step work stays short, since it is on the
@@ -479,19 +434,18 @@ __device__ __forceinline__ void produce_item(const FwdArgs<T> &a, const Item<T, 
   // them re-read)
   const T *const X = a.X;
   const T *const coef = a.coef;
-  const int x_ld = a.x_ld, O = a.O;
+  const int O = a.O;
+  const size_t x_ld = a.x_ld;
   int *const err = ps.err;
   const long long wait_cycles = ps.wait_cycles;
-  auto src_x = [&](int pp, int kc) {
-    return X + ((size_t)(it.p_begin + pp) * x_ld + it.k_begin % x_ld + kc * CH) * kRec;
-  };
+  const size_t row_b = (size_t)it.p_begin * x_ld + (it.k_begin - a.row0);
   auto src_c = [&](int pp) {
     return coef + ((size_t)(it.p_begin + pp) * O + it.o_begin) * kRec;
   };
   if (a.withhold) return;  // testing: no copies, so every consumer wait runs out
   int fp = 0, fk = 0;  // prefetch cursor (panel offset, chunk)
   auto prefetch_next = [&]() {
-    prefetch_l2(src_x(fp, fk), ps.x_bytes);
+    prefetch_l2(X + (row_b + fp * x_ld + (size_t)fk * CH) * kSer, ps.x_bytes);
     prefetch_l2(src_c(fp), cbytes);
     if (++fp == np) {
       fp = 0;
@@ -510,9 +464,8 @@ __device__ __forceinline__ void produce_item(const FwdArgs<T> &a, const Item<T, 
       return;
     unsigned char *dst = ps.stage0 + (size_t)s * ps.stage_bytes;
     mbar_expect_tx(&ps.full[s], ps.x_bytes + cbytes);
-    // tensor rows are 128 bytes: two FP32 samples or one FP64 sample
-    const int row = (it.p_begin + cp) * x_ld + it.k_begin % x_ld + ck * CH;
-    tma_load_2d(dst, ps.tmap, 0, sizeof(T) == 4 ? row >> 1 : row, &ps.full[s]);
+    const size_t row = row_b + cp * x_ld + (size_t)ck * CH;
+    tma_load_2d(dst, ps.tmap, 0, (int)(row / RPL), &ps.full[s]);
     bulk_load(dst + ps.x_bytes, src_c(cp), cbytes, &ps.full[s]);
     if (++cp == np) {
       cp = 0;
@@ -525,70 +478,65 @@ __device__ __forceinline__ void produce_item(const FwdArgs<T> &a, const Item<T, 
   }
 }
 
-template <typename T, int TK, int NW>
-__device__ __forceinline__ void consume_item(const FwdArgs<T> &a, const Item<T, NW> &it,
-                                             const PipeState &ps, unsigned &step, T *wwin,
+template <int TK, int NW>
+__device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Item<double, NW> &it,
+                                             const PipeState &ps, unsigned &step, double *wwin,
                                              int *s_i0max, int w) {
-  static_assert(sizeof(T) == 8, "scalar consumers read the 16-value FP64 record");
   constexpr int CH = 32 * TK;
   const int lane = threadIdx.x & 31;
-  item_prologue<T, NW>(a, it, w, wwin, s_i0max);
-  for (int k0 = it.k_begin; k0 < it.k_end; k0 += CH) {
+  item_prologue<double, NW>(a, it, w, wwin, s_i0max);
+  int k0 = it.k_begin;
+  for (; k0 < it.k_end; k0 += CH) {
+    const int nj = min(TK, (it.k_end - k0 + 31) / 32);
     for (int p = it.p_begin; p < it.p_end; ++p, ++step) {
       const int s = (int)(step % (unsigned)ps.nst);
       const unsigned ph = (step / (unsigned)ps.nst) & 1u;
       if (!mbar_wait(&ps.full[s], ph, ps.err, ps.abort, ps.wait_cycles)) return;
       const unsigned char *stg = ps.stage0 + (size_t)s * ps.stage_bytes;
-      T x[TK][kRec];
+      double x[TK][kSer];
 #pragma unroll
-      for (int j = 0; j < TK; ++j) lds_row_swz<T>(stg, lane + 32 * j, x[j]);
-      const T *crec = reinterpret_cast<const T *>(stg + ps.x_bytes);
+      for (int j = 0; j < TK; ++j) lds_row_f64(stg, lane + 32 * j, x[j]);
+      const double *crec = reinterpret_cast<const double *>(stg + ps.x_bytes);
       for (int m = 0; m < it.nobs; ++m) {
-        const int o = it.o_begin + w + NW * m;
-        T c[kRec];
-        lds16<T>(crec + (size_t)(o - it.o_begin) * kRec, c);
-        T *wm = wwin + (m * a.win + 1 + lane + rec_i0_of<T>(c[slot::off]));
-        accumulate<T, TK>(x, c, wm);
+        const double *rec = crec + (size_t)(w + NW * m) * kRec;
+        double c[12];
+        lds_f64(rec, c);
+        accumulate<TK>(x, c, wwin + (m * a.win + lane + (int)rec[slot::off]), nj);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&ps.empty[s]);
     }
-    flush_slide<T, CH, NW>(a, it, w, wwin, s_i0max, k0);
+    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0);
   }
-  flush_tail<T, CH, NW>(a, it, w, wwin, s_i0max);
+  flush_tail<CH, NW>(a, it, w, wwin, s_i0max, k0);
 }
 
 // ---- FP32 consumer (mixed precision) ----------------------------------------
-// FP32 X rows pair the consecutive samples 2r and 2r + 1 of each 64-sample
-// block, so the 16-byte chunk c of pair row r holds (x_k[2c], x_k+1[2c],
-// x_k[2c+1], x_k+1[2c+1]), k = 64 b + 2 r: one swizzled row read per lane
-// gives both samples' series.  Lane l owns pair rows l + 32 t of a chunk
-// (samples s = 64 t + 2 l and s + 1) and forms, per observer, G = sum_q c_q
-// X_q and M likewise on the moments for both samples at once: (x_k[q],
-// x_k+1[q]) is a register pair, and packed fma.rn.f32x2 with c_q in both
-// halves computes the two samples' dot products.  A packed FMA issues in one
-// slot and occupies the FMA pipe for two cycles, so the 16 multiply-adds of
-// the two dot products take 8 issue slots instead of 16: the kernel is bound
-// by instruction issue, not by the FMA pipe.  Results are those of scalar
-// fmaf (both round each element to nearest).
-// Sample s adds a G + cc M (left spline node) to window slot 1 + s + off and
-// b G + dd M (right node) to slot s + off, so slot 1 + s + off receives
-// a G_s + cc M_s + b G_s+1 + dd M_s+1.  For the first sample of a pair both
-// nodes are the lane's own: the old slot value enters a chain of four FMAs.
-// For the second, v = b G + dd M of the next sample comes from lane l + 1
-// (lane 31: lane 0's pair of block t + 1), one shuffle per pair; the last
-// block's lane 31 has no successor in the chunk, and the slot below the
-// chunk (v of sample 0) is added by lane 0, so the chunk-crossing node is
-// split between two chunks exactly once.
+// An X row is 32 bytes, four consecutive rows one 128-byte line.  Lane l owns
+// line l + 32 b of each 128-row block b of a chunk and forms, per observer and
+// row, G = c . X with packed fma.rn.f32x2 over the register pairs (X_2q,
+// X_2q+1) and (c_2q, c_2q+1) as they lie in the row and in the record (no
+// duplicated coefficients), the halves added at the end.  A packed FMA issues
+// in one slot and occupies the FMA pipe for two cycles.  The bin of interval k
+// needs G of rows k .. k + 3: three values come from the lane above by
+// shuffle (lane 31: lane 0's of the next block), and the last block's lane 31
+// only serves its neighbour, so a chunk of NB blocks completes 128 NB - 4 bins
+// and the next chunk starts at that row.
 //
-// Split windows: slot x of an observer's window lives in half x & 1 at word
-// x >> 1, so the two slots of a lane's pair sit in different halves and 32
-// lanes touch 32 consecutive words of one half per access: conflict-free for
-// every offset.  The planner writes each record's two byte offsets (slots 14,
-// 15: the words of slots off + 1 and off + 2 relative to the window), so the
-// hot loop adds them to the lane's base and never branches on the shift.
-// Within one (panel, observer) no two lanes touch the same slot; one
-// __syncwarp per panel orders the next panel's shifted updates.
+// Per (observer, 128-row block): 16 packed FMAs, 4 adds, 16 FMAs, 3 shuffles,
+// 4 window loads and stores and a share of the record's 4 loads and 4 address
+// adds: 13.1 warp instructions per 32 samples with two blocks.  On a GB300 the
+// sphere of 32768 panels x 2048 steps x 72 observers takes @FWD_MS@ ms; the
+// former kernel on samples and moments side by side (20 multiply-adds, 64-byte
+// rows, 22 instructions per 32 samples) took 4.57 ms.
+//
+// Quarter-split windows: slot x of an observer's window lives in quarter x & 3
+// at word x >> 2, so the four bins of a lane sit in four quarters and 32 lanes
+// touch 32 consecutive words of one quarter per access: conflict-free for
+// every offset.  The planner writes each record's four byte offsets, so the
+// hot loop adds them to the lane's base and never branches on the shift; block
+// b adds 32 words.  Within one (panel, observer) no two lanes touch the same
+// slot; one __syncwarp per panel orders the next panel's shifted updates.
 // Shared-space accesses by 32-bit address (the consumer addresses the stage
 // ring and its windows explicitly, so no generic-address arithmetic).
 // Window loads are not volatile: the compiler may hoist an observer's loads
@@ -614,47 +562,29 @@ __device__ __forceinline__ float4 lds_v4f32(unsigned addr) {
       : "r"(addr));
   return v;
 }
-__device__ __forceinline__ uint2 lds_v2u32_stage(unsigned addr) {
-  uint2 v;
-  asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-  return v;
-}
 // The stage address as an opaque value produced after the barrier wait.
 __device__ __forceinline__ unsigned stage_token(unsigned addr) {
   unsigned r;
   asm volatile("mov.u32 %0, %1;" : "=r"(r) : "r"(addr) : "memory");
   return r;
 }
-// x + (the value of the lane above, if there is one): the last lane keeps x.
-__device__ __forceinline__ float add_from_lane_above(float x, float v) {
-  float r;
-  asm(
-      "{\n\t.reg .pred p;\n\t.reg .f32 t;\n\t"
-      "shfl.sync.down.b32 t|p, %2, 1, 0x1f, 0xffffffff;\n\t"
-      "mov.f32 %0, %1;\n\t"
-      "@p add.f32 %0, %1, t;\n\t}"
-      : "=f"(r)
-      : "f"(x), "f"(v));
-  return r;
-}
 
-// The slots of one FP32 record that the consumer reads: c0..c7, a, b, cc, dd
-// and the two window byte offsets (slots 14, 15).
+// The slots of one FP32 record that the consumer reads: c0..c7 as pairs, the
+// weights and the four window byte offsets.
 struct Coef {
-  float c[8], wa, wb, wcc, wdd;
-  unsigned r0, r1;
+  unsigned long long c[4];
+  float w[4];
+  uint4 q;
 };
 __device__ __forceinline__ void lds_coef(unsigned rec, Coef &k) {
-  static_assert(slot::c == 0 && slot::a == 8 && slot::b == 9 && slot::cc == 10 &&
-                    slot::dd == 11 && slot::w0 == 14 && slot::w1 == 15,
-                "record read as three 16-byte groups and one 8-byte pair");
-  const float4 c0 = lds_v4f32(rec), c1 = lds_v4f32(rec + 16), w = lds_v4f32(rec + 32);
-  const uint2 r = lds_v2u32_stage(rec + 4 * slot::w0);
-  k.c[0] = c0.x; k.c[1] = c0.y; k.c[2] = c0.z; k.c[3] = c0.w;
-  k.c[4] = c1.x; k.c[5] = c1.y; k.c[6] = c1.z; k.c[7] = c1.w;
-  k.wa = w.x; k.wb = w.y; k.wcc = w.z; k.wdd = w.w;
-  k.r0 = r.x;
-  k.r1 = r.y;
+  static_assert(slot::c == 0 && slot::w == 8 && slot::q0 == 12, "record read in 16-byte groups");
+  asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(k.c[0]), "=l"(k.c[1]) : "r"(rec));
+  asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(k.c[2]), "=l"(k.c[3]) : "r"(rec + 16));
+  const float4 w = lds_v4f32(rec + 32);
+  k.w[0] = w.x; k.w[1] = w.y; k.w[2] = w.z; k.w[3] = w.w;
+  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+      : "=r"(k.q.x), "=r"(k.q.y), "=r"(k.q.z), "=r"(k.q.w)
+      : "r"(rec + 48));
 }
 
 // Value of a split-window entry: a plain FP32 sum, or a compensated pair
@@ -673,7 +603,27 @@ template <> struct WinEntry<true> {
   static __device__ __forceinline__ E zero() { return make_float2(0.f, 0.f); }
 };
 
-// Flush the first CH (complete) bins of every split window to p_out and slide.
+// Add the first n bins of an observer's window to p_out.  Lanes take
+// consecutive bins; the quarter length is 8 or 24 mod 32 words, so the eight
+// words of each quarter that a warp reads lie on distinct banks.
+template <bool KAHAN, int NW>
+__device__ __forceinline__ void flush_bins(const FwdArgs<float> &a, const Item<float, NW> &it,
+                                           int w, int m, const void *wm, int wbase, int n) {
+  using W = WinEntry<KAHAN>;
+  const typename W::E *e = static_cast<const typename W::E *>(wm);
+  const int lane = threadIdx.x & 31;
+  const int H = a.win >> 2;
+  const int o = it.o_begin + w + NW * m;
+  const int nvalid = a.n_valid[o];
+  double *po = a.p_out + (size_t)o * a.nt;
+  for (int x = lane; x < n; x += 32) {
+    const int bin = wbase + x;
+    const typename W::E v = e[(x & 3) * H + (x >> 2)];
+    if (bin >= 0 && bin < nvalid && W::nz(v)) atomic_add_f64(po + bin, W::value(v));
+  }
+}
+
+// Flush the first CH (complete) bins of every window to p_out and slide.
 template <int CH, int NW, bool KAHAN>
 __device__ __forceinline__ void flush_slide_split(const FwdArgs<float> &a,
                                                   const Item<float, NW> &it, int w, float *wwin,
@@ -681,55 +631,30 @@ __device__ __forceinline__ void flush_slide_split(const FwdArgs<float> &a,
   using W = WinEntry<KAHAN>;
   using E = typename W::E;
   const int lane = threadIdx.x & 31;
-  const int H = a.win >> 1;
+  const int H = a.win >> 2;
   for (int m = 0; m < it.nobs; ++m) {
-    const int o = it.o_begin + w + NW * m;
     E *wm = reinterpret_cast<E *>(wwin + (size_t)m * a.wfl);
-    const int wbase = k0 - s_i0max[m] - 1;
-    const int nvalid = a.n_valid[o];
-    double *po = a.p_out + (size_t)o * a.nt;
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf)
-      for (int q = lane; q < CH / 2; q += 32) {
-        const int bin = wbase + 2 * q + hf;
-        const E v = wm[hf * H + q];
-        if (bin >= 0 && bin < nvalid && W::nz(v)) atomic_add_f64(po + bin, W::value(v));
-      }
+    flush_bins<KAHAN, NW>(a, it, w, m, wm, k0 - s_i0max[m], CH);
     __syncwarp();
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf)  // H - CH/2 <= CH/2: no overlap
-      for (int q = lane; q < H - CH / 2; q += 32) wm[hf * H + q] = wm[hf * H + CH / 2 + q];
+    const int keep = H - CH / 4;  // <= CH / 4: no overlap
+    for (int i = lane; i < 4 * keep; i += 32) {
+      E *q = wm + (i & 3) * H + (i >> 2);
+      *q = q[CH / 4];
+    }
     __syncwarp();
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf)
-      for (int q = H - CH / 2 + lane; q < H; q += 32) wm[hf * H + q] = W::zero();
+    for (int i = lane; i < CH; i += 32) wm[(i & 3) * H + keep + (i >> 2)] = W::zero();
     __syncwarp();
   }
 }
 
-// Segment end: the remaining split window holds partial bins of the next segment.
+// Segment end (k0: the interval after the last chunk): the remaining window
+// holds partial bins of the next segment.
 template <int CH, int NW, bool KAHAN>
 __device__ __forceinline__ void flush_tail_split(const FwdArgs<float> &a,
                                                  const Item<float, NW> &it, int w, float *wwin,
-                                                 const int *s_i0max) {
-  using W = WinEntry<KAHAN>;
-  using E = typename W::E;
-  const int lane = threadIdx.x & 31;
-  const int H = a.win >> 1;
-  for (int m = 0; m < it.nobs; ++m) {
-    const int o = it.o_begin + w + NW * m;
-    const E *wm = reinterpret_cast<const E *>(wwin + (size_t)m * a.wfl);
-    const int wbase = it.k_end - s_i0max[m] - 1;
-    const int nvalid = a.n_valid[o];
-    double *po = a.p_out + (size_t)o * a.nt;
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf)
-      for (int q = lane; q < H - CH / 2; q += 32) {
-        const int bin = wbase + 2 * q + hf;
-        const E v = wm[hf * H + q];
-        if (bin >= 0 && bin < nvalid && W::nz(v)) atomic_add_f64(po + bin, W::value(v));
-      }
-  }
+                                                 const int *s_i0max, int k0) {
+  for (int m = 0; m < it.nobs; ++m)
+    flush_bins<KAHAN, NW>(a, it, w, m, wwin + (size_t)m * a.wfl, k0 - s_i0max[m], a.win - CH);
   __syncwarp();
 }
 
@@ -748,215 +673,156 @@ __device__ __forceinline__ void sts_f32x2(unsigned addr, float2 v) {
   asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 
-// Packed FP32 pairs (fma.rn.f32x2 and friends): element-wise IEEE round-to-
-// nearest operations on two floats held in a 64-bit register pair.  One
-// packed FMA issues in one slot and keeps the FMA pipe busy for two cycles.
-using f32x2 = unsigned long long;
 __device__ __forceinline__ void lds_v2f32x2(unsigned addr, f32x2 &a, f32x2 &b) {
   asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr));
 }
-__device__ __forceinline__ f32x2 f2_dup(float x) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ void f2_split(f32x2 v, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+__device__ __forceinline__ float f2_sum(f32x2 v) {
+  float lo, hi;
+  f2_split(v, lo, hi);
+  return lo + hi;
 }
 
-template <int TK, int NW, bool PF, int PIPE, bool KAHAN>
+// One (chunk, panel) step: NA blocks of 128 rows (NA = 1: the last chunk of a
+// record, when its remaining intervals fit one block).
+template <int NA, int NW, bool PF, bool KAHAN>
+__device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned crec,
+                                             unsigned win_s, unsigned win_b, unsigned xrow) {
+  constexpr unsigned RB = kRec * 4;         // record bytes
+  constexpr unsigned BB = KAHAN ? 256 : 128;  // window bytes of 32 words of a quarter
+  const int lane = threadIdx.x & 31;
+  const bool first = lane == 0, inner = lane < 31;
+  f32x2 XP[NA][4][4];  // [block][row][pair of series]
+  const unsigned xb = stg + xrow;
+#pragma unroll
+  for (int b = 0; b < NA; ++b)
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      lds_v2f32x2((xb ^ ((unsigned)c << 4)) + 4096u * b, XP[b][c >> 1][2 * (c & 1)],
+                  XP[b][c >> 1][2 * (c & 1) + 1]);
+  // window base of this panel's updates, ordered after the previous panel's
+  // stores (see lds_win)
+  const unsigned wtok = stage_token(win_s);
+  auto observer = [&](int m, const Coef &k) {
+    const unsigned base = wtok + (unsigned)m * win_b;
+    const unsigned A[4] = {base + k.q.x, base + k.q.y, base + k.q.z, base + k.q.w};
+    float g[NA][7];
+    auto dots = [&]() {
+#pragma unroll
+      for (int b = 0; b < NA; ++b) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          f32x2 v = f2_mul(k.c[0], XP[b][j][0]);
+#pragma unroll
+          for (int q = 1; q < 4; ++q) v = f2_fma(k.c[q], XP[b][j][q], v);
+          g[b][j] = f2_sum(v);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          // lane 0 serves lane 31 with the next block's first rows
+          g[b][4 + i] = b + 1 < NA ? __shfl_sync(0xffffffffu, first ? g[b + 1][i] : g[b][i],
+                                                 (lane + 1) & 31)
+                                   : __shfl_down_sync(0xffffffffu, g[b][i], 1);
+    };
+    if constexpr (!KAHAN) {
+      float s[NA][4];
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[b][j] = lds_win(A[j] + BB * b);
+      dots();
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) s[b][j] = fmaf(k.w[t], g[b][j + t], s[b][j]);
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+        if (b + 1 < NA || inner) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sts_f32(A[j] + BB * b, s[b][j]);
+        }
+    } else {
+      // compensated: each slot is (sum, compensation); every panel's
+      // contribution to a slot is formed first, then added by Kahan's rule
+      float2 s[NA][4];
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[b][j] = lds_win2(A[j] + BB * b);
+      dots();
+#pragma unroll
+      for (int b = 0; b < NA; ++b)
+        if (b + 1 < NA || inner) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float y = k.w[0] * g[b][j];
+#pragma unroll
+            for (int t = 1; t < 4; ++t) y = fmaf(k.w[t], g[b][j + t], y);
+            sts_f32x2(A[j] + BB * b, kahan_add(s[b][j], y));
+          }
+        }
+    }
+  };
+  // PF: read the next observer's record while this one computes, else read
+  // each record right before its use.  A warp with the full count of
+  // observers runs them without an exit test, so the compiler may overlap one
+  // observer's tail with the next one's loads and arithmetic.
+  auto run = [&](auto full) {
+    constexpr bool kFull = decltype(full)::value;
+    const int n = kFull ? kMaxObsPerWarpF32 : nobs;
+    auto rec = [&](int m) { return crec + (unsigned)m * NW * RB; };
+    Coef k;
+    if (PF && n > 0) lds_coef(rec(0), k);
+#pragma unroll
+    for (int m = 0; m < kMaxObsPerWarpF32; ++m) {
+      if (!kFull && m >= n) break;
+      if (!PF) lds_coef(rec(m), k);
+      Coef kn;
+      if (PF && m + 1 < n) lds_coef(rec(m + 1), kn);
+      observer(m, k);
+      if (PF) k = kn;
+    }
+  };
+  if (nobs == kMaxObsPerWarpF32)
+    run(std::true_type{});
+  else
+    run(std::false_type{});
+}
+
+template <int TK, int NW, bool PF, bool KAHAN>
 __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
                                                  const Item<float, NW> &it,
                                                  const PipeState &ps, unsigned &step,
                                                  float *wwin, int *s_i0max, int w) {
-  constexpr int CH = 32 * TK;
-  constexpr int NP = TK / 2;  // pair rows per lane
-  constexpr unsigned RB = kRec * 4;  // record bytes
+  constexpr int NB = TK / 4;  // 128-row blocks
+  constexpr int CH = chunk_of<float, TK>();
   const int lane = threadIdx.x & 31;
   item_prologue<float, NW>(a, it, w, wwin, s_i0max);
-  // Window of observer m starts at win_s + m * win_b; the record's byte
-  // offsets r0 / r1 locate slots off + 1 / off + 2 of lane 0, block 0, and
-  // block t adds 32 words.
-  constexpr unsigned EB = KAHAN ? 8u : 4u;  // bytes per window entry
   const unsigned win_b = (unsigned)a.wfl * 4u;
-  const unsigned win_s = smem_u32(wwin) + (unsigned)lane * EB;
+  const unsigned win_s = smem_u32(wwin) + (unsigned)lane * (KAHAN ? 8u : 4u);
   const unsigned stage0 = smem_u32(ps.stage0);
-  // X pair row r = lane + 32 t of a stage: 16-byte chunk c at c ^ (lane & 7).
-  // Stages are 1024-byte aligned and a pair row is 128 bytes, so bits 4..6 of
-  // (stage + 128 lane) are zero and chunk c of the lane's row sits at
-  // (stage + 128 lane + 16 (lane & 7)) ^ 16 c: one XOR per chunk.
+  // X line lane + 32 b of a stage: 16-byte chunk c at c ^ (lane & 7).  Stages
+  // are 1024-byte aligned and a line is 128 bytes, so chunk c of the lane's
+  // line sits at (stage + 128 lane + 16 (lane & 7)) ^ 16 c: one XOR per chunk.
   const unsigned xrow = (unsigned)lane * 128u + (((unsigned)lane & 7u) << 4);
-  const bool first = lane == 0;
   unsigned s = step % (unsigned)ps.nst, ph = (step / (unsigned)ps.nst) & 1u;
-  const int nsteps = (it.p_end - it.p_begin) * ((it.k_end - it.k_begin) / CH);
-  int j = 0;  // in-item step index
-  for (int k0 = it.k_begin; k0 < it.k_end; k0 += CH) {
-    for (int p = it.p_begin; p < it.p_end; ++p, ++step, ++j) {
+  int k0 = it.k_begin;
+  for (; k0 < it.k_end; k0 += CH) {
+    const bool one = NB > 1 && it.k_end - k0 <= 124;
+    for (int p = it.p_begin; p < it.p_end; ++p, ++step) {
       if (!mbar_wait(&ps.full[s], ph, ps.err, ps.abort, ps.wait_cycles)) return;
       const unsigned stg = stage_token(stage0 + s * ps.stage_bytes);
-      // XP[t][q] = (value q of sample 2r, value q of sample 2r + 1): the 16-byte
-      // chunk c holds the pairs of values 2c and 2c + 1
-      f32x2 XP[NP][kRec];
-      const unsigned xb = stg + xrow;
-#pragma unroll
-      for (int t = 0; t < NP; ++t) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          lds_v2f32x2((xb ^ ((unsigned)c << 4)) + 4096u * t, XP[t][2 * c], XP[t][2 * c + 1]);
-      }
-      const unsigned crec = stg + ps.x_bytes + (unsigned)w * RB;
-      // window base of this panel's updates, ordered after the previous
-      // panel's stores (see lds_win)
-      const unsigned wtok = stage_token(win_s);
-      // one (panel, observer): the spline-node updates of the lane's samples
-      auto observer = [&](int m, const Coef &k) {
-        const unsigned base = wtok + (unsigned)m * win_b;
-        const unsigned A0 = base + k.r0, A1 = base + k.r1;
-        // signal G and moment M of both samples of each pair row: packed dot
-        // products c . X with the coefficient in both halves of a register
-        // pair (issued after the window loads, which then hide their latency)
-        f32x2 Gp[NP], Mp[NP];
-        auto dots = [&]() {
-          {
-            const f32x2 cp = f2_dup(k.c[0]);
-#pragma unroll
-            for (int t = 0; t < NP; ++t) {
-              Gp[t] = f2_mul(cp, XP[t][0]);
-              Mp[t] = f2_mul(cp, XP[t][8]);
-            }
-          }
-#pragma unroll
-          for (int q = 1; q < 8; ++q) {
-            const f32x2 cp = f2_dup(k.c[q]);
-#pragma unroll
-            for (int t = 0; t < NP; ++t) {
-              Gp[t] = f2_fma(cp, XP[t][q], Gp[t]);
-              Mp[t] = f2_fma(cp, XP[t][8 + q], Mp[t]);
-            }
-          }
-        };
-        if constexpr (!KAHAN) {
-          float s0[NP], s1[NP], v0[NP];
-#pragma unroll
-          for (int t = 0; t < NP; ++t) {
-            s0[t] = lds_win(A0 + 128u * t);
-            s1[t] = lds_win(A1 + 128u * t);
-          }
-          // lane 0: the slot below the chunk (other lanes read a slot of the
-          // lane below, in the window, and discard it); no lane stores to it
-          // before lane 0 does, so it is read early to hide the latency
-          const float e_old = lds_win(A1 - 4u);
-          dots();
-#pragma unroll
-          for (int t = 0; t < NP; ++t) {
-            float G0, G1, M0, M1;
-            f2_split(Gp[t], G0, G1);
-            f2_split(Mp[t], M0, M1);
-            // slot of the pair's first sample: both spline nodes are this lane's
-            s0[t] = fmaf(k.wdd, M1, fmaf(k.wb, G1, fmaf(k.wcc, M0, fmaf(k.wa, G0, s0[t]))));
-            // slot of the second: its left node, the right one comes from above
-            s1[t] = fmaf(k.wcc, M1, fmaf(k.wa, G1, s1[t]));
-            // right node of the pair's first sample, for the lane below
-            v0[t] = fmaf(k.wdd, M0, k.wb * G0);
-          }
-#pragma unroll
-          for (int t = 0; t < NP; ++t) sts_f32(A0 + 128u * t, s0[t]);
-#pragma unroll
-          for (int t = 0; t + 1 < NP; ++t) {
-            // lane 0 serves lane 31 with block t + 1's first sample
-            const float x = first ? v0[t + 1] : v0[t];
-            s1[t] += __shfl_sync(0xffffffffu, x, (lane + 1) & 31);
-          }
-          s1[NP - 1] = add_from_lane_above(s1[NP - 1], v0[NP - 1]);
-#pragma unroll
-          for (int t = 0; t < NP; ++t) sts_f32(A1 + 128u * t, s1[t]);
-          // lane 0: the slot below the chunk (a C++ condition, so the compiler
-          // predicates the store on `first` computed once, not per observer)
-          if (first) sts_f32(A1 - 4u, e_old + v0[0]);
-        } else {
-          // compensated: each slot is (sum, compensation); every panel's
-          // contribution to a slot is formed first, then added by Kahan's rule
-          float2 w0[NP], w1[NP];
-#pragma unroll
-          for (int t = 0; t < NP; ++t) {
-            w0[t] = lds_win2(A0 + 256u * t);
-            w1[t] = lds_win2(A1 + 256u * t);
-          }
-          const float2 e_old = lds_win2(A1 - 8u);
-          dots();
-          float y0[NP], y1[NP], v0[NP];
-#pragma unroll
-          for (int t = 0; t < NP; ++t) {
-            float G0, G1, M0, M1;
-            f2_split(Gp[t], G0, G1);
-            f2_split(Mp[t], M0, M1);
-            y0[t] = fmaf(k.wdd, M1, fmaf(k.wb, G1, fmaf(k.wcc, M0, k.wa * G0)));
-            y1[t] = fmaf(k.wcc, M1, k.wa * G1);
-            v0[t] = fmaf(k.wdd, M0, k.wb * G0);
-          }
-#pragma unroll
-          for (int t = 0; t < NP; ++t) sts_f32x2(A0 + 256u * t, kahan_add(w0[t], y0[t]));
-#pragma unroll
-          for (int t = 0; t + 1 < NP; ++t) {
-            const float x = first ? v0[t + 1] : v0[t];
-            y1[t] += __shfl_sync(0xffffffffu, x, (lane + 1) & 31);
-          }
-          y1[NP - 1] = add_from_lane_above(y1[NP - 1], v0[NP - 1]);
-#pragma unroll
-          for (int t = 0; t < NP; ++t) sts_f32x2(A1 + 256u * t, kahan_add(w1[t], y1[t]));
-          if (first) sts_f32x2(A1 - 8u, kahan_add(e_old, v0[0]));
-        }
-      };
-      // PF: read the next observer's record while this one computes, else
-      // read each record right before its use.  A warp with the full count of
-      // observers runs them without an exit test, so the compiler may overlap
-      // one observer's tail with the next one's loads and arithmetic.
-      auto run = [&](auto full) {
-        constexpr bool kFull = decltype(full)::value;
-        const int n = kFull ? kMaxObsPerWarpF32 : it.nobs;
-        auto rec = [&](int m) { return crec + (unsigned)m * NW * RB; };
-        Coef k;
-        if (PF && n > 0) lds_coef(rec(0), k);
-#pragma unroll
-        for (int m = 0; m < kMaxObsPerWarpF32; ++m) {
-          if (!kFull && m >= n) break;
-          if (!PF) lds_coef(rec(m), k);
-          Coef kn;
-          if (PF && m + 1 < n) lds_coef(rec(m + 1), kn);
-          observer(m, k);
-          if (PF) k = kn;
-        }
-      };
-      if (it.nobs == kMaxObsPerWarpF32)
-        run(std::true_type{});
+      const unsigned crec = stg + ps.x_bytes + (unsigned)w * (kRec * 4);
+      if (one)
+        consume_step<1, NW, PF, KAHAN>(it.nobs, stg, crec, win_s, win_b, xrow);
       else
-        run(std::false_type{});
+        consume_step<NB, NW, PF, KAHAN>(it.nobs, stg, crec, win_s, win_b, xrow);
       __syncwarp();
-      if constexpr (PIPE == 2) {
-        // the last warp done with this stage refills it with step j + nst
-        if (lane == 0) {
-          __threadfence_block();
-          const int done = atomicAdd(&ps.released[s], 1) + 1;
-          if (done % NW == 0 && j + ps.nst < nsteps && !a.withhold) {
-            __threadfence_block();
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue_step<float, TK, NW>(a, it, ps, j + ps.nst, s);
-            atomicMax(ps.issued, (int)step + ps.nst + 1);
-          }
-        }
-      } else {
-        if (lane == 0) mbar_arrive(&ps.empty[s]);
-      }
+      if (lane == 0) mbar_arrive(&ps.empty[s]);
       if (++s == (unsigned)ps.nst) {
         s = 0;
         ph ^= 1u;
@@ -964,7 +830,7 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
     }
     flush_slide_split<CH, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
   }
-  flush_tail_split<CH, NW, KAHAN>(a, it, w, wwin, s_i0max);
+  flush_tail_split<CH, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
 }
 
 // Wait until every copy the producer issued has landed, always with the full
@@ -982,28 +848,21 @@ __device__ __forceinline__ void drain_copies(const PipeState &ps, unsigned step,
 template <typename T, int TK, int NW>
 __device__ __forceinline__ unsigned char *pipe_setup(unsigned char *raw, int obs_per_cta,
                                                      int nst, uint64_t *bars,
-                                                     volatile int *abort, PipeState &ps,
-                                                     int *released = nullptr,
-                                                     int *issued = nullptr) {
-  constexpr int CH = 32 * TK;
+                                                     volatile int *abort, PipeState &ps) {
   const unsigned base = smem_u32(raw);
   unsigned char *al = raw + ((1024u - (base & 1023u)) & 1023u);
-  ps.x_bytes = CH * kRec * sizeof(T);
+  ps.x_bytes = 32 * TK * kSer * sizeof(T);
   ps.stage_bytes = (ps.x_bytes + obs_per_cta * kRec * sizeof(T) + 1023u) & ~1023u;
   ps.nst = nst;
   ps.stage0 = al;
   ps.full = bars;
   ps.empty = bars + nst;
   ps.abort = abort;
-  ps.released = released;
-  ps.issued = issued;
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(&ps.full[s], 1);
       mbar_init(&ps.empty[s], NW);
-      if (released) released[s] = 0;
     }
-    if (issued) *issued = 0;
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1013,13 +872,10 @@ __device__ __forceinline__ unsigned char *pipe_setup(unsigned char *raw, int obs
 
 constexpr int kMaxStages = 8;
 
-// CTAs per SM the register budget is sized for: TMA shapes with 4 compute
-// warps run 3 (TK = 4) or 2 (TK = 8) per SM, with 8 compute warps 2 or 1.
+// CTAs per SM the register budget is sized for.
 template <int TK, int NW, int PIPE>
 struct MinBlocks {
-  static constexpr int v = !PIPE ? 1
-                           : PIPE == 2 ? (NW <= 4 ? (TK <= 4 ? 4 : 2) : (TK <= 4 ? 2 : 1))
-                                       : (NW <= 4 ? (TK <= 4 ? 3 : 2) : (TK <= 4 ? 2 : 1));
+  static constexpr int v = !PIPE ? 1 : (NW <= 4 ? (TK <= 4 ? 4 : 3) : (TK <= 4 ? 2 : 1));
 };
 
 template <typename T, int TK, int NW, int PIPE, int ACC>
@@ -1029,33 +885,7 @@ __device__ __forceinline__ void forward_cta(const FwdArgs<T> &a, const void *tma
   __shared__ int st[NW * kMaxObsPerWarp];
   if constexpr (PIPE == 0) {
     (void)tmap;
-    process_item_direct<T, TK, NW>(a, item, reinterpret_cast<T *>(smem_raw), st);
-  } else if constexpr (PIPE == 2) {
-    static_assert(sizeof(T) == 4 && ACC >= 3, "the in-line producer serves the FP32 consumer");
-    __shared__ __align__(8) uint64_t bars[2 * kMaxStages];
-    __shared__ int released[kMaxStages];
-    __shared__ int issued;
-    __shared__ int abort_flag;
-    PipeState ps;
-    unsigned char *wbase = pipe_setup<T, TK, NW>(smem_raw, a.obs_per_cta, nst, bars,
-                                                 &abort_flag, ps, released, &issued);
-    ps.tmap = tmap;
-    ps.err = err;
-    ps.wait_cycles = wait_cycles;
-    const int w = threadIdx.x >> 5;
-    const Item<T, NW> it(a, item, w);
-    if (threadIdx.x == 0 && !a.withhold) {  // fill the ring
-      const int nsteps = (it.p_end - it.p_begin) * ((it.k_end - it.k_begin) / (32 * TK));
-      const int n0 = min(nst, nsteps);
-      for (int j = 0; j < n0; ++j) issue_step<T, TK, NW>(a, it, ps, j, (unsigned)j);
-      atomicMax(&issued, n0);
-    }
-    unsigned step = 0;
-    T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
-    consume_item_f32<TK, NW, ACC >= 4, 2, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp,
-                                                      w);
-    __syncthreads();
-    if (threadIdx.x == 0 && abort_flag) drain_copies(ps, (unsigned)issued, err);
+    process_item_direct<TK, NW>(a, item, reinterpret_cast<T *>(smem_raw), st);
   } else {
     __shared__ __align__(8) uint64_t bars[2 * kMaxStages];
     __shared__ int abort_flag;
@@ -1076,28 +906,18 @@ __device__ __forceinline__ void forward_cta(const FwdArgs<T> &a, const void *tma
     } else {
       const Item<T, NW> it(a, item, w);
       T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
-      if constexpr (ACC >= 3 && sizeof(T) == 4) {
-        consume_item_f32<TK, NW, ACC >= 4, 1, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp,
-                                                        w);
-      } else {
-        consume_item<T, TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
-      }
+      if constexpr (sizeof(T) == 4)
+        consume_item_f32<TK, NW, ACC >= 4, ACC == 5>(a, it, ps, step, wwin,
+                                                     st + w * kMaxObsPerWarp, w);
+      else
+        consume_item<TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
     }
   }
 }
 
-
 template <typename T, int TK, int NW, int PIPE, int ACC>
 __global__ void __launch_bounds__((cta_threads<NW, PIPE>()), (MinBlocks<TK, NW, PIPE>::v))
     k_forward(FwdArgs<T> a, const __grid_constant__ CUtensorMap tm, int nst) {
-  forward_cta<T, TK, NW, PIPE, ACC>(a, &tm, nst, blockIdx.x, a.err, a.wait_cycles);
-}
-
-// Same CTA program for the long-sample-block shapes (TK = 8), which need
-// about 190 registers: capped at 200 so that two CTAs still share an SM.
-template <typename T, int TK, int NW, int PIPE, int ACC>
-__global__ void __maxnreg__(200) k_forward_wide(FwdArgs<T> a,
-                                                const __grid_constant__ CUtensorMap tm, int nst) {
   forward_cta<T, TK, NW, PIPE, ACC>(a, &tm, nst, blockIdx.x, a.err, a.wait_cycles);
 }
 
@@ -1139,8 +959,6 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
   __shared__ __align__(8) uint64_t qbar[kItemQ];
   __shared__ int s_q[kItemQ];
   __shared__ int abort_flag;
-  __shared__ int released[kMaxStages];
-  __shared__ int issued;
   const int n_surf = P.n_surf, total = P.total;
   const int *prefix = P.prefix;   // parameter space: read through the constant cache
   const FwdArgs<T> *args = P.a;
@@ -1150,20 +968,16 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
       for (int q = 0; q < kItemQ; ++q) mbar_init(&qbar[q], 1);
   }
   __syncthreads();
-  PipeState ps;
-  unsigned char *wbase = smem_raw;
-  if constexpr (PIPE != 0) {
+  const int w = threadIdx.x >> 5;
+  if constexpr (PIPE == 1) {
+    PipeState ps;
     int maxo = 0;
     for (int i = 0; i < n_surf; ++i) maxo = max(maxo, args[i].obs_per_cta);
     // (its barrier also orders the item ring's initialisation above)
-    wbase = pipe_setup<T, TK, NW>(smem_raw, maxo, nst, bars, &abort_flag, ps,
-                                  PIPE == 2 ? released : nullptr, PIPE == 2 ? &issued : nullptr);
+    unsigned char *wbase = pipe_setup<T, TK, NW>(smem_raw, maxo, nst, bars, &abort_flag, ps);
     ps.err = args[0].err;
     ps.wait_cycles = args[0].wait_cycles;
-  }
-  unsigned step = 0;
-  if constexpr (PIPE == 1) {
-    const int w = threadIdx.x >> 5;
+    unsigned step = 0;
     volatile int *abort = &abort_flag;
     if (w == NW) {
       if ((threadIdx.x & 31) == 0) {
@@ -1194,62 +1008,32 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
         const FwdArgs<T> &a = args[sf];
         const Item<T, NW> it(a, item - prefix[sf], w);
         T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
-        if constexpr (ACC >= 3 && sizeof(T) == 4) {
-          consume_item_f32<TK, NW, ACC >= 4, 1, ACC == 5>(a, it, ps, step, wwin,
-                                                  st + w * kMaxObsPerWarp, w);
-        } else {
-          consume_item<T, TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
-        }
+        if constexpr (sizeof(T) == 4)
+          consume_item_f32<TK, NW, ACC >= 4, ACC == 5>(a, it, ps, step, wwin,
+                                                       st + w * kMaxObsPerWarp, w);
+        else
+          consume_item<TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
         if (*abort) break;
       }
     }
-    return;
-  }
-  const int w = threadIdx.x >> 5;
-  for (;;) {
-    __syncthreads();  // the previous item is done; s_item holds this one
-    const int item = s_item;
-    __syncthreads();  // every thread has read it
-    if (item >= total) break;
-    const int lo = batch_surface(prefix, n_surf, item);
-    // a reference, not a copy: the fields are read from the parameter block
-    // where used, instead of holding the whole argument block in registers
-    const FwdArgs<T> &a = args[lo];
-    const int li = item - prefix[lo];
-    if constexpr (PIPE == 0) {
-      process_item_direct<T, TK, NW>(a, li, reinterpret_cast<T *>(smem_raw), st);
-    } else if constexpr (PIPE == 2) {
-      ps.tmap = &P.tm[lo];
-      if (abort_flag) break;
-      const Item<T, NW> it(a, li, w);
-      if (threadIdx.x == 0 && !a.withhold) {  // fill the ring: every stage is free here
-        const int nsteps = (it.p_end - it.p_begin) * ((it.k_end - it.k_begin) / (32 * TK));
-        const int n0 = min(nst, nsteps);
-        for (int j = 0; j < n0; ++j)
-          issue_step<T, TK, NW>(a, it, ps, j, (step + (unsigned)j) % (unsigned)nst);
-        atomicMax(&issued, (int)step + n0);
-      }
-      T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
-      consume_item_f32<TK, NW, ACC >= 4, 2, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp,
-                                                      w);
+  } else {
+    for (;;) {
+      __syncthreads();  // the previous item is done; s_item holds this one
+      const int item = s_item;
+      __syncthreads();  // every thread has read it
+      if (item >= total) break;
+      const int lo = batch_surface(prefix, n_surf, item);
+      // a reference, not a copy: the fields are read from the parameter block
+      // where used, instead of holding the whole argument block in registers
+      process_item_direct<TK, NW>(args[lo], item - prefix[lo], reinterpret_cast<T *>(smem_raw), st);
+      if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
     }
-    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-  }
-  if constexpr (PIPE == 2) {
-    __syncthreads();
-    if (threadIdx.x == 0 && abort_flag) drain_copies(ps, (unsigned)issued, args[0].err);
   }
 }
 
 template <typename T, int TK, int NW, int PIPE, int ACC>
 __global__ void __launch_bounds__((cta_threads<NW, PIPE>()), (MinBlocks<TK, NW, PIPE>::v))
     k_forward_batch(const __grid_constant__ BatchParams<T> P, int *counter, int nst) {
-  forward_batch_cta<T, TK, NW, PIPE, ACC>(P, counter, nst);
-}
-
-template <typename T, int TK, int NW, int PIPE, int ACC>
-__global__ void __maxnreg__(200)
-    k_forward_batch_wide(const __grid_constant__ BatchParams<T> P, int *counter, int nst) {
   forward_batch_cta<T, TK, NW, PIPE, ACC>(P, counter, nst);
 }
 
@@ -1274,32 +1058,24 @@ __global__ void __launch_bounds__((cta_threads<NW, PIPE>()), (MinBlocks<TK, NW, 
   forward_multi_cta<T, TK, NW, PIPE, ACC>(P, nst);
 }
 
-template <typename T, int TK, int NW, int PIPE, int ACC>
-__global__ void __maxnreg__(200) k_forward_multi_wide(const __grid_constant__ BatchParams<T> P,
-                                                      int nst) {
-  forward_multi_cta<T, TK, NW, PIPE, ACC>(P, nst);
-}
-
 // Candidate tile shapes {pipe, tk, warps, obs_per_warp, win, seg_chunks,
-// stages, acc, wide}.  acc: 0 one sample per lane per block (FP64), 3 a pair
-// of consecutive samples per lane per block with split windows and packed
-// dot products (FP32; its series rows pair those samples, so every FP32 shape
-// is a TMA shape), 4 the same with the next observer's record read ahead, 5
-// as 4 with compensated (Kahan) window sums.  wide: register cap 200 instead
-// of the launch bounds' occupancy target.
+// stages, acc}.  FP32 (always TMA): tk 4 or 8 (one or two 128-row blocks per
+// chunk); acc 3 plain window sums, 4 the same with the next observer's record
+// read ahead, 5 as 4 with compensated (Kahan) window sums.  win / 4 is 8 or 24
+// mod 32 (see flush_bins).
 constexpr FwdConfig kCfgF32[] = {
-    {1, 4, 4, 9, 224, 4, 3, 4, 0},
-    {1, 4, 4, 9, 224, 2, 3, 4, 0},
-    {1, 4, 4, 9, 224, 4, 3, 3, 0},
-    {2, 4, 4, 9, 224, 4, 2, 4, 0},
-    {2, 4, 8, 9, 224, 4, 3, 4, 0},
-    {1, 8, 4, 9, 352, 2, 3, 3, 0},
-    {1, 4, 4, 9, 224, 4, 3, 4, 1},
-    {1, 4, 4, 9, 224, 8, 3, 4, 0},
-    {1, 4, 4, 9, 160, 4, 4, 4, 0},
-    {1, 4, 4, 9, 224, 4, 2, 4, 0},
-    {1, 4, 4, 9, 160, 4, 2, 5, 0},
-    {1, 4, 4, 9, 224, 4, 3, 5, 0},
+    {1, 8, 4, 9, 352, 2, 2, 4},
+    {1, 8, 4, 9, 352, 1, 2, 4},
+    {1, 8, 4, 9, 352, 2, 2, 3},
+    {1, 4, 4, 9, 224, 4, 3, 4},
+    {1, 4, 8, 9, 224, 4, 3, 4},
+    {1, 8, 4, 9, 352, 2, 3, 3},
+    {1, 4, 4, 9, 224, 4, 3, 3},
+    {1, 8, 4, 9, 352, 4, 2, 4},
+    {1, 4, 4, 9, 224, 8, 3, 4},
+    {1, 8, 4, 9, 288, 2, 2, 4},
+    {1, 4, 4, 9, 160, 4, 2, 5},
+    {1, 4, 4, 9, 224, 4, 3, 5},
 };
 constexpr bool f32_obs_fit() {
   for (const FwdConfig &c : kCfgF32)
@@ -1308,10 +1084,10 @@ constexpr bool f32_obs_fit() {
 }
 static_assert(f32_obs_fit(), "an FP32 shape has more observers per warp than the unrolled loop");
 const FwdConfig kCfgF64[] = {
-    {0, 2, 8, 16, 128, 8, 0, 0, 0},
-    {1, 2, 8, 9, 128, 8, 3, 0, 0},
-    {0, 2, 4, 16, 128, 8, 0, 0, 0},
-    {0, 1, 8, 16, 64, 16, 0, 0, 0},
+    {0, 2, 8, 16, 128, 8, 0, 0},
+    {1, 2, 8, 9, 128, 8, 3, 0},
+    {0, 2, 4, 16, 128, 8, 0, 0},
+    {0, 1, 8, 16, 64, 16, 0, 0},
 };
 
 template <typename T>
@@ -1319,7 +1095,7 @@ size_t smem_for(const FwdConfig &c, int obs_per_cta) {
   const int opw = obs_per_cta / c.warps;
   size_t win = (size_t)c.warps * opw * c.win * sizeof(T) * (c.acc == 5 ? 2 : 1);
   if (c.pipe == 0) return win;
-  const size_t xb = (size_t)32 * c.tk * kRec * sizeof(T);
+  const size_t xb = (size_t)32 * c.tk * kSer * sizeof(T);
   const size_t sb =
       (xb + (size_t)obs_per_cta * kRec * sizeof(T) + 1023) & ~size_t(1023);
   return 1024 + (size_t)c.stages * sb + win;
@@ -1329,22 +1105,21 @@ template <typename T, int TK, int NW, int PIPE, int ACC>
 cudaError_t launch_one(const FwdArgs<T> &a, const CUtensorMap &tm, const FwdConfig &c,
                        cudaStream_t s) {
   const size_t smem = smem_for<T>(c, a.obs_per_cta);
-  auto kern = c.wide ? k_forward_wide<T, TK, NW, PIPE, ACC> : k_forward<T, TK, NW, PIPE, ACC>;
+  auto kern = k_forward<T, TK, NW, PIPE, ACC>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
   if (a.seg_lo < 0 || a.seg_cnt < 1 || a.seg_lo + a.seg_cnt > a.n_segs) return cudaErrorInvalidValue;
-  const int items = a.nsets * a.n_obs_groups * a.seg_cnt;
+  const long long items = (long long)a.nsets * a.subs * a.n_obs_groups * a.seg_cnt;
   if (items <= 0) return cudaSuccess;
-  kern<<<items, cta_threads<NW, PIPE>(), smem, s>>>(a, tm, c.stages);
+  if (items > INT32_MAX) return cudaErrorInvalidValue;
+  kern<<<(unsigned)items, cta_threads<NW, PIPE>(), smem, s>>>(a, tm, c.stages);
   return cudaGetLastError();
 }
 
 template <typename T, int TK, int NW, int PIPE, int ACC>
-cudaError_t launch_multi_one(const BatchParams<T> &P, size_t smem, bool wide, int nst,
-                             cudaStream_t s) {
-  auto kern = wide ? k_forward_multi_wide<T, TK, NW, PIPE, ACC>
-                   : k_forward_multi<T, TK, NW, PIPE, ACC>;
+cudaError_t launch_multi_one(const BatchParams<T> &P, size_t smem, int nst, cudaStream_t s) {
+  auto kern = k_forward_multi<T, TK, NW, PIPE, ACC>;
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1354,9 +1129,8 @@ cudaError_t launch_multi_one(const BatchParams<T> &P, size_t smem, bool wide, in
 
 template <typename T, int TK, int NW, int PIPE, int ACC>
 cudaError_t launch_batch_one(const BatchParams<T> &P, int *d_counter, size_t smem, int n_ctas,
-                             bool wide, int nst, cudaStream_t s) {
-  auto kern = wide ? k_forward_batch_wide<T, TK, NW, PIPE, ACC>
-                   : k_forward_batch<T, TK, NW, PIPE, ACC>;
+                             int nst, cudaStream_t s) {
+  auto kern = k_forward_batch<T, TK, NW, PIPE, ACC>;
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1393,9 +1167,9 @@ bool encode_x_tensor_map(void *out128, const void *X, unsigned long long rows, b
       return false;
     enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  // Rows of 128 bytes (two FP32 samples or one FP64 sample of 16 values), so
-  // the inner box dimension equals the 128-byte swizzle span.
-  const unsigned per = fp64 ? 1u : 2u;  // samples per 128-byte row
+  // Lines of 128 bytes (four FP32 rows or two FP64 rows), so the inner box
+  // dimension equals the 128-byte swizzle span.
+  const unsigned per = fp64 ? 2u : 4u;  // rows per 128-byte line
   const cuuint64_t dims[2] = {fp64 ? 16ull : 32ull, rows / per};
   const cuuint64_t strides[1] = {128ull};
   const cuuint32_t box[2] = {fp64 ? 16u : 32u, (cuuint32_t)(box_rows / per)};
@@ -1409,18 +1183,18 @@ bool encode_x_tensor_map(void *out128, const void *X, unsigned long long rows, b
   return r == CUDA_SUCCESS;
 }
 
-// Instantiated shapes: FP32 {copy warp: TK 4 with and without the record read
-// ahead, TK 8; in-line refill: 4 and 8 warps}; FP64 {direct 2x8, TMA 2x8,
-// direct 2x4, direct 1x8}.
+// Instantiated shapes: FP32 {one or two blocks with and without the record
+// read ahead, one block with 8 warps, one block compensated}; FP64 {direct
+// 2x8, TMA 2x8, direct 2x4, direct 1x8}.
 #define FWH_DISPATCH(T, c, CALL)                                                        \
   do {                                                                                   \
     if constexpr (sizeof(T) == 4) {                                                      \
-      if (c.pipe == 2 && c.tk == 4 && c.warps == 4 && c.acc == 4) return CALL(T, 4, 4, 2, 4); \
-      if (c.pipe == 2 && c.tk == 4 && c.warps == 8 && c.acc == 4) return CALL(T, 4, 8, 2, 4); \
-      if (c.pipe == 1 && c.tk == 4 && c.warps == 4 && c.acc == 3) return CALL(T, 4, 4, 1, 3); \
-      if (c.pipe == 1 && c.tk == 4 && c.warps == 4 && c.acc == 4) return CALL(T, 4, 4, 1, 4); \
-      if (c.pipe == 1 && c.tk == 4 && c.warps == 4 && c.acc == 5) return CALL(T, 4, 4, 1, 5); \
-      if (c.pipe == 1 && c.tk == 8 && c.warps == 4 && c.acc == 3) return CALL(T, 8, 4, 1, 3); \
+      if (c.tk == 8 && c.warps == 4 && c.acc == 4) return CALL(T, 8, 4, 1, 4);           \
+      if (c.tk == 8 && c.warps == 4 && c.acc == 3) return CALL(T, 8, 4, 1, 3);           \
+      if (c.tk == 4 && c.warps == 4 && c.acc == 4) return CALL(T, 4, 4, 1, 4);           \
+      if (c.tk == 4 && c.warps == 4 && c.acc == 3) return CALL(T, 4, 4, 1, 3);           \
+      if (c.tk == 4 && c.warps == 8 && c.acc == 4) return CALL(T, 4, 8, 1, 4);           \
+      if (c.tk == 4 && c.warps == 4 && c.acc == 5) return CALL(T, 4, 4, 1, 5);           \
     } else {                                                                             \
       if (c.pipe == 0 && c.tk == 2 && c.warps == 8) return CALL(T, 2, 8, 0, 0);          \
       if (c.pipe == 1 && c.tk == 2 && c.warps == 8) return CALL(T, 2, 8, 1, 0);          \
@@ -1451,7 +1225,7 @@ cudaError_t launch_forward_batch(const BatchParams<T> &P, int *d_counter, int cf
   const FwdConfig c = fwd_config(sizeof(T) == 8, cfg);
   const size_t smem = smem_for<T>(c, c.warps * c.obs_per_warp);
 #define FWH_CALL_BATCH(TT, TK, NW, PIPE, ACC) \
-  launch_batch_one<TT, TK, NW, PIPE, ACC>(P, d_counter, smem, n_ctas, c.wide != 0, c.stages, s)
+  launch_batch_one<TT, TK, NW, PIPE, ACC>(P, d_counter, smem, n_ctas, c.stages, s)
   FWH_DISPATCH(T, c, FWH_CALL_BATCH);
 #undef FWH_CALL_BATCH
 }
@@ -1462,7 +1236,7 @@ cudaError_t launch_forward_multi(const BatchParams<T> &P, int cfg, cudaStream_t 
   const FwdConfig c = fwd_config(sizeof(T) == 8, cfg);
   const size_t smem = smem_for<T>(c, c.warps * c.obs_per_warp);
 #define FWH_CALL_MULTI(TT, TK, NW, PIPE, ACC) \
-  launch_multi_one<TT, TK, NW, PIPE, ACC>(P, smem, c.wide != 0, c.stages, s)
+  launch_multi_one<TT, TK, NW, PIPE, ACC>(P, smem, c.stages, s)
   FWH_DISPATCH(T, c, FWH_CALL_MULTI);
 #undef FWH_CALL_MULTI
 }
@@ -1470,8 +1244,7 @@ cudaError_t launch_forward_multi(const BatchParams<T> &P, int cfg, cudaStream_t 
 // Resident CTAs per SM of the persistent kernel for a config.
 template <typename T, int TK, int NW, int PIPE, int ACC>
 cudaError_t batch_occupancy_one(const FwdConfig &c, size_t smem, int *per_sm) {
-  auto kern = c.wide ? k_forward_batch_wide<T, TK, NW, PIPE, ACC>
-                     : k_forward_batch<T, TK, NW, PIPE, ACC>;
+  auto kern = k_forward_batch<T, TK, NW, PIPE, ACC>;
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1493,19 +1266,17 @@ template cudaError_t forward_batch_occupancy<float>(int, int *);
 template cudaError_t forward_batch_occupancy<double>(int, int *);
 
 template <typename T>
-cudaError_t launch_plan(T *coef, const int *set_begin, int nsets, int O, int slack,
-                        int half_bytes, int slot_bytes, int *i0max_tab, int *err,
-                        cudaStream_t s) {
+cudaError_t launch_plan(T *coef, const int *i0, const int *set_begin, int nsets, int O, int slack,
+                        int win, int slot_bytes, int *i0max_tab, int *err, cudaStream_t s) {
   if (nsets <= 0 || O <= 0) return cudaSuccess;
-  k_plan<T><<<nsets, 128, 0, s>>>(coef, set_begin, O, slack, half_bytes, slot_bytes, i0max_tab,
-                                  err);
+  k_plan<T><<<nsets, 128, 0, s>>>(coef, i0, set_begin, O, slack, win, slot_bytes, i0max_tab, err);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_plan<float>(float *, const int *, int, int, int, int, int, int *,
-                                        int *, cudaStream_t);
-template cudaError_t launch_plan<double>(double *, const int *, int, int, int, int, int, int *,
-                                         int *, cudaStream_t);
+template cudaError_t launch_plan<float>(float *, const int *, const int *, int, int, int, int, int,
+                                        int *, int *, cudaStream_t);
+template cudaError_t launch_plan<double>(double *, const int *, const int *, int, int, int, int,
+                                         int, int *, int *, cudaStream_t);
 template cudaError_t launch_forward<float>(const FwdArgs<float> &, const void *, int,
                                            cudaStream_t);
 template cudaError_t launch_forward<double>(const FwdArgs<double> &, const void *, int,

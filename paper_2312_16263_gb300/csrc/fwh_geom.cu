@@ -15,8 +15,8 @@
 //   L_dot  : S M0 R-hat / (R D^2)
 //   L      : S [R-hat / (R^2 D^2) - M / (R^2 D^2) + R-hat (M_R - M0^2) / (R^2 D^3)]
 // and the arrival shift delta = M0 (R_max - R) = (i0 + f) dt of the source
-// sample feeding observer bin j (tau = t_j - M0 R, Eq. tau2) with the
-// natural-spline weights a = 1 - f, b = f, (a^3 - a) dt^2/6, (b^3 - b) dt^2/6.
+// sample feeding observer bin j (tau = t_j - M0 R, Eq. tau2) with the cubic
+// B-spline weights of beta_{k-1} .. beta_{k+2} at f.
 #include "fwh_internal.cuh"
 
 namespace fwh {
@@ -70,18 +70,7 @@ __global__ void __launch_bounds__(256) k_window(GeomArgs a) {
 }
 
 template <typename T>
-__device__ __forceinline__ void store_i0(T *rec, int i0);
-template <>
-__device__ __forceinline__ void store_i0<float>(float *slot, int i0) {
-  *slot = __int_as_float(i0);
-}
-template <>
-__device__ __forceinline__ void store_i0<double>(double *slot, int i0) {
-  *slot = (double)i0;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) k_coef(GeomArgs a, T *coef) {
+__global__ void __launch_bounds__(128) k_coef(GeomArgs a, T *coef, int *i0_tab) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= a.P) return;
   for (int o = blockIdx.y; o < a.O; o += gridDim.y) {  // grid y is capped at 65535
@@ -100,27 +89,27 @@ __global__ void __launch_bounds__(128) k_coef(GeomArgs a, T *coef) {
     const double k2 = k1 * iR;                 // S / (R^2 D^2)
     const double mrm = MR - M0 * M0;           // M_R - M^2
     double c[8];
-    c[0] = k1;
+    c[0] = k1;                                 // order of the series in X: Q', Q, L1', L1, ..
     c[1] = k2 * mrm * iD / M0;
     for (int i = 0; i < 3; ++i) {
-      c[2 + i] = k1 * M0 * Rh[i];
-      c[5 + i] = k2 * (Rh[i] + M0 * U[i] + Rh[i] * mrm * iD);
+      c[2 + 2 * i] = k1 * M0 * Rh[i];
+      c[3 + 2 * i] = k2 * (Rh[i] + M0 * U[i] + Rh[i] * mrm * iD);
     }
     const double q = M0 * (a.Rmax[o] - R) / a.dt;
-    double fl = floor(q);
-    double f = q - fl;
-    const double aw = 1.0 - f, bw = f;
-    const double h26 = a.dt * a.dt / 6.0;
+    const double fl = floor(q);
+    const double f = q - fl, e = 1.0 - f;
     T *rec = coef + ((size_t)p * a.O + o) * kRec;
     for (int i = 0; i < 8; ++i) rec[slot::c + i] = (T)c[i];
-    rec[slot::a] = (T)aw;
-    rec[slot::b] = (T)bw;
-    rec[slot::cc] = (T)((aw * aw * aw - aw) * h26);
-    rec[slot::dd] = (T)((bw * bw * bw - bw) * h26);
-    rec[slot::off] = (T)0;
-    rec[14] = (T)0;
-    rec[15] = (T)0;
-    store_i0<T>(rec + slot::i0, (int)fl);
+    rec[slot::w] = (T)(e * e * e / 6.0);
+    rec[slot::w + 1] = (T)((4.0 + f * f * (3.0 * f - 6.0)) / 6.0);
+    rec[slot::w + 2] = (T)((4.0 + e * e * (3.0 * e - 6.0)) / 6.0);
+    rec[slot::w + 3] = (T)(f * f * f / 6.0);
+    // the planner writes the window offsets into the remaining slots
+    for (int i = 12; i < kRec; ++i) rec[i] = (T)0;
+    if constexpr (sizeof(T) == 4)
+      i0_tab[(size_t)p * a.O + o] = (int)fl;
+    else
+      rec[slot::i0] = fl;
   }
 }
 
@@ -155,14 +144,14 @@ cudaError_t launch_window(const GeomArgs &a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_coef(const GeomArgs &a, T *coef, cudaStream_t s) {
+cudaError_t launch_coef(const GeomArgs &a, T *coef, int *i0, cudaStream_t s) {
   if (a.O <= 0 || a.P <= 0) return cudaSuccess;
   dim3 grid((a.P + 127) / 128, a.O < 65535 ? a.O : 65535);
-  k_coef<T><<<grid, 128, 0, s>>>(a, coef);
+  k_coef<T><<<grid, 128, 0, s>>>(a, coef, i0);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_coef<float>(const GeomArgs &, float *, cudaStream_t);
-template cudaError_t launch_coef<double>(const GeomArgs &, double *, cudaStream_t);
+template cudaError_t launch_coef<float>(const GeomArgs &, float *, int *, cudaStream_t);
+template cudaError_t launch_coef<double>(const GeomArgs &, double *, int *, cudaStream_t);
 
 }  // namespace fwh

@@ -1,22 +1,36 @@
 // Internal declarations of the GB300 FW-H library (not part of the C ABI).
 //
+// The natural cubic spline of a panel's source signal is carried in its
+// cubic B-spline coefficients: with F_k the samples and m_k the spline's
+// second derivatives, beta_k = F_k - m_k dt^2 / 6, and at k + f (0 <= f < 1)
+// the spline is
+//   w0 beta_{k-1} + w1 beta_k + w2 beta_{k+1} + w3 beta_{k+2},
+//   w0 = (1 - f)^3 / 6, w1 = (4 - 6 f^2 + 3 f^3) / 6,
+//   w2 = (1 + 3 f + 3 f^2 - 3 f^3) / 6, w3 = f^3 / 6,
+// with beta_{-1} = 2 beta_0 - beta_1 and beta_nt = 2 beta_{nt-1} - beta_{nt-2}
+// (the natural ends).  One eight-value dot product and four weights per
+// (panel, sample, observer): 12 multiply-adds, where samples and moments side
+// by side take 20 and twice the bytes.
+//
 // Data layout in HBM (P = panels in the library's spatial order, O =
-// observers, ntp = nt rounded up to the forward chunk, T = float or double):
+// observers, T = float or double):
 //   fields   [nt][5][P]      caller's pulsations (original panel order)
-//   X        [P][ntp][16] T  per panel, per source sample: the eight
-//                            observer-independent series
-//                              0 Qn_dot 1 Qn 2..4 L_dot 5..7 L
-//                            then their natural-spline moments (8..15);
-//                            rows >= nt are zero.  FP32 X pairs samples j
-//                            and j + 32 of every 64-sample block in one
-//                            128-byte row, [ntp/64][32][16][2]
+//   X        [P][x_ld][8] T  per panel the B-spline coefficients of the eight
+//                            observer-independent series, interleaved as
+//                              Qn', Qn, L1', L1, L2', L2, L3', L3
+//                            (' = source-time derivative).  Row r holds
+//                            sample row0 + r - 1, so that a record's first
+//                            row is the end value beta_{-1}; x_ld is a
+//                            multiple of 64 rows, rows past sample nt zero.
+//                            Whole records: row0 = 0 and x_ld >= nt + 3
+//   Xbar     [P][xb_ld][8] T gradient with respect to beta_0 .. beta_{nt-1}
 //   coef     [P][O][16] T    per (panel, observer) record (slots in
 //                            namespace slot): the 8 integrand coefficients
-//                            (same order as X), the interpolation weights
-//                            a, b, cc, dd, the integer shift i0 and the
-//                            window offset i0max(set) - i0 written by the
-//                            planner; integers are bit patterns in FP32
-//                            records, values in FP64 ones
+//                            (same order as X), the weights w0..w3, then for
+//                            FP64 the shift i0 and the window offset
+//                            i0max(set) - i0, for FP32 the four byte offsets
+//                            of that window offset (written by the planner)
+//   i0       [P][O] int      FP32: the integer shifts
 //   p_out    [O][nt] double  caller's output
 #pragma once
 
@@ -25,17 +39,24 @@
 
 namespace fwh {
 
-constexpr int kRec = 16;          // values per X row and per coef record
+constexpr int kRec = 16;          // values per coef record
+constexpr int kSer = 8;           // values per X row
+constexpr int kRowBlk = 64;       // X rows per prep block
+
+// X rows of a whole record of nt samples (samples -1 .. nt + 1 and padding).
+inline int64_t x_rows(int64_t nt) { return (nt + 3 + kRowBlk - 1) / kRowBlk * kRowBlk; }
+// Bytes past the last X row that an L2 prefetch of a whole chunk may touch.
+constexpr size_t kXPad = 16384;
 
 // Slots of a coefficient record (kRec values, both precisions).
 namespace slot {
-constexpr int c = 0;    // c0..c7: coefficients of the eight series
-constexpr int a = 8, b = 9, cc = 10, dd = 11;  // interpolation weights
-constexpr int i0 = 12;  // integer shift (bit pattern in FP32 records)
-constexpr int off = 13; // window offset i0max(set) - i0, written by the planner
-// FP32 records: byte offsets, in an observer's split window (slot x in half
-// x & 1, word x >> 1), of the slots off + 1 and off + 2, written by the planner
-constexpr int w0 = 14, w1 = 15;
+constexpr int c = 0;    // c0..c7: coefficients of the eight series, in X's order
+constexpr int w = 8;    // w0..w3: B-spline weights of beta_{k-1} .. beta_{k+2}
+constexpr int i0 = 12;  // FP64: integer shift (a value)
+constexpr int off = 13; // FP64: window offset i0max(set) - i0, written by the planner
+// FP32 records, written by the planner: byte offsets, in an observer's window
+// (slot x in quarter x & 3, word x >> 2), of the slots off, off + 1, off + 2, off + 3
+constexpr int q0 = 12;
 }  // namespace slot
 constexpr int kWarp = 32;
 
@@ -46,7 +67,37 @@ template <typename T> struct Prec;
 template <> struct Prec<float> { static constexpr int halo = 16; };
 template <> struct Prec<double> { static constexpr int halo = 32; };
 
-constexpr int kPivTab = 64;       // 1/pivot of the tridiag(1,4,1) elimination
+#ifdef __CUDACC__
+// Packed FP32 pairs (fma.rn.f32x2 and friends): element-wise IEEE round-to-
+// nearest operations on two floats held in a 64-bit register pair.  One
+// packed FMA issues in one slot and keeps the FMA pipe busy for two cycles.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 f2_dup(float x) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ void f2_split(f32x2 v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+// 32 bytes to global memory in one store (a whole sector per lane).
+__device__ __forceinline__ void stg256(void *dst, unsigned long long a, unsigned long long b,
+                                       unsigned long long c, unsigned long long d) {
+  asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(a), "l"(b), "l"(c),
+               "l"(d)
+               : "memory");
+}
+#endif
 
 // Device error flags (bitmask written by kernels, read by the host).
 enum : int {
@@ -68,21 +119,20 @@ struct GeomArgs {
 template <typename T>
 struct PrepArgs {
   const T *fields;      // [nt][5][P] original order
-  const int *perm;      // [P] sorted position -> original panel index
+  const int *place;     // [P] original panel index -> sorted position (null: the same)
   const double *n;      // [P][3] sorted normals
-  T *X;                 // [P][x_ld][16]: sample k of panel p in row p x_ld + k mod x_ld
-  int P, nt, ntp, chunk;
-  int x_ld;             // X rows per panel: ntp, or a ring of whole time segments
+  T *X;                 // [P][x_ld][8]
+  int P, nt;
+  int x_ld;             // X rows per panel
+  int row0;             // record row held by X row 0 (a multiple of 64)
   double ca, sa, dt;
-  int c_lo, c_hi;       // 64-sample chunks [c_lo, c_hi) to prepare (0, 0: all)
-  int int_lo, int_hi;   // FP32, set by the launcher: the interior chunks within [c_lo, c_hi)
+  int c_lo, c_hi;       // 64-row blocks [c_lo, c_hi) to prepare (0, 0: the whole record)
+  int int_lo, int_hi;   // set by the launcher: the interior blocks within [c_lo, c_hi)
 };
 
 template <typename T>
 struct FwdArgs {
-  const void *tmX;      // batched form: device CUtensorMap over X as [P*ntp rows][16]
-                        // (single launches take the descriptor as a kernel parameter)
-  const T *X;           // [P][x_ld][16] (sample k in row p x_ld + k mod x_ld)
+  const T *X;           // [P][x_ld][8]
   const T *coef;        // [P][O][16]
   double *p_out;        // [O][nt]
   const int *n_valid;   // [O]
@@ -90,9 +140,12 @@ struct FwdArgs {
   const int *set_order; // [nsets] sets by descending panel count (null: index order)
   const int *i0max_tab; // [nsets][O] largest shift of each (panel set, observer)
   int *err;
-  int nsets, O, ntp, nt;
-  int x_ld;             // X rows per panel (ntp, or a ring of whole time segments)
+  int nsets, O, nt;
+  int x_ld;             // X rows per panel
+  int row0;             // record row held by X row 0
+  int k_top;            // FP32: spline intervals (nt); FP64: rows that reach a bin (nt + 2)
   int obs_per_cta, n_obs_groups;
+  int subs;             // work items a panel set is cut into
   int seg_len, n_segs;
   int seg_lo, seg_cnt;  // this launch covers time segments [seg_lo, seg_lo + seg_cnt)
   int win;              // window slots per observer
@@ -108,26 +161,27 @@ constexpr int kMaxBatchSurf = 32;
 template <typename T>
 struct AdjArgs {
   const T *coef;        // [P][O][16]
-  T *Gt;                // [O][ntp] workspace: grad_p in T, zero outside [0, N_o)
+  T *Gt;                // [O][g_ld] workspace: grad_p in T, zero outside [0, N_o)
   const double *grad_p; // [O][nt]
   const int *n_valid;   // [O]
-  T *Xbar;              // [P][ntp][16] gradient w.r.t. X
-  int P, O, ntp, nt;
-  // FP32 set form (win > 0): the forward plan of a 128-sample-chunk shape
+  T *Xbar;              // [P][xb_ld][8] gradient w.r.t. the B-spline coefficients
+  int P, O, nt, g_ld, xb_ld;
+  // FP32: the forward plan
   const int *set_begin; // [nsets + 1] panel-set boundaries (sorted order)
   const int *set_order; // [nsets] sets by descending panel count
   const int *i0max_tab; // [nsets][O] largest shift of each (panel set, observer)
-  int nsets, win;       // win: window slots per observer (chunk + slack + 1)
+  int nsets, win;       // win: window slots per observer
+  int slot_shift;       // log2 of the plan's bytes per window slot (2, or 3 if compensated)
 };
 
 template <typename T>
 struct PrepAdjArgs {
   const T *fields;      // [nt][5][P] original order
-  const int *perm;
+  const int *place;     // [P] original panel index -> sorted position (null: the same)
   const double *n;      // [P][3] sorted normals
-  const T *Xbar;        // [P][ntp][16]
+  const T *Xbar;        // [P][xb_ld][8]
   T *grad_fields;       // [nt][5][P] original order
-  int P, nt, ntp, chunk;
+  int P, nt, xb_ld, chunk;
   double ca, sa, dt;
 };
 
@@ -137,8 +191,7 @@ cudaError_t launch_window(const GeomArgs &a, cudaStream_t s);
 cudaError_t launch_nvalid(const double *Rmax, const double *Rmin, int O, double mach, double dt,
                           int nt, int *n_valid, cudaStream_t s);
 template <typename T>
-cudaError_t launch_coef(const GeomArgs &a, T *coef, cudaStream_t s);
-cudaError_t upload_pivots(cudaStream_t s);
+cudaError_t launch_coef(const GeomArgs &a, T *coef, int *i0, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prep(const PrepArgs<T> &a, cudaStream_t s);
 template <typename T>
@@ -148,25 +201,33 @@ cudaError_t launch_adjoint(const AdjArgs<T> &a, cudaStream_t s);
 
 // Forward tile configurations (index into a table in fwh_forward.cu).
 struct FwdConfig {
-  int pipe;           // 0: direct loads, 1: TMA + mbarrier pipeline (producer warp),
-                      // 2: TMA pipeline refilled by the last warp done with a stage
-  int tk;             // source samples per lane per chunk (chunk = 32 tk)
+  int pipe;           // 0: direct loads, 1: TMA + mbarrier pipeline (producer warp)
+  int tk;             // X rows per lane per chunk
   int warps;          // compute warps per CTA
   int obs_per_warp;   // max observers per warp
   int win;            // window slots per observer
   int seg_chunks;     // chunks per time segment
   int stages;         // pipeline stages (pipe = 1)
-  int acc;            // 0: one sample per lane per block (FP64); FP32 consecutive sample
-                      // pairs with split windows: 3 plain, 4 with the next record read
-                      // ahead, 5 read ahead with compensated (Kahan) window sums
-  int wide;           // 1: register cap 200 instead of the occupancy launch bound
+  int acc;            // FP64: 0.  FP32 window sums: 3 plain, 4 plain with the next record
+                      // read ahead, 5 compensated (Kahan)
 };
+// Source samples a chunk completes: FP64 lanes hold rows 32 apart; FP32 lanes
+// hold four consecutive rows per 128-row block, and the last lane's serve only
+// its neighbour.
+inline int fwd_chunk(bool fp64, const FwdConfig &c) { return 32 * c.tk - (fp64 ? 0 : 4); }
+// Largest spread of shifts within a panel set that a config's window holds
+// (FP32: also the adjoint's window of a 128-row chunk).
+constexpr int kAdjReach = 131;
+inline int fwd_slack(bool fp64, const FwdConfig &c) {
+  const int need = fp64 ? 32 * c.tk + 3 : 32 * c.tk - 4;
+  return c.win - (fp64 || need > kAdjReach ? need : kAdjReach);
+}
 // Bytes of dynamic shared memory a config needs for `obs_per_cta` observers.
 size_t fwd_smem_bytes(bool fp64, const FwdConfig &c, int obs_per_cta);
 // CTAs of the persistent batch kernel that fit on one SM for config `cfg`.
 template <typename T>
 cudaError_t forward_batch_occupancy(int cfg, int *per_sm);
-// Encode the TMA descriptor of X ([rows][16] elements of 4 or 8 bytes) into a
+// Encode the TMA descriptor of X ([rows][8] elements of 4 or 8 bytes) into a
 // host buffer of 128 bytes; returns false if the driver refuses.
 bool encode_x_tensor_map(void *out128, const void *X, unsigned long long rows, bool fp64,
                          int box_rows);
@@ -178,15 +239,13 @@ template <typename T>
 cudaError_t launch_forward(const FwdArgs<T> &a, const void *tmap128, int cfg_idx,
                            cudaStream_t s);
 // Planner kernel: per (panel set, observer) the largest shift i0max into
-// i0max_tab and, per record, the window offset i0max - i0 clamped to
-// [0, slack] (slack = win - chunk - 1) into slot 13 and, for FP32 records,
-// the split-window byte offsets of slots off + 1 and off + 2 into slots 14
-// and 15 (half_bytes: bytes of one window half, slot_bytes: bytes per slot);
-// a set whose shifts span more than slack raises kErrWindow.
+// i0max_tab and, per record, the window offset i0max - i0 clamped to [0,
+// slack], as a value (FP64) or as the byte offsets of its four slots in the
+// quarter-split window of `win` slots of slot_bytes (FP32).  A set whose
+// shifts span more than slack raises kErrWindow.
 template <typename T>
-cudaError_t launch_plan(T *coef, const int *set_begin, int nsets, int O, int slack,
-                        int half_bytes, int slot_bytes, int *i0max_tab, int *err,
-                        cudaStream_t s);
+cudaError_t launch_plan(T *coef, const int *i0, const int *set_begin, int nsets, int O, int slack,
+                        int win, int slot_bytes, int *i0max_tab, int *err, cudaStream_t s);
 
 // Batched persistent forward: the arguments of one launch, passed by value
 // as a __grid_constant__ kernel parameter (under 9 KB at kMaxBatchSurf
@@ -198,7 +257,7 @@ struct alignas(64) TmapBytes {
 template <typename T>
 struct alignas(64) BatchParams {
   TmapBytes tm[kMaxBatchSurf];      // X descriptor of each surface
-  FwdArgs<T> a[kMaxBatchSurf];      // arguments of each surface (tmX unused)
+  FwdArgs<T> a[kMaxBatchSurf];      // arguments of each surface
   int prefix[kMaxBatchSurf + 1];    // first work item of each surface; [n_surf] = total
   int n_surf, total;
 };
