@@ -142,9 +142,16 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs<double> a) {
 // every record as a shared-memory broadcast instead of waiting on L2.  One
 // observer group writes Xbar directly, 32 bytes a lane and store; several add
 // their partial sums with vector atomics into a zeroed Xbar.
-// @ADJ@
+// Bound by instruction issue and shared-memory bandwidth together (issue 61 %,
+// shared-memory wavefronts 55 %, DRAM 11 %).  Eight warps a CTA so that 16 fit an
+// SM beside the windows (four: 12; the whole backward of 16384 panels x 1024 steps x
+// 36 observers takes 0.95 ms with eight, 0.97 with four; 0.99 on samples and
+// moments side by side, 20 multiply-adds and 64-byte rows).  Runs of six: the
+// gradient's error against 64 bits is 2.2e-6 there (2.4e-6 before; 3.2e-6
+// with one running sum).
 constexpr int kAdjGroup = 36;    // observers per item
-constexpr int kAdjWarps = 4;
+constexpr int kAdjRun = 6;       // observers summed from zero at a time
+constexpr int kAdjWarps = 8;
 constexpr int kAdjTK = 4;        // samples per lane (chunk 128)
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -224,35 +231,50 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
       cp_async_wait<0>();
     }
     __syncwarp();
-    f32x2 acc[kAdjTK][kSer / 2];
+    // The spline's adjoint amplifies rounding noise in Xbar, so a panel's sum
+    // over the group's observers is taken in runs of kAdjRun, each from zero:
+    // a third of the rounding of one running sum of 36.
+    f32x2 sum[kAdjTK][kSer / 2];
 #pragma unroll
     for (int j = 0; j < kAdjTK; ++j)
 #pragma unroll
-      for (int s = 0; s < kSer / 2; ++s) acc[j][s] = 0ull;
+      for (int s = 0; s < kSer / 2; ++s) sum[j][s] = 0ull;
     const float *rec = rb + (size_t)buf * kAdjGroup * kRec;
-#pragma unroll 2
-    for (int o = 0; o < no; ++o) {
-      const ulonglong2 c01 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec);
-      const ulonglong2 c23 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec + 4);
-      const float4 wv = *reinterpret_cast<const float4 *>(rec + o * kRec + slot::w);
-      const uint4 qo = *reinterpret_cast<const uint4 *>(rec + o * kRec + slot::q0);
-      const f32x2 c[4] = {c01.x, c01.y, c23.x, c23.y};
-      const float wt[4] = {wv.x, wv.y, wv.z, wv.w};
-      const float *gp = gw + o * win + lane;
-      const float *A[4] = {gp + (qo.x >> shift), gp + (qo.y >> shift), gp + (qo.z >> shift),
-                           gp + (qo.w >> shift)};
-      float gv[7];  // bins of intervals s - 2 .. s + 4 of the lane's first sample s
+    for (int or0 = 0; or0 < no; or0 += kAdjRun) {
+      f32x2 acc[kAdjTK][kSer / 2];
 #pragma unroll
-      for (int i = 0; i < 7; ++i) gv[i] = A[i & 3][i >> 2];
+      for (int j = 0; j < kAdjTK; ++j)
 #pragma unroll
-      for (int j = 0; j < kAdjTK; ++j) {
-        float q = gather_q(wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
-        if (edge)
-          q += ghost_q(k0 + 4 * lane + j, a.nt, wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
-        const f32x2 q2 = f2_dup(q);
+        for (int s = 0; s < kSer / 2; ++s) acc[j][s] = 0ull;
+      const int oe = min(no, or0 + kAdjRun);
+#pragma unroll 3
+      for (int o = or0; o < oe; ++o) {
+        const ulonglong2 c01 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec);
+        const ulonglong2 c23 = *reinterpret_cast<const ulonglong2 *>(rec + o * kRec + 4);
+        const float4 wv = *reinterpret_cast<const float4 *>(rec + o * kRec + slot::w);
+        const uint4 qo = *reinterpret_cast<const uint4 *>(rec + o * kRec + slot::q0);
+        const f32x2 c[4] = {c01.x, c01.y, c23.x, c23.y};
+        const float wt[4] = {wv.x, wv.y, wv.z, wv.w};
+        const float *gp = gw + o * win + lane;
+        const float *A[4] = {gp + (qo.x >> shift), gp + (qo.y >> shift), gp + (qo.z >> shift),
+                             gp + (qo.w >> shift)};
+        float gv[7];  // bins of intervals s - 2 .. s + 4 of the lane's first sample s
 #pragma unroll
-        for (int s = 0; s < kSer / 2; ++s) acc[j][s] = f2_fma(c[s], q2, acc[j][s]);
+        for (int i = 0; i < 7; ++i) gv[i] = A[i & 3][i >> 2];
+#pragma unroll
+        for (int j = 0; j < kAdjTK; ++j) {
+          float q = gather_q(wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
+          if (edge)
+            q += ghost_q(k0 + 4 * lane + j, a.nt, wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
+          const f32x2 q2 = f2_dup(q);
+#pragma unroll
+          for (int s = 0; s < kSer / 2; ++s) acc[j][s] = f2_fma(c[s], q2, acc[j][s]);
+        }
       }
+#pragma unroll
+      for (int j = 0; j < kAdjTK; ++j)
+#pragma unroll
+        for (int s = 0; s < kSer / 2; ++s) sum[j][s] = f2_add(sum[j][s], acc[j][s]);
     }
     float *out = a.Xbar + ((size_t)p * a.xb_ld + k0 + 4 * lane) * kSer;
 #pragma unroll
@@ -261,12 +283,12 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float4 v;
-          f2_split(acc[j][2 * h], v.x, v.y);
-          f2_split(acc[j][2 * h + 1], v.z, v.w);
+          f2_split(sum[j][2 * h], v.x, v.y);
+          f2_split(sum[j][2 * h + 1], v.z, v.w);
           red_add_v4(out + j * kSer + 4 * h, v);
         }
       } else {
-        stg256(out + j * kSer, acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+        stg256(out + j * kSer, sum[j][0], sum[j][1], sum[j][2], sum[j][3]);
       }
     }
     __syncwarp();  // every lane is done with this buffer before it is refilled

@@ -432,12 +432,22 @@ fwh_status ensure_events(fwh_handle h, int n) {
   return FWH_OK;
 }
 
-// Host fields of a mixed handle are copied in slabs of kSlab source frames; the
+// Host fields of a mixed handle are copied in slabs of source frames; the
 // series of slab q are prepared as soon as slab q + 1 (which holds the filters'
-// reach beyond it) has landed, and the forward scatter runs in segments of two
-// chunks, each as soon as its rows are prepared, so copy, prep and scatter
-// overlap and only the last slab's prep and segment follow the last copy.
-constexpr int kSlab = 128;
+// reach beyond it) has landed, and the forward scatter runs in segments of one
+// or two 128-row blocks, each as soon as its rows are prepared, so copy, prep
+// and scatter overlap and only the last slab's prep and segment follow the last
+// copy.  A slab is 64 frames where that is 16 MB or more (75 us at the link's 211
+// GB/s; 64 frames: 7.34 ms for 32768 panels x 2048 steps x 72 observers, 128 frames:
+// 7.70, 256: 8.01), else as many as hold 4 MB: the launches of a slab take about 20 us
+// of host time.
+constexpr int64_t kSlabMin = 128;  // frames: shorter records than two of these go in one copy
+int slab_frames(const fwh_ctx *h) {
+  const int64_t bytes = (int64_t)kRowBlk * 5 * h->P * (int64_t)sizeof(float);
+  if (bytes >= ((int64_t)16 << 20)) return kRowBlk;
+  const int64_t blocks = std::max<int64_t>(2, (((int64_t)4 << 20) + bytes - 1) / bytes);
+  return (int)std::min<int64_t>(blocks * kRowBlk, (int64_t)1 << 20);
+}
 
 template <typename T>
 fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStream_t s,
@@ -513,24 +523,29 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     // The copy stream first waits for the work already on `s` (the previous
     // call's scatter reads X and its prep the staging buffer), so every later
     // step of this call is ordered after it.
-    const int nslab = (int)((h->nt + kSlab - 1) / kSlab);
+    const int slab = slab_frames(h);
+    const int nslab = (int)((h->nt + slab - 1) / slab);
     const size_t row = (size_t)5 * h->P * sizeof(T);
     if (!h->copy) CK(h, cudaStreamCreateWithFlags(&h->copy, cudaStreamNonBlocking));
     fwh_status st1 = ensure_pstream(h);
     if (st1 != FWH_OK) return st1;
-    fa.seg_len = (c.tk > 4 ? 1 : 2) * fwd_chunk(fp64, c);
+    fa.seg_len = slab > 128 && c.tk > 4 ? fwd_chunk(fp64, c) : 124;  // one block: 124 intervals
     fa.n_segs = (fa.k_top + fa.seg_len - 1) / fa.seg_len;
-    st1 = ensure_events(h, 2 * nslab + 1);
+    // the short segment first: it runs under the copies, and what follows the
+    // last copy is one segment of whole chunks
+    fa.seg_shift = (fa.n_segs * fa.seg_len - fa.k_top) / 4 * 4;
+    st1 = ensure_events(h, 2 * nslab + 2);
     if (st1 != FWH_OK) return st1;
-    cudaEvent_t *ev_in = h->slab_ev.data(), *ev_x = ev_in + nslab, ev_go = ev_in[2 * nslab];
+    cudaEvent_t *ev_in = h->slab_ev.data(), *ev_x = ev_in + nslab, ev_go = ev_in[2 * nslab],
+                ev_end = ev_in[2 * nslab + 1];
     CK(h, cudaEventRecord(ev_go, s));
     CK(h, cudaStreamWaitEvent(h->copy, ev_go, 0));
-    constexpr int cps = kSlab / kRowBlk;  // prep blocks per slab
-    static_assert(kSlab % kRowBlk == 0, "slabs are whole prep blocks");
+    const int cps = slab / kRowBlk;  // prep blocks per slab
     int seg_done = 0;
     // scatter the segments whose rows lie below rows_ready (prepared by slab j)
     auto scatter_upto = [&](int rows_ready, int j) -> fwh_status {
-      const int ready = rows_ready >= x_ld ? fa.n_segs : (rows_ready - 3) / fa.seg_len;
+      const int ready =
+          rows_ready >= x_ld ? fa.n_segs : (rows_ready - 3 + fa.seg_shift) / fa.seg_len;
       if (ready <= seg_done) return FWH_OK;
       CK(h, cudaStreamWaitEvent(s, ev_x[j], 0));
       if (tev && seg_done == 0) CK(h, cudaEventRecord(tev[1], s));
@@ -542,7 +557,7 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     };
     for (int q = 0; q <= nslab; ++q) {
       if (q < nslab) {
-        const int64_t r0 = (int64_t)q * kSlab, r1 = std::min<int64_t>(h->nt, r0 + kSlab);
+        const int64_t r0 = (int64_t)q * slab, r1 = std::min<int64_t>(h->nt, r0 + slab);
         CK(h, cudaMemcpyAsync(const_cast<T *>(d_fields) + r0 * 5 * h->P,
                               host_fields + r0 * 5 * h->P, (size_t)(r1 - r0) * row,
                               cudaMemcpyHostToDevice, h->copy));
@@ -553,9 +568,21 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
       CK(h, cudaStreamWaitEvent(h->pstream, ev_in[std::min(q, nslab - 1)], 0));
       pa.c_lo = j * cps;
       pa.c_hi = q < nslab ? std::min(n_rb, q * cps) : n_rb;
+      const int c_end = pa.c_hi;
+      if (q == nslab) {
+        // the last slab: its record-end blocks beside its interior ones
+        pa.c_lo = std::max(j * cps, std::min(n_rb, prep_interior_end<T>(pa.nt)));
+        if (pa.c_lo > j * cps && pa.c_lo < n_rb) {
+          CK(h, launch_prep<T>(pa, h->copy));
+          CK(h, cudaEventRecord(ev_end, h->copy));
+          CK(h, cudaStreamWaitEvent(s, ev_end, 0));
+          pa.c_hi = pa.c_lo;
+        }
+        pa.c_lo = j * cps;
+      }
       CK(h, launch_prep<T>(pa, h->pstream));
       CK(h, cudaEventRecord(ev_x[j], h->pstream));
-      const fwh_status st2 = scatter_upto(pa.c_hi * kRowBlk, j);
+      const fwh_status st2 = scatter_upto(c_end * kRowBlk, j);
       if (st2 != FWH_OK) return st2;
     }
   }
@@ -967,7 +994,8 @@ fwh_status fwh_forward(fwh_handle h, const void *fields, int64_t nt, double *p_o
   const void *df = fields;
   double *dp = p_out;
   // mixed handles overlap the copy of host fields with the series prep
-  const bool slabs = !din && h->precision == FWH_MIXED && nt >= 2 * kSlab;
+  const bool slabs = !din && h->precision == FWH_MIXED && nt >= 2 * kSlabMin &&
+                     nt > slab_frames(h);
   if (!din) {
     CK(h, ensure(h->stage_in, fbytes));
     if (!slabs)

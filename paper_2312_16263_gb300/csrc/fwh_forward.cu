@@ -263,8 +263,8 @@ struct Item {
     opw = a.obs_per_cta / NW;
     o_begin = g * a.obs_per_cta;
     o_end = min(a.O, o_begin + a.obs_per_cta);
-    k_begin = q * a.seg_len;
-    k_end = min(a.k_top, k_begin + a.seg_len);
+    k_begin = max(0, q * a.seg_len - a.seg_shift);
+    k_end = min(a.k_top, (q + 1) * a.seg_len - a.seg_shift);
     nobs = 0;
     for (int m = 0; m < opw; ++m)
       if (o_begin + w + NW * m < o_end) nobs = m + 1;
@@ -525,8 +525,12 @@ __device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Ite
 //
 // Per (observer, 128-row block): 16 packed FMAs, 4 adds, 16 FMAs, 3 shuffles,
 // 4 window loads and stores and a share of the record's 4 loads and 4 address
-// adds: 13.1 warp instructions per 32 samples with two blocks.  On a GB300 the
-// sphere of 32768 panels x 2048 steps x 72 observers takes @FWD_MS@ ms; the
+// adds.  No one unit bounds it: with two blocks the shared-memory pipe is busy
+// about 77 % of the time (20 wavefronts per block: windows 8, records 4, X rows
+// 3.6, shuffles 3, flushes), issue 58 %, the FMA pipe 46 %; one block a chunk
+// lets 16 warps fit an SM instead of 12 but reads each record twice as often
+// (24 wavefronts): 3.58 ms.  On a GB300 the
+// sphere of 32768 panels x 2048 steps x 72 observers takes 3.43 ms; the
 // former kernel on samples and moments side by side (20 multiply-adds, 64-byte
 // rows, 22 instructions per 32 samples) took 4.57 ms.
 //
@@ -569,50 +573,90 @@ __device__ __forceinline__ unsigned stage_token(unsigned addr) {
   return r;
 }
 
-// The slots of one FP32 record that the consumer reads: c0..c7 as pairs, the
-// weights and the four window byte offsets.
+// The slots of one FP32 record that the consumer reads, in the groups it loads
+// them by: c0..c7 as pairs, the four window byte offsets, the weights.
+static_assert(slot::c == 0 && slot::w == 8 && slot::q0 == 12, "record read in 16-byte groups");
 struct Coef {
   unsigned long long c[4];
   float w[4];
   uint4 q;
+  __device__ __forceinline__ void load_c(unsigned rec) {
+    asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(c[0]), "=l"(c[1]) : "r"(rec));
+    asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(c[2]), "=l"(c[3]) : "r"(rec + 16));
+  }
+  __device__ __forceinline__ void load_w(unsigned rec) {
+    const float4 v = lds_v4f32(rec + 32);
+    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+  }
+  static __device__ __forceinline__ uint4 load_q(unsigned rec) {
+    uint4 v;
+    asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "r"(rec + 48));
+    return v;
+  }
 };
-__device__ __forceinline__ void lds_coef(unsigned rec, Coef &k) {
-  static_assert(slot::c == 0 && slot::w == 8 && slot::q0 == 12, "record read in 16-byte groups");
-  asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(k.c[0]), "=l"(k.c[1]) : "r"(rec));
-  asm("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(k.c[2]), "=l"(k.c[3]) : "r"(rec + 16));
-  const float4 w = lds_v4f32(rec + 32);
-  k.w[0] = w.x; k.w[1] = w.y; k.w[2] = w.z; k.w[3] = w.w;
-  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-      : "=r"(k.q.x), "=r"(k.q.y), "=r"(k.q.z), "=r"(k.q.w)
-      : "r"(rec + 48));
+
+// Compensated (Kahan) update of a window entry (sum, compensation) by y.
+__device__ __forceinline__ float2 kahan_add(float2 w, float y) {
+  const float yc = __fsub_rn(y, w.y);
+  const float t = __fadd_rn(w.x, yc);
+  return make_float2(t, __fsub_rn(__fsub_rn(t, w.x), yc));
 }
 
-// Value of a split-window entry: a plain FP32 sum, or a compensated pair
-// (sum, compensation) whose value is sum - compensation (formed in FP64).
+// A window entry: a plain FP32 sum, or a compensated pair (sum, compensation)
+// whose value is sum - compensation (formed in FP64).  add(): the four taps of
+// one bin (a compensated entry takes a panel's whole contribution at once).
 template <bool KAHAN> struct WinEntry;
 template <> struct WinEntry<false> {
   using E = float;
   static __device__ __forceinline__ bool nz(E e) { return e != 0.f; }
   static __device__ __forceinline__ double value(E e) { return (double)e; }
   static __device__ __forceinline__ E zero() { return 0.f; }
+  static __device__ __forceinline__ E load(unsigned addr) { return lds_win(addr); }
+  static __device__ __forceinline__ void store(unsigned addr, E v) { sts_f32(addr, v); }
+  static __device__ __forceinline__ E add(E s, const float (&w)[4], const float *g) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) s = fmaf(w[t], g[t], s);
+    return s;
+  }
 };
 template <> struct WinEntry<true> {
   using E = float2;
   static __device__ __forceinline__ bool nz(E e) { return e.x != 0.f || e.y != 0.f; }
   static __device__ __forceinline__ double value(E e) { return (double)e.x - (double)e.y; }
   static __device__ __forceinline__ E zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ E load(unsigned addr) {
+    float2 v;
+    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+  }
+  static __device__ __forceinline__ void store(unsigned addr, E v) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+  }
+  static __device__ __forceinline__ E add(E s, const float (&w)[4], const float *g) {
+    float y = w[0] * g[0];
+#pragma unroll
+    for (int t = 1; t < 4; ++t) y = fmaf(w[t], g[t], y);
+    return kahan_add(s, y);
+  }
 };
+
+// Window slots per observer of the FP32 shapes, fixed per chunk length so that
+// the hot loop addresses the windows with immediates.
+template <int TK>
+constexpr int win_f32() { return TK == 4 ? 224 : 352; }
 
 // Add the first n bins of an observer's window to p_out.  Lanes take
 // consecutive bins; the quarter length is 8 or 24 mod 32 words, so the eight
 // words of each quarter that a warp reads lie on distinct banks.
-template <bool KAHAN, int NW>
+template <int TK, bool KAHAN, int NW>
 __device__ __forceinline__ void flush_bins(const FwdArgs<float> &a, const Item<float, NW> &it,
                                            int w, int m, const void *wm, int wbase, int n) {
   using W = WinEntry<KAHAN>;
   const typename W::E *e = static_cast<const typename W::E *>(wm);
   const int lane = threadIdx.x & 31;
-  const int H = a.win >> 2;
+  constexpr int H = win_f32<TK>() / 4;
   const int o = it.o_begin + w + NW * m;
   const int nvalid = a.n_valid[o];
   double *po = a.p_out + (size_t)o * a.nt;
@@ -624,19 +668,20 @@ __device__ __forceinline__ void flush_bins(const FwdArgs<float> &a, const Item<f
 }
 
 // Flush the first CH (complete) bins of every window to p_out and slide.
-template <int CH, int NW, bool KAHAN>
+template <int TK, int NW, bool KAHAN>
 __device__ __forceinline__ void flush_slide_split(const FwdArgs<float> &a,
                                                   const Item<float, NW> &it, int w, float *wwin,
                                                   const int *s_i0max, int k0) {
   using W = WinEntry<KAHAN>;
   using E = typename W::E;
+  constexpr int H = win_f32<TK>() / 4, CH = chunk_of<float, TK>();
   const int lane = threadIdx.x & 31;
-  const int H = a.win >> 2;
   for (int m = 0; m < it.nobs; ++m) {
-    E *wm = reinterpret_cast<E *>(wwin + (size_t)m * a.wfl);
-    flush_bins<KAHAN, NW>(a, it, w, m, wm, k0 - s_i0max[m], CH);
+    E *wm = reinterpret_cast<E *>(wwin) + m * 4 * H;
+    flush_bins<TK, KAHAN, NW>(a, it, w, m, wm, k0 - s_i0max[m], CH);
     __syncwarp();
-    const int keep = H - CH / 4;  // <= CH / 4: no overlap
+    constexpr int keep = H - CH / 4;
+    static_assert(keep <= CH / 4, "no overlap");
     for (int i = lane; i < 4 * keep; i += 32) {
       E *q = wm + (i & 3) * H + (i >> 2);
       *q = q[CH / 4];
@@ -649,28 +694,15 @@ __device__ __forceinline__ void flush_slide_split(const FwdArgs<float> &a,
 
 // Segment end (k0: the interval after the last chunk): the remaining window
 // holds partial bins of the next segment.
-template <int CH, int NW, bool KAHAN>
+template <int TK, int NW, bool KAHAN>
 __device__ __forceinline__ void flush_tail_split(const FwdArgs<float> &a,
                                                  const Item<float, NW> &it, int w, float *wwin,
                                                  const int *s_i0max, int k0) {
+  constexpr int WIN = win_f32<TK>();
   for (int m = 0; m < it.nobs; ++m)
-    flush_bins<KAHAN, NW>(a, it, w, m, wwin + (size_t)m * a.wfl, k0 - s_i0max[m], a.win - CH);
+    flush_bins<TK, KAHAN, NW>(a, it, w, m, wwin + m * WIN * (KAHAN ? 2 : 1), k0 - s_i0max[m],
+                              WIN - chunk_of<float, TK>());
   __syncwarp();
-}
-
-// Compensated (Kahan) update of a window entry (sum, compensation) by y.
-__device__ __forceinline__ float2 kahan_add(float2 w, float y) {
-  const float yc = __fsub_rn(y, w.y);
-  const float t = __fadd_rn(w.x, yc);
-  return make_float2(t, __fsub_rn(__fsub_rn(t, w.x), yc));
-}
-__device__ __forceinline__ float2 lds_win2(unsigned addr) {
-  float2 v;
-  asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ void sts_f32x2(unsigned addr, float2 v) {
-  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 
 __device__ __forceinline__ void lds_v2f32x2(unsigned addr, f32x2 &a, f32x2 &b) {
@@ -683,14 +715,23 @@ __device__ __forceinline__ float f2_sum(f32x2 v) {
 }
 
 // One (chunk, panel) step: NA blocks of 128 rows (NA = 1: the last chunk of a
-// record, when its remaining intervals fit one block).
-template <int NA, int NW, bool PF, bool KAHAN>
+// segment, when its remaining intervals fit one block); `lanes` lanes of the
+// last block add their bins.
+//
+// The next observer's record is loaded piece by piece as this one's is used
+// up, always before this observer's stores: the compiler cannot move a shared
+// load above a store it cannot tell apart (3.43 ms; 3.50 with the record read
+// at the top of each observer).  Two observers at a time (168 registers): 4.1
+// ms; the last lane's stores predicated or sent to a spare slot instead of the
+// branch: 3.8 and 3.7 ms.
+template <int TK, int NA, int NW, bool KAHAN>
 __device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned crec,
-                                             unsigned win_s, unsigned win_b, unsigned xrow) {
-  constexpr unsigned RB = kRec * 4;         // record bytes
+                                             unsigned win_s, unsigned xrow, int lanes) {
+  constexpr unsigned RB = kRec * 4;           // record bytes
   constexpr unsigned BB = KAHAN ? 256 : 128;  // window bytes of 32 words of a quarter
+  constexpr unsigned WB = win_f32<TK>() * (KAHAN ? 8u : 4u);  // window bytes
   const int lane = threadIdx.x & 31;
-  const bool first = lane == 0, inner = lane < 31;
+  const bool first = lane == 0, inner = lane < lanes;
   f32x2 XP[NA][4][4];  // [block][row][pair of series]
   const unsigned xb = stg + xrow;
 #pragma unroll
@@ -702,89 +743,65 @@ __device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned cr
   // window base of this panel's updates, ordered after the previous panel's
   // stores (see lds_win)
   const unsigned wtok = stage_token(win_s);
-  auto observer = [&](int m, const Coef &k) {
-    const unsigned base = wtok + (unsigned)m * win_b;
-    const unsigned A[4] = {base + k.q.x, base + k.q.y, base + k.q.z, base + k.q.w};
+  // one observer: window m, its record in k; `next`: the record to load
+  using W = WinEntry<KAHAN>;
+  auto observer = [&](int m, Coef &k, unsigned next) {
+    const unsigned A[4] = {wtok + k.q.x + m * WB, wtok + k.q.y + m * WB, wtok + k.q.z + m * WB,
+                           wtok + k.q.w + m * WB};
+    typename W::E s[NA][4];
+#pragma unroll
+    for (int b = 0; b < NA; ++b)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[b][j] = W::load(A[j] + BB * b);
+    k.q = Coef::load_q(next);
     float g[NA][7];
-    auto dots = [&]() {
 #pragma unroll
-      for (int b = 0; b < NA; ++b) {
+    for (int b = 0; b < NA; ++b)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          f32x2 v = f2_mul(k.c[0], XP[b][j][0]);
+      for (int j = 0; j < 4; ++j) {
+        f32x2 v = f2_mul(k.c[0], XP[b][j][0]);
 #pragma unroll
-          for (int q = 1; q < 4; ++q) v = f2_fma(k.c[q], XP[b][j][q], v);
-          g[b][j] = f2_sum(v);
-        }
+        for (int q = 1; q < 4; ++q) v = f2_fma(k.c[q], XP[b][j][q], v);
+        g[b][j] = f2_sum(v);
       }
+    k.load_c(next);
 #pragma unroll
-      for (int b = 0; b < NA; ++b)
+    for (int b = 0; b < NA; ++b)
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-          // lane 0 serves lane 31 with the next block's first rows
-          g[b][4 + i] = b + 1 < NA ? __shfl_sync(0xffffffffu, first ? g[b + 1][i] : g[b][i],
-                                                 (lane + 1) & 31)
-                                   : __shfl_down_sync(0xffffffffu, g[b][i], 1);
-    };
-    if constexpr (!KAHAN) {
-      float s[NA][4];
+      for (int t = 0; t < 3; ++t)
+        // lane 0 serves lane 31 with the next block's first rows
+        g[b][4 + t] = b + 1 < NA ? __shfl_sync(0xffffffffu, first ? g[b + 1][t] : g[b][t],
+                                               (lane + 1) & 31)
+                                 : __shfl_down_sync(0xffffffffu, g[b][t], 1);
 #pragma unroll
-      for (int b = 0; b < NA; ++b)
+    for (int b = 0; b < NA; ++b)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[b][j] = lds_win(A[j] + BB * b);
-      dots();
+      for (int j = 0; j < 4; ++j) s[b][j] = W::add(s[b][j], k.w, &g[b][j]);
+    k.load_w(next);
 #pragma unroll
-      for (int b = 0; b < NA; ++b)
+    for (int b = 0; b < NA; ++b)
+      if (b + 1 < NA || inner) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int t = 0; t < 4; ++t) s[b][j] = fmaf(k.w[t], g[b][j + t], s[b][j]);
-#pragma unroll
-      for (int b = 0; b < NA; ++b)
-        if (b + 1 < NA || inner) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) sts_f32(A[j] + BB * b, s[b][j]);
-        }
-    } else {
-      // compensated: each slot is (sum, compensation); every panel's
-      // contribution to a slot is formed first, then added by Kahan's rule
-      float2 s[NA][4];
-#pragma unroll
-      for (int b = 0; b < NA; ++b)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) s[b][j] = lds_win2(A[j] + BB * b);
-      dots();
-#pragma unroll
-      for (int b = 0; b < NA; ++b)
-        if (b + 1 < NA || inner) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            float y = k.w[0] * g[b][j];
-#pragma unroll
-            for (int t = 1; t < 4; ++t) y = fmaf(k.w[t], g[b][j + t], y);
-            sts_f32x2(A[j] + BB * b, kahan_add(s[b][j], y));
-          }
-        }
-    }
+        for (int j = 0; j < 4; ++j) W::store(A[j] + BB * b, s[b][j]);
+      }
   };
-  // PF: read the next observer's record while this one computes, else read
-  // each record right before its use.  A warp with the full count of
-  // observers runs them without an exit test, so the compiler may overlap one
-  // observer's tail with the next one's loads and arithmetic.
+  // A warp with the full count of observers runs them without an exit test,
+  // so the compiler may overlap one observer's tail with the next one's loads
+  // and arithmetic.
   auto run = [&](auto full) {
     constexpr bool kFull = decltype(full)::value;
     const int n = kFull ? kMaxObsPerWarpF32 : nobs;
+    if (n == 0) return;
     auto rec = [&](int m) { return crec + (unsigned)m * NW * RB; };
     Coef k;
-    if (PF && n > 0) lds_coef(rec(0), k);
+    k.q = Coef::load_q(rec(0));
+    k.load_c(rec(0));
+    k.load_w(rec(0));
 #pragma unroll
     for (int m = 0; m < kMaxObsPerWarpF32; ++m) {
       if (!kFull && m >= n) break;
-      if (!PF) lds_coef(rec(m), k);
-      Coef kn;
-      if (PF && m + 1 < n) lds_coef(rec(m + 1), kn);
-      observer(m, k);
-      if (PF) k = kn;
+      // (the last one loads its own record again)
+      observer(m, k, rec(m + 1 < n ? m + 1 : m));
     }
   };
   if (nobs == kMaxObsPerWarpF32)
@@ -793,7 +810,7 @@ __device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned cr
     run(std::false_type{});
 }
 
-template <int TK, int NW, bool PF, bool KAHAN>
+template <int TK, int NW, bool KAHAN>
 __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
                                                  const Item<float, NW> &it,
                                                  const PipeState &ps, unsigned &step,
@@ -802,7 +819,6 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
   constexpr int CH = chunk_of<float, TK>();
   const int lane = threadIdx.x & 31;
   item_prologue<float, NW>(a, it, w, wwin, s_i0max);
-  const unsigned win_b = (unsigned)a.wfl * 4u;
   const unsigned win_s = smem_u32(wwin) + (unsigned)lane * (KAHAN ? 8u : 4u);
   const unsigned stage0 = smem_u32(ps.stage0);
   // X line lane + 32 b of a stage: 16-byte chunk c at c ^ (lane & 7).  Stages
@@ -813,14 +829,17 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
   int k0 = it.k_begin;
   for (; k0 < it.k_end; k0 += CH) {
     const bool one = NB > 1 && it.k_end - k0 <= 124;
+    // lanes of the last block whose bins belong to this chunk (a segment that
+    // ends inside the record ends at a multiple of four intervals)
+    const int lanes = min(31, (it.k_end - k0 - (one ? 0 : 128 * (NB - 1)) + 3) >> 2);
     for (int p = it.p_begin; p < it.p_end; ++p, ++step) {
       if (!mbar_wait(&ps.full[s], ph, ps.err, ps.abort, ps.wait_cycles)) return;
       const unsigned stg = stage_token(stage0 + s * ps.stage_bytes);
       const unsigned crec = stg + ps.x_bytes + (unsigned)w * (kRec * 4);
       if (one)
-        consume_step<1, NW, PF, KAHAN>(it.nobs, stg, crec, win_s, win_b, xrow);
+        consume_step<TK, 1, NW, KAHAN>(it.nobs, stg, crec, win_s, xrow, lanes);
       else
-        consume_step<NB, NW, PF, KAHAN>(it.nobs, stg, crec, win_s, win_b, xrow);
+        consume_step<TK, NB, NW, KAHAN>(it.nobs, stg, crec, win_s, xrow, lanes);
       __syncwarp();
       if (lane == 0) mbar_arrive(&ps.empty[s]);
       if (++s == (unsigned)ps.nst) {
@@ -828,9 +847,9 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
         ph ^= 1u;
       }
     }
-    flush_slide_split<CH, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
+    flush_slide_split<TK, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
   }
-  flush_tail_split<CH, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
+  flush_tail_split<TK, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
 }
 
 // Wait until every copy the producer issued has landed, always with the full
@@ -890,8 +909,8 @@ __device__ __forceinline__ void forward_cta(const FwdArgs<T> &a, const void *tma
     __shared__ __align__(8) uint64_t bars[2 * kMaxStages];
     __shared__ int abort_flag;
     PipeState ps;
-    unsigned char *wbase = pipe_setup<T, TK, NW>(smem_raw, a.obs_per_cta, nst, bars,
-                                                 &abort_flag, ps);
+    unsigned char *wbase = pipe_setup<T, TK, NW>(smem_raw, a.obs_per_cta, nst, bars, &abort_flag,
+                                                 ps);
     ps.tmap = tmap;
     ps.err = err;
     ps.wait_cycles = wait_cycles;
@@ -907,8 +926,7 @@ __device__ __forceinline__ void forward_cta(const FwdArgs<T> &a, const void *tma
       const Item<T, NW> it(a, item, w);
       T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
       if constexpr (sizeof(T) == 4)
-        consume_item_f32<TK, NW, ACC >= 4, ACC == 5>(a, it, ps, step, wwin,
-                                                     st + w * kMaxObsPerWarp, w);
+        consume_item_f32<TK, NW, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
       else
         consume_item<TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
     }
@@ -969,15 +987,18 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
   }
   __syncthreads();
   const int w = threadIdx.x >> 5;
-  if constexpr (PIPE == 1) {
-    PipeState ps;
+  PipeState ps;
+  unsigned char *wbase = smem_raw;
+  unsigned step = 0;
+  if constexpr (PIPE != 0) {
     int maxo = 0;
     for (int i = 0; i < n_surf; ++i) maxo = max(maxo, args[i].obs_per_cta);
     // (its barrier also orders the item ring's initialisation above)
-    unsigned char *wbase = pipe_setup<T, TK, NW>(smem_raw, maxo, nst, bars, &abort_flag, ps);
+    wbase = pipe_setup<T, TK, NW>(smem_raw, maxo, nst, bars, &abort_flag, ps);
     ps.err = args[0].err;
     ps.wait_cycles = args[0].wait_cycles;
-    unsigned step = 0;
+  }
+  if constexpr (PIPE == 1) {
     volatile int *abort = &abort_flag;
     if (w == NW) {
       if ((threadIdx.x & 31) == 0) {
@@ -1009,8 +1030,7 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
         const Item<T, NW> it(a, item - prefix[sf], w);
         T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
         if constexpr (sizeof(T) == 4)
-          consume_item_f32<TK, NW, ACC >= 4, ACC == 5>(a, it, ps, step, wwin,
-                                                       st + w * kMaxObsPerWarp, w);
+          consume_item_f32<TK, NW, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
         else
           consume_item<TK, NW>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
         if (*abort) break;
@@ -1022,10 +1042,10 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
       const int item = s_item;
       __syncthreads();  // every thread has read it
       if (item >= total) break;
-      const int lo = batch_surface(prefix, n_surf, item);
+      const int sf = batch_surface(prefix, n_surf, item);
       // a reference, not a copy: the fields are read from the parameter block
       // where used, instead of holding the whole argument block in registers
-      process_item_direct<TK, NW>(args[lo], item - prefix[lo], reinterpret_cast<T *>(smem_raw), st);
+      process_item_direct<TK, NW>(args[sf], item - prefix[sf], reinterpret_cast<T *>(smem_raw), st);
       if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
     }
   }
@@ -1060,29 +1080,30 @@ __global__ void __launch_bounds__((cta_threads<NW, PIPE>()), (MinBlocks<TK, NW, 
 
 // Candidate tile shapes {pipe, tk, warps, obs_per_warp, win, seg_chunks,
 // stages, acc}.  FP32 (always TMA): tk 4 or 8 (one or two 128-row blocks per
-// chunk); acc 3 plain window sums, 4 the same with the next observer's record
-// read ahead, 5 as 4 with compensated (Kahan) window sums.  win / 4 is 8 or 24
-// mod 32 (see flush_bins).
+// chunk); acc 3 plain window sums, 5 compensated (Kahan) ones.  win / 4 is 8
+// or 24 mod 32 (see flush_bins).
 constexpr FwdConfig kCfgF32[] = {
-    {1, 8, 4, 9, 352, 2, 2, 4},
-    {1, 8, 4, 9, 352, 1, 2, 4},
     {1, 8, 4, 9, 352, 2, 2, 3},
-    {1, 4, 4, 9, 224, 4, 3, 4},
-    {1, 4, 8, 9, 224, 4, 3, 4},
-    {1, 8, 4, 9, 352, 2, 3, 3},
+    {1, 8, 4, 9, 352, 1, 2, 3},
     {1, 4, 4, 9, 224, 4, 3, 3},
-    {1, 8, 4, 9, 352, 4, 2, 4},
-    {1, 4, 4, 9, 224, 8, 3, 4},
-    {1, 8, 4, 9, 288, 2, 2, 4},
-    {1, 4, 4, 9, 160, 4, 2, 5},
+    {1, 4, 8, 9, 224, 4, 3, 3},
+    {1, 8, 4, 9, 352, 3, 2, 3},
+    {1, 8, 4, 9, 352, 2, 3, 3},
+    {1, 4, 4, 9, 224, 2, 3, 3},
+    {1, 8, 4, 9, 352, 4, 2, 3},
+    {1, 4, 4, 9, 224, 8, 3, 3},
+    {1, 4, 4, 9, 224, 4, 2, 3},
+    {1, 4, 4, 9, 224, 4, 2, 5},
     {1, 4, 4, 9, 224, 4, 3, 5},
 };
 constexpr bool f32_obs_fit() {
   for (const FwdConfig &c : kCfgF32)
-    if (c.obs_per_warp > kMaxObsPerWarpF32) return false;
+    if (c.obs_per_warp > kMaxObsPerWarpF32 ||
+        c.win != (c.tk == 4 ? win_f32<4>() : win_f32<8>()))
+      return false;
   return true;
 }
-static_assert(f32_obs_fit(), "an FP32 shape has more observers per warp than the unrolled loop");
+static_assert(f32_obs_fit(), "FP32 shapes: observers per warp and window slots of the unrolled loop");
 const FwdConfig kCfgF64[] = {
     {0, 2, 8, 16, 128, 8, 0, 0},
     {1, 2, 8, 9, 128, 8, 3, 0},
@@ -1183,17 +1204,14 @@ bool encode_x_tensor_map(void *out128, const void *X, unsigned long long rows, b
   return r == CUDA_SUCCESS;
 }
 
-// Instantiated shapes: FP32 {one or two blocks with and without the record
-// read ahead, one block with 8 warps, one block compensated}; FP64 {direct
-// 2x8, TMA 2x8, direct 2x4, direct 1x8}.
+// Instantiated shapes: FP32 {two blocks; one block with 4 and 8 warps; one
+// block compensated}; FP64 {direct 2x8, TMA 2x8, direct 2x4, direct 1x8}.
 #define FWH_DISPATCH(T, c, CALL)                                                        \
   do {                                                                                   \
     if constexpr (sizeof(T) == 4) {                                                      \
-      if (c.tk == 8 && c.warps == 4 && c.acc == 4) return CALL(T, 8, 4, 1, 4);           \
       if (c.tk == 8 && c.warps == 4 && c.acc == 3) return CALL(T, 8, 4, 1, 3);           \
-      if (c.tk == 4 && c.warps == 4 && c.acc == 4) return CALL(T, 4, 4, 1, 4);           \
       if (c.tk == 4 && c.warps == 4 && c.acc == 3) return CALL(T, 4, 4, 1, 3);           \
-      if (c.tk == 4 && c.warps == 8 && c.acc == 4) return CALL(T, 4, 8, 1, 4);           \
+      if (c.tk == 4 && c.warps == 8 && c.acc == 3) return CALL(T, 4, 8, 1, 3);           \
       if (c.tk == 4 && c.warps == 4 && c.acc == 5) return CALL(T, 4, 4, 1, 5);           \
     } else {                                                                             \
       if (c.pipe == 0 && c.tk == 2 && c.warps == 8) return CALL(T, 2, 8, 0, 0);          \

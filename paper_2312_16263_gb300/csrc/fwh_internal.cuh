@@ -82,6 +82,11 @@ __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
@@ -147,6 +152,7 @@ struct FwdArgs {
   int obs_per_cta, n_obs_groups;
   int subs;             // work items a panel set is cut into
   int seg_len, n_segs;
+  int seg_shift;        // segment q ends at interval (q + 1) seg_len - seg_shift (a multiple of 4)
   int seg_lo, seg_cnt;  // this launch covers time segments [seg_lo, seg_lo + seg_cnt)
   int win;              // window slots per observer
   int wfl;              // values per observer window: win, or 2 win for compensated
@@ -194,6 +200,12 @@ template <typename T>
 cudaError_t launch_coef(const GeomArgs &a, T *coef, int *i0, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prep(const PrepArgs<T> &a, cudaStream_t s);
+// The interior blocks of a record's prep are [1, this).
+template <typename T>
+constexpr int prep_interior_end(int nt) {
+  const int top = nt - kRowBlk - Prec<T>::halo - 1;
+  return top >= kRowBlk ? top / kRowBlk + 1 : 1;
+}
 template <typename T>
 cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s);
 template <typename T>
@@ -208,8 +220,7 @@ struct FwdConfig {
   int win;            // window slots per observer
   int seg_chunks;     // chunks per time segment
   int stages;         // pipeline stages (pipe = 1)
-  int acc;            // FP64: 0.  FP32 window sums: 3 plain, 4 plain with the next record
-                      // read ahead, 5 compensated (Kahan)
+  int acc;            // FP64: 0.  FP32 window sums: 3 plain, 5 compensated (Kahan)
 };
 // Source samples a chunk completes: FP64 lanes hold rows 32 apart; FP32 lanes
 // hold four consecutive rows per 128-row block, and the last lane's serve only

@@ -64,7 +64,7 @@ constexpr int kIntThreads = kIntPanels * 4;
 constexpr int kIntRow = kIntPanels * 4;              // staged row: [panel][integrand]
 constexpr int kIntRows = kIirChunk + 2 * kIirH + 3;  // samples c0 - H - 2 .. c0 + 64 + H
 constexpr int kIntKeep = kIntRows - kIirChunk;       // rows shared by consecutive blocks
-constexpr int kIntUnit = 8;                          // blocks per work unit
+constexpr int kIntUnit = 8;                          // most blocks per work unit
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool ok) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -86,7 +86,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float> a) {
+__global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float> a, int unit) {
   constexpr int NP = kIntPanels, H = kIirH, C = kIirChunk;
   constexpr float rho = -0.267949192431122706f;  // sqrt(3) - 2
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
   const int n_blk = a.int_hi - a.int_lo;
-  const int n_us = (n_blk + kIntUnit - 1) / kIntUnit;
+  const int n_us = (n_blk + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   // phase A thread: panel pa, rows tid / NP + 4 u
   const int pa = tid % NP;
@@ -107,8 +107,8 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     // panel group fastest: concurrent units read neighbouring segments of the same rows
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = a.int_lo + (int)(u / n_pg) * kIntUnit;
-    const int b1 = min(a.int_lo + n_blk, b0 + kIntUnit);
+    const int b0 = a.int_lo + (int)(u / n_pg) * unit;
+    const int b1 = min(a.int_lo + n_blk, b0 + unit);
     const int p = p0 + pa;
     const bool live = p < a.P;
     float n0 = 0.f, n1 = 0.f, n2 = 0.f, Un = 0.f;
@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
 // block, in place of the integrand), so per sample the integrands are formed
 // once, the causal step runs once and the anti-causal one 1.5 times (64 + 34
 // rows per 64): about 36 FP64 operations per (panel, sample).
-// @PREP64@
+// 32768 panels x 2048 steps: 8.7 ms with the record ends (15.2 ms by windowed
+// elimination, 142 operations and 128-byte rows).
 // ---------------------------------------------------------------------------
 constexpr int kF64H = Prec<double>::halo;
 constexpr int kF64Rows = kIirChunk + kF64H + 2;  // samples c0 - 1 .. c0 + 64 + H
@@ -250,14 +251,14 @@ __device__ __forceinline__ void issue_rows_f64(const double *fields, int P, int 
   }
 }
 
-__global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a) {
+__global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a, int unit) {
   constexpr int NP = kIntPanels, C = kIirChunk, H = kF64H, R = kF64Rows;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *win = reinterpret_cast<double *>(smem_raw);  // [R][NP][4]
   double *raw = win + R * kIntRow;                     // [C][5][NP]
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
-  const int n_us = (a.int_hi - a.int_lo + kIntUnit - 1) / kIntUnit;
+  const int n_us = (a.int_hi - a.int_lo + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   const int pa = tid % NP;               // integrand phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
@@ -265,8 +266,8 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   const bool vec = (a.P & 1) == 0 && ((size_t)a.fields & 15) == 0;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = a.int_lo + (int)(u / n_pg) * kIntUnit;
-    const int b1 = min(a.int_hi, b0 + kIntUnit);
+    const int b0 = a.int_lo + (int)(u / n_pg) * unit;
+    const int b1 = min(a.int_hi, b0 + unit);
     const int p = p0 + pa, pb = p0 + pl;
     double n0 = 0, n1 = 0, n2 = 0, Un = 0;
     if (p < a.P) {
@@ -548,7 +549,9 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_ii
 // column of the window holds the causal recursion's y (carried on from block
 // to block), then the integrand gradients, in place; the Jacobian phase takes
 // (sample, panel) pairs, so field reads and gradient writes are coalesced.
-// @PADJ@
+// Each thread's Xbar rows of the next 16 samples are in flight while it works on
+// these, and the block's fields are copied to shared memory behind the
+// anti-causal pass.
 // ---------------------------------------------------------------------------
 template <typename T> struct Pair;
 template <> struct Pair<float> { using V = float2; };
@@ -572,8 +575,8 @@ __device__ __forceinline__ void put_grad(T *g, size_t P, const T *f, T qb, T lb0
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
-    k_prep_adj_int(PrepAdjArgs<T> a, int int_lo, int int_hi) {
+__global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
+    k_prep_adj_int(PrepAdjArgs<T> a, int int_lo, int int_hi, int unit) {
   constexpr int NP = kIntPanels, C = kIirChunk, H = Prec<T>::halo, R = C + H;
   constexpr int BT = 16;  // rows in flight per thread
   static_assert(C % BT == 0 && H % BT == 0, "row batches");
@@ -581,9 +584,10 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
   constexpr T rho = (T)kRho, six = (T)(-6.0 * kRho);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *win = reinterpret_cast<T *>(smem_raw);  // [R][NP][4]: samples c0 .. c0 + R - 1
+  T *fld = win + R * kIntRow;                // [C][4][NP]: rho', u' of the block
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
-  const int n_us = (int_hi - int_lo + kIntUnit - 1) / kIntUnit;
+  const int n_us = (int_hi - int_lo + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   const int pa = tid % NP;               // Jacobian phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
@@ -591,8 +595,8 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
   const size_t P = a.P;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = int_lo + (int)(u / n_pg) * kIntUnit;
-    const int b1 = min(int_hi, b0 + kIntUnit);
+    const int b0 = int_lo + (int)(u / n_pg) * unit;
+    const int b1 = min(int_hi, b0 + unit);
     const int p = p0 + pa, pb = min(p0 + pl, a.P - 1);
     const bool live = p < a.P;
     T n0 = 0, n1 = 0, n2 = 0, Un = 0;
@@ -609,13 +613,21 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
     T *const col = win + pl * 4 + qi;
     T yy = T(0);
     int k = b0 * C - H;  // next sample of the causal recursion
+    const int k_last = (b1 - 1) * C + R;  // last sample it reads
     V cur = X(k);
     T dm = X(k - 1).x;   // derivative gradient one sample back
+    V nx[BT];            // the next batch, in flight
+    auto fetch = [&]() {
+#pragma unroll
+      for (int i = 0; i < BT; ++i) nx[i] = X(min(k + 1 + i, k_last));
+    };
     // BT samples of the recursion; y of each to col (row `w` on) unless w < 0
     auto causal = [&](int w) {
       V x[BT];
 #pragma unroll
-      for (int i = 0; i < BT; ++i) x[i] = X(k + 1 + i);
+      for (int i = 0; i < BT; ++i) x[i] = nx[i];
+      k += BT;
+      fetch();
 #pragma unroll
       for (int i = 0; i < BT; ++i) {
         yy = fma(rho, yy, fma(dm - x[i].x, inv2h, cur.y));
@@ -623,12 +635,25 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
         dm = cur.x;
         cur = x[i];
       }
-      k += BT;
+    };
+    fetch();
+    // the block's fields in flight to shared memory (read by the Jacobian phase)
+    auto issue_fields = [&](int b) {
+      const T *f0 = a.fields + (size_t)b * C * 5 * P + (live ? p : 0);
+#pragma unroll 4
+      for (int rc = tid / NP; rc < 4 * C; rc += kIntThreads / NP) {
+        const T *src = f0 + (size_t)((rc >> 2) * 5 + (rc & 3)) * P;
+        if constexpr (sizeof(T) == 4)
+          cp_async4(fld + rc * NP + pa, src, live);
+        else
+          cp_async8(fld + rc * NP + pa, src, live);
+      }
     };
     __syncthreads();  // the previous unit's Jacobian phase is done with win
     for (int i = 0; i < H; i += BT) causal(-1);
     for (int i = 0; i < R; i += BT) causal(i);
     for (int b = b0; b < b1; ++b) {
+      issue_fields(b);
       T xx = T(0);
 #pragma unroll 16
       for (int r = R - 1; r >= C; --r) xx = fma(rho, xx, col[r * kIntRow]);
@@ -637,12 +662,13 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 10 : 4)
         xx = fma(rho, xx, col[r * kIntRow]);
         col[r * kIntRow] = six * xx;
       }
+      cp_async_wait_all();
       __syncthreads();
       if (live) {
 #pragma unroll 4
         for (int r = tid / NP; r < C; r += kIntThreads / NP) {
-          const T *f = a.fields + (size_t)(b * C + r) * 5 * P + p;
-          const T fv[4] = {f[0], f[P], f[2 * P], f[3 * P]};
+          const T *f = fld + r * 4 * NP + pa;
+          const T fv[4] = {f[0], f[NP], f[2 * NP], f[3 * NP]};
           const T *q = win + r * kIntRow + pa * 4;
           put_grad<T>(a.grad_fields + (size_t)(b * C + r) * 5 * P + p, P, fv, q[0], q[1], q[2],
                       q[3], n0, n1, n2, Un);
@@ -859,9 +885,12 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 5 : 2)
 
 }  // namespace
 
-// Persistent CTAs of an interior kernel: as many as fit the GPU at once.
+// Persistent CTAs of an interior kernel over `blocks` blocks of n_pg panel
+// groups: as many as fit the GPU at once, and the blocks of a work unit (at
+// most kIntUnit: a unit starts with half a block's worth of extra rows), fewer
+// where the GPU would otherwise not be filled twice over.
 template <typename K>
-cudaError_t persistent_grid(K kern, size_t smem, long units, long *grid) {
+cudaError_t persistent_grid(K kern, size_t smem, long n_pg, int blocks, int *unit, long *grid) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -871,13 +900,16 @@ cudaError_t persistent_grid(K kern, size_t smem, long units, long *grid) {
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIntThreads, smem)) !=
       cudaSuccess)
     return e;
-  *grid = std::min<long>(units, (long)std::max(per_sm, 1) * sms);
+  const long fit = (long)std::max(per_sm, 1) * sms;
+  *unit = (int)std::clamp<long>(n_pg * blocks / (2 * fit), 1, kIntUnit);
+  *grid = std::min<long>(n_pg * ((blocks + *unit - 1) / *unit), fit);
   return cudaSuccess;
 }
 
 template <typename T>
 cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
-  constexpr int H = Prec<T>::halo, C = kIirChunk;
+  constexpr int C = kIirChunk;
+  static_assert(C == kRowBlk && C - 1 >= Prec<T>::halo + 2, "block 1 is an interior one");
   PrepArgs<T> a = a0;
   const int n_rb = (int)(x_rows(a.nt) / C);
   if (a.c_hi == 0) {
@@ -889,24 +921,25 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
     return cudaErrorInvalidValue;
   // interior blocks (first sample c0 = 64 b - 1): filter reach inside samples
   // 1 .. nt - 2, c0 >= H + 2 and c0 + C + H + 1 <= nt - 1
-  static_assert(C - 1 >= H + 2, "block 1 is an interior one");
-  const int last_int = a.nt >= C + H + 1 ? (a.nt - C - H - 1) / C : -1;
   a.int_lo = std::max(a.c_lo, 1);
-  a.int_hi = std::min(a.c_hi, last_int + 1);
+  a.int_hi = std::min(a.c_hi, prep_interior_end<T>(a.nt));
   if (a.int_lo >= a.int_hi) a.int_lo = a.int_hi = a.c_hi;
   cudaError_t e;
   if (a.int_hi > a.int_lo) {
-    const long units = (long)((a.P + kIntPanels - 1) / kIntPanels) *
-                       ((a.int_hi - a.int_lo + kIntUnit - 1) / kIntUnit);
+    const long n_pg = (a.P + kIntPanels - 1) / kIntPanels;
+    const int n_blk = a.int_hi - a.int_lo;
     long grid = 0;
+    int unit = 1;
     if constexpr (sizeof(T) == 4) {
       const size_t smem = ((size_t)kIntRows * kIntRow + (size_t)C * 5 * kIntPanels) * sizeof(T);
-      if ((e = persistent_grid(k_prep_iir_int, smem, units, &grid)) != cudaSuccess) return e;
-      k_prep_iir_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a);
+      if ((e = persistent_grid(k_prep_iir_int, smem, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+        return e;
+      k_prep_iir_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     } else {
       const size_t smem = ((size_t)kF64Rows * kIntRow + (size_t)C * 5 * kIntPanels) * sizeof(T);
-      if ((e = persistent_grid(k_prep_f64_int, smem, units, &grid)) != cudaSuccess) return e;
-      k_prep_f64_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a);
+      if ((e = persistent_grid(k_prep_f64_int, smem, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+        return e;
+      k_prep_f64_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -935,12 +968,14 @@ cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s) {
   if (int_hi <= int_lo) int_lo = int_hi = 0;
   cudaError_t e;
   if (int_hi > int_lo) {
-    const long units = (long)((a.P + kIntPanels - 1) / kIntPanels) *
-                       ((int_hi - int_lo + kIntUnit - 1) / kIntUnit);
-    const size_t smem = (size_t)(C + H) * kIntRow * sizeof(T);
+    const long n_pg = (a.P + kIntPanels - 1) / kIntPanels;
+    const size_t smem = ((size_t)(C + H) * kIntRow + (size_t)C * 4 * kIntPanels) * sizeof(T);
     long grid = 0;
-    if ((e = persistent_grid(k_prep_adj_int<T>, smem, units, &grid)) != cudaSuccess) return e;
-    k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, int_lo, int_hi);
+    int unit = 1;
+    if ((e = persistent_grid(k_prep_adj_int<T>, smem, n_pg, int_hi - int_lo, &unit, &grid)) !=
+        cudaSuccess)
+      return e;
+    k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, int_lo, int_hi, unit);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const long ends = (long)(n_ct - (int_hi - int_lo)) * tiles;
