@@ -303,9 +303,9 @@ fwh_status fwh_forward_noalloc(fwh_handle h, const void *fields, int64_t nt, dou
  * fwh_observer_window), fs > 0 the sampling rate (1/dt for the observer
  * grid), nperseg a power of two in [16, 4096], psd [n_sig][nperseg/2 + 1]
  * doubles (host or device) at frequencies k fs / nperseg.  A signal shorter
- * than one segment gets NaN in every bin.  Computed in FP64, one CTA per
- * signal, on `stream`; host buffers are staged and the call then
- * synchronises.  Errors: FWH_ERR_ARG (sizes, ranges, null pointers),
+ * than one segment gets NaN in every bin.  Computed in FP64 on `stream`; host
+ * buffers are staged and the call then synchronises (host n_valid of up to
+ * 1024 signals is passed by value instead).  Errors: FWH_ERR_ARG (sizes, ranges, null pointers),
  * FWH_ERR_OOM / FWH_ERR_CUDA (message via fwh_last_error(NULL)).
  */
 fwh_status fwh_psd(int64_t n_sig, const double *p, int64_t ld, const int64_t *n_valid,
@@ -335,17 +335,19 @@ fwh_status fwh_psd(int64_t n_sig, const double *p, int64_t ld, const int64_t *n_
  * of the last frame's, N_o = floor((t_end - t_start) / dt) + 1.  Each panel's
  * signal and arrival time are natural cubic splines over tau; bin j takes the
  * signal at the tau* whose arrival is t_j.  The motion must stay subsonic
- * (|M_r| < 1).  Device scratch of 32 nt P bytes per observer, up to
- * the budget of fwh_set_moving_scratch (16 GiB by default; observers are
- * split over launches that fit it, at least one observer per launch), is
- * taken with cudaMallocAsync on `stream`; the call synchronises.
+ * (|M_r| < 1).  Device scratch of 16 nt P bytes per observer (counted as 32 in
+ * the budget of fwh_set_moving_scratch, 16 GiB by default; observers are
+ * split over launches that fit it, at least one observer per launch) and
+ * 128 nt P bytes is taken on `stream` from a memory pool of the library, which
+ * keeps up to 8 GiB between calls; the call synchronises.
  * Errors: FWH_ERR_ARG (sizes, |w| >= c0, non-positive c0, rho0, dt),
  * FWH_ERR_OOM / FWH_ERR_CUDA (message via fwh_last_error(NULL)).
  */
 /*
  * Scratch budget in bytes of later fwh_forward_moving calls, process-wide
  * (0 restores the default of 16 GiB).  Smaller budgets split the observers
- * over more, smaller launches.  Errors: FWH_ERR_ARG for a negative budget.
+ * over more, smaller launches.  Also gives the pool's unused memory back to the
+ * device.  Errors: FWH_ERR_ARG for a negative budget.
  */
 fwh_status fwh_set_moving_scratch(int64_t bytes);
 

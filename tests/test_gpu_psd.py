@@ -94,3 +94,19 @@ def test_psd_of_far_field_dipole(dev):
     f = np.arange(257) / (512 * w.dt)
     assert np.all(np.abs(f[np.argmax(got, axis=1)] - 2.0) <= 1.0 / (512 * w.dt))
     s.close()
+
+
+@pytest.mark.parametrize("n_sig,ld,L", [(1, 4096, 64), (40, 900, 128), (320, 700, 64),
+                                        (700, 300, 32), (1030, 100, 16)])
+def test_psd_split_over_ctas(dev, n_sig, ld, L):
+    """One to eight CTAs a signal (few signals with many segments, or signals
+    enough for one CTA each), lengths by value (up to 1024 signals) and in a
+    device buffer, from host and from device memory."""
+    from paper_2312_16263_gb300 import welch_psd
+    rng = np.random.default_rng(n_sig)
+    p = rng.normal(size=(n_sig, ld)) + 0.3
+    nv = rng.integers(L - 2, ld + 1, size=n_sig)
+    ref = observer_psd(p, nv, 3.0, L)
+    d = torch.as_tensor(p, device=dev)
+    _close(welch_psd(d, 3.0, L, nv).cpu().numpy(), ref)
+    _close(welch_psd(d, 3.0, L, torch.as_tensor(nv, device=dev)).cpu().numpy(), ref)
