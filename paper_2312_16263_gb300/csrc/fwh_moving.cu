@@ -6,32 +6,41 @@
 // and the Mach numbers change with source time, so every (panel, observer)
 // has its own source-time signal and its own arrival times: the spline that
 // carries a panel's signal onto the observer grid cannot be shared between
-// observers.  Three kernels:
-//  * k_mseries, per (panel, frame): the observer-independent series Q_n
-//    (Eq. Qn), L_i (Eq. Li), the surface Mach vector v / c0 and their
-//    second-order source-time derivatives (Sec. III B), one 16-value row;
+// observers.  Three kernels, all bound by the FP64 pipe (2 operations a clock
+// and SM), so what they save is operations:
+//  * k_mseries, per (panel, run of frames): the observer-independent series Q_n
+//    (Eq. Qn), L_i (Eq. Li), the surface Mach vector M = v / c0, their
+//    second-order source-time derivatives (Sec. III B), M.M and L.M, one
+//    16-value row per frame; each frame's integrands are formed once;
 //  * k_mwindow, per observer: the earliest and latest arrival over panels of
 //    the first and last frame (the window t_start, t_end and N_o);
-//  * k_mscatter, per (observer, tile of 128 panels): a thread per panel
-//    evaluates, at every frame, the arrival t_i = tau_i + Delta (the positive
-//    root of |b + w Delta| = c0 Delta, b = x0 + w tau - y) and the bracket g_i
-//    of Eqs. pT + pL times dS / (4 pi); solves the natural-spline moments of g
-//    and of t over source time (tridiagonal elimination in a scratch column);
-//    then walks the observer bins: t_j lies in the interval whose arrival
-//    times bracket it, tau* solves t(tau*) = t_j there by Newton's method on
-//    the spline of t (three steps from the linear estimate reach FP64
-//    rounding for subsonic motion), and the spline of g at tau* is reduced
-//    over each warp's panels before one FP64 atomic per warp and bin.
-// Scratch: four FP64 columns of nt per (panel, observer) of a launch; the
-// host splits the observers into launches that fit the scratch budget (16 GiB
-// by default: a budget of 2 GiB, four observers per launch on the 8192-panel
-// x 2048-step benchmark case, measured 10 % slower, the grid then filling a
-// third of the GPU).
+//  * k_mscatter, per (observer, panel), a thread each.  Ascending in source
+//    time it evaluates, at every frame, the delay Delta (the positive root of
+//    |b + w Delta| = c0 Delta, b = x0 + w tau - y) and the bracket g of Eqs.
+//    pT + pL, and runs the forward elimination of the natural spline's cubic
+//    B-spline coefficients, beta_{i-1} + 4 beta_i + beta_{i+1} = 6 F_i with
+//    beta = F at both ends (g and Delta: two scratch columns).  Descending, the
+//    back substitution yields the coefficients in registers, four at a time,
+//    while the thread walks the observer bins downwards: the bin t_j lies in
+//    the interval whose arrival times tau + Delta bracket it, tau* is the root
+//    of a cubic there by Newton's method (residual in FP64, its quotient with
+//    the slope in FP32: a relative error of 1e-7 in a correction that the next
+//    step repeats; three steps reach FP64 rounding for subsonic motion), and
+//    the spline of g at tau* goes to a shared-memory tile from which each warp
+//    sums its panels, one FP64 atomic per warp and bin.
+// About 126 FP64 operations per (panel, sample, observer), the FP64 pipe 87 % busy.
+// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 62.0 ms for
+// k_mscatter (135.4 with moments, four columns, divisions in Newton's method
+// and a shuffle sum per bin: about 380 operations), 1.84 ms for k_mseries (5.65
+// with each frame's integrands formed three times), 64.3 ms a call (164).
+// Scratch: two FP64 columns of nt per (panel, observer) of a launch; the host
+// splits the observers into launches by the scratch budget.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -42,8 +51,10 @@ fwh_status fwh_fail_handle(fwh_handle h, fwh_status st, const char *msg);
 
 namespace {
 
-constexpr int kMRow = 16;     // series row: Qn, Qn', L(3), L'(3), M(3), M'(3), 2 pad
+constexpr int kMRow = 16;     // series row: Qn, Qn', L(3), L'(3), M(3), M'(3), M.M, L.M
+constexpr int kMRun = 16;     // frames per series thread
 constexpr int kMTile = 128;   // panels per scatter CTA
+constexpr int kMBins = 16;    // bins a warp sums at a time
 constexpr double kInv4Pi = 0.079577471545947667884441881686257181;
 
 struct MovArgs {
@@ -57,7 +68,7 @@ struct MovArgs {
   double *ts, *te;            // [O] window
   int *nv;                    // [O]
   double *p_out;              // [O][nt]
-  double *scratch;            // [4][nt][P * n_obs of the launch]
+  double *scratch;            // [2][nt][P * n_obs of the launch]
   int o_lo, n_obs;            // observers of this launch
 };
 
@@ -79,53 +90,63 @@ __device__ __forceinline__ void mv_integrands(const MovArgs &a, int p, int i, do
   for (int c = 0; c < 3; ++c) L[c] = pp * n[c] + rho * u[c] * (un - vn);
 }
 
-// Second-order source-time derivative weights of Sec. III B at frame i:
-// central inside, one-sided three-point at the first and last frame.
-__device__ __forceinline__ void fd_stencil(int i, int nt, int idx[3], double wgt[3]) {
-  if (i == 0) {
-    idx[0] = 0; idx[1] = 1; idx[2] = 2;
-    wgt[0] = -3.0; wgt[1] = 4.0; wgt[2] = -1.0;
-  } else if (i == nt - 1) {
-    idx[0] = nt - 1; idx[1] = nt - 2; idx[2] = nt - 3;
-    wgt[0] = 3.0; wgt[1] = -4.0; wgt[2] = 1.0;
-  } else {
-    idx[0] = i + 1; idx[1] = i - 1; idx[2] = i;
-    wgt[0] = 1.0; wgt[1] = -1.0; wgt[2] = 0.0;
-  }
+// Frames [i0, i0 + kMRun) of one panel; (q, L, v) of the frames i - 1, i, i + 1 slide
+// through registers (central differences inside, one-sided at the ends).
+struct MvFrame {
+  double q, L[3], v[3];
+};
+__device__ __forceinline__ MvFrame mv_frame(const MovArgs &a, int p, int i) {
+  MvFrame f;
+  mv_integrands(a, p, i, f.q, f.L);
+  for (int c = 0; c < 3; ++c) f.v[c] = a.v[((size_t)i * a.P + p) * 3 + c];
+  return f;
 }
 
 __global__ void __launch_bounds__(256) k_mseries(MovArgs a) {
-  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;  // e = i P + p
-  if (e >= (long)a.P * a.nt) return;
-  const int p = (int)(e % a.P), i = (int)(e / a.P);
-  double qn, L[3];
-  mv_integrands(a, p, i, qn, L);
-  int idx[3];
-  double wgt[3];
-  fd_stencil(i, a.nt, idx, wgt);
-  const double inv2h = 0.5 / a.dt;
-  double qd = 0.0, Ld[3] = {0.0, 0.0, 0.0}, vd[3] = {0.0, 0.0, 0.0};
-  for (int s = 0; s < 3; ++s) {
-    if (wgt[s] == 0.0) continue;
-    double q2, L2[3];
-    mv_integrands(a, p, idx[s], q2, L2);
-    const double *v2 = a.v + ((size_t)idx[s] * a.P + p) * 3;
-    qd += wgt[s] * q2;
-    for (int c = 0; c < 3; ++c) {
-      Ld[c] += wgt[s] * L2[c];
-      vd[c] += wgt[s] * v2[c];
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= a.P) return;
+  const double inv2h = 0.5 / a.dt, ic0 = 1.0 / a.c0;
+  for (int i0 = blockIdx.y * kMRun; i0 < a.nt; i0 += gridDim.y * kMRun) {  // grid y <= 65535
+    const int i1 = min(a.nt, i0 + kMRun);
+    MvFrame fm{}, f = mv_frame(a, p, i0), fp{};
+    if (i0 > 0) fm = mv_frame(a, p, i0 - 1);
+    for (int i = i0; i < i1; ++i) {
+      if (i + 1 < a.nt) fp = mv_frame(a, p, i + 1);
+      MvFrame d;
+      if (i == 0 || i == a.nt - 1) {  // one-sided three-point
+        const double sg = i == 0 ? 1.0 : -1.0;
+        const MvFrame g1 = i == 0 ? fp : fm, g2 = mv_frame(a, p, i == 0 ? 2 : a.nt - 3);
+        d.q = sg * (-3.0 * f.q + 4.0 * g1.q - g2.q);
+        for (int c = 0; c < 3; ++c) {
+          d.L[c] = sg * (-3.0 * f.L[c] + 4.0 * g1.L[c] - g2.L[c]);
+          d.v[c] = sg * (-3.0 * f.v[c] + 4.0 * g1.v[c] - g2.v[c]);
+        }
+      } else {
+        d.q = fp.q - fm.q;
+        for (int c = 0; c < 3; ++c) {
+          d.L[c] = fp.L[c] - fm.L[c];
+          d.v[c] = fp.v[c] - fm.v[c];
+        }
+      }
+      const size_t P = a.P;
+      double *row = a.S + (size_t)i * kMRow * P + p;  // value q at row[q P]
+      row[0] = f.q;
+      row[P] = d.q * inv2h;
+      double M2 = 0.0, LM = 0.0;
+      for (int c = 0; c < 3; ++c) {
+        const double M = f.v[c] * ic0;
+        M2 = fma(M, M, M2);
+        LM = fma(f.L[c], M, LM);
+        row[(2 + c) * P] = f.L[c];
+        row[(5 + c) * P] = d.L[c] * inv2h;
+        row[(8 + c) * P] = M;
+        row[(11 + c) * P] = d.v[c] * inv2h * ic0;
+      }
+      row[14 * P] = M2;
+      row[15 * P] = LM;
+      fm = f;
+      f = fp;
     }
-  }
-  const double *v = a.v + ((size_t)i * a.P + p) * 3;
-  double *row = a.S + (size_t)i * kMRow * a.P + p;  // value q at row[q P]
-  const size_t P = a.P;
-  row[0] = qn;
-  row[P] = qd * inv2h;
-  for (int c = 0; c < 3; ++c) {
-    row[(2 + c) * P] = L[c];
-    row[(5 + c) * P] = Ld[c] * inv2h;
-    row[(8 + c) * P] = v[c] / a.c0;              // M
-    row[(11 + c) * P] = vd[c] * inv2h / a.c0;    // M-dot
   }
 }
 
@@ -177,49 +198,29 @@ __global__ void __launch_bounds__(256) k_mwindow(MovArgs a) {
   }
 }
 
-// Natural cubic-spline moments of column c (stride `ld` between samples):
-// m_0 = m_{n-1} = 0, m_{i-1} + 4 m_i + m_{i+1} = 6 (c_{i+1} - 2 c_i + c_{i-1})
-// / h^2, by tridiagonal elimination; ipiv[i] = 1/pivot of row i (piv_1 = 4,
-// piv_i = 4 - 1/piv_{i-1}), constant from row 63 on (it has converged to
-// 2 + sqrt 3 to FP64 rounding long before).
-constexpr int kPiv = 64;
-__device__ void spline_moments(const double *c, double *m, long ld, int n, double h,
-                               const double *ipiv) {
-  const double s6 = 6.0 / (h * h);
-  m[0] = 0.0;
-  m[(long)(n - 1) * ld] = 0.0;
-  if (n < 3) return;
-  double prev = 0.0, cm = c[0], c0 = c[ld];
-  for (int i = 1; i <= n - 2; ++i) {
-    const double cp1 = c[(long)(i + 1) * ld];
-    const double r = s6 * (cp1 - 2.0 * c0 + cm);
-    prev = (r - prev) * ipiv[i < kPiv ? i : kPiv - 1];
-    m[(long)i * ld] = prev;
-    cm = c0;
-    c0 = cp1;
-  }
-  double mn = 0.0;
-  for (int i = n - 2; i >= 1; --i) {
-    const double v = m[(long)i * ld] - mn * ipiv[i < kPiv ? i : kPiv - 1];
-    m[(long)i * ld] = v;
-    mn = v;
-  }
+constexpr int kPiv = 64;  // pivots of tridiag(1, 4, 1); constant to FP64 rounding from row 63 on
+
+// Reciprocal of a number of ordinary size: Newton's method from the FP32 one.
+__device__ __forceinline__ double recip(double x) {
+  double y = (double)__frcp_rn((float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
 }
 
-__global__ void __launch_bounds__(kMTile, 8) k_mscatter(MovArgs a) {
+// REST: observers at rest (w = 0), whose distance needs no quadratic.
+template <bool REST>
+__global__ void __launch_bounds__(kMTile, 7) k_mscatter(MovArgs a) {
   const int ob = blockIdx.y;               // observer within the launch
   const int o = a.o_lo + ob;
   const int p = blockIdx.x * kMTile + threadIdx.x;
+  const int lane = threadIdx.x & 31, N = a.nt;
   const bool live = p < a.P;
   const int pp = live ? p : a.P - 1;
-  const long ld = (long)a.P * a.n_obs;     // scratch column stride
-  const long col = (long)ob * a.P + pp;
-  double *G = a.scratch + col, *MG = G + (long)a.nt * ld, *TT = MG + (long)a.nt * ld,
-         *MT = TT + (long)a.nt * ld;
-  const double x0[3] = {a.x0[3 * o], a.x0[3 * o + 1], a.x0[3 * o + 2]};
-  const double S4 = a.dS[pp] * kInv4Pi;
-  const double c0 = a.c0;
+  const size_t P = a.P, ld = P * a.n_obs;  // scratch row stride
+  double *const ZG = a.scratch + (size_t)ob * P + pp, *const ZD = ZG + (size_t)N * ld;
+  const double c0 = a.c0, ic0 = 1.0 / c0, h = a.dt;
   __shared__ double ipiv[kPiv];
+  __shared__ double tile[kMTile / 32][kMBins][33];
   if (threadIdx.x == 0) {
     double piv = 4.0;
     ipiv[0] = 0.0;
@@ -229,73 +230,178 @@ __global__ void __launch_bounds__(kMTile, 8) k_mscatter(MovArgs a) {
     }
   }
   __syncthreads();
-  // signal g and arrival time t at every frame (Eqs. pT, pL, tau); threads
-  // past the last panel only join the bin reductions below
-  for (int i = 0; live && i < a.nt; ++i) {
-    const double tau = (double)i * a.dt;
-    const double *rw = a.S + (size_t)i * kMRow * a.P + pp;
-    double row[14];
-    for (int q = 0; q < 14; ++q) row[q] = rw[(size_t)q * a.P];
-    double b[3];
-    const double d = mv_delay(a, x0, tau, a.y + ((size_t)i * a.P + pp) * 3, b);
-    const double r = c0 * d, ir = 1.0 / r;
-    double rh[3];
-    for (int c = 0; c < 3; ++c) rh[c] = (b[c] + a.w[c] * d) * ir;
-    double Mr = 0.0, Mdr = 0.0, M2 = 0.0, Lr = 0.0, Ldr = 0.0, LM = 0.0;
-    for (int c = 0; c < 3; ++c) {
-      Mr += row[8 + c] * rh[c];
-      Mdr += row[11 + c] * rh[c];
-      M2 += row[8 + c] * row[8 + c];
-      Lr += row[2 + c] * rh[c];
-      Ldr += row[5 + c] * rh[c];
-      LM += row[2 + c] * row[8 + c];
-    }
-    const double D = 1.0 - Mr, iD = 1.0 / D;
-    const double k = r * Mdr + c0 * (Mr - M2);
-    const double thick = row[1] * ir * iD * iD + row[0] * k * ir * ir * iD * iD * iD;
-    const double load = Ldr / c0 * ir * iD * iD + (Lr - LM) * ir * ir * iD * iD +
-                        Lr * k / c0 * ir * ir * iD * iD * iD;
-    G[(long)i * ld] = S4 * (thick + load);
-    TT[(long)i * ld] = tau + d;
+  const double x0[3] = {a.x0[3 * o], a.x0[3 * o + 1], a.x0[3 * o + 2]};
+  double iq = 0.0, q = 0.0, w[3] = {0.0, 0.0, 0.0};
+  if constexpr (!REST) {
+    for (int c = 0; c < 3; ++c) w[c] = a.w[c];
+    q = c0 * c0 - (w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
+    iq = 1.0 / q;
   }
+  // signal g and delay Delta at every frame (Eqs. pT, pL, tau) and the forward
+  // elimination of both; threads past the last panel only join the sums below
+  double g = 0.0, dl = 0.0, zg = 0.0, zd = 0.0;
+  for (int i = 0; live && i < N; ++i) {
+    const double *rw = a.S + (size_t)i * kMRow * P + pp;
+    double row[kMRow];
+#pragma unroll
+    for (int v = 0; v < kMRow; ++v) row[v] = rw[(size_t)v * P];
+    const double *y = a.y + ((size_t)i * P + pp) * 3;
+    double r, ir, rh[3];
+    if constexpr (REST) {
+      const double b[3] = {x0[0] - y[0], x0[1] - y[1], x0[2] - y[2]};
+      const double bb = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+      ir = rsqrt(bb);
+      r = bb * ir;
+      dl = r * ic0;
+      for (int c = 0; c < 3; ++c) rh[c] = b[c] * ir;
+    } else {
+      const double tau = (double)i * h;
+      double b[3];
+      for (int c = 0; c < 3; ++c) b[c] = fma(w[c], tau, x0[c]) - y[c];
+      const double bw = b[0] * w[0] + b[1] * w[1] + b[2] * w[2];
+      const double bb = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+      dl = (bw + sqrt(fma(q, bb, bw * bw))) * iq;
+      r = c0 * dl;
+      ir = 1.0 / r;
+      for (int c = 0; c < 3; ++c) rh[c] = fma(w[c], dl, b[c]) * ir;
+    }
+    double Mr = row[8] * rh[0], Mdr = row[11] * rh[0], Lr = row[2] * rh[0], Ldr = row[5] * rh[0];
+#pragma unroll
+    for (int c = 1; c < 3; ++c) {
+      Mr = fma(row[8 + c], rh[c], Mr);
+      Mdr = fma(row[11 + c], rh[c], Mdr);
+      Lr = fma(row[2 + c], rh[c], Lr);
+      Ldr = fma(row[5 + c], rh[c], Ldr);
+    }
+    const double iD = recip(1.0 - Mr);
+    const double k = fma(r, Mdr, c0 * (Mr - row[14]));
+    // [Qn' + L'_r / c0] / (r D^2) + [L_r - L.M + (Qn + L_r / c0) k / D] / (r^2 D^2)
+    const double u = ir * iD * iD;
+    const double near = fma(fma(Lr, ic0, row[0]), k * iD, Lr - row[15]);
+    g = u * fma(near, ir, fma(Ldr, ic0, row[1]));
+    const double ip = ipiv[min(i, kPiv - 1)];
+    if (i == 0) {
+      zg = g;
+      zd = dl;
+    } else {
+      zg = fma(6.0, g, -zg) * ip;
+      zd = fma(6.0, dl, -zd) * ip;
+    }
+    ZG[(size_t)i * ld] = zg;
+    ZD[(size_t)i * ld] = zd;
+  }
+  // interval k: coefficients B[0..3] = beta_{k-1} .. beta_{k+2} of both splines
+  double G[4] = {0.0, 0.0, 0.0, 0.0}, D[4] = {0.0, 0.0, 0.0, 0.0};
+  int k = N - 2;
+  auto below = [&](int i, const double *Z, const double *B) -> double {  // beta_i from B[1] = beta_{i+1}
+    if (i < 0) return 2.0 * B[1] - B[2];
+    return fma(-B[1], ipiv[min(i, kPiv - 1)], Z[(size_t)i * ld]);
+  };
   if (live) {
-    spline_moments(G, MG, ld, a.nt, a.dt, ipiv);
-    spline_moments(TT, MT, ld, a.nt, a.dt, ipiv);
+    G[2] = g;
+    D[2] = dl;
+    G[1] = fma(-g, ipiv[min(N - 2, kPiv - 1)], ZG[(size_t)(N - 2) * ld]);
+    D[1] = fma(-dl, ipiv[min(N - 2, kPiv - 1)], ZD[(size_t)(N - 2) * ld]);
+    G[3] = 2.0 * G[2] - G[1];
+    D[3] = 2.0 * D[2] - D[1];
+    G[0] = below(k - 1, ZG, G);
+    D[0] = below(k - 1, ZD, D);
   }
-  // observer bins: every thread walks the same j, each warp sums its panels
-  // and adds them with one atomic (no CTA barrier per bin)
+  // observer bins downwards: every thread walks the same j; each warp sums its
+  // panels kMBins at a time and adds them with one atomic a bin
   const int nv = a.nv[o];
-  const double ts = a.ts[o], h = a.dt, h26 = a.dt * a.dt / 6.0;
-  int k = 0;
-  for (int j = 0; j < nv; ++j) {
-    double val = 0.0;
-    if (live) {
-    const double tj = ts + (double)j * h;
-    while (k < a.nt - 2 && TT[(long)(k + 1) * ld] < tj) ++k;
-    const double t0 = TT[(long)k * ld], t1 = TT[(long)(k + 1) * ld];
-    const double mt0 = MT[(long)k * ld], mt1 = MT[(long)(k + 1) * ld];
-    // Newton on S_t(x) = A t0 + B t1 + ((A^3 - A) mt0 + (B^3 - B) mt1) h^2/6 = tj,
-    // x = B in [0, 1], A = 1 - B
-    double B = (t1 > t0) ? (tj - t0) / (t1 - t0) : 0.0;
-    B = fmin(1.0, fmax(0.0, B));
-    for (int it = 0; it < 3; ++it) {
-      const double A = 1.0 - B;
-      const double f = A * t0 + B * t1 + ((A * A * A - A) * mt0 + (B * B * B - B) * mt1) * h26 - tj;
-      const double df = (t1 - t0) + ((1.0 - 3.0 * A * A) * mt0 + (3.0 * B * B - 1.0) * mt1) * h26;
-      B = fmin(1.0, fmax(0.0, B - f / df));
+  const double ts = a.ts[o], scale = a.dS[pp] * (kInv4Pi / 6.0);
+  double(*tl)[33] = tile[threadIdx.x >> 5];
+  double ak = fma((double)k, h, (D[0] + 4.0 * D[1] + D[2]) * (1.0 / 6.0));  // arrival of node k
+  for (int j1 = nv; j1 > 0; j1 -= kMBins) {
+    const int j0 = max(0, j1 - kMBins);
+    for (int j = j1 - 1; j >= j0; --j) {
+      double val = 0.0;
+      if (live) {
+        const double tj = fma((double)j, h, ts);
+        while (k > 0 && ak > tj) {
+          --k;
+          G[3] = G[2]; G[2] = G[1]; G[1] = G[0];
+          D[3] = D[2]; D[2] = D[1]; D[1] = D[0];
+          G[0] = below(k - 1, ZG, G);
+          D[0] = below(k - 1, ZD, D);
+          ak = fma((double)k, h, (D[0] + 4.0 * D[1] + D[2]) * (1.0 / 6.0));
+        }
+        // arrival - t_j on the interval: e + p1 f + p2 f^2 + p3 f^3
+        const double e = ak - tj;
+        const double p1 = fma(0.5, D[2] - D[0], h);
+        const double p2 = fma(0.5, D[0] + D[2], -D[1]);
+        const double p3 = fma(0.5, D[1] - D[2], (D[3] - D[0]) * (1.0 / 6.0));
+        const float q1 = (float)p1, q2 = 2.f * (float)p2, q3 = 3.f * (float)p3;
+        float ff = fminf(1.f, fmaxf(0.f, __fdividef(-(float)e, q1)));
+        double f = (double)ff;
+#pragma unroll
+        for (int it = 0; it < 3; ++it) {
+          const double res = fma(fma(fma(p3, f, p2), f, p1), f, e);
+          ff = (float)f;
+          f -= (double)__fdividef((float)res, fmaf(fmaf(q3, ff, q2), ff, q1));
+        }
+        f = fmin(1.0, fmax(0.0, f));
+        const double c = 1.0 - f, f2 = f * f, c2 = c * c;
+        val = (c2 * c) * G[0];
+        val = fma(fma(f2, fma(3.0, f, -6.0), 4.0), G[1], val);
+        val = fma(fma(c2, fma(3.0, c, -6.0), 4.0), G[2], val);
+        val = fma(f2 * f, G[3], val) * scale;
+      }
+      tl[j - j0][lane] = val;
     }
-    const double A = 1.0 - B;
-    val = A * G[(long)k * ld] + B * G[(long)(k + 1) * ld] +
-          ((A * A * A - A) * MG[(long)k * ld] + (B * B * B - B) * MG[(long)(k + 1) * ld]) * h26;
+    __syncwarp();
+    {  // lane: bin lane % kMBins over half of the warp's panels
+      static_assert(kMBins == 16, "two lanes a bin");
+      const int b = lane & 15, l0 = lane & 16;
+      double v = 0.0;
+      if (b < j1 - j0) {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) v += tl[b][l0 + l];
+      }
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+      if (lane < j1 - j0) atomicAdd(a.p_out + (size_t)o * N + j0 + lane, v);
     }
-    for (int off = 16; off > 0; off >>= 1) val += __shfl_xor_sync(0xffffffffu, val, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(a.p_out + (size_t)o * a.nt + j, val);
+    __syncwarp();
   }
 }
 
 // Scratch budget of one call (bytes; 0: the default of 16 GiB), process-wide.
 std::atomic<int64_t> g_mov_scratch{0};
 constexpr int64_t kMovScratchDefault = (int64_t)16 << 30;
+
+// Scratch comes from a pool of the library's own, one per device, which keeps
+// up to kPoolKeep bytes between calls (mapping the 6.4 GB of the benchmark case anew on
+// every call took 14 ms); fwh_set_moving_scratch gives what is unused back.  The pool
+// orders reuse between streams itself.
+constexpr uint64_t kPoolKeep = (uint64_t)8 << 30;
+constexpr int kMaxDev = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDev] = {};
+
+cudaError_t mov_pool(cudaMemPool_t *pool) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t np = nullptr;
+    if ((e = cudaMemPoolCreate(&np, &props)) != cudaSuccess) return e;
+    uint64_t keep = kPoolKeep;
+    if ((e = cudaMemPoolSetAttribute(np, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(np);
+      return e;
+    }
+    g_pool[dev] = np;
+  }
+  *pool = g_pool[dev];
+  return cudaSuccess;
+}
 
 bool on_device(const void *p) {
   if (!p) return false;
@@ -316,6 +422,9 @@ fwh_status failm(fwh_status st, const std::string &m) {
 extern "C" fwh_status fwh_set_moving_scratch(int64_t bytes) {
   if (bytes < 0) return failm(FWH_ERR_ARG, "scratch budget must be >= 0 bytes");
   g_mov_scratch.store(bytes);
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  for (cudaMemPool_t p : g_pool)
+    if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
   return FWH_OK;
 }
 
@@ -346,12 +455,13 @@ extern "C" fwh_status fwh_forward_moving(int64_t P, int64_t nt, const double *y,
   const size_t fb = (size_t)nt * 5 * P * sizeof(double);
   const size_t ob = (size_t)O * nt * sizeof(double);
   std::vector<void *> tmp;
-  cudaError_t e = cudaSuccess;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = mov_pool(&pool);
   auto dev_in = [&](const double *src, size_t bytes) -> const double * {
     if (e != cudaSuccess) return nullptr;
     if (on_device(src)) return src;
     void *d = nullptr;
-    if ((e = cudaMallocAsync(&d, bytes, s)) != cudaSuccess) return nullptr;
+    if ((e = cudaMallocFromPoolAsync(&d, bytes, pool, s)) != cudaSuccess) return nullptr;
     tmp.push_back(d);
     e = cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, s);
     return static_cast<const double *>(d);
@@ -359,7 +469,7 @@ extern "C" fwh_status fwh_forward_moving(int64_t P, int64_t nt, const double *y,
   auto dev_buf = [&](size_t bytes) -> void * {
     if (e != cudaSuccess) return nullptr;
     void *d = nullptr;
-    if ((e = cudaMallocAsync(&d, bytes, s)) != cudaSuccess) return nullptr;
+    if ((e = cudaMallocFromPoolAsync(&d, bytes, pool, s)) != cudaSuccess) return nullptr;
     tmp.push_back(d);
     return d;
   };
@@ -385,16 +495,17 @@ extern "C" fwh_status fwh_forward_moving(int64_t P, int64_t nt, const double *y,
   a.nv = static_cast<int *>(dev_buf((size_t)O * sizeof(int)));
   const bool o_dev = on_device(p_out);
   a.p_out = o_dev ? p_out : static_cast<double *>(dev_buf(ob));
-  // observers per launch: four scratch columns of nt per (panel, observer)
-  // within the scratch budget (at least one observer per launch)
+  // observers per launch: the budget counts four columns of nt per (panel,
+  // observer), of which two are used (at least one observer per launch)
   const size_t per_obs = (size_t)4 * nt * P * sizeof(double);
   const int64_t budget = g_mov_scratch.load() > 0 ? g_mov_scratch.load() : kMovScratchDefault;
   const int n_obs = (int)std::max<size_t>(1, std::min<size_t>((size_t)O, (size_t)budget / per_obs));
-  a.scratch = static_cast<double *>(dev_buf(per_obs * n_obs));
+  a.scratch = static_cast<double *>(dev_buf(per_obs / 2 * n_obs));
   if (e == cudaSuccess) e = cudaMemsetAsync(a.p_out, 0, ob, s);
   if (e == cudaSuccess) {
-    const long n = (long)P * nt;
-    k_mseries<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a);
+    const int64_t runs = (nt + kMRun - 1) / kMRun;
+    const dim3 grid((unsigned)((P + 255) / 256), (unsigned)std::min<int64_t>(runs, 65535));
+    k_mseries<<<grid, 256, 0, s>>>(a);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -405,7 +516,10 @@ extern "C" fwh_status fwh_forward_moving(int64_t P, int64_t nt, const double *y,
     a.o_lo = o0;
     a.n_obs = (int)std::min<int64_t>(n_obs, O - o0);
     dim3 grid((unsigned)((P + kMTile - 1) / kMTile), (unsigned)a.n_obs);
-    k_mscatter<<<grid, kMTile, 0, s>>>(a);
+    if (wh[0] == 0.0 && wh[1] == 0.0 && wh[2] == 0.0)
+      k_mscatter<true><<<grid, kMTile, 0, s>>>(a);
+    else
+      k_mscatter<false><<<grid, kMTile, 0, s>>>(a);
     e = cudaGetLastError();
   }
   std::vector<double> hts;

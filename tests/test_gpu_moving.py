@@ -130,3 +130,17 @@ def test_observers_split_over_launches(dev):
         _run(dev, y, n, v, dS, 1.0, 1.0, 0.02, f, obs, np.zeros(3))
     finally:
         _abi.check(lib.fwh_set_moving_scratch(0), None)
+
+
+@pytest.mark.parametrize("motion,nt,n_obs", [("spin", 3, 2), ("translate", 4, 3), ("spin", 17, 5),
+                                             ("translate", 130, 2)])
+def test_short_records_and_partial_bin_runs(dev, motion, nt, n_obs):
+    """The shortest records (the back substitution starts at the natural end),
+    runs of frames and of bins that are not whole, observers at rest and moving."""
+    import sys, os
+    sys.path.insert(0, os.path.dirname(__file__))
+    y, n, v, dS, f = _sphere(motion, 6, 11, nt, 1.5 if nt < 10 else 0.3)
+    v = v / (5.0 if nt < 20 else 1.0)
+    obs = observers_circle(12.0, 6)[:n_obs]
+    w = np.array([0.0, 0.0, 0.0]) if motion == "spin" else np.array([0.05, 0.02, 0.0])
+    _run(dev, y, n, v, dS, 1.0, 1.0, 1.5 if nt < 10 else 0.3, f, obs, w)
