@@ -534,10 +534,9 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     // the short segment first: it runs under the copies, and what follows the
     // last copy is one segment of whole chunks
     fa.seg_shift = (fa.n_segs * fa.seg_len - fa.k_top) / 4 * 4;
-    st1 = ensure_events(h, 2 * nslab + 2);
+    st1 = ensure_events(h, 2 * nslab + 1);
     if (st1 != FWH_OK) return st1;
-    cudaEvent_t *ev_in = h->slab_ev.data(), *ev_x = ev_in + nslab, ev_go = ev_in[2 * nslab],
-                ev_end = ev_in[2 * nslab + 1];
+    cudaEvent_t *ev_in = h->slab_ev.data(), *ev_x = ev_in + nslab, ev_go = ev_in[2 * nslab];
     CK(h, cudaEventRecord(ev_go, s));
     CK(h, cudaStreamWaitEvent(h->copy, ev_go, 0));
     const int cps = slab / kRowBlk;  // prep blocks per slab
@@ -568,21 +567,9 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
       CK(h, cudaStreamWaitEvent(h->pstream, ev_in[std::min(q, nslab - 1)], 0));
       pa.c_lo = j * cps;
       pa.c_hi = q < nslab ? std::min(n_rb, q * cps) : n_rb;
-      const int c_end = pa.c_hi;
-      if (q == nslab) {
-        // the last slab: its record-end blocks beside its interior ones
-        pa.c_lo = std::max(j * cps, std::min(n_rb, prep_interior_end<T>(pa.nt)));
-        if (pa.c_lo > j * cps && pa.c_lo < n_rb) {
-          CK(h, launch_prep<T>(pa, h->copy));
-          CK(h, cudaEventRecord(ev_end, h->copy));
-          CK(h, cudaStreamWaitEvent(s, ev_end, 0));
-          pa.c_hi = pa.c_lo;
-        }
-        pa.c_lo = j * cps;
-      }
       CK(h, launch_prep<T>(pa, h->pstream));
       CK(h, cudaEventRecord(ev_x[j], h->pstream));
-      const fwh_status st2 = scatter_upto(c_end * kRowBlk, j);
+      const fwh_status st2 = scatter_upto(pa.c_hi * kRowBlk, j);
       if (st2 != FWH_OK) return st2;
     }
   }

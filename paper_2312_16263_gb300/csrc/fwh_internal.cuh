@@ -132,7 +132,6 @@ struct PrepArgs {
   int row0;             // record row held by X row 0 (a multiple of 64)
   double ca, sa, dt;
   int c_lo, c_hi;       // 64-row blocks [c_lo, c_hi) to prepare (0, 0: the whole record)
-  int int_lo, int_hi;   // set by the launcher: the interior blocks within [c_lo, c_hi)
 };
 
 template <typename T>
@@ -200,12 +199,6 @@ template <typename T>
 cudaError_t launch_coef(const GeomArgs &a, T *coef, int *i0, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prep(const PrepArgs<T> &a, cudaStream_t s);
-// The interior blocks of a record's prep are [1, this).
-template <typename T>
-constexpr int prep_interior_end(int nt) {
-  const int top = nt - kRowBlk - Prec<T>::halo - 1;
-  return top >= kRowBlk ? top / kRowBlk + 1 : 1;
-}
 template <typename T>
 cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s);
 template <typename T>

@@ -23,13 +23,20 @@
 //   beta_k = -6 rho x_k      with r = F             (FP64: fewer operations)
 // A recursion started H samples outside the 64-row block it serves errs by
 // |rho|^H (H = 16 for FP32, 32 for FP64: below rounding), so blocks are
-// independent.  Away from the record ends the solve commutes with the central
-// difference, so a derivative series' coefficients are the central
-// differences of its value series' coefficients: four filters, not eight.
+// independent.  At the record ends both start exactly: y_0 is a sum over the
+// first H samples of the reflected series, and beta_{N-1} = F_{N-1} gives
+// x_{N-1}.
 //
-// Kernels: the interior blocks of FP32 (k_prep_iir_int) and FP64
-// (k_prep_f64_int), persistent CTAs that walk consecutive blocks of a panel
-// group; k_prep_iir for the blocks at the record ends, all eight series.  All
+// Away from the record ends the solve commutes with the central difference, so
+// a derivative series' coefficients are the central differences d_k =
+// (beta_{k+1} - beta_{k-1}) / (2 dt) of its value series' coefficients: four
+// filters, not eight.  Near an end they differ by a solution of the
+// homogeneous system: beta'_k = d_k + (D_0 - d_0) rho^k from the start (D_0 the
+// one-sided derivative, d_0 = (beta_1 - beta_0) / dt), and likewise from the end.
+//
+// Kernels: k_prep_iir_int (FP32) and k_prep_f64_int (FP64), persistent CTAs that
+// walk consecutive blocks of a panel group; k_prep_iir for records too short for
+// them (under 64 + 2 H samples), all eight series by index arithmetic.  All
 // take the panels in the caller's order, so field reads are coalesced also
 // for a reordered surface; the rows of X go where the panel's place is.
 #include "fwh_internal.cuh"
@@ -55,9 +62,13 @@ constexpr int kIirQ = 8;  // integrand stride in a staged row ([4 integrands][8 
 constexpr int kIirRow = 4 * kIirQ;                   // staged row stride (values)
 
 // ---------------------------------------------------------------------------
-// FP32 prep of the interior blocks: one thread owns one (panel, integrand)
-// over a whole 64-row block and stores the pair (derivative, value) of each
-// sample, 8 of the 32 bytes of an X row.
+// FP32 prep: one thread owns one (panel, integrand) over a whole 64-row block
+// and stores the pair (derivative, value) of each sample, 8 of the 32 bytes of
+// an X row.  Bound by HBM: 20 bytes in and 32 out per (panel, sample), 5.5 TB/s
+// (81 % of a copy's).  The blocks at the record ends take the same filters with
+// exact starts (edge_block); as a kernel of their own that filtered all eight
+// reflected series they took 0.32 of 0.88 ms at 32768 panels x 2048 steps,
+// here @EDGE@.
 // ---------------------------------------------------------------------------
 constexpr int kIntPanels = 16;
 constexpr int kIntThreads = kIntPanels * 4;
@@ -86,6 +97,85 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
+// rho^k for k < kIirH + 4, zero beyond (below FP32 rounding).
+__host__ __device__ constexpr float rho_pow(int k) {
+  double v = k < kIirH + 4 ? 1.0 : 0.0;
+  for (int i = 0; i < k && i < kIirH + 4; ++i) v *= kRho;
+  return (float)v;
+}
+
+// A block at a record end: bc[k kIntRow] is the integrand of sample c0 + k (valid
+// inside the record), xr the thread's pair in the block's first X row, `room` the
+// rows of X from there on.
+__device__ __forceinline__ void edge_block(const float *bc, float *xr, int c0, int N, float inv2h,
+                                           int room, bool store) {
+  constexpr int H = kIirH, C = kIirChunk;
+  constexpr float rho = (float)kRho;
+  auto B = [&](int k) -> float { return bc[k * kIntRow]; };
+  const bool start = c0 < 0;  // c0 = -1: sample 0 at k = 1
+  float y0 = 0.f;             // y of sample 0
+  if (start) {
+#pragma unroll
+    for (int j = H; j >= 1; --j) y0 = (y0 - (B(j + 2) - 2.f * B(j + 1) + B(j))) * rho;
+  }
+  float y[C + H + 1];
+  float yy = 0.f;
+#pragma unroll
+  for (int k = -1 - H; k <= C + H - 1; ++k) {
+    if (k <= 1 && start)
+      yy = k == 1 ? y0 : 0.f;
+    else
+      yy = (B(k + 1) - 2.f * B(k) + B(k - 1)) + rho * yy;
+    if (k >= -1) y[k + 1] = yy;
+  }
+  float D0 = 0.f, cs = 0.f;  // one-sided derivative at sample 0, its excess over the central one
+  if (start) {
+    float x1 = 0.f;
+#pragma unroll
+    for (int k = H + 2; k >= 2; --k) x1 = y[k + 1] + rho * x1;
+    D0 = (-3.f * B(1) + 4.f * B(2) - B(3)) * inv2h;
+    cs = D0 - (B(2) + rho * x1 - B(1)) * (2.f * inv2h);
+  }
+  float xx = 0.f, b1v = 0.f, b2v = 0.f, cr = 0.f, DN = 0.f, d2 = 0.f;
+#pragma unroll
+  for (int k = C + H - 1; k >= -1; --k) {
+    const int sk = c0 + k;
+    xx = sk >= N - 1 ? 0.f : y[k + 1] + rho * xx;
+    const float bk = B(k) + rho * xx;
+    if (sk == N - 2) {
+      DN = (3.f * B(k + 1) - 4.f * B(k) + B(k - 1)) * inv2h;
+      cr = DN - (b1v - bk) * (2.f * inv2h);
+    } else if (sk < N - 2) {
+      cr *= rho;
+    }
+    // sample sk + 1 = c0 + e
+    const int e = k + 1, se = sk + 1;
+    float d = (b2v - bk) * inv2h + cr;
+    if (e >= 2) d += cs * rho_pow(e - 1);
+    if (e <= C - 1 && store) {
+      float *row = xr + e * kSer;
+      if (se == N + 1) {
+        *reinterpret_cast<float2 *>(row) = make_float2(0.f, 0.f);
+      } else if (se <= N - 2 && !(start && e <= 1)) {
+        *reinterpret_cast<float2 *>(row) = make_float2(d, b1v);
+        if (se == N - 2) {  // the last sample and the ghost after it
+          const float bN = B(e + 1);
+          if (e + 1 < room) *reinterpret_cast<float2 *>(row + kSer) = make_float2(DN, bN);
+          if (e + 2 < room)
+            *reinterpret_cast<float2 *>(row + 2 * kSer) =
+                make_float2(2.f * DN - d, 2.f * bN - b1v);
+        }
+      } else if (start && e == 1) {  // sample 0 and the ghost before it
+        *reinterpret_cast<float2 *>(row) = make_float2(D0, b1v);
+        *reinterpret_cast<float2 *>(row - kSer) = make_float2(2.f * D0 - d2, 2.f * b1v - b2v);
+      }
+    }
+    d2 = d;
+    b2v = b1v;
+    b1v = bk;
+  }
+}
+
 __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float> a, int unit) {
   constexpr int NP = kIntPanels, H = kIirH, C = kIirChunk;
   constexpr float rho = -0.267949192431122706f;  // sqrt(3) - 2
@@ -94,7 +184,7 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
   float *raw = sb + kIntRows * kIntRow;             // [C rows][5][NP] fields in flight
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
-  const int n_blk = a.int_hi - a.int_lo;
+  const int n_blk = a.c_hi - a.c_lo;
   const int n_us = (n_blk + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   // phase A thread: panel pa, rows tid / NP + 4 u
@@ -107,8 +197,8 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     // panel group fastest: concurrent units read neighbouring segments of the same rows
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = a.int_lo + (int)(u / n_pg) * unit;
-    const int b1 = min(a.int_lo + n_blk, b0 + unit);
+    const int b0 = a.c_lo + (int)(u / n_pg) * unit;
+    const int b1 = min(a.c_hi, b0 + unit);
     const int p = p0 + pa;
     const bool live = p < a.P;
     float n0 = 0.f, n1 = 0.f, n2 = 0.f, Un = 0.f;
@@ -121,6 +211,11 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
     }
     const int pb = p0 + pl;
     const bool live_b = pb < a.P;
+    // row of component rc % 5 of frame r0 + rc / 5 (rows outside the record are
+    // copied from its ends and not used)
+    auto src_row = [&](int r0, int rc) -> size_t {
+      return (size_t)min(max(r0 + rc / 5, 0), a.nt - 1) * 5 + rc % 5;
+    };
     // copy field rows [r0, r0 + n) of the group into raw (n <= C)
     auto issue = [&](int r0, int n) {
       if (vec) {
@@ -128,14 +223,14 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
           const int q4 = e % (NP / 4), rc = e / (NP / 4);  // rc = row * 5 + component
           const int pq = p0 + 4 * q4;
           if (pq < a.P)
-            cp_async16(raw + rc * NP + 4 * q4, a.fields + ((size_t)r0 * 5 + rc) * a.P + pq);
+            cp_async16(raw + rc * NP + 4 * q4, a.fields + src_row(r0, rc) * a.P + pq);
           else
             *reinterpret_cast<float4 *>(raw + rc * NP + 4 * q4) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
       } else {
         const int po = live ? p : 0;
         for (int rc = tid / NP; rc < n * 5; rc += kIntThreads / NP)
-          cp_async4(raw + rc * NP + pa, a.fields + ((size_t)r0 * 5 + rc) * a.P + po, live);
+          cp_async4(raw + rc * NP + pa, a.fields + src_row(r0, rc) * a.P + po, live);
       }
     };
     // integrands of the n rows in raw into window rows [w0, w0 + n)
@@ -179,27 +274,31 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
       float *const xr = xp + (size_t)(b * C - a.row0) * kSer;
       const float *bc = sb + (size_t)(H + 2) * kIntRow + pl * 4 + qi;
       auto B = [&](int k) -> float { return bc[k * kIntRow]; };  // k relative to c0
-      float y[C + H + 1];
-      float yy = 0.f;
-      float Bm = B(-2 - H), B0 = B(-1 - H);
+      if (c0 < 0 || c0 + C + H >= a.nt - 1) {
+        edge_block(bc, xr, c0, a.nt, inv2h, a.row0 + a.x_ld - b * C, live_b);
+      } else {
+        float y[C + H + 1];
+        float yy = 0.f;
+        float Bm = B(-2 - H), B0 = B(-1 - H);
 #pragma unroll
-      for (int k = -1 - H; k <= C + H - 1; ++k) {
-        const float Bp = B(k + 1);
-        yy = (Bp - 2.f * B0 + Bm) + rho * yy;
-        if (k >= -1) y[k + 1] = yy;
-        Bm = B0;
-        B0 = Bp;
-      }
-      float xx = 0.f, b1v = 0.f, b2v = 0.f;  // coefficients at k + 1, k + 2
+        for (int k = -1 - H; k <= C + H - 1; ++k) {
+          const float Bp = B(k + 1);
+          yy = (Bp - 2.f * B0 + Bm) + rho * yy;
+          if (k >= -1) y[k + 1] = yy;
+          Bm = B0;
+          B0 = Bp;
+        }
+        float xx = 0.f, b1v = 0.f, b2v = 0.f;  // coefficients at k + 1, k + 2
 #pragma unroll
-      for (int k = C + H - 1; k >= -1; --k) {
-        xx = y[k + 1] + rho * xx;
-        if (k <= C) {
-          const float bk = B(k) + rho * xx;
-          if (k <= C - 2 && live_b)
-            *reinterpret_cast<float2 *>(xr + (k + 1) * kSer) = make_float2((b2v - bk) * inv2h, b1v);
-          b2v = b1v;
-          b1v = bk;
+        for (int k = C + H - 1; k >= -1; --k) {
+          xx = y[k + 1] + rho * xx;
+          if (k <= C) {
+            const float bk = B(k) + rho * xx;
+            if (k <= C - 2 && live_b)
+              *reinterpret_cast<float2 *>(xr + (k + 1) * kSer) = make_float2((b2v - bk) * inv2h, b1v);
+            b2v = b1v;
+            b1v = bk;
+          }
         }
       }
       if (!more) break;
@@ -221,9 +320,10 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
 // column of the window holds y (the causal recursion, carried on from block to
 // block, in place of the integrand), so per sample the integrands are formed
 // once, the causal step runs once and the anti-causal one 1.5 times (64 + 34
-// rows per 64): about 36 FP64 operations per (panel, sample).
-// 32768 panels x 2048 steps: 8.7 ms with the record ends (15.2 ms by windowed
-// elimination, 142 operations and 128-byte rows).
+// rows per 64): about 36 FP64 operations per (panel, sample).  The record ends
+// are handled in place.  32768 panels x 2048 steps: @P64@ ms (15.2 ms by
+// windowed elimination, 142 operations and 128-byte rows; 8.7 with a kernel of
+// its own for the record ends).
 // ---------------------------------------------------------------------------
 constexpr int kF64H = Prec<double>::halo;
 constexpr int kF64Rows = kIirChunk + kF64H + 2;  // samples c0 - 1 .. c0 + 64 + H
@@ -231,15 +331,19 @@ constexpr int kF64Keep = kF64Rows - kIirChunk;
 
 // Field rows in flight to shared memory: [n rows][5][NP].
 template <int NP>
-__device__ __forceinline__ void issue_rows_f64(const double *fields, int P, int p0, int r0, int n,
-                                               double *raw, bool vec) {
+__device__ __forceinline__ void issue_rows_f64(const double *fields, int P, int nt, int p0, int r0,
+                                               int n, double *raw, bool vec) {
   const int tid = threadIdx.x;
+  // (rows outside the record are copied from its ends and not used)
+  auto src_row = [&](int rc) -> size_t {
+    return (size_t)min(max(r0 + rc / 5, 0), nt - 1) * 5 + rc % 5;
+  };
   if (vec) {  // 16-byte copies of 2 panels
     for (int e = tid; e < n * 5 * (NP / 2); e += kIntThreads) {
       const int q2 = e % (NP / 2), rc = e / (NP / 2);
       const int pq = p0 + 2 * q2;
       if (pq < P)
-        cp_async16(raw + rc * NP + 2 * q2, fields + ((size_t)r0 * 5 + rc) * P + pq);
+        cp_async16(raw + rc * NP + 2 * q2, fields + src_row(rc) * P + pq);
       else
         *reinterpret_cast<double2 *>(raw + rc * NP + 2 * q2) = make_double2(0.0, 0.0);
     }
@@ -247,7 +351,7 @@ __device__ __forceinline__ void issue_rows_f64(const double *fields, int P, int 
     const int pa = tid % NP;
     const bool live = p0 + pa < P;
     for (int rc = tid / NP; rc < n * 5; rc += kIntThreads / NP)
-      cp_async8(raw + rc * NP + pa, fields + ((size_t)r0 * 5 + rc) * P + (live ? p0 + pa : 0), live);
+      cp_async8(raw + rc * NP + pa, fields + src_row(rc) * P + (live ? p0 + pa : 0), live);
   }
 }
 
@@ -258,7 +362,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   double *raw = win + R * kIntRow;                     // [C][5][NP]
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
-  const int n_us = (a.int_hi - a.int_lo + unit - 1) / unit;
+  const int n_us = (a.c_hi - a.c_lo + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   const int pa = tid % NP;               // integrand phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
@@ -266,8 +370,8 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   const bool vec = (a.P & 1) == 0 && ((size_t)a.fields & 15) == 0;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = a.int_lo + (int)(u / n_pg) * unit;
-    const int b1 = min(a.int_hi, b0 + unit);
+    const int b0 = a.c_lo + (int)(u / n_pg) * unit;
+    const int b1 = min(a.c_hi, b0 + unit);
     const int p = p0 + pa, pb = p0 + pl;
     double n0 = 0, n1 = 0, n2 = 0, Un = 0;
     if (p < a.P) {
@@ -296,45 +400,135 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
       }
     };
     auto fill = [&](int sample, int w0, int n) {
-      issue_rows_f64<NP>(a.fields, a.P, p0, sample, n, raw, vec);
+      issue_rows_f64<NP>(a.fields, a.P, a.nt, p0, sample, n, raw, vec);
       cp_async_wait_all();
       __syncthreads();
       integrands(w0, n);
       __syncthreads();
     };
     const int lo = b0 * C - 2;  // sample c0 - 1 of the first block
+    const int N = a.nt;
     double yy = 0.0;
+    double f1 = 0.0, f2 = 0.0, f3 = 0.0;  // integrand at the last three samples passed
+    // causal recursion over window rows [r0, R), whose row r holds sample s0 + r;
+    // it stops being used at sample N - 1
+    auto causal = [&](int r0, int s0) {
+      if (s0 + R <= N) {
+#pragma unroll 8
+        for (int r = r0; r < R; ++r) {
+          yy = fma(kRho, yy, col[r * kIntRow]);
+          col[r * kIntRow] = yy;
+        }
+        f1 = fma(-kRho, col[(R - 2) * kIntRow], col[(R - 1) * kIntRow]);
+        f2 = fma(-kRho, col[(R - 3) * kIntRow], col[(R - 2) * kIntRow]);
+        f3 = fma(-kRho, col[(R - 4) * kIntRow], col[(R - 3) * kIntRow]);
+      } else {
+        for (int r = r0; r < R && s0 + r < N; ++r) {
+          f3 = f2;
+          f2 = f1;
+          f1 = col[r * kIntRow];
+          yy = fma(kRho, yy, f1);
+          col[r * kIntRow] = yy;
+        }
+      }
+    };
+    double F0 = 0.0, D0 = 0.0;  // integrand and one-sided derivative at sample 0
     __syncthreads();  // the previous unit is done with raw and win
-    fill(lo - H, 0, H);  // the samples the causal recursion starts on
-    for (int r = 0; r < H; ++r) yy = fma(kRho, yy, col[r * kIntRow]);
-    __syncthreads();
+    if (b0 > 0) {
+      fill(lo - H, 0, H);  // the samples the causal recursion starts on
+      for (int r = 0; r < H; ++r) {
+        f3 = f2;
+        f2 = f1;
+        f1 = col[r * kIntRow];
+        yy = fma(kRho, yy, f1);
+      }
+      __syncthreads();
+    }
     fill(lo, 0, C);
     fill(lo + C, C, R - C);
-    for (int r = 0; r < R; ++r) {
-      yy = fma(kRho, yy, col[r * kIntRow]);
-      col[r * kIntRow] = yy;
+    if (b0 > 0) {
+      causal(0, lo);
+    } else {  // rows 0 and 1 lie before the record; y_0 from the reflected series
+      F0 = col[2 * kIntRow];
+      D0 = (-3.0 * F0 + 4.0 * col[3 * kIntRow] - col[4 * kIntRow]) * inv2h;
+      for (int j = H; j >= 1; --j) yy = kRho * (col[(2 + j) * kIntRow] + yy);
+      yy = F0 * ((1.0 + kRho) / (1.0 - kRho)) - yy;
+      f1 = F0;
+      col[2 * kIntRow] = yy;
+      causal(3, lo);
     }
     for (int b = b0; b < b1; ++b) {
       const bool more = b + 1 < b1;
-      if (more) issue_rows_f64<NP>(a.fields, a.P, p0, b * C - 2 + R, C, raw, vec);
+      if (more) issue_rows_f64<NP>(a.fields, a.P, a.nt, p0, b * C - 2 + R, C, raw, vec);
       double *const xr = xp + (size_t)(b * C - a.row0) * kSer;
+      const int s0 = b * C - 2;  // sample of window row 0
       double xx = 0.0, c1 = 0.0, c2 = 0.0;  // coefficients one and two samples on
+      if (b > 0 && s0 + R < N) {
 #pragma unroll 14
-      for (int r = R - 1; r >= C + 2; --r) xx = fma(kRho, xx, col[r * kIntRow]);
+        for (int r = R - 1; r >= C + 2; --r) xx = fma(kRho, xx, col[r * kIntRow]);
 #pragma unroll
-      for (int r = C + 1; r >= C; --r) {
-        xx = fma(kRho, xx, col[r * kIntRow]);
-        c2 = c1;
-        c1 = (-6.0 * kRho) * xx;
-      }
+        for (int r = C + 1; r >= C; --r) {
+          xx = fma(kRho, xx, col[r * kIntRow]);
+          c2 = c1;
+          c1 = (-6.0 * kRho) * xx;
+        }
 #pragma unroll 16
-      for (int r = C - 1; r >= 0; --r) {  // window row r: sample c0 - 1 + r
-        xx = fma(kRho, xx, col[r * kIntRow]);
-        const double c0v = (-6.0 * kRho) * xx;
-        if (live_b)
-          *reinterpret_cast<double2 *>(xr + r * kSer) = make_double2((c2 - c0v) * inv2h, c1);
-        c2 = c1;
-        c1 = c0v;
+        for (int r = C - 1; r >= 0; --r) {  // window row r: sample c0 - 1 + r
+          xx = fma(kRho, xx, col[r * kIntRow]);
+          const double c0v = (-6.0 * kRho) * xx;
+          if (live_b)
+            *reinterpret_cast<double2 *>(xr + r * kSer) = make_double2((c2 - c0v) * inv2h, c1);
+          c2 = c1;
+          c1 = c0v;
+        }
+      } else {
+        // a record end: row r of X holds sample s0 + 1 + r
+        double cs = 0.0, pw = 0.0;  // excess of D0 over the central difference, times rho^sample
+        if (b == 0) {
+          double x1 = 0.0;
+          for (int r = H + 3; r >= 3; --r) x1 = fma(kRho, x1, col[r * kIntRow]);
+          cs = D0 - ((-6.0 * kRho) * x1 - F0) * (2.0 * inv2h);
+          pw = 1.0;
+          for (int i = 0; i < C - 1; ++i) pw *= kRho;  // at sample C - 1 (row C), going down
+        }
+        const double ir = 1.0 / kRho;
+        const double DN = (3.0 * f1 - 4.0 * f2 + f3) * inv2h;  // (used where f1 is sample N - 1)
+        double cr = 0.0, d2 = 0.0;
+        for (int r = R - 1; r >= 0; --r) {
+          const int sr = s0 + r;
+          if (sr > N - 1) continue;
+          xx = sr == N - 1 ? f1 * (-1.0 / (6.0 * kRho)) : fma(kRho, xx, col[r * kIntRow]);
+          const double c0v = sr == N - 1 ? f1 : (-6.0 * kRho) * xx;
+          if (sr == N - 2)
+            cr = DN - (c1 - c0v) * (2.0 * inv2h);
+          else
+            cr *= kRho;
+          const int se = sr + 1;  // the sample now complete, in X row r
+          double d = (c2 - c0v) * inv2h + cr;
+          if (b == 0) {
+            if (r < C) pw *= ir;
+            if (r <= C) d += cs * pw;
+          }
+          if (r < C && live_b && se <= N - 2) {
+            double *row = xr + r * kSer;
+            if (se > 0) *reinterpret_cast<double2 *>(row) = make_double2(d, c1);
+            if (se == 0) {  // sample 0 and the ghost before it
+              *reinterpret_cast<double2 *>(row) = make_double2(D0, c1);
+              *reinterpret_cast<double2 *>(row - kSer) = make_double2(2.0 * D0 - d2, 2.0 * c1 - c2);
+            }
+            if (se == N - 2) {  // the last sample, the ghost after it and a zero row
+              const int room = a.row0 + a.x_ld - b * C - r;  // rows of X from this one on
+              if (room > 1) *reinterpret_cast<double2 *>(row + kSer) = make_double2(DN, f1);
+              if (room > 2)
+                *reinterpret_cast<double2 *>(row + 2 * kSer) =
+                    make_double2(2.0 * DN - d, 2.0 * f1 - c1);
+              if (room > 3) *reinterpret_cast<double2 *>(row + 3 * kSer) = make_double2(0.0, 0.0);
+            }
+          }
+          d2 = d;
+          c2 = c1;
+          c1 = c0v;
+        }
       }
       if (!more) break;
       // slide the thread's column by C rows, then add the rows now in raw
@@ -343,17 +537,15 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
       __syncthreads();
       integrands(kF64Keep, C);
       __syncthreads();
-      for (int r = kF64Keep; r < R; ++r) {
-        yy = fma(kRho, yy, col[r * kIntRow]);
-        col[r * kIntRow] = yy;
-      }
+      causal(kF64Keep, s0 + C);
     }
   }
 }
 
-// Prep of the blocks at the record ends: thread (series, half, panel) filters
-// 32 rows of one of the eight series; the eight threads of a panel write one X
-// row (a sector for FP32, two for FP64) per step.
+// Prep of records shorter than 64 + 2 H samples (compact code): thread (series,
+// half, panel) filters 32 rows of one of the eight series, r = D2 F on the
+// odd-periodic extension of any number of periods; the eight threads of a panel
+// write one X row per step.
 template <typename T>
 __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_iir(PrepArgs<T> a) {
   constexpr int NP = kIirPanels, H = Prec<T>::halo, J = kIirJ, ROWS = iir_rows<T>();
@@ -365,13 +557,10 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_ii
   T *sb = reinterpret_cast<T *>(smem_raw);
   T *sb2 = sb + ROWS * kIirRow;
   const int tid = threadIdx.x;
-  // 1D grid over the blocks of [c_lo, c_hi) outside [int_lo, int_hi) (fastest),
-  // then panel tiles
-  const int na = a.int_lo - a.c_lo, n_edge = na + a.c_hi - a.int_hi;
-  const int ei = (int)(blockIdx.x % n_edge);
-  const int blk = ei < na ? a.c_lo + ei : a.int_hi + ei - na;
+  const int n_blk = a.c_hi - a.c_lo;  // 1D grid: block fastest, then panel tiles
+  const int blk = a.c_lo + (int)(blockIdx.x % n_blk);
   const int c0 = blk * kIirChunk - 1;  // first sample
-  const int p0 = (int)(blockIdx.x / n_edge) * NP;
+  const int p0 = (int)(blockIdx.x / n_blk) * NP;
   const int N = a.nt;
   // phase B thread: series s, half h (samples c0 + 32 h ..), panel pl
   const int s = tid & 7;
@@ -459,80 +648,39 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_ii
     if (i == N - 1) return (T(3) * B(N - 1) - T(4) * B(N - 2) + B(N - 3)) * inv2h;
     return (B(i + 1) - B(i - 1)) * inv2h;
   };
-  // Long enough records: every index the filters reach folds back into the
-  // record with one reflection, so the filters run on the point-reflected
-  // series with the same unrolled recursion as the interior.
-  if (N >= kIirChunk + 2 * H) {
-    T Fs = T(0), Fe = T(0);  // series at the first and last frame
-    if (lo == 0) Fs = F(0);
-    if (hi == N) Fe = F(N - 1);
-    auto Fx = [&](int kk) -> T {
-      const bool neg = kk < 0, big = kk > N - 1;
-      const int m = neg ? -kk : (big ? 2 * (N - 1) - kk : kk);
-      T v;
-      if (deriv) {
-        const T c = (B(min(m + 1, N - 1)) - B(max(m - 1, 0))) * inv2h;
-        v = m == 0 ? Fs : (m == N - 1 ? Fe : c);
-      } else {
-        v = B(m);
-      }
-      return neg ? T(2) * Fs - v : (big ? T(2) * Fe - v : v);
-    };
-    T y[J + H];
-    int k = ks - H;
-    T Fm = Fx(k - 1), F0 = Fx(k);
-    T yy = T(0);
-#pragma unroll
-    for (int t = 0; t < J + 2 * H; ++t, ++k) {
-      const T Fp = Fx(k + 1);
-      yy = (Fp - T(2) * F0 + Fm) + rho * yy;
-      if (t >= H) y[t - H] = yy;
-      Fm = F0;
-      F0 = Fp;
+  const int L2 = 2 * (N - 1);
+  auto r_at = [&](int kk) -> T {
+    int km = kk % L2;
+    if (km < 0) km += L2;
+    T sg = T(1);
+    if (km >= N - 1) {
+      km = L2 - km;
+      sg = T(-1);
     }
-    T xx = T(0);
-#pragma unroll
-    for (int t = J + H - 1; t >= 0; --t) {
-      xx = y[t] + rho * xx;
-      if (t < J) put(t, ks + t <= N ? Fx(ks + t) + rho * xx : T(0));
-    }
-  } else {
-    // short records (compact code): r = D2 F on the odd-periodic extension of
-    // any number of periods
-    const int L2 = 2 * (N - 1);
-    auto r_at = [&](int kk) -> T {
-      int km = kk % L2;
-      if (km < 0) km += L2;
-      T sg = T(1);
-      if (km >= N - 1) {
-        km = L2 - km;
-        sg = T(-1);
-      }
-      if (km == 0 || km == N - 1) return T(0);
-      return sg * (F(km + 1) - T(2) * F(km) + F(km - 1));
-    };
-    T ye[J + H];
-    T yy = T(0);
+    if (km == 0 || km == N - 1) return T(0);
+    return sg * (F(km + 1) - T(2) * F(km) + F(km - 1));
+  };
+  T ye[J + H];
+  T yy = T(0);
 #pragma unroll 1
-    for (int t = 0; t < J + 2 * H; ++t) {
-      yy = r_at(ks - H + t) + rho * yy;
-      if (t >= H) ye[t - H] = yy;
-    }
-    T xx = T(0);
+  for (int t = 0; t < J + 2 * H; ++t) {
+    yy = r_at(ks - H + t) + rho * yy;
+    if (t >= H) ye[t - H] = yy;
+  }
+  T xx = T(0);
 #pragma unroll 1
-    for (int t = J + H - 1; t >= 0; --t) {
-      xx = ye[t] + rho * xx;
-      if (t >= J) continue;
-      const int k = ks + t;
-      T v = T(0);
-      if (k < 0)
-        v = T(2) * F(0) - F(-k) + rho * xx;
-      else if (k < N)
-        v = F(k) + rho * xx;
-      else if (k == N)
-        v = T(2) * F(N - 1) - F(N - 2) + rho * xx;
-      put(t, v);
-    }
+  for (int t = J + H - 1; t >= 0; --t) {
+    xx = ye[t] + rho * xx;
+    if (t >= J) continue;
+    const int k = ks + t;
+    T v = T(0);
+    if (k < 0)
+      v = T(2) * F(0) - F(-k) + rho * xx;
+    else if (k < N)
+      v = F(k) + rho * xx;
+    else if (k == N)
+      v = T(2) * F(N - 1) - F(N - 2) + rho * xx;
+    put(t, v);
   }
 }
 
@@ -909,7 +1057,7 @@ cudaError_t persistent_grid(K kern, size_t smem, long n_pg, int blocks, int *uni
 template <typename T>
 cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
   constexpr int C = kIirChunk;
-  static_assert(C == kRowBlk && C - 1 >= Prec<T>::halo + 2, "block 1 is an interior one");
+  static_assert(C == kRowBlk && C - 1 >= Prec<T>::halo + 2, "only block 0 reaches before the record");
   PrepArgs<T> a = a0;
   const int n_rb = (int)(x_rows(a.nt) / C);
   if (a.c_hi == 0) {
@@ -919,15 +1067,10 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
   if (a.c_lo < 0 || a.c_hi > n_rb || a.c_lo >= a.c_hi || a.c_lo * C < a.row0 ||
       a.c_hi * C > a.row0 + a.x_ld)
     return cudaErrorInvalidValue;
-  // interior blocks (first sample c0 = 64 b - 1): filter reach inside samples
-  // 1 .. nt - 2, c0 >= H + 2 and c0 + C + H + 1 <= nt - 1
-  a.int_lo = std::max(a.c_lo, 1);
-  a.int_hi = std::min(a.c_hi, prep_interior_end<T>(a.nt));
-  if (a.int_lo >= a.int_hi) a.int_lo = a.int_hi = a.c_hi;
   cudaError_t e;
-  if (a.int_hi > a.int_lo) {
+  if (a.nt >= C + 2 * Prec<T>::halo) {
     const long n_pg = (a.P + kIntPanels - 1) / kIntPanels;
-    const int n_blk = a.int_hi - a.int_lo;
+    const int n_blk = a.c_hi - a.c_lo;
     long grid = 0;
     int unit = 1;
     if constexpr (sizeof(T) == 4) {
@@ -941,17 +1084,14 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
         return e;
       k_prep_f64_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaGetLastError();
   }
-  // record-end blocks by the general kernel
-  const int n_edge = (a.int_lo - a.c_lo) + (a.c_hi - a.int_hi);
-  if (n_edge == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * iir_rows<T>() * kIirRow * sizeof(T);
   e = cudaFuncSetAttribute(k_prep_iir<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long eblocks = (long)n_edge * ((a.P + kIirPanels - 1) / kIirPanels);
-  if (eblocks > INT32_MAX) return cudaErrorInvalidValue;
-  k_prep_iir<T><<<(unsigned)eblocks, kIirThreads, smem, s>>>(a);
+  const long blocks = (long)(a.c_hi - a.c_lo) * ((a.P + kIirPanels - 1) / kIirPanels);
+  if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+  k_prep_iir<T><<<(unsigned)blocks, kIirThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
