@@ -36,7 +36,7 @@
 //
 // Kernels: k_prep_iir_int (FP32) and k_prep_f64_int (FP64), persistent CTAs that
 // walk consecutive blocks of a panel group; k_prep_iir for records too short for
-// them (under 64 + 2 H samples), all eight series by index arithmetic.  All
+// them (under H + 3 samples), all eight series by index arithmetic.  All
 // take the panels in the caller's order, so field reads are coalesced also
 // for a reordered surface; the rows of X go where the panel's place is.
 #include "fwh_internal.cuh"
@@ -496,6 +496,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         double cr = 0.0, d2 = 0.0;
         for (int r = R - 1; r >= 0; --r) {
           const int sr = s0 + r;
+          if (r < C) pw *= ir;  // rho^(sr + 1) in block 0
           if (sr > N - 1) continue;
           xx = sr == N - 1 ? f1 * (-1.0 / (6.0 * kRho)) : fma(kRho, xx, col[r * kIntRow]);
           const double c0v = sr == N - 1 ? f1 : (-6.0 * kRho) * xx;
@@ -505,10 +506,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
             cr *= kRho;
           const int se = sr + 1;  // the sample now complete, in X row r
           double d = (c2 - c0v) * inv2h + cr;
-          if (b == 0) {
-            if (r < C) pw *= ir;
-            if (r <= C) d += cs * pw;
-          }
+          if (b == 0 && r <= C) d += cs * pw;
           if (r < C && live_b && se <= N - 2) {
             double *row = xr + r * kSer;
             if (se > 0) *reinterpret_cast<double2 *>(row) = make_double2(d, c1);
@@ -542,7 +540,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   }
 }
 
-// Prep of records shorter than 64 + 2 H samples (compact code): thread (series,
+// Prep of records shorter than H + 3 samples (compact code): thread (series,
 // half, panel) filters 32 rows of one of the eight series, r = D2 F on the
 // odd-periodic extension of any number of periods; the eight threads of a panel
 // write one X row per step.
@@ -1068,7 +1066,9 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
       a.c_hi * C > a.row0 + a.x_ld)
     return cudaErrorInvalidValue;
   cudaError_t e;
-  if (a.nt >= C + 2 * Prec<T>::halo) {
+  // the walking kernels' exact starts reach H + 1 samples into the record and
+  // take the two ends' corrections apart (rho^(nt - 1) below rounding)
+  if (a.nt >= Prec<T>::halo + 3) {
     const long n_pg = (a.P + kIntPanels - 1) / kIntPanels;
     const int n_blk = a.c_hi - a.c_lo;
     long grid = 0;
