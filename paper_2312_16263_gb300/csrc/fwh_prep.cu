@@ -42,6 +42,7 @@
 #include "fwh_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 #include <cstdint>
 
@@ -67,14 +68,17 @@ constexpr int kIirRow = 4 * kIirQ;                   // staged row stride (value
 // an X row.  Bound by HBM: 20 bytes in and 32 out per (panel, sample), 5.5 TB/s
 // (81 % of a copy's).  The blocks at the record ends take the same filters with
 // exact starts (edge_block); as a kernel of their own that filtered all eight
-// reflected series they took 0.32 of 0.88 ms at 32768 panels x 2048 steps,
-// here @EDGE@.
+// reflected series they took 0.32 of 0.88 ms at 32768 panels x 2048 steps; the
+// whole prep now takes 0.68.
 // ---------------------------------------------------------------------------
 constexpr int kIntPanels = 16;
 constexpr int kIntThreads = kIntPanels * 4;
 constexpr int kIntRow = kIntPanels * 4;              // staged row: [panel][integrand]
 constexpr int kIntRows = kIirChunk + 2 * kIirH + 3;  // samples c0 - H - 2 .. c0 + 64 + H
 constexpr int kIntKeep = kIntRows - kIirChunk;       // rows shared by consecutive blocks
+// fields of 64 frames in flight, or (record ends) y of 81 rows of the window
+constexpr int kIntRaw = kIirChunk * 5 * kIntPanels + kIntRow;
+static_assert(kIntRaw >= (kIirChunk + kIirH + 1) * kIntRow, "y of an end block fits");
 constexpr int kIntUnit = 8;                          // most blocks per work unit
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool ok) {
@@ -97,77 +101,83 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// rho^k for k < kIirH + 4, zero beyond (below FP32 rounding).
-__host__ __device__ constexpr float rho_pow(int k) {
-  double v = k < kIirH + 4 ? 1.0 : 0.0;
-  for (int i = 0; i < k && i < kIirH + 4; ++i) v *= kRho;
-  return (float)v;
-}
+// rho^k, k < kIirH + 4 (below FP32 rounding from there on).
+struct RhoPow {
+  float v[kIirH + 4];
+  constexpr RhoPow() : v() {
+    double p = 1.0;
+    for (int i = 0; i < kIirH + 4; ++i, p *= kRho) v[i] = (float)p;
+  }
+};
+__constant__ RhoPow c_rho_pow = RhoPow();
 
 // A block at a record end: bc[k kIntRow] is the integrand of sample c0 + k (valid
-// inside the record), xr the thread's pair in the block's first X row, `room` the
-// rows of X from there on.
-__device__ __forceinline__ void edge_block(const float *bc, float *xr, int c0, int N, float inv2h,
-                                           int room, bool store) {
+// inside the record), ys[(k + 1) kIntRow] takes y, xr is the thread's pair in the
+// block's first X row, `room` the rows of X from there on.  Compact loops: a
+// small problem has little else to do, and unrolled code reaches it through
+// cold instruction caches (24 us for 64 panels x 48 steps unrolled, 18 so).
+__device__ __forceinline__ void edge_block(const float *bc, float *ys, float *xr, int c0, int N,
+                                           float inv2h, int room, bool store) {
   constexpr int H = kIirH, C = kIirChunk;
   constexpr float rho = (float)kRho;
   auto B = [&](int k) -> float { return bc[k * kIntRow]; };
-  const bool start = c0 < 0;  // c0 = -1: sample 0 at k = 1
-  float y0 = 0.f;             // y of sample 0
-  if (start) {
-#pragma unroll
-    for (int j = H; j >= 1; --j) y0 = (y0 - (B(j + 2) - 2.f * B(j + 1) + B(j))) * rho;
-  }
-  float y[C + H + 1];
+  auto y = [&](int k) -> float & { return ys[(k + 1) * kIntRow]; };
+  const bool start = c0 < 0;                    // c0 = -1: sample 0 at k = 1
+  const int top = min(C + H, N - 1 - c0);       // the anti-causal recursion starts here
   float yy = 0.f;
-#pragma unroll
-  for (int k = -1 - H; k <= C + H - 1; ++k) {
-    if (k <= 1 && start)
-      yy = k == 1 ? y0 : 0.f;
-    else
-      yy = (B(k + 1) - 2.f * B(k) + B(k - 1)) + rho * yy;
-    if (k >= -1) y[k + 1] = yy;
+  int k = -1 - H;
+  if (start) {  // y of sample 0 from the reflected series
+    for (int j = H; j >= 1; --j) yy = (yy - (B(j + 2) - 2.f * B(j + 1) + B(j))) * rho;
+    y(-1) = y(0) = 0.f;
+    y(1) = yy;
+    k = 2;
   }
-  float D0 = 0.f, cs = 0.f;  // one-sided derivative at sample 0, its excess over the central one
+  {
+    float Bm = B(k - 1), B0 = B(k);
+#pragma unroll 4
+    for (; k < top; ++k) {
+      const float Bp = B(k + 1);
+      yy = (Bp - 2.f * B0 + Bm) + rho * yy;
+      if (k >= -1) y(k) = yy;
+      Bm = B0;
+      B0 = Bp;
+    }
+  }
+  float D0 = 0.f, ex = 0.f;  // one-sided derivative at sample 0, its excess over the central one
   if (start) {
     float x1 = 0.f;
-#pragma unroll
-    for (int k = H + 2; k >= 2; --k) x1 = y[k + 1] + rho * x1;
+    for (int j = H + 2; j >= 2; --j) x1 = y(j) + rho * x1;
     D0 = (-3.f * B(1) + 4.f * B(2) - B(3)) * inv2h;
-    cs = D0 - (B(2) + rho * x1 - B(1)) * (2.f * inv2h);
+    ex = D0 - (B(2) + rho * x1 - B(1)) * (2.f * inv2h);
   }
   float xx = 0.f, b1v = 0.f, b2v = 0.f, cr = 0.f, DN = 0.f, d2 = 0.f;
-#pragma unroll
-  for (int k = C + H - 1; k >= -1; --k) {
+#pragma unroll 2
+  for (k = top; k >= -1; --k) {
     const int sk = c0 + k;
-    xx = sk >= N - 1 ? 0.f : y[k + 1] + rho * xx;
+    if (k < top) xx = y(k) + rho * xx;
     const float bk = B(k) + rho * xx;
+    cr *= rho;
     if (sk == N - 2) {
       DN = (3.f * B(k + 1) - 4.f * B(k) + B(k - 1)) * inv2h;
       cr = DN - (b1v - bk) * (2.f * inv2h);
-    } else if (sk < N - 2) {
-      cr *= rho;
     }
-    // sample sk + 1 = c0 + e
+    // sample se = sk + 1, row e of the block, is now complete
     const int e = k + 1, se = sk + 1;
     float d = (b2v - bk) * inv2h + cr;
-    if (e >= 2) d += cs * rho_pow(e - 1);
-    if (e <= C - 1 && store) {
-      float *row = xr + e * kSer;
-      if (se == N + 1) {
-        *reinterpret_cast<float2 *>(row) = make_float2(0.f, 0.f);
-      } else if (se <= N - 2 && !(start && e <= 1)) {
-        *reinterpret_cast<float2 *>(row) = make_float2(d, b1v);
-        if (se == N - 2) {  // the last sample and the ghost after it
-          const float bN = B(e + 1);
-          if (e + 1 < room) *reinterpret_cast<float2 *>(row + kSer) = make_float2(DN, bN);
-          if (e + 2 < room)
-            *reinterpret_cast<float2 *>(row + 2 * kSer) =
-                make_float2(2.f * DN - d, 2.f * bN - b1v);
-        }
-      } else if (start && e == 1) {  // sample 0 and the ghost before it
-        *reinterpret_cast<float2 *>(row) = make_float2(D0, b1v);
-        *reinterpret_cast<float2 *>(row - kSer) = make_float2(2.f * D0 - d2, 2.f * b1v - b2v);
+    if (start && se < H + 4 && se > 0) d += ex * c_rho_pow.v[se];
+    if (e < C && se <= N - 2 && store) {
+      float2 *row = reinterpret_cast<float2 *>(xr + e * kSer);
+      constexpr int NR = kSer / 2;  // a row in pairs
+      if (!(start && e <= 1)) *row = make_float2(d, b1v);
+      if (start && e == 1) {  // sample 0 and the ghost before it
+        row[0] = make_float2(D0, b1v);
+        row[-NR] = make_float2(2.f * D0 - d2, 2.f * b1v - b2v);
+      }
+      if (se == N - 2) {  // the last sample, the ghost after it and a zero row
+        const float bN = B(e + 1);
+        if (e + 1 < room) row[NR] = make_float2(DN, bN);
+        if (e + 2 < room) row[2 * NR] = make_float2(2.f * DN - d, 2.f * bN - b1v);
+        if (e + 3 < room) row[3 * NR] = make_float2(0.f, 0.f);
       }
     }
     d2 = d;
@@ -269,13 +279,15 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
     for (int b = b0; b < b1; ++b) {
       const int c0 = b * C - 1;  // first sample: row b C holds it
       const bool more = b + 1 < b1;
-      if (more) issue(c0 + C + H + 1, C);  // rows of the next window, in flight meanwhile
+      const bool edge = c0 < 0 || c0 + C + H >= a.nt - 1;
+      // rows of the next window, in flight meanwhile (a record end keeps y in raw)
+      if (more && !edge) issue(c0 + C + H + 1, C);
       // ---- phase B: filters of block b ----------------------------------------
       float *const xr = xp + (size_t)(b * C - a.row0) * kSer;
       const float *bc = sb + (size_t)(H + 2) * kIntRow + pl * 4 + qi;
       auto B = [&](int k) -> float { return bc[k * kIntRow]; };  // k relative to c0
-      if (c0 < 0 || c0 + C + H >= a.nt - 1) {
-        edge_block(bc, xr, c0, a.nt, inv2h, a.row0 + a.x_ld - b * C, live_b);
+      if (edge) {
+        edge_block(bc, raw + pl * 4 + qi, xr, c0, a.nt, inv2h, a.row0 + a.x_ld - b * C, live_b);
       } else {
         float y[C + H + 1];
         float yy = 0.f;
@@ -304,6 +316,7 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
       if (!more) break;
       // ---- slide the window by C rows and add the rows now in raw --------------
       __syncthreads();  // every thread is done reading the window
+      if (edge) issue(c0 + C + H + 1, C);
       for (int e = tid; e < kIntKeep * kIntRow / 4; e += kIntThreads)
         reinterpret_cast<float4 *>(sb)[e] = reinterpret_cast<const float4 *>(sb + C * kIntRow)[e];
       cp_async_wait_all();
@@ -321,7 +334,7 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
 // block, in place of the integrand), so per sample the integrands are formed
 // once, the causal step runs once and the anti-causal one 1.5 times (64 + 34
 // rows per 64): about 36 FP64 operations per (panel, sample).  The record ends
-// are handled in place.  32768 panels x 2048 steps: @P64@ ms (15.2 ms by
+// are handled in place.  32768 panels x 2048 steps: 6.8 ms (15.2 ms by
 // windowed elimination, 142 operations and 128-byte rows; 8.7 with a kernel of
 // its own for the record ends).
 // ---------------------------------------------------------------------------
@@ -483,30 +496,34 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         }
       } else {
         // a record end: row r of X holds sample s0 + 1 + r
-        double cs = 0.0, pw = 0.0;  // excess of D0 over the central difference, times rho^sample
+        double pw = 0.0;  // excess of D0 over the central difference, times rho^sample
         if (b == 0) {
           double x1 = 0.0;
           for (int r = H + 3; r >= 3; --r) x1 = fma(kRho, x1, col[r * kIntRow]);
-          cs = D0 - ((-6.0 * kRho) * x1 - F0) * (2.0 * inv2h);
-          pw = 1.0;
-          for (int i = 0; i < C - 1; ++i) pw *= kRho;  // at sample C - 1 (row C), going down
+          pw = D0 - ((-6.0 * kRho) * x1 - F0) * (2.0 * inv2h);
+          for (int i = 0; i < H + 4; ++i) pw *= kRho;  // below rounding from sample H + 4 on
         }
         const double ir = 1.0 / kRho;
         const double DN = (3.0 * f1 - 4.0 * f2 + f3) * inv2h;  // (used where f1 is sample N - 1)
         double cr = 0.0, d2 = 0.0;
         for (int r = R - 1; r >= 0; --r) {
           const int sr = s0 + r;
-          if (r < C) pw *= ir;  // rho^(sr + 1) in block 0
           if (sr > N - 1) continue;
           xx = sr == N - 1 ? f1 * (-1.0 / (6.0 * kRho)) : fma(kRho, xx, col[r * kIntRow]);
           const double c0v = sr == N - 1 ? f1 : (-6.0 * kRho) * xx;
           if (sr == N - 2)
             cr = DN - (c1 - c0v) * (2.0 * inv2h);
-          else
+          else if (sr > N - 3 - (H + 4))  // below rounding further on
             cr *= kRho;
+          else
+            cr = 0.0;
           const int se = sr + 1;  // the sample now complete, in X row r
-          double d = (c2 - c0v) * inv2h + cr;
-          if (b == 0 && r <= C) d += cs * pw;
+          double d = (c2 - c0v) * inv2h;
+          if (cr != 0.0) d += cr;
+          if (b == 0 && se < H + 4) {
+            pw *= ir;
+            d += pw;
+          }
           if (r < C && live_b && se <= N - 2) {
             double *row = xr + r * kSer;
             if (se > 0) *reinterpret_cast<double2 *>(row) = make_double2(d, c1);
@@ -1031,24 +1048,44 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 5 : 2)
 
 }  // namespace
 
-// Persistent CTAs of an interior kernel over `blocks` blocks of n_pg panel
-// groups: as many as fit the GPU at once, and the blocks of a work unit (at
-// most kIntUnit: a unit starts with half a block's worth of extra rows), fewer
-// where the GPU would otherwise not be filled twice over.
-template <typename K>
-cudaError_t persistent_grid(K kern, size_t smem, long n_pg, int blocks, int *unit, long *grid) {
+// Persistent CTAs of a walking kernel over `blocks` blocks of n_pg panel groups:
+// as many as fit the GPU at once, and the blocks of a work unit (at most
+// kIntUnit), by the rounds of units each CTA takes times a unit's cost, its
+// blocks and `start` blocks' worth of rows to start on (0.68 ms at 32768 panels
+// x 2048 steps; 0.71 with the units that fill the GPU twice).  A small problem
+// gets one block a unit, so that its blocks run side by side.
+template <auto kern>
+cudaError_t persistent_grid(size_t smem, double start, long n_pg, int blocks, int *unit,
+                            long *grid) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
+  // CTAs that fit the device, looked up once per kernel and device
+  constexpr int kMaxDev = 64;
+  static std::atomic<int> fits[kMaxDev];
+  int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIntThreads, smem)) !=
-      cudaSuccess)
-    return e;
-  const long fit = (long)std::max(per_sm, 1) * sms;
-  *unit = (int)std::clamp<long>(n_pg * blocks / (2 * fit), 1, kIntUnit);
-  *grid = std::min<long>(n_pg * ((blocks + *unit - 1) / *unit), fit);
+  int fit = dev < kMaxDev ? fits[dev].load(std::memory_order_relaxed) : 0;
+  if (fit == 0) {
+    int sms = 0, per_sm = 0;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIntThreads, smem)) !=
+        cudaSuccess)
+      return e;
+    fit = std::max(per_sm, 1) * sms;
+    if (dev < kMaxDev) fits[dev].store(fit, std::memory_order_relaxed);
+  }
+  double best = 0.0;
+  *unit = 0;
+  for (int u = 1; u <= kIntUnit && u <= std::max(blocks, 1); ++u) {
+    const long units = n_pg * ((blocks + u - 1) / u);
+    const double cost = (double)((units + fit - 1) / fit) * (u + start);
+    if (*unit == 0 || cost < best) {
+      best = cost;
+      *unit = u;
+    }
+  }
+  *grid = std::min<long>(n_pg * ((blocks + *unit - 1) / *unit), (long)fit);
   return cudaSuccess;
 }
 
@@ -1074,13 +1111,13 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
     long grid = 0;
     int unit = 1;
     if constexpr (sizeof(T) == 4) {
-      const size_t smem = ((size_t)kIntRows * kIntRow + (size_t)C * 5 * kIntPanels) * sizeof(T);
-      if ((e = persistent_grid(k_prep_iir_int, smem, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+      const size_t smem = ((size_t)kIntRows * kIntRow + (size_t)kIntRaw) * sizeof(T);
+      if ((e = persistent_grid<k_prep_iir_int>(smem, 0.6, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
         return e;
       k_prep_iir_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     } else {
       const size_t smem = ((size_t)kF64Rows * kIntRow + (size_t)C * 5 * kIntPanels) * sizeof(T);
-      if ((e = persistent_grid(k_prep_f64_int, smem, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+      if ((e = persistent_grid<k_prep_f64_int>(smem, 1.0, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
         return e;
       k_prep_f64_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     }
@@ -1112,7 +1149,7 @@ cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s) {
     const size_t smem = ((size_t)(C + H) * kIntRow + (size_t)C * 4 * kIntPanels) * sizeof(T);
     long grid = 0;
     int unit = 1;
-    if ((e = persistent_grid(k_prep_adj_int<T>, smem, n_pg, int_hi - int_lo, &unit, &grid)) !=
+    if ((e = persistent_grid<k_prep_adj_int<T>>(smem, 0.5, n_pg, int_hi - int_lo, &unit, &grid)) !=
         cudaSuccess)
       return e;
     k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, int_lo, int_hi, unit);
