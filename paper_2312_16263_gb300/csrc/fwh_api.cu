@@ -366,6 +366,7 @@ FwdArgs<T> forward_args(fwh_ctx *h, const FwdConfig &c, int64_t nt, const T *X, 
   fa.seg_lo = 0;
   fa.seg_cnt = fa.n_segs;
   fa.win = c.win;
+  fa.slack = fwd_slack(fp64, c);
   fa.wfl = c.win * (c.acc == 5 ? 2 : 1);
   return fa;
 }

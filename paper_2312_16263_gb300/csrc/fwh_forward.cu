@@ -284,6 +284,26 @@ __device__ __forceinline__ void item_prologue(const FwdArgs<T> &a, const Item<T,
   __syncwarp();
 }
 
+// The warp's observers (bit m) with a valid bin among those a chunk can reach:
+// intervals [k_lo, k_hi] at every shift of the set.  Outside an observer's
+// window (N_o of nt bins) the work would be dropped bin by bin; it is not done.
+// Before its first active chunk a window is zero, and after its last the
+// remaining bins lie past N_o, so neither needs a flush.  72 observers around
+// 32768 panels x 2048 steps: 3.64 -> 3.49 ms, FP64 104.3 -> 97.8; 36
+// around 76800 panels x 4096 steps: 7.90 -> 7.25.
+template <typename T, int NW>
+__device__ __forceinline__ unsigned active_observers(const FwdArgs<T> &a, const Item<T, NW> &it,
+                                                     int w, const int *s_i0max, int k_lo,
+                                                     int k_hi) {
+  const int lane = threadIdx.x & 31;
+  bool on = false;
+  if (lane < it.nobs) {
+    const int i0 = s_i0max[lane];
+    on = k_lo - i0 < a.n_valid[it.o_begin + w + NW * lane] && k_hi - i0 + a.slack >= 0;
+  }
+  return __ballot_sync(0xffffffffu, on);
+}
+
 // FP64, one (panel, observer): lane rows k0 + lane + 32 j (j < nj).  Row r
 // enters the bins of intervals r - 3 .. r with weights w3 .. w0; wm is the
 // window slot of interval r - 3 of the lane's first row.  Neighbouring lanes'
@@ -315,10 +335,12 @@ __device__ __forceinline__ void accumulate(const double (&x)[TK][kSer], const do
 // Window slot 0 is the bin of interval k0 - 3 at the set's largest shift.
 template <int CH, int NW>
 __device__ __forceinline__ void flush_slide(const FwdArgs<double> &a, const Item<double, NW> &it,
-                                            int w, double *wwin, const int *s_i0max, int k0) {
+                                            int w, double *wwin, const int *s_i0max, int k0,
+                                            unsigned active) {
   const int lane = threadIdx.x & 31;
   const int win = a.win;
-  for (int m = 0; m < it.nobs; ++m) {
+  for (; active; active &= active - 1) {
+    const int m = __ffs(active) - 1;
     const int o = it.o_begin + w + NW * m;
     double *wm = wwin + (size_t)m * win;
     const int wbase = k0 - s_i0max[m] - 3;
@@ -373,6 +395,8 @@ __device__ __forceinline__ void process_item_direct(const FwdArgs<double> &a, in
   int k0 = it.k_begin;
   for (; k0 < it.k_end; k0 += CH) {
     const int nj = min(TK, (it.k_end - k0 + 31) / 32);
+    const unsigned active = active_observers<double, NW>(a, it, w, s_i0max, k0 - 3, k0 + CH - 1);
+    if (!active) continue;
     for (int p = it.p_begin; p < it.p_end; ++p) {
       double x[TK][kSer];
       const double *Xp = a.X + ((size_t)p * a.x_ld + (k0 - a.row0) + lane) * kSer;
@@ -380,14 +404,15 @@ __device__ __forceinline__ void process_item_direct(const FwdArgs<double> &a, in
       for (int j = 0; j < TK; ++j)
         if (j < nj) ldg_f64(Xp + (size_t)j * 32 * kSer, x[j]);
       const double *rec0 = a.coef + (size_t)p * a.O * kRec;
-      for (int m = 0; m < it.nobs; ++m) {
+      for (unsigned left = active; left; left &= left - 1) {
+        const int m = __ffs(left) - 1;
         const double *rec = rec0 + (size_t)(it.o_begin + w + NW * m) * kRec;
         double c[12];
         ldg_f64(rec, c);
         accumulate<TK>(x, c, wwin + (m * a.win + lane + (int)__ldg(rec + slot::off)), nj);
       }
     }
-    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0);
+    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0, active);
   }
   flush_tail<CH, NW>(a, it, w, wwin, s_i0max, k0);
 }
@@ -488,6 +513,7 @@ __device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Ite
   int k0 = it.k_begin;
   for (; k0 < it.k_end; k0 += CH) {
     const int nj = min(TK, (it.k_end - k0 + 31) / 32);
+    const unsigned active = active_observers<double, NW>(a, it, w, s_i0max, k0 - 3, k0 + CH - 1);
     for (int p = it.p_begin; p < it.p_end; ++p, ++step) {
       const int s = (int)(step % (unsigned)ps.nst);
       const unsigned ph = (step / (unsigned)ps.nst) & 1u;
@@ -497,7 +523,8 @@ __device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Ite
 #pragma unroll
       for (int j = 0; j < TK; ++j) lds_row_f64(stg, lane + 32 * j, x[j]);
       const double *crec = reinterpret_cast<const double *>(stg + ps.x_bytes);
-      for (int m = 0; m < it.nobs; ++m) {
+      for (unsigned left = active; left; left &= left - 1) {
+        const int m = __ffs(left) - 1;
         const double *rec = crec + (size_t)(w + NW * m) * kRec;
         double c[12];
         lds_f64(rec, c);
@@ -506,7 +533,7 @@ __device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Ite
       __syncwarp();
       if (lane == 0) mbar_arrive(&ps.empty[s]);
     }
-    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0);
+    flush_slide<CH, NW>(a, it, w, wwin, s_i0max, k0, active);
   }
   flush_tail<CH, NW>(a, it, w, wwin, s_i0max, k0);
 }
@@ -529,8 +556,8 @@ __device__ __forceinline__ void consume_item(const FwdArgs<double> &a, const Ite
 // about 77 % of the time (20 wavefronts per block: windows 8, records 4, X rows
 // 3.6, shuffles 3, flushes), issue 58 %, the FMA pipe 46 %; one block a chunk
 // lets 16 warps fit an SM instead of 12 but reads each record twice as often
-// (24 wavefronts): 3.58 ms.  On a GB300 the
-// sphere of 32768 panels x 2048 steps x 72 observers takes 3.43 ms; the
+// (24 wavefronts): 0.15 ms more.  On a GB300 the
+// sphere of 32768 panels x 2048 steps x 72 observers takes 3.49 ms; the
 // former kernel on samples and moments side by side (20 multiply-adds, 64-byte
 // rows, 22 instructions per 32 samples) took 4.57 ms.
 //
@@ -605,8 +632,11 @@ __device__ __forceinline__ float2 kahan_add(float2 w, float y) {
 }
 
 // A window entry: a plain FP32 sum, or a compensated pair (sum, compensation)
-// whose value is sum - compensation (formed in FP64).  add(): the four taps of
-// one bin (a compensated entry takes a panel's whole contribution at once).
+// whose value is sum - compensation (formed in FP64).  add() takes a panel's
+// whole contribution to the bin at once: the four taps are summed first, so the
+// running sum, much larger than one panel's share, is rounded once per panel
+// and not four times (error against 64 bits 7.2e-8 instead of 8.0e-8 at 8192
+// panels x 512 steps, for 0.13 of 3.5 ms).
 template <bool KAHAN> struct WinEntry;
 template <> struct WinEntry<false> {
   using E = float;
@@ -615,11 +645,7 @@ template <> struct WinEntry<false> {
   static __device__ __forceinline__ E zero() { return 0.f; }
   static __device__ __forceinline__ E load(unsigned addr) { return lds_win(addr); }
   static __device__ __forceinline__ void store(unsigned addr, E v) { sts_f32(addr, v); }
-  static __device__ __forceinline__ E add(E s, const float (&w)[4], const float *g) {
-#pragma unroll
-    for (int t = 0; t < 4; ++t) s = fmaf(w[t], g[t], s);
-    return s;
-  }
+  static __device__ __forceinline__ E add(E s, float y) { return s + y; }
 };
 template <> struct WinEntry<true> {
   using E = float2;
@@ -634,12 +660,7 @@ template <> struct WinEntry<true> {
   static __device__ __forceinline__ void store(unsigned addr, E v) {
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
   }
-  static __device__ __forceinline__ E add(E s, const float (&w)[4], const float *g) {
-    float y = w[0] * g[0];
-#pragma unroll
-    for (int t = 1; t < 4; ++t) y = fmaf(w[t], g[t], y);
-    return kahan_add(s, y);
-  }
+  static __device__ __forceinline__ E add(E s, float y) { return kahan_add(s, y); }
 };
 
 // Window slots per observer of the FP32 shapes, fixed per chunk length so that
@@ -671,12 +692,13 @@ __device__ __forceinline__ void flush_bins(const FwdArgs<float> &a, const Item<f
 template <int TK, int NW, bool KAHAN>
 __device__ __forceinline__ void flush_slide_split(const FwdArgs<float> &a,
                                                   const Item<float, NW> &it, int w, float *wwin,
-                                                  const int *s_i0max, int k0) {
+                                                  const int *s_i0max, int k0, unsigned active) {
   using W = WinEntry<KAHAN>;
   using E = typename W::E;
   constexpr int H = win_f32<TK>() / 4, CH = chunk_of<float, TK>();
   const int lane = threadIdx.x & 31;
-  for (int m = 0; m < it.nobs; ++m) {
+  for (; active; active &= active - 1) {
+    const int m = __ffs(active) - 1;
     E *wm = reinterpret_cast<E *>(wwin) + m * 4 * H;
     flush_bins<TK, KAHAN, NW>(a, it, w, m, wm, k0 - s_i0max[m], CH);
     __syncwarp();
@@ -720,12 +742,12 @@ __device__ __forceinline__ float f2_sum(f32x2 v) {
 //
 // The next observer's record is loaded piece by piece as this one's is used
 // up, always before this observer's stores: the compiler cannot move a shared
-// load above a store it cannot tell apart (3.43 ms; 3.50 with the record read
-// at the top of each observer).  Two observers at a time (168 registers): 4.1
-// ms; the last lane's stores predicated or sent to a spare slot instead of the
-// branch: 3.8 and 3.7 ms.
+// load above a store it cannot tell apart (3.43 ms so, 3.50 with the record
+// read at the top of each observer, before the taps were summed apart).  Two
+// observers at a time (168 registers): 4.1 ms; the last lane's stores predicated
+// or sent to a spare slot instead of the branch: 3.8 and 3.7 ms.
 template <int TK, int NA, int NW, bool KAHAN>
-__device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned crec,
+__device__ __forceinline__ void consume_step(unsigned active, unsigned stg, unsigned crec,
                                              unsigned win_s, unsigned xrow, int lanes) {
   constexpr unsigned RB = kRec * 4;           // record bytes
   constexpr unsigned BB = KAHAN ? 256 : 128;  // window bytes of 32 words of a quarter
@@ -776,7 +798,12 @@ __device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned cr
 #pragma unroll
     for (int b = 0; b < NA; ++b)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s[b][j] = W::add(s[b][j], k.w, &g[b][j]);
+      for (int j = 0; j < 4; ++j) {
+        float y = k.w[0] * g[b][j];
+#pragma unroll
+        for (int t = 1; t < 4; ++t) y = fmaf(k.w[t], g[b][j + t], y);
+        s[b][j] = W::add(s[b][j], y);
+      }
     k.load_w(next);
 #pragma unroll
     for (int b = 0; b < NA; ++b)
@@ -785,29 +812,32 @@ __device__ __forceinline__ void consume_step(int nobs, unsigned stg, unsigned cr
         for (int j = 0; j < 4; ++j) W::store(A[j] + BB * b, s[b][j]);
       }
   };
-  // A warp with the full count of observers runs them without an exit test,
-  // so the compiler may overlap one observer's tail with the next one's loads
-  // and arithmetic.
-  auto run = [&](auto full) {
-    constexpr bool kFull = decltype(full)::value;
-    const int n = kFull ? kMaxObsPerWarpF32 : nobs;
-    if (n == 0) return;
-    auto rec = [&](int m) { return crec + (unsigned)m * NW * RB; };
-    Coef k;
-    k.q = Coef::load_q(rec(0));
-    k.load_c(rec(0));
-    k.load_w(rec(0));
-#pragma unroll
-    for (int m = 0; m < kMaxObsPerWarpF32; ++m) {
-      if (!kFull && m >= n) break;
-      // (the last one loads its own record again)
-      observer(m, k, rec(m + 1 < n ? m + 1 : m));
-    }
+  auto rec = [&](int m) { return crec + (unsigned)m * NW * RB; };
+  Coef k;
+  auto load = [&](unsigned r) {
+    k.q = Coef::load_q(r);
+    k.load_c(r);
+    k.load_w(r);
   };
-  if (nobs == kMaxObsPerWarpF32)
-    run(std::true_type{});
-  else
-    run(std::false_type{});
+  // A warp with the full count of observers runs them unrolled, so the
+  // compiler may overlap one observer's tail with the next one's loads and
+  // arithmetic.  (The last one loads its own record again.)
+  if (active == (1u << kMaxObsPerWarpF32) - 1) {
+    load(rec(0));
+#pragma unroll
+    for (int m = 0; m < kMaxObsPerWarpF32; ++m)
+      observer(m, k, rec(m + 1 < kMaxObsPerWarpF32 ? m + 1 : m));
+  } else {
+    int m = __ffs(active) - 1;
+    load(rec(m));
+    for (;;) {
+      active &= active - 1;
+      const int next = active ? __ffs(active) - 1 : m;
+      observer(m, k, rec(next));
+      if (!active) break;
+      m = next;
+    }
+  }
 }
 
 template <int TK, int NW, bool KAHAN>
@@ -832,14 +862,17 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
     // lanes of the last block whose bins belong to this chunk (a segment that
     // ends inside the record ends at a multiple of four intervals)
     const int lanes = min(31, (it.k_end - k0 - (one ? 0 : 128 * (NB - 1)) + 3) >> 2);
+    const unsigned active = active_observers<float, NW>(a, it, w, s_i0max, k0, k0 + CH - 1);
     for (int p = it.p_begin; p < it.p_end; ++p, ++step) {
       if (!mbar_wait(&ps.full[s], ph, ps.err, ps.abort, ps.wait_cycles)) return;
       const unsigned stg = stage_token(stage0 + s * ps.stage_bytes);
       const unsigned crec = stg + ps.x_bytes + (unsigned)w * (kRec * 4);
-      if (one)
-        consume_step<TK, 1, NW, KAHAN>(it.nobs, stg, crec, win_s, xrow, lanes);
-      else
-        consume_step<TK, NB, NW, KAHAN>(it.nobs, stg, crec, win_s, xrow, lanes);
+      if (active) {
+        if (one)
+          consume_step<TK, 1, NW, KAHAN>(active, stg, crec, win_s, xrow, lanes);
+        else
+          consume_step<TK, NB, NW, KAHAN>(active, stg, crec, win_s, xrow, lanes);
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&ps.empty[s]);
       if (++s == (unsigned)ps.nst) {
@@ -847,7 +880,7 @@ __device__ __forceinline__ void consume_item_f32(const FwdArgs<float> &a,
         ph ^= 1u;
       }
     }
-    flush_slide_split<TK, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
+    flush_slide_split<TK, NW, KAHAN>(a, it, w, wwin, s_i0max, k0, active);
   }
   flush_tail_split<TK, NW, KAHAN>(a, it, w, wwin, s_i0max, k0);
 }

@@ -154,6 +154,7 @@ struct FwdArgs {
   int seg_shift;        // segment q ends at interval (q + 1) seg_len - seg_shift (a multiple of 4)
   int seg_lo, seg_cnt;  // this launch covers time segments [seg_lo, seg_lo + seg_cnt)
   int win;              // window slots per observer
+  int slack;            // largest spread of shifts within a panel set
   int wfl;              // values per observer window: win, or 2 win for compensated
                         // FP32 windows (a sum and its compensation per slot)
   long long wait_cycles; // bound of each pipeline wait in SM clocks (the handle's limit)
