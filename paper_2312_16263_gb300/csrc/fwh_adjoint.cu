@@ -9,8 +9,10 @@
 // so each (panel, sample) output is owned by one lane and summed over the
 // observers in registers, 12 multiply-adds per (panel, sample, observer).
 // The ghost rows beta_{-1} = 2 beta_0 - beta_1 and beta_nt = 2 beta_{nt-1} -
-// beta_{nt-2} hand their gradients to the two samples next to them: q of those
-// samples takes the ghost's q times 2 and -1 (edge chunks only).  Two forms:
+// beta_{nt-2} hand their gradients to the two samples next to them, times 2
+// and -1: a warp whose chunk holds one of those sums the ghost's gradient with
+// its lanes over the observers, beside the main loop.  An observer whose valid
+// bins the chunk cannot reach is left out (its g there is zero).  Two forms:
 // k_adjoint_set (FP32) gathers per panel set from a window of g staged in
 // shared memory, with atomics only to add the partial sums of several
 // 36-observer groups; k_adjoint (FP64) is one CTA per panel reading g from
@@ -39,15 +41,33 @@ template <typename T>
 __device__ __forceinline__ T gather_q(const T *w, T gm2, T gm1, T g0, T g1) {
   return fma(w[0], g1, fma(w[1], g0, fma(w[2], gm1, w[3] * gm2)));
 }
-// The ghost rows' share of sample s (see above).
+// Sums v[8] over the warp; every lane gets all eight.
 template <typename T>
-__device__ __forceinline__ T ghost_q(int s, int nt, const T *w, T gm2, T gm1, T g0, T g1) {
-  T v = T(0);
-  if (s == 0) v += T(2) * (w[0] * g0);
-  if (s == 1) v -= w[0] * gm1;
-  if (s == nt - 1) v += T(2) * (w[3] * gm1 + w[2] * g0);
-  if (s == nt - 2) v -= w[3] * g0 + w[2] * g1;
-  return v;
+__device__ __forceinline__ void warp_sum8(T (&v)[kSer]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = kSer / 2, m = 16; n >= 1; n >>= 1, m >>= 1)
+#pragma unroll
+    for (int i = 0; i < n; ++i) {  // hand one half of the components to lane ^ m
+      const T send = lane & m ? v[i] : v[i + n];
+      v[i] = (lane & m ? v[i + n] : v[i]) + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+  T r = v[0];  // component lane >> 2
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+#pragma unroll
+  for (int s = 0; s < kSer; ++s) v[s] = __shfl_sync(0xffffffffu, r, 4 * s);
+}
+// Ghost rows next to the samples of [k0, k0 + ch): bit 0 the one before the
+// record, bit 1 the one after it.
+__device__ __forceinline__ int ghosts(int k0, int ch, int nt) {
+  return (k0 < 2 ? 1 : 0) | (k0 < nt && k0 + ch >= nt - 1 ? 2 : 0);
+}
+// The share of ghost row `end` (0 or 1) that sample s takes.
+template <typename T>
+__device__ __forceinline__ T ghost_share(int end, int s, int nt) {
+  const int d = end ? nt - 1 - s : s;
+  return d == 0 ? T(2) : d == 1 ? T(-1) : T(0);
 }
 
 // FP64: one CTA per (panel, group of 8 chunks of 64 samples), one warp per
@@ -67,7 +87,6 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs<double> a) {
   const int ch = (blockIdx.x % ngrp) * 8 + w;
   const bool live = ch < nch;  // warps past the last chunk only help staging
   const int k0 = ch * CH;
-  const bool edge = k0 == 0 || k0 + CH >= a.nt - 1;
   double acc[TK][kSer];
 #pragma unroll
   for (int j = 0; j < TK; ++j)
@@ -92,31 +111,64 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs<double> a) {
           g[j][t] = jb >= 0 && jb < a.g_ld ? __ldg(G + jb) : 0.0;
         }
     };
-    double g[TK][4];
-    bins(0, g);
-    for (int o = 0; o < no; ++o) {
-      double gn[TK][4];
-      if (o + 1 < no) bins(o + 1, gn);
-      double c[12];
-#pragma unroll
-      for (int s = 0; s < 12; ++s) c[s] = srec[o * kRec + s];
-#pragma unroll
-      for (int j = 0; j < TK; ++j) {
-        double q = gather_q(c + slot::w, g[j][0], g[j][1], g[j][2], g[j][3]);
-        if (edge)
-          q += ghost_q(k0 + lane + 32 * j, a.nt, c + slot::w, g[j][0], g[j][1], g[j][2], g[j][3]);
-#pragma unroll
-        for (int s = 0; s < kSer; ++s) acc[j][s] = fma(c[s], q, acc[j][s]);
+    for (int of = 0; of < no; of += 32) {
+      // observers of the 32 from `of` on with a valid bin in reach
+      bool on = false;
+      if (of + lane < no) {
+        const int i0 = (int)srec[(of + lane) * kRec + slot::i0];
+        on = k0 - 2 - i0 < a.n_valid[ob + of + lane] && k0 + CH - i0 >= 0;
       }
-      if (o + 1 < no) {
+      unsigned left = __ballot_sync(0xffffffffu, on);
+      if (!left) continue;
+      double g[TK][4];
+      bins(of + __ffs(left) - 1, g);
+      while (left) {
+        const int o = of + __ffs(left) - 1;
+        left &= left - 1;
+        double gn[TK][4];
+        if (left) bins(of + __ffs(left) - 1, gn);
+        double c[12];
 #pragma unroll
-        for (int j = 0; j < TK; ++j)
+        for (int s = 0; s < 12; ++s) c[s] = srec[o * kRec + s];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) g[j][t] = gn[j][t];
+        for (int j = 0; j < TK; ++j) {
+          const double q = gather_q(c + slot::w, g[j][0], g[j][1], g[j][2], g[j][3]);
+#pragma unroll
+          for (int s = 0; s < kSer; ++s) acc[j][s] = fma(c[s], q, acc[j][s]);
+        }
+        if (left) {
+#pragma unroll
+          for (int j = 0; j < TK; ++j)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) g[j][t] = gn[j][t];
+        }
       }
     }
   }
   if (!live) return;
+  const int gh = ghosts(k0, CH, a.nt);
+  for (int e = 0; e < 2; ++e)
+    if (gh >> e & 1) {
+      double v[kSer] = {};
+      for (int o = lane; o < a.O; o += 32) {
+        const double *r = rec0 + (size_t)o * kRec, *w4 = r + slot::w;
+        const double *G = a.Gt + (size_t)o * a.g_ld;
+        auto bin = [&](int k) {  // g of interval k
+          const int j = k - (int)r[slot::i0];
+          return j >= 0 && j < a.g_ld ? __ldg(G + j) : 0.0;
+        };
+        const double q = e ? fma(w4[2], bin(a.nt - 1), w4[3] * bin(a.nt - 2)) : w4[0] * bin(0);
+#pragma unroll
+        for (int s = 0; s < kSer; ++s) v[s] = fma(r[s], q, v[s]);
+      }
+      warp_sum8(v);
+#pragma unroll
+      for (int j = 0; j < TK; ++j) {
+        const double f = ghost_share<double>(e, k0 + lane + 32 * j, a.nt);
+#pragma unroll
+        for (int s = 0; s < kSer; ++s) acc[j][s] = fma(f, v[s], acc[j][s]);
+      }
+    }
   double *out = a.Xbar + ((size_t)p * a.xb_ld + k0 + lane) * kSer;
 #pragma unroll
   for (int j = 0; j < TK; ++j)
@@ -144,11 +196,11 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs<double> a) {
 // their partial sums with vector atomics into a zeroed Xbar.
 // Bound by instruction issue and shared-memory bandwidth together (issue 61 %,
 // shared-memory wavefronts 55 %, DRAM 11 %).  Eight warps a CTA so that 16 fit an
-// SM beside the windows (four: 12; the whole backward of 16384 panels x 1024 steps x
-// 36 observers takes 0.95 ms with eight, 0.97 with four; 0.99 on samples and
-// moments side by side, 20 multiply-adds and 64-byte rows).  Runs of six: the
-// gradient's error against 64 bits is 2.2e-6 there (2.4e-6 before; 3.2e-6
-// with one running sum).
+// SM beside the windows (four: 12, 2 % slower).  16384 panels x 1024 steps x 36
+// observers: 0.50 ms; 0.58 with the ghosts' share computed for every sample of an
+// edge chunk and every observer taken in every chunk (FP64, 5151 x 701 x 19:
+// 1.78 -> 1.49 ms).  Runs of six: the gradient's error against 64 bits is 2.2e-6
+// there (3.2e-6 with one running sum).
 constexpr int kAdjGroup = 36;    // observers per item
 constexpr int kAdjRun = 6;       // observers summed from zero at a time
 constexpr int kAdjWarps = 8;
@@ -182,6 +234,7 @@ template <bool kAtomic>
 __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a) {
   constexpr int CH = 32 * kAdjTK;
   extern __shared__ __align__(16) float gw[];  // [kAdjGroup][win], then the record buffers
+  __shared__ int s_obs[kAdjGroup];             // the group's observers with a bin in reach
   const int win = a.win, H = win >> 2;
   const int lane = threadIdx.x & 31;
   const int w = threadIdx.x >> 5;
@@ -193,15 +246,28 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
   const int ch = rest % nch;
   const int sidx = a.set_order[rest / nch];
   const int k0 = ch * CH;
-  const bool edge = k0 == 0 || k0 + CH >= a.nt - 1;
+  const int gh = ghosts(k0, CH, a.nt);
   const int o0 = g * kAdjGroup;
-  const int no = min(kAdjGroup, a.O - o0);
+  const int *i0max = a.i0max_tab + (size_t)sidx * a.O + o0;
+  int no = 0;  // observers with a valid bin in reach of the set's samples here
+  for (int of = 0; of < min(kAdjGroup, a.O - o0); of += 32) {
+    const int o = of + lane;
+    bool on = false;
+    if (o < min(kAdjGroup, a.O - o0)) {
+      const int i0 = i0max[o];
+      on = k0 - 2 - i0 < a.n_valid[o0 + o] && k0 + CH - i0 + a.slack >= 0;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (on && w == 0) s_obs[no + __popc(m & ((1u << lane) - 1))] = o;
+    no += __popc(m);
+  }
+  __syncthreads();
   const int p_begin = a.set_begin[sidx], p_end = a.set_begin[sidx + 1];
   // stage the window of each observer of the group (cp.async: every copy in
   // flight at once; zero outside the record)
   for (int o = 0; o < no; ++o) {
-    const int base = k0 - 2 - a.i0max_tab[(size_t)sidx * a.O + o0 + o];
-    const float *G = a.Gt + (size_t)(o0 + o) * a.g_ld;
+    const int base = k0 - 2 - i0max[s_obs[o]];
+    const float *G = a.Gt + (size_t)(o0 + s_obs[o]) * a.g_ld;
     for (int t = threadIdx.x; t < win; t += blockDim.x) {
       const int j = base + t;
       const bool ok = j >= 0 && j < a.g_ld;
@@ -214,7 +280,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
   auto stage = [&](int p, int buf) {  // the group's records of panel p, 16 bytes a copy
     const float *src = a.coef + ((size_t)p * a.O + o0) * kRec;
     float *dst = rb + (size_t)buf * kAdjGroup * kRec;
-    for (int c = lane; c < no * (kRec / 4); c += 32) cp_async16(dst + 4 * c, src + 4 * c);
+    for (int c = lane; c < no * (kRec / 4); c += 32)
+      cp_async16(dst + 4 * c, src + s_obs[c / (kRec / 4)] * kRec + 4 * (c % (kRec / 4)));
     cp_async_commit();
   };
   const int shift = a.slot_shift;  // the records' offsets are in slots of 2^shift bytes
@@ -263,10 +330,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
         for (int i = 0; i < 7; ++i) gv[i] = A[i & 3][i >> 2];
 #pragma unroll
         for (int j = 0; j < kAdjTK; ++j) {
-          float q = gather_q(wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
-          if (edge)
-            q += ghost_q(k0 + 4 * lane + j, a.nt, wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]);
-          const f32x2 q2 = f2_dup(q);
+          const f32x2 q2 = f2_dup(gather_q(wt, gv[j], gv[j + 1], gv[j + 2], gv[j + 3]));
 #pragma unroll
           for (int s = 0; s < kSer / 2; ++s) acc[j][s] = f2_fma(c[s], q2, acc[j][s]);
         }
@@ -276,6 +340,33 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adjoint_set(AdjArgs<float> a
 #pragma unroll
         for (int s = 0; s < kSer / 2; ++s) sum[j][s] = f2_add(sum[j][s], acc[j][s]);
     }
+    for (int e = 0; e < 2; ++e)
+      if (gh >> e & 1) {
+        float v[kSer] = {};
+        for (int o = lane; o < no; o += 32) {
+          const float *r = rec + o * kRec;
+          const unsigned *qo = reinterpret_cast<const unsigned *>(r + slot::q0);
+          auto bin = [&](int k) {  // g of interval k
+            const int y = k - k0 + 2;
+            return gw[o * win + (qo[y & 3] >> shift) + (y >> 2)];
+          };
+          const float *w4 = r + slot::w;
+          const float q =
+              e ? fmaf(w4[2], bin(a.nt - 1), w4[3] * bin(a.nt - 2)) : w4[0] * bin(0);
+#pragma unroll
+          for (int s = 0; s < kSer; ++s) v[s] = fmaf(r[s], q, v[s]);
+        }
+        warp_sum8(v);
+        f32x2 v2[kSer / 2];
+#pragma unroll
+        for (int s = 0; s < kSer / 2; ++s) v2[s] = f2_pack(v[2 * s], v[2 * s + 1]);
+#pragma unroll
+        for (int j = 0; j < kAdjTK; ++j) {
+          const f32x2 f = f2_dup(ghost_share<float>(e, k0 + 4 * lane + j, a.nt));
+#pragma unroll
+          for (int s = 0; s < kSer / 2; ++s) sum[j][s] = f2_fma(f, v2[s], sum[j][s]);
+        }
+      }
     float *out = a.Xbar + ((size_t)p * a.xb_ld + k0 + 4 * lane) * kSer;
 #pragma unroll
     for (int j = 0; j < kAdjTK; ++j) {

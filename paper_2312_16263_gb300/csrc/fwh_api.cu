@@ -604,6 +604,7 @@ fwh_status run_backward(fwh_handle h, const T *fields, const double *grad_p, T *
     aa.nsets = (int)h->set_begin.size() - 1;
     aa.win = c.win;
     aa.slot_shift = c.acc == 5 ? 3 : 2;
+    aa.slack = fwd_slack(false, c);
   }
   CK(h, launch_adjoint<T>(aa, s));
   PrepAdjArgs<T> pa{};

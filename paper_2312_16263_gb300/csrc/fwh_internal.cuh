@@ -77,6 +77,11 @@ __device__ __forceinline__ f32x2 f2_dup(float x) {
   asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
 __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
   f32x2 d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -178,6 +183,7 @@ struct AdjArgs {
   const int *i0max_tab; // [nsets][O] largest shift of each (panel set, observer)
   int nsets, win;       // win: window slots per observer
   int slot_shift;       // log2 of the plan's bytes per window slot (2, or 3 if compensated)
+  int slack;            // largest spread of shifts within a panel set
 };
 
 template <typename T>
