@@ -333,12 +333,16 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
 // column of the window holds y (the causal recursion, carried on from block to
 // block, in place of the integrand), so per sample the integrands are formed
 // once, the causal step runs once and the anti-causal one 1.5 times (64 + 34
-// rows per 64): about 36 FP64 operations per (panel, sample).  The record ends
-// are handled in place.  32768 panels x 2048 steps: 6.8 ms (15.2 ms by
-// windowed elimination, 142 operations and 128-byte rows; 8.7 with a kernel of
-// its own for the record ends).
+// rows per 64): about 32 FP64 operations per (panel, sample).  The record ends
+// are handled in place.  Field rows arrive 32 at a time, half of a block's ahead
+// of the block, so that three CTAs fit an SM and hide each other's chains.
+// 32768 panels x 2048 steps: 5.3 ms (6.8 with 64 rows in flight, two CTAs and
+// the filter's gain applied per sample; 8.7 with a kernel of its own for the
+// record ends; 15.2 by windowed elimination, 142 operations and 128-byte rows).
 // ---------------------------------------------------------------------------
 constexpr int kF64H = Prec<double>::halo;
+constexpr int kF64Raw = 32;  // field rows in flight
+static_assert(kF64H <= kF64Raw, "the rows a unit starts on are issued at once");
 constexpr int kF64Rows = kIirChunk + kF64H + 2;  // samples c0 - 1 .. c0 + 64 + H
 constexpr int kF64Keep = kF64Rows - kIirChunk;
 
@@ -372,13 +376,16 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   constexpr int NP = kIntPanels, C = kIirChunk, H = kF64H, R = kF64Rows;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *win = reinterpret_cast<double *>(smem_raw);  // [R][NP][4]
-  double *raw = win + R * kIntRow;                     // [C][5][NP]
+  double *raw = win + R * kIntRow;                     // [kF64Raw][5][NP]
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
   const int n_us = (a.c_hi - a.c_lo + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   const int pa = tid % NP;               // integrand phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
+  // Normals scaled by -6 rho scale all four integrands by it, so the filter's
+  // output is the coefficient itself: F below is -6 rho times the integrand.
+  constexpr double kScale = -6.0 * kRho, kUnscale = 1.0 / kScale;
   const double inv2h = 0.5 / a.dt;
   const bool vec = (a.P & 1) == 0 && ((size_t)a.fields & 15) == 0;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
@@ -389,9 +396,9 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
     double n0 = 0, n1 = 0, n2 = 0, Un = 0;
     if (p < a.P) {
       const double *n = a.n + 3 * (size_t)(a.place ? a.place[p] : p);
-      n0 = n[0];
-      n1 = n[1];
-      n2 = n[2];
+      n0 = kScale * n[0];
+      n1 = kScale * n[1];
+      n2 = kScale * n[2];
       Un = a.ca * n0 + a.sa * n1;
     }
     const bool live_b = pb < a.P;
@@ -412,12 +419,20 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         *reinterpret_cast<double2 *>(w + 2) = make_double2(pp * n1 + u1 * t, pp * n2 + u2 * t);
       }
     };
-    auto fill = [&](int sample, int w0, int n) {
+    auto issue = [&](int sample, int n) {
       issue_rows_f64<NP>(a.fields, a.P, a.nt, p0, sample, n, raw, vec);
-      cp_async_wait_all();
-      __syncthreads();
-      integrands(w0, n);
-      __syncthreads();
+    };
+    // integrands of n samples from `sample` on into window rows from w0 on; the
+    // first min(n, kF64Raw) are in flight already
+    auto fill = [&](int sample, int w0, int n) {
+      for (int r = 0; r < n; r += kF64Raw) {
+        const int m = min(kF64Raw, n - r);
+        if (r > 0) issue(sample + r, m);
+        cp_async_wait_all();
+        __syncthreads();
+        integrands(w0 + r, m);
+        __syncthreads();
+      }
     };
     const int lo = b0 * C - 2;  // sample c0 - 1 of the first block
     const int N = a.nt;
@@ -448,6 +463,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
     double F0 = 0.0, D0 = 0.0;  // integrand and one-sided derivative at sample 0
     __syncthreads();  // the previous unit is done with raw and win
     if (b0 > 0) {
+      issue(lo - H, H);
       fill(lo - H, 0, H);  // the samples the causal recursion starts on
       for (int r = 0; r < H; ++r) {
         f3 = f2;
@@ -457,13 +473,13 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
       }
       __syncthreads();
     }
-    fill(lo, 0, C);
-    fill(lo + C, C, R - C);
+    issue(lo, kF64Raw);
+    fill(lo, 0, R);
     if (b0 > 0) {
       causal(0, lo);
     } else {  // rows 0 and 1 lie before the record; y_0 from the reflected series
       F0 = col[2 * kIntRow];
-      D0 = (-3.0 * F0 + 4.0 * col[3 * kIntRow] - col[4 * kIntRow]) * inv2h;
+      D0 = (-3.0 * F0 + 4.0 * col[3 * kIntRow] - col[4 * kIntRow]) * (kUnscale * inv2h);
       for (int j = H; j >= 1; --j) yy = kRho * (col[(2 + j) * kIntRow] + yy);
       yy = F0 * ((1.0 + kRho) / (1.0 - kRho)) - yy;
       f1 = F0;
@@ -472,7 +488,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
     }
     for (int b = b0; b < b1; ++b) {
       const bool more = b + 1 < b1;
-      if (more) issue_rows_f64<NP>(a.fields, a.P, a.nt, p0, b * C - 2 + R, C, raw, vec);
+      if (more) issue(b * C - 2 + R, kF64Raw);
       double *const xr = xp + (size_t)(b * C - a.row0) * kSer;
       const int s0 = b * C - 2;  // sample of window row 0
       double xx = 0.0, c1 = 0.0, c2 = 0.0;  // coefficients one and two samples on
@@ -483,16 +499,15 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         for (int r = C + 1; r >= C; --r) {
           xx = fma(kRho, xx, col[r * kIntRow]);
           c2 = c1;
-          c1 = (-6.0 * kRho) * xx;
+          c1 = xx;
         }
 #pragma unroll 16
         for (int r = C - 1; r >= 0; --r) {  // window row r: sample c0 - 1 + r
           xx = fma(kRho, xx, col[r * kIntRow]);
-          const double c0v = (-6.0 * kRho) * xx;
           if (live_b)
-            *reinterpret_cast<double2 *>(xr + r * kSer) = make_double2((c2 - c0v) * inv2h, c1);
+            *reinterpret_cast<double2 *>(xr + r * kSer) = make_double2((c2 - xx) * inv2h, c1);
           c2 = c1;
-          c1 = c0v;
+          c1 = xx;
         }
       } else {
         // a record end: row r of X holds sample s0 + 1 + r
@@ -500,25 +515,25 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         if (b == 0) {
           double x1 = 0.0;
           for (int r = H + 3; r >= 3; --r) x1 = fma(kRho, x1, col[r * kIntRow]);
-          pw = D0 - ((-6.0 * kRho) * x1 - F0) * (2.0 * inv2h);
+          pw = D0 - (x1 - kUnscale * F0) * (2.0 * inv2h);
           for (int i = 0; i < H + 4; ++i) pw *= kRho;  // below rounding from sample H + 4 on
         }
         const double ir = 1.0 / kRho;
-        const double DN = (3.0 * f1 - 4.0 * f2 + f3) * inv2h;  // (used where f1 is sample N - 1)
+        // (used where f1 is sample N - 1)
+        const double DN = (3.0 * f1 - 4.0 * f2 + f3) * (kUnscale * inv2h), FN = kUnscale * f1;
         double cr = 0.0, d2 = 0.0;
         for (int r = R - 1; r >= 0; --r) {
           const int sr = s0 + r;
           if (sr > N - 1) continue;
-          xx = sr == N - 1 ? f1 * (-1.0 / (6.0 * kRho)) : fma(kRho, xx, col[r * kIntRow]);
-          const double c0v = sr == N - 1 ? f1 : (-6.0 * kRho) * xx;
+          xx = sr == N - 1 ? FN : fma(kRho, xx, col[r * kIntRow]);
           if (sr == N - 2)
-            cr = DN - (c1 - c0v) * (2.0 * inv2h);
+            cr = DN - (c1 - xx) * (2.0 * inv2h);
           else if (sr > N - 3 - (H + 4))  // below rounding further on
             cr *= kRho;
           else
             cr = 0.0;
           const int se = sr + 1;  // the sample now complete, in X row r
-          double d = (c2 - c0v) * inv2h;
+          double d = (c2 - xx) * inv2h;
           if (cr != 0.0) d += cr;
           if (b == 0 && se < H + 4) {
             pw *= ir;
@@ -533,25 +548,22 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
             }
             if (se == N - 2) {  // the last sample, the ghost after it and a zero row
               const int room = a.row0 + a.x_ld - b * C - r;  // rows of X from this one on
-              if (room > 1) *reinterpret_cast<double2 *>(row + kSer) = make_double2(DN, f1);
+              if (room > 1) *reinterpret_cast<double2 *>(row + kSer) = make_double2(DN, FN);
               if (room > 2)
                 *reinterpret_cast<double2 *>(row + 2 * kSer) =
-                    make_double2(2.0 * DN - d, 2.0 * f1 - c1);
+                    make_double2(2.0 * DN - d, 2.0 * FN - c1);
               if (room > 3) *reinterpret_cast<double2 *>(row + 3 * kSer) = make_double2(0.0, 0.0);
             }
           }
           d2 = d;
           c2 = c1;
-          c1 = c0v;
+          c1 = xx;
         }
       }
       if (!more) break;
       // slide the thread's column by C rows, then add the rows now in raw
       for (int r = 0; r < kF64Keep; ++r) col[r * kIntRow] = col[(r + C) * kIntRow];
-      cp_async_wait_all();
-      __syncthreads();
-      integrands(kF64Keep, C);
-      __syncthreads();
+      fill(s0 + R, kF64Keep, C);
       causal(kF64Keep, s0 + C);
     }
   }
@@ -1055,8 +1067,8 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 5 : 2)
 // x 2048 steps; 0.71 with the units that fill the GPU twice).  A small problem
 // gets one block a unit, so that its blocks run side by side.
 template <auto kern>
-cudaError_t persistent_grid(size_t smem, double start, long n_pg, int blocks, int *unit,
-                            long *grid) {
+cudaError_t persistent_grid(size_t smem, double start, long n_pg, int blocks,
+                            int *unit, long *grid) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // CTAs that fit the device, looked up once per kernel and device
@@ -1112,12 +1124,15 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
     int unit = 1;
     if constexpr (sizeof(T) == 4) {
       const size_t smem = ((size_t)kIntRows * kIntRow + (size_t)kIntRaw) * sizeof(T);
-      if ((e = persistent_grid<k_prep_iir_int>(smem, 0.6, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+      if ((e = persistent_grid<k_prep_iir_int>(smem, 0.6, n_pg, n_blk, &unit, &grid)) !=
+          cudaSuccess)
         return e;
       k_prep_iir_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     } else {
-      const size_t smem = ((size_t)kF64Rows * kIntRow + (size_t)C * 5 * kIntPanels) * sizeof(T);
-      if ((e = persistent_grid<k_prep_f64_int>(smem, 1.0, n_pg, n_blk, &unit, &grid)) != cudaSuccess)
+      const size_t smem =
+          ((size_t)kF64Rows * kIntRow + (size_t)kF64Raw * 5 * kIntPanels) * sizeof(T);
+      if ((e = persistent_grid<k_prep_f64_int>(smem, 1.0, n_pg, n_blk, &unit, &grid)) !=
+          cudaSuccess)
         return e;
       k_prep_f64_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     }
@@ -1149,8 +1164,8 @@ cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s) {
     const size_t smem = ((size_t)(C + H) * kIntRow + (size_t)C * 4 * kIntPanels) * sizeof(T);
     long grid = 0;
     int unit = 1;
-    if ((e = persistent_grid<k_prep_adj_int<T>>(smem, 0.5, n_pg, int_hi - int_lo, &unit, &grid)) !=
-        cudaSuccess)
+    if ((e = persistent_grid<k_prep_adj_int<T>>(smem, 0.5, n_pg, int_hi - int_lo, &unit,
+                                                &grid)) != cudaSuccess)
       return e;
     k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, int_lo, int_hi, unit);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
