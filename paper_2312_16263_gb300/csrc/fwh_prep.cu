@@ -718,15 +718,26 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_ii
 // value and derivative series' rows of Xbar), and the four integrand gradients
 // of a (panel, sample) map to the five field gradients.
 //
-// Interior blocks: S and D commute, so one filter per integrand on
-// Xbar_v + D^T Xbar_d, in the form -6 rho (1 - rho z)^-1 (1 - rho z^-1)^-1.  A
-// thread owns one (panel, integrand) and walks the blocks of a work unit: its
+// S and D commute away from the ends, so one filter per integrand on
+//   w = Xbar_v + D^T Xbar_d,
+// in the form -6 rho (1 - rho z)^-1 (1 - rho z^-1)^-1.  The ends transpose the
+// forward's: with a0 = sum rho^k Xbar_d,k (the sum that D_0 - d_0 multiplies
+// there), the two samples of d_0 see Xbar_d,0 - a0 instead of Xbar_d,0, a0 goes
+// through D_0's one-sided weights straight into the gradient, the recursions
+// run on the odd extension of w (zero at the end samples), and the end sample's
+// own gradient is w minus the moment next to it; likewise aN.
+//
+// A thread owns one (panel, integrand) and walks the blocks of a work unit: its
 // column of the window holds the causal recursion's y (carried on from block
 // to block), then the integrand gradients, in place; the Jacobian phase takes
 // (sample, panel) pairs, so field reads and gradient writes are coalesced.
 // Each thread's Xbar rows of the next 16 samples are in flight while it works on
-// these, and the block's fields are copied to shared memory behind the
-// anti-causal pass.
+// these, and half of the block's fields are copied to shared memory behind the
+// anti-causal pass, the other half behind the first half's gradients (six CTAs
+// an SM instead of five, three instead of two in FP64).  Bound by HBM and the
+// latency of the chains together.  16384 panels x 1024 steps: 0.25 ms (0.36 with
+// the record ends in a kernel of their own that filtered all eight series, and
+// all the fields at once); FP64, 5151 x 701: 0.41 ms (0.68).
 // ---------------------------------------------------------------------------
 template <typename T> struct Pair;
 template <> struct Pair<float> { using V = float2; };
@@ -749,29 +760,33 @@ __device__ __forceinline__ void put_grad(T *g, size_t P, const T *f, T qb, T lb0
   g[4 * P] = lb0 * n0 + lb1 * n1 + lb2 * n2;   // d/dp' (dL_c/dp' = n_c)
 }
 
+constexpr int kAdjFieldRows = 32;  // field rows of a block staged at a time
+
 template <typename T>
 __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
-    k_prep_adj_int(PrepAdjArgs<T> a, int int_lo, int int_hi, int unit) {
+    k_prep_adj_int(PrepAdjArgs<T> a, int n_blk, int unit) {
   constexpr int NP = kIntPanels, C = kIirChunk, H = Prec<T>::halo, R = C + H;
   constexpr int BT = 16;  // rows in flight per thread
-  static_assert(C % BT == 0 && H % BT == 0, "row batches");
+  constexpr int FR = kAdjFieldRows;
+  static_assert(C % BT == 0 && H % BT == 0 && C % FR == 0, "row batches");
   using V = typename Pair<T>::V;
   constexpr T rho = (T)kRho, six = (T)(-6.0 * kRho);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *win = reinterpret_cast<T *>(smem_raw);  // [R][NP][4]: samples c0 .. c0 + R - 1
-  T *fld = win + R * kIntRow;                // [C][4][NP]: rho', u' of the block
+  T *fld = win + R * kIntRow;                // [FR][4][NP]: rho', u' of the block
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
-  const int n_us = (int_hi - int_lo + unit - 1) / unit;
+  const int n_us = (n_blk + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
+  const int N = a.nt;
   const int pa = tid % NP;               // Jacobian phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
   const T inv2h = (T)(0.5 / a.dt);
   const size_t P = a.P;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     const int p0 = (int)(u % n_pg) * NP;
-    const int b0 = int_lo + (int)(u / n_pg) * unit;
-    const int b1 = min(int_hi, b0 + unit);
+    const int b0 = (int)(u / n_pg) * unit;
+    const int b1 = min(n_blk, b0 + unit);
     const int p = p0 + pa, pb = min(p0 + pl, a.P - 1);
     const bool live = p < a.P;
     T n0 = 0, n1 = 0, n2 = 0, Un = 0;
@@ -787,10 +802,42 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
     auto X = [&](int k) -> V { return __ldg(reinterpret_cast<const V *>(xb + (size_t)k * kSer)); };
     T *const col = win + pl * 4 + qi;
     T yy = T(0);
-    int k = b0 * C - H;  // next sample of the causal recursion
-    const int k_last = (b1 - 1) * C + R;  // last sample it reads
-    V cur = X(k);
-    T dm = X(k - 1).x;   // derivative gradient one sample back
+    int k;               // next sample of the causal recursion
+    const int k_last = min((b1 - 1) * C + R, N - 1);  // last sample it reads
+    V cur;
+    T dm;                // derivative gradient one sample back
+    T a0 = T(0), w0 = T(0);             // the start's sum, w of sample 0
+    T aN = T(0), wN = T(0), yN = T(0);  // the end's sum, w of the last sample, y before it
+    if (b0 > 0) {
+      k = b0 * C - H;
+      cur = X(k);
+      dm = X(k - 1).x;
+    } else {  // exact start: y of sample 0 on the odd extension of w
+      k = 0;
+      T e = T(0);
+      V x1 = V{}, x2 = V{};
+#pragma unroll
+      for (int j = H + 1; j >= 0; --j) {
+        const V x = X(j);
+        a0 = fma(rho, a0, x.x);
+        if (j >= 1 && j < H) e = rho * (e + fma(x.x - x2.x, inv2h, x1.y));
+        if (j > 0) {
+          x2 = x1;
+          x1 = x;
+        } else {
+          const T d0 = T(2) * (x.x - a0);  // what sample 1 sees as the one before it
+          e = rho * (e + fma(d0 - x2.x, inv2h, x1.y));
+          w0 = fma(-inv2h, x1.x + d0, x.y);
+          cur.x = d0;
+          cur.y = -e;
+          dm = x1.x;  // no difference: the first step gives y_0 = -e itself
+        }
+      }
+    }
+    if (k_last == N - 1) {
+#pragma unroll
+      for (int j = H + 2; j >= 0; --j) aN = fma(rho, aN, X(N - 1 - j).x);
+    }
     V nx[BT];            // the next batch, in flight
     auto fetch = [&]() {
 #pragma unroll
@@ -801,23 +848,41 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
       V x[BT];
 #pragma unroll
       for (int i = 0; i < BT; ++i) x[i] = nx[i];
+      const int k0 = k;
       k += BT;
       fetch();
+      if (k0 + BT < N - 1) {
 #pragma unroll
-      for (int i = 0; i < BT; ++i) {
-        yy = fma(rho, yy, fma(dm - x[i].x, inv2h, cur.y));
-        if (w >= 0) col[(w + i) * kIntRow] = yy;
-        dm = cur.x;
-        cur = x[i];
+        for (int i = 0; i < BT; ++i) {
+          yy = fma(rho, yy, fma(dm - x[i].x, inv2h, cur.y));
+          if (w >= 0) col[(w + i) * kIntRow] = yy;
+          dm = cur.x;
+          cur = x[i];
+        }
+      } else {  // x of sample N - 1 is zero: so is y from there on
+#pragma unroll
+        for (int i = 0; i < BT; ++i) {
+          const bool last = k0 + i == N - 2;
+          const T xn = last ? T(2) * (x[i].x - aN) : x[i].x;
+          yy = k0 + i <= N - 2 ? fma(rho, yy, fma(dm - xn, inv2h, cur.y)) : T(0);
+          if (last) {
+            yN = yy;
+            wN = fma(inv2h, cur.x + xn, x[i].y);
+          }
+          if (w >= 0) col[(w + i) * kIntRow] = yy;
+          dm = cur.x;
+          cur = x[i];
+        }
       }
     };
     fetch();
-    // the block's fields in flight to shared memory (read by the Jacobian phase)
-    auto issue_fields = [&](int b) {
-      const T *f0 = a.fields + (size_t)b * C * 5 * P + (live ? p : 0);
+    // fields of FR samples from row r0 of a block on, in flight to shared memory
+    // (read by the Jacobian phase)
+    auto issue_fields = [&](int b, int r0) {
+      const T *f0 = a.fields + (live ? p : 0);
 #pragma unroll 4
-      for (int rc = tid / NP; rc < 4 * C; rc += kIntThreads / NP) {
-        const T *src = f0 + (size_t)((rc >> 2) * 5 + (rc & 3)) * P;
+      for (int rc = tid / NP; rc < 4 * FR; rc += kIntThreads / NP) {
+        const T *src = f0 + ((size_t)min(b * C + r0 + (rc >> 2), N - 1) * 5 + (rc & 3)) * P;
         if constexpr (sizeof(T) == 4)
           cp_async4(fld + rc * NP + pa, src, live);
         else
@@ -825,10 +890,11 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
       }
     };
     __syncthreads();  // the previous unit's Jacobian phase is done with win
-    for (int i = 0; i < H; i += BT) causal(-1);
+    if (b0 > 0)
+      for (int i = 0; i < H; i += BT) causal(-1);
     for (int i = 0; i < R; i += BT) causal(i);
     for (int b = b0; b < b1; ++b) {
-      issue_fields(b);
+      issue_fields(b, 0);
       T xx = T(0);
 #pragma unroll 16
       for (int r = R - 1; r >= C; --r) xx = fma(rho, xx, col[r * kIntRow]);
@@ -837,16 +903,33 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
         xx = fma(rho, xx, col[r * kIntRow]);
         col[r * kIntRow] = six * xx;
       }
-      cp_async_wait_all();
-      __syncthreads();
-      if (live) {
+      if (b == 0) {
+        col[0] = w0 - col[kIntRow] * T(1.0 / 6.0) - T(3) * inv2h * a0;
+        col[kIntRow] += T(4) * inv2h * a0;
+        col[2 * kIntRow] -= inv2h * a0;
+      }
+      const int rN = N - 1 - b * C;  // row of the last sample
+      if (rN < C + 2) {
+        if (rN < C) col[rN * kIntRow] = wN + rho * yN + T(3) * inv2h * aN;
+        if (rN >= 1 && rN <= C) col[(rN - 1) * kIntRow] -= T(4) * inv2h * aN;
+        if (rN >= 2) col[(rN - 2) * kIntRow] += inv2h * aN;
+      }
+      for (int r0 = 0; r0 < C; r0 += FR) {
+        if (r0 > 0) {
+          __syncthreads();  // every thread is done with the fields before these
+          issue_fields(b, r0);
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        if (live) {
 #pragma unroll 4
-        for (int r = tid / NP; r < C; r += kIntThreads / NP) {
-          const T *f = fld + r * 4 * NP + pa;
-          const T fv[4] = {f[0], f[NP], f[2 * NP], f[3 * NP]};
-          const T *q = win + r * kIntRow + pa * 4;
-          put_grad<T>(a.grad_fields + (size_t)(b * C + r) * 5 * P + p, P, fv, q[0], q[1], q[2],
-                      q[3], n0, n1, n2, Un);
+          for (int r = r0 + tid / NP; r < min(r0 + FR, N - b * C); r += kIntThreads / NP) {
+            const T *f = fld + (r - r0) * 4 * NP + pa;
+            const T fv[4] = {f[0], f[NP], f[2 * NP], f[3 * NP]};
+            const T *q = win + r * kIntRow + pa * 4;
+            put_grad<T>(a.grad_fields + (size_t)(b * C + r) * 5 * P + p, P, fv, q[0], q[1], q[2],
+                        q[3], n0, n1, n2, Un);
+          }
         }
       }
       if (b + 1 == b1) break;
@@ -857,7 +940,7 @@ __global__ void __launch_bounds__(kIntThreads, sizeof(T) == 4 ? 6 : 2)
   }
 }
 
-// Blocks at the record ends: all eight series, S with the natural ends as
+// Records shorter than H + 3 samples: all eight series, S with the natural ends as
 //   G_s = Xbar_s - D2^T A Xbar_s,
 // A = tridiag(1, 4, 1)^-1 on rows 1 .. N - 2 by the same pair of recursions on
 // the odd-periodic extension of Xbar_s (zero at 0 and N - 1), then D^T with its
@@ -931,10 +1014,10 @@ __device__ __forceinline__ void adj_values_ends(T (&z)[kAdjZ], const T *xv, bool
   }
 }
 
-// Blocks outside [int_lo, int_hi) of each panel tile.  1D grid, block fastest.
+// 1D grid, block fastest.
 template <typename T>
 __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 5 : 2)
-    k_prep_adj_iir(PrepAdjArgs<T> a, int int_lo, int int_hi) {
+    k_prep_adj_iir(PrepAdjArgs<T> a) {
   constexpr int NP = kIirPanels, H = Prec<T>::halo, J = kIirJ;
   constexpr int NR = kAdjZ + 2 * H;  // samples each thread filters
   constexpr int MR = iir_rows<T>(), MPS = adj_mps<T>();
@@ -946,11 +1029,8 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 5 : 2)
   T *cs = sm;
   const int tid = threadIdx.x;
   const int n_ct = (a.nt + kIirChunk - 1) / kIirChunk;
-  const int n_mid = int_hi - int_lo;
-  const int n_sel = n_ct - n_mid;
-  const int e = (int)(blockIdx.x % n_sel);
-  const int c0 = (e < int_lo ? e : e + n_mid) * kIirChunk;
-  const int p0 = (int)(blockIdx.x / n_sel) * NP;
+  const int c0 = (int)(blockIdx.x % n_ct) * kIirChunk;
+  const int p0 = (int)(blockIdx.x / n_ct) * NP;
   const int N = a.nt;
   const int L2 = 2 * (N - 1);
   // sample k of the odd-periodic extension as a row of the record: km in
@@ -1153,32 +1233,26 @@ cudaError_t launch_prep_adjoint(const PrepAdjArgs<T> &a, cudaStream_t s) {
   const int n_ct = (a.nt + C - 1) / C;
   const long tiles = (a.P + kIirPanels - 1) / kIirPanels;
   if (n_ct <= 0 || tiles <= 0) return cudaSuccess;
-  // interior blocks: the filters' reach c0 - H - 1 .. c0 + C + H inside 1 .. nt - 2
-  static_assert(C >= H + 2, "block 1 is an interior one");
-  const int top = a.nt - 2 - C - H;  // largest interior c0
-  int int_lo = 1, int_hi = top >= 0 ? top / C + 1 : 0;
-  if (int_hi <= int_lo) int_lo = int_hi = 0;
   cudaError_t e;
-  if (int_hi > int_lo) {
+  if (a.nt >= H + 3) {  // as in launch_prep
     const long n_pg = (a.P + kIntPanels - 1) / kIntPanels;
-    const size_t smem = ((size_t)(C + H) * kIntRow + (size_t)C * 4 * kIntPanels) * sizeof(T);
+    const size_t smem =
+        ((size_t)(C + H) * kIntRow + (size_t)kAdjFieldRows * 4 * kIntPanels) * sizeof(T);
     long grid = 0;
     int unit = 1;
-    if ((e = persistent_grid<k_prep_adj_int<T>>(smem, 0.5, n_pg, int_hi - int_lo, &unit,
-                                                &grid)) != cudaSuccess)
+    if ((e = persistent_grid<k_prep_adj_int<T>>(smem, 0.5, n_pg, n_ct, &unit, &grid)) !=
+        cudaSuccess)
       return e;
-    k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, int_lo, int_hi, unit);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_prep_adj_int<T><<<(unsigned)grid, kIntThreads, smem, s>>>(a, n_ct, unit);
+    return cudaGetLastError();
   }
-  const long ends = (long)(n_ct - (int_hi - int_lo)) * tiles;
+  const long ends = (long)n_ct * tiles;
   if (ends > INT32_MAX) return cudaErrorInvalidValue;
-  if (ends > 0) {
-    const size_t smem = (size_t)kIirPanels * (adj_mps<T>() + kAdjVPS) * sizeof(T);
-    e = cudaFuncSetAttribute(k_prep_adj_iir<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    k_prep_adj_iir<T><<<(unsigned)ends, kIirThreads, smem, s>>>(a, int_lo, int_hi);
-  }
+  const size_t smem = (size_t)kIirPanels * (adj_mps<T>() + kAdjVPS) * sizeof(T);
+  e = cudaFuncSetAttribute(k_prep_adj_iir<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem);
+  if (e != cudaSuccess) return e;
+  k_prep_adj_iir<T><<<(unsigned)ends, kIirThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
