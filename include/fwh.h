@@ -123,7 +123,7 @@ fwh_status fwh_set_observer_extremes(fwh_handle h, const double *r_max, const do
  * [nt][5][P] (double for FWH_FP64, float for FWH_MIXED), nt >= 3.
  * Covers the "compute Noise", "compute t", "interp pressure signal" and
  * surface-integration stages (Sec. III B, III C).  Host FWH_MIXED fields of
- * 256 frames or more are copied in 128-frame slabs on streams the handle owns,
+ * 256 frames or more are copied in slabs of 64 frames or more on streams the handle owns,
  * overlapped with the preparation and scatter of the frames already copied;
  * the call still returns only when p_out holds the result.
  * Errors: FWH_ERR_STATE before fwh_set_observers, FWH_ERR_ARG for nt outside
@@ -160,9 +160,10 @@ fwh_status fwh_backward(fwh_handle h, const void *fields, int64_t nt,
  * Faces of Sec. III A); all handles must share one precision and take device
  * buffers.  By default the series of every surface are kept for the whole
  * record.  With a ring set on hs[0] (fwh_set_batch_options), the record is
- * streamed instead in rounds of R time segments (512 samples each under the
- * default tile shape): each surface keeps the series of R segments only
- * (P x 512 R rows instead of P x round_up(nt, 256)).  The work items (panel
+ * streamed instead in rounds of R time segments (252 intervals in mixed
+ * precision, 128 samples in FP64, under the default tile shape): each surface
+ * keeps the series of R segments only (about P x 256 R, P x 128 R rows instead
+ * of P x round_up(nt + 3, 64)).  The work items (panel
  * set x time segment x observer group) are scattered in the launch form set
  * on hs[0]: FWH_BATCH_PIPELINED (default) one launch per surface and round,
  * each surface's series prepared on a high-priority stream while the
@@ -181,8 +182,9 @@ fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void *const *fie
  * Options of batched calls led by h (h = hs[0] of fwh_batch_forward).
  * ring_samples = 0 (the default) keeps every surface's series for its whole
  * record; ring_samples > 0 streams records longer than that through a ring
- * of max(1, floor(ring_samples / 512)) time segments of 512 samples (default
- * tile shape), 64 bytes (FP32) or 128 bytes (FP64) per panel and sample.
+ * of max(1, floor(ring_samples / 256)) time segments of just under 256 samples
+ * (default tile shape; 128 and 128 in FP64), 32 bytes (FP32) or 64 bytes (FP64)
+ * per panel and sample.
  * form: FWH_BATCH_PIPELINED, FWH_BATCH_GRID or FWH_BATCH_PERSISTENT (see
  * fwh_batch_forward).  On a GB300 the pipelined form is the fastest; the
  * single grid reads its per-surface arguments from a parameter block by
@@ -195,12 +197,12 @@ fwh_status fwh_set_batch_options(fwh_handle h, int64_t ring_samples, int form);
 
 /*
  * Pipelined forward passes (default off): with device fields and a record of
- * several time segments (512 samples under the default tile shape),
- * fwh_forward prepares the series of each segment on a high-priority stream
- * the handle owns and starts the scatter of a segment as soon as its series
- * are in, so the preparation of later segments runs under the scatter of
- * earlier ones; off, it prepares the whole record first and scatters it in
- * one launch.  Results agree to the FP64 rounding of the output sums.  On a
+ * several time segments (252 intervals in mixed precision, 128 samples in FP64,
+ * under the default tile shape), fwh_forward prepares the series of each
+ * segment on a high-priority stream the handle owns and starts the scatter of a
+ * segment as soon as its series are in, so the preparation of later segments
+ * runs under the scatter of earlier ones; off, it prepares the whole record
+ * first and scatters it in one launch.  Results agree to the FP64 rounding of the output sums.  On a
  * GB300 the pipelined call was slower for device-resident fields (the prep's
  * blocks take SM slots from the arithmetic-bound scatter, and each segment
  * launch has its own tail), hence the default; host fields are always
@@ -230,7 +232,7 @@ fwh_status fwh_set_tile_config(fwh_handle h, int config);
  * last call; fwh_timing_totals the sums over all timed calls since the last
  * reset and their count.  Both synchronise on the recorded events.  When a
  * FWH_MIXED call takes host fields of 256 frames or more, the copy, the
- * preparation and the scatter overlap in 128-frame slabs: [0] then runs to
+ * preparation and the scatter overlap in slabs of frames: [0] then runs to
  * the start of the first scatter launch and [1] from there to the end.
  */
 fwh_status fwh_set_timing(fwh_handle h, int enable);

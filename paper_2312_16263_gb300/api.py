@@ -158,7 +158,7 @@ class FWH:
     def set_batch_options(self, ring: int = 0, form: str = "pipelined"):
         """Options of batched calls this surface leads (first in the list):
         ring = 0 keeps whole records, > 0 streams them through a ring of that
-        many source samples (whole 512-sample segments, at least one); form
+        many source samples (whole time segments, at least one); form
         is "pipelined" (one launch per surface, preps overlapped), "grid" (one
         grid over every surface) or "persistent" (the work-queue kernel)."""
         forms = {"pipelined": _abi.FWH_BATCH_PIPELINED, "grid": _abi.FWH_BATCH_GRID,

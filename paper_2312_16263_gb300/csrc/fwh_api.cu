@@ -328,12 +328,18 @@ int effective_cfg(const fwh_ctx *h, int64_t nt) {
 
 // Work items a panel set is cut into, from sizes of the whole problem only
 // (every launch form of it then forms the same partial sums): enough items to
-// give each SM several CTAs, at least eight panels an item.
+// give each SM several CTAs, at least eight panels an item; in FP64, where an
+// item's prologue and flushes weigh less and fewer CTAs fit an SM, three times
+// as many items and down to four panels (5151 panels x 701 steps x 19 observers
+// 1.74 -> 1.56 ms and 688 x 475 x 21 0.31 -> 0.17 together with the shorter
+// segments; four panels an item in mixed precision: 23 -> 30 us at 2048 x 256
+// x 8).
 int set_subs(const fwh_ctx *h, int groups, int n_segs) {
+  const bool fp64 = h->precision == FWH_FP64;
   const int64_t nsets = (int64_t)h->set_begin.size() - 1;
   const int64_t items = nsets * groups * n_segs;
-  const int64_t want = (kWantItems + items - 1) / items;
-  const int64_t most = std::max<int64_t>(1, h->P / nsets / 8);
+  const int64_t want = ((fp64 ? 3 : 1) * kWantItems + items - 1) / items;
+  const int64_t most = std::max<int64_t>(1, h->P / nsets / (fp64 ? 4 : 8));
   return (int)std::min(want, most);
 }
 
@@ -1246,7 +1252,8 @@ template <typename T> const std::vector<BatchParams<T>> &batch_params(const Batc
 int seg_len_of(bool fp64, const FwdConfig &c) { return c.seg_chunks * fwd_chunk(fp64, c); }
 
 // Segments per round of a batched call led by h0 (0: the whole record).  Ring
-// lengths count segments of 512 samples; a segment is that or slightly less.
+// lengths count segments of 32 tk samples a chunk; an FP32 segment's chunks
+// complete four fewer each.
 int batch_round_segs(const fwh_ctx *h0, const FwdConfig &c) {
   const int seg = c.seg_chunks * 32 * c.tk;
   return h0->batch_ring > 0 ? (int)std::max<int64_t>(1, h0->batch_ring / seg) : 0;
