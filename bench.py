@@ -33,7 +33,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "FW-H panel·τ·observer evals/s, mixed vs FP64 at ≤1e-4 rel L2; % roofline"
 UNIT = "evals/s"
-FLOP_PER_EVAL = 40          # 20 FMA: 8 + 8 (signal, spline moment) + 4 (interpolation)
+FLOP_PER_EVAL = 24          # 12 FMA: 8 (signal) + 4 (B-spline taps)
 # FP32 FMA roof: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz (maximum SM clock)
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # FP64 FMA roof: nominal GB300 FP64 rate
@@ -327,9 +327,9 @@ def extra_legs(dev):
         ms = _time_calls(lambda: s.forward(fx, o), 20)
         _, nv = s.window(w.nt)
         # few observers: the series bytes per call (one row per panel and
-        # sample per observer group; 64 B mixed, 128 B FP64) against HBM too
+        # sample per observer group; 32 B mixed, 64 B FP64) against HBM too
         groups = -(-w.observers.shape[0] // 36)
-        xbytes = (64 if prec == "mixed" else 128) * w.surface.n_panels * w.nt * groups
+        xbytes = (32 if prec == "mixed" else 64) * w.surface.n_panels * w.nt * groups
         leg[prec] = {"ms": ms, "evals_per_s": w.evals / (ms / 1e3),
                      "series_bytes": xbytes,
                      "hbm_frac": xbytes / (ms / 1e3) / 1e9 / hbm_peak_gbs()[0],
@@ -387,9 +387,8 @@ def extra_legs(dev):
     torch.cuda.empty_cache()
     # workload 5: eight uneven surfaces in one graph-captured call (whole
     # records, pipelined form), one fwh_forward call per surface, the single
-    # grid and persistent forms, and the series streamed through a ring of two
-    # 512-sample segments per surface (four rounds); the smallest surface
-    # against the oracle
+    # grid and persistent forms, and the series streamed through a ring of 1024
+    # samples per surface; the smallest surface against the oracle
     ws5 = batch_workloads()
     surfs = [FWH.from_workload(x, "mixed") for x in ws5]
     fields = [x.fields(device=dev, dtype="float32") for x in ws5]
@@ -438,7 +437,7 @@ def extra_legs(dev):
                     "grid_vs_oracle_rel_l2": err_f["grid"],
                     "persistent_vs_oracle_rel_l2": err_f["persistent"],
                     "streamed_ms": ms_r, "streamed_evals_per_s": ev5 / (ms_r / 1e3),
-                    "streamed_form": "pipelined, ring of 2 x 512 samples per surface, 4 rounds",
+                    "streamed_form": "pipelined, ring of 1024 samples per surface",
                     "device_free_gb_whole_records": free_b / 1e9,
                     "device_free_gb_streamed": free_r / 1e9,
                     "mixed_vs_oracle_rel_l2": err_b, "streamed_vs_oracle_rel_l2": err_r,
@@ -634,10 +633,9 @@ def main():
     fwd_ms = tt["forward_ms"] / max(1, tt["calls"])
     prep_ms = tt["prep_ms"] / max(1, tt["calls"])
     achieved = evals * FLOP_PER_EVAL / (fwd_ms / 1e3) / 1e12
-    # series prep: FP32 fields read once, FP32 series rows (16 values per panel
-    # and padded step) written once
-    ntp = (w.nt + 255) // 256 * 256
-    prep_bytes = w.nt * 5 * w.surface.n_panels * 4 + w.surface.n_panels * ntp * 16 * 4
+    # series prep: FP32 fields read once, FP32 series rows (8 values per panel and
+    # step) written once
+    prep_bytes = w.nt * 5 * w.surface.n_panels * 4 + w.surface.n_panels * w.nt * 8 * 4
     hbm_gbs, hbm_src = hbm_peak_gbs()
     traffic = profile_traffic()
     p_mixed = out.cpu().numpy()
@@ -693,7 +691,7 @@ def main():
         "config": {"workload": w.name, "panels": w.surface.n_panels, "nt": w.nt,
                    "observers_per_gpu": s.O, "precision": "mixed (FP32 series and integrand "
                    "arithmetic, FP64 arrival times/weights and output)",
-                   "l2": "inputs larger than L2 (1.34 GB fields, 4.3 GB series per step)",
+                   "l2": "inputs larger than L2 (1.34 GB fields, 2.2 GB series per step)",
                    "parallelism": f"observer sets x{ws}, no collective"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS,
                      "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_TFLOPS,
@@ -718,13 +716,12 @@ def main():
                 "h2d_bytes_per_step": int(fh.numel() * fh.element_size()),
                 "d2h_bytes_per_step": int(oh.numel() * oh.element_size()),
                 "ms_per_step": e2e_ms_max},
-        "prep": {"bound": "hbm", "kernels": "k_prep_iir_int (interior blocks) + k_prep_iir "
-                 "(record ends)", "ms": prep_ms, "bytes": prep_bytes,
+        "prep": {"bound": "hbm", "kernels": "k_prep_iir_int", "ms": prep_ms, "bytes": prep_bytes,
                  "achieved": prep_bytes / (prep_ms / 1e3) / 1e9, "peak": hbm_gbs,
                  "unit": "GB/s", "frac": prep_bytes / (prep_ms / 1e3) / 1e9 / hbm_gbs,
                  "peak_source": hbm_src},
-        # per step: the two prep kernels and the forward scatter
-        "gpu_launches": 3 * args.steps,
+        # per step: the prep kernel and the forward scatter
+        "gpu_launches": 2 * args.steps,
         "clocks": clocks,
     }
     # PSD of the far-field signals (Sec. IV C): Welch, 512-sample segments
