@@ -983,9 +983,14 @@ __global__ void __launch_bounds__((cta_threads<NW, PIPE>()), (MinBlocks<TK, NW, 
 // has flushed its windows for the previous one.  There is no CTA-wide barrier
 // between items, so the copies of an item's first stages are in flight while
 // the compute warps finish the item before it.  A slot is rewritten kItemQ
-// publications later; the producer can run at most `nst` steps (hence items)
-// ahead of the slowest compute warp, so kItemQ > kMaxStages keeps every
-// publication readable until each warp has taken it.
+// publications later.  What holds the producer back is the stage ring: it can
+// run at most `nst` steps ahead of the slowest compute warp, and every published
+// item has at least one step, so it is at most `nst` items ahead and kItemQ >
+// kMaxStages keeps every publication readable until each warp has taken it.  A
+// panel set of fewer panels than the parts it is cut into leaves parts without
+// panels; such an item takes no stage, so any number of them could pass while the
+// compute warps still work: the producer drops them and claims on (65 panels in
+// sets of 64 and 1, four parts each: over 300 in a row).
 constexpr int kItemQ = 16;
 // kernel parameters may take up to 32764 bytes (CUDA 12.1 and later)
 static_assert(sizeof(BatchParams<double>) + 64 <= 32764, "batched launch parameters too large");
@@ -1035,20 +1040,23 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
     volatile int *abort = &abort_flag;
     if (w == NW) {
       if ((threadIdx.x & 31) == 0) {
-        int item = s_item;
-        for (int k = 0;; ++k) {
-          s_q[k % kItemQ] = item;
-          mbar_arrive(&qbar[k % kItemQ]);  // release: the index is visible to the waiters
-          if (item >= total) break;
+        int k = 0;  // publications
+        // after a timeout, or with copies withheld (testing), the queue ends: the
+        // compute warps stop at the sentinel below or at the abort flag
+        for (int item = s_item; item < total;
+             item = (*abort || args[0].withhold) ? total : atomicAdd(counter, 1)) {
           const int sf = batch_surface(prefix, n_surf, item);
           const FwdArgs<T> &a = args[sf];
-          ps.tmap = &P.tm[sf];
           const Item<T, 1> it(a, item - prefix[sf], 0);
+          if (it.p_begin == it.p_end) continue;  // no panels, hence no steps: not published
+          s_q[k % kItemQ] = item;
+          mbar_arrive(&qbar[k % kItemQ]);  // release: the index is visible to the waiters
+          ++k;
+          ps.tmap = &P.tm[sf];
           produce_item<T, TK, NW>(a, it, ps, step);
-          // after a timeout, or with copies withheld (testing), end the queue
-          // here: the compute warps stop at this sentinel or at the abort flag
-          item = (*abort || a.withhold) ? total : atomicAdd(counter, 1);
         }
+        s_q[k % kItemQ] = total;  // the sentinel that ends the queue
+        mbar_arrive(&qbar[k % kItemQ]);
         drain_copies(ps, step, args[0].err);
       }
     } else {
