@@ -1269,9 +1269,13 @@ int batch_x_ld(const fwh_ctx *h, int seg, int R) {
                      : whole);
 }
 
-// First record row in X of round r.
+// First record row in X of round r: the block of the round's first row, or of row
+// nt - 1 where the round starts past it (an FP64 round of the last one or two rows;
+// the last sample's row and the rows after it are written with row nt - 1's block,
+// and x_ld has room for the block more).
 int batch_row0(const BatchPlan &bp, int i, int64_t nt, int r) {
-  return bp.x_ld[i] == x_rows(nt) ? 0 : (int)((int64_t)r * bp.R * bp.seg / kRowBlk * kRowBlk);
+  if (bp.x_ld[i] == x_rows(nt)) return 0;
+  return (int)(std::min<int64_t>((int64_t)r * bp.R * bp.seg, nt - 1) / kRowBlk * kRowBlk);
 }
 
 template <typename T>

@@ -137,6 +137,7 @@ struct PrepArgs {
   int row0;             // record row held by X row 0 (a multiple of 64)
   double ca, sa, dt;
   int c_lo, c_hi;       // 64-row blocks [c_lo, c_hi) to prepare (0, 0: the whole record)
+                        // (rows nt .. nt + 2 are written with the block of row nt - 1)
 };
 
 template <typename T>
