@@ -23,16 +23,17 @@
 //    back substitution yields the coefficients in registers, four at a time,
 //    while the thread walks the observer bins downwards: the bin t_j lies in
 //    the interval whose arrival times tau + Delta bracket it, tau* is the root
-//    of a cubic there by Newton's method (residual in FP64, its quotient with
-//    the slope in FP32: a relative error of 1e-7 in a correction that the next
-//    step repeats; three steps reach FP64 rounding for subsonic motion), and
-//    the spline of g at tau* goes to a shared-memory tile from which each warp
-//    sums its panels, one FP64 atomic per warp and bin.
-// About 126 FP64 operations per (panel, sample, observer), the FP64 pipe 87 % busy.
-// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 62.0 ms for
+//    of a cubic there by Newton's method (three steps from the chord, the last
+//    one in FP64; the two before it need not be exact, and their FP32 parts leave
+//    the FP64 pipe alone: against long double the result is that of three FP64
+//    steps, to rounding up to tip Mach numbers of 0.9 at 30 frames a revolution,
+//    1e-11 at 18), and the spline of g at tau* goes to a shared-memory tile from
+//    which each warp sums its panels, one FP64 atomic per warp and bin.
+// About 130 FP64 operations per (panel, sample, observer); bound by the FP64 pipe.
+// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 63.0 ms for
 // k_mscatter (135.4 with moments, four columns, divisions in Newton's method
 // and a shuffle sum per bin: about 380 operations), 1.84 ms for k_mseries (5.65
-// with each frame's integrands formed three times), 64.3 ms a call (164).
+// with each frame's integrands formed three times), 65.0 ms a call (164).
 // Scratch: two FP64 columns of nt per (panel, observer) of a launch; the host
 // splits the observers into launches by the scratch budget.
 #include <cuda_runtime.h>
@@ -332,15 +333,19 @@ __global__ void __launch_bounds__(kMTile, 7) k_mscatter(MovArgs a) {
         const double p1 = fma(0.5, D[2] - D[0], h);
         const double p2 = fma(0.5, D[0] + D[2], -D[1]);
         const double p3 = fma(0.5, D[1] - D[2], (D[3] - D[0]) * (1.0 / 6.0));
-        const float q1 = (float)p1, q2 = 2.f * (float)p2, q3 = 3.f * (float)p3;
-        float ff = fminf(1.f, fmaxf(0.f, __fdividef(-(float)e, q1)));
+        // Newton's method, three steps from the chord, each clamped to the interval:
+        // the first in FP32, the second an FP64 residual over an FP32 slope, the
+        // last in FP64
+        const float r1 = (float)p1, r2 = (float)p2, r3 = (float)p3, re = (float)e;
+        auto slope = [&](float x) { return fmaf(fmaf(3.f * r3, x, 2.f * r2), x, r1); };
+        float ff = fminf(1.f, fmaxf(0.f, __fdividef(-re, r1 + r2 + r3)));
+        ff -= __fdividef(fmaf(fmaf(fmaf(r3, ff, r2), ff, r1), ff, re), slope(ff));
+        ff = fminf(1.f, fmaxf(0.f, ff));
+        auto residual = [&](double x) { return fma(fma(fma(p3, x, p2), x, p1), x, e); };
         double f = (double)ff;
-#pragma unroll
-        for (int it = 0; it < 3; ++it) {
-          const double res = fma(fma(fma(p3, f, p2), f, p1), f, e);
-          ff = (float)f;
-          f -= (double)__fdividef((float)res, fmaf(fmaf(q3, ff, q2), ff, q1));
-        }
+        f -= (double)__fdividef((float)residual(f), slope(ff));
+        f = fmin(1.0, fmax(0.0, f));
+        f = fma(-residual(f), recip(fma(fma(3.0 * p3, f, 2.0 * p2), f, p1)), f);
         f = fmin(1.0, fmax(0.0, f));
         const double c = 1.0 - f, f2 = f * f, c2 = c * c;
         val = (c2 * c) * G[0];
