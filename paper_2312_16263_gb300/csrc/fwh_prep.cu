@@ -20,7 +20,8 @@
 // a causal recursion y_k = r_k + rho y_{k-1} followed by an anti-causal one
 // x_k = y_k + rho x_{k+1}:
 //   beta_k = F_k + rho x_k   with r = D2 F          (FP32: no loss at low frequency)
-//   beta_k = -6 rho x_k      with r = F             (FP64: fewer operations)
+//   beta_k = F_0 - 6 rho x_k with r = F - F_0       (FP64: fewer operations; F_0
+//                                                    a constant, see below)
 // A recursion started H samples outside the 64-row block it serves errs by
 // |rho|^H (H = 16 for FP32, 32 for FP64: below rounding), so blocks are
 // independent.  At the record ends both start exactly: y_0 is a sum over the
@@ -30,12 +31,18 @@
 // Away from the record ends the solve commutes with the central difference, so
 // a derivative series' coefficients are the central differences d_k =
 // (beta_{k+1} - beta_{k-1}) / (2 dt) of its value series' coefficients: four
-// filters, not eight.  In FP32 d_k is formed from the differences of F and of x,
-// not of the rounded beta: under a mean value of F far above its changes (a mean
-// pressure on a flat face) the rounding of beta is what a difference of beta would
-// keep (error 4e-5 instead of 6e-4 at a mean of 1000 amplitudes, no time lost).  Near an end they differ by a solution of the
+// filters, not eight.  Near an end they differ by a solution of the
 // homogeneous system: beta'_k = d_k + (D_0 - d_0) rho^k from the start (D_0 the
 // one-sided derivative, d_0 = (beta_1 - beta_0) / dt), and likewise from the end.
+//
+// A mean of F far above its changes (a mean pressure on a flat face) must not round
+// into the differences.  FP32 forms d_k from the differences of F and of x, not of the
+// rounded beta (a fluctuation under a mean of 1000 amplitudes: error 4e-5, 6e-4 with
+// differences of beta; no time lost).  FP64 filters F less its value at the work
+// unit's first sample, which the integrands' last multiply-adds subtract: 5e-14, and
+// 1.2e-12 with the filter's gain folded into the normals, which saved a multiply-add
+// per value (32768 panels x 2048 steps 5.28 against 5.70 ms, 2048 x 256 113 against
+// 118 us).
 //
 // Kernels: k_prep_iir_int (FP32) and k_prep_f64_int (FP64), persistent CTAs that
 // walk consecutive blocks of a panel group; k_prep_iir for records too short for
@@ -346,12 +353,12 @@ __global__ void __launch_bounds__(kIntThreads, 4) k_prep_iir_int(PrepArgs<float>
 // column of the window holds y (the causal recursion, carried on from block to
 // block, in place of the integrand), so per sample the integrands are formed
 // once, the causal step runs once and the anti-causal one 1.5 times (64 + 34
-// rows per 64): about 32 FP64 operations per (panel, sample).  The record ends
+// rows per 64): about 36 FP64 operations per (panel, sample).  The record ends
 // are handled in place.  Field rows arrive 32 at a time, half of a block's ahead
 // of the block, so that three CTAs fit an SM and hide each other's chains.
-// 32768 panels x 2048 steps: 5.3 ms (6.8 with 64 rows in flight, two CTAs and
-// the filter's gain applied per sample; 8.7 with a kernel of its own for the
-// record ends; 15.2 by windowed elimination, 142 operations and 128-byte rows).
+// 32768 panels x 2048 steps: 5.7 ms (6.8 with 64 rows in flight and two CTAs; 8.7
+// with a kernel of its own for the record ends; 15.2 by windowed elimination, 142
+// operations and 128-byte rows).
 // ---------------------------------------------------------------------------
 constexpr int kF64H = Prec<double>::halo;
 constexpr int kF64Raw = 32;  // field rows in flight
@@ -390,16 +397,18 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *win = reinterpret_cast<double *>(smem_raw);  // [R][NP][4]
   double *raw = win + R * kIntRow;                     // [kF64Raw][5][NP]
+  double *base = raw + kF64Raw * 5 * NP;               // [NP][4]: F0
   const int tid = threadIdx.x;
   const int n_pg = (a.P + NP - 1) / NP;
   const int n_us = (a.c_hi - a.c_lo + unit - 1) / unit;
   const long n_units = (long)n_pg * n_us;
   const int pa = tid % NP;               // integrand phase: panel, rows tid / NP + 4 u
   const int qi = tid & 3, pl = tid >> 2; // filter phase: integrand, panel
-  // Normals scaled by -6 rho scale all four integrands by it, so the filter's
-  // output is the coefficient itself: F below is -6 rho times the integrand.
-  constexpr double kScale = -6.0 * kRho, kUnscale = 1.0 / kScale;
-  const double inv2h = 0.5 / a.dt;
+  // What is filtered is F - F0, F0 the integrand of the unit's first sample: the
+  // differences then round with the changes of F, not with its mean (see above).
+  // Coefficients are F0 + kGain x, their differences kGain times those of x.
+  constexpr double kGain = -6.0 * kRho, kUngain = 1.0 / kGain;
+  const double inv2h = 0.5 / a.dt, g2h = kGain * inv2h;
   const bool vec = (a.P & 1) == 0 && ((size_t)a.fields & 15) == 0;
   for (long u = blockIdx.x; u < n_units; u += gridDim.x) {
     const int p0 = (int)(u % n_pg) * NP;
@@ -409,40 +418,56 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
     double n0 = 0, n1 = 0, n2 = 0, Un = 0;
     if (p < a.P) {
       const double *n = a.n + 3 * (size_t)(a.place ? a.place[p] : p);
-      n0 = kScale * n[0];
-      n1 = kScale * n[1];
-      n2 = kScale * n[2];
+      n0 = n[0];
+      n1 = n[1];
+      n2 = n[2];
       Un = a.ca * n0 + a.sa * n1;
     }
     const bool live_b = pb < a.P;
     double *const xp =
         a.X + ((size_t)(live_b ? (a.place ? a.place[pb] : pb) : 0) * a.x_ld) * kSer + 2 * qi;
     double *const col = win + pl * 4 + qi;
-    // integrands of the n rows in raw into window rows [w0, w0 + n)
+    // integrands, less F0, of the n rows in raw into window rows [w0, w0 + n)
+    double q0[4] = {0.0, 0.0, 0.0, 0.0};  // F0 of this thread's panel (integrand phase)
+    auto form = [&](int r, double (&q)[4]) {
+      const double *f = raw + r * 5 * NP + pa;
+      const double rho_ = f[0], u0 = f[NP], u1 = f[2 * NP], u2 = f[3 * NP], pp = f[4 * NP];
+      const double un = u0 * n0 + u1 * n1 + u2 * n2;
+      const double r1 = 1.0 + rho_;
+      const double t = r1 * (Un + un);
+      q[0] = fma(rho_, Un, fma(r1, un, -q0[0]));  // Qn
+      q[1] = fma(pp, n0, fma(u0, t, -q0[1]));     // L_1
+      q[2] = fma(pp, n1, fma(u1, t, -q0[2]));
+      q[3] = fma(pp, n2, fma(u2, t, -q0[3]));
+    };
     auto integrands = [&](int w0, int n) {
       for (int r = tid / NP; r < n; r += kIntThreads / NP) {
-        const double *f = raw + r * 5 * NP + pa;
-        const double rho_ = f[0], u0 = f[NP], u1 = f[2 * NP], u2 = f[3 * NP], pp = f[4 * NP];
-        const double un = u0 * n0 + u1 * n1 + u2 * n2;
-        const double r1 = 1.0 + rho_;
-        const double t = r1 * (Un + un);
+        double q[4];
+        form(r, q);
         double *w = win + (w0 + r) * kIntRow + pa * 4;
-        *reinterpret_cast<double2 *>(w) = make_double2(rho_ * Un + r1 * un,   // Qn
-                                                       pp * n0 + u0 * t);     // L_1
-        *reinterpret_cast<double2 *>(w + 2) = make_double2(pp * n1 + u1 * t, pp * n2 + u2 * t);
+        *reinterpret_cast<double2 *>(w) = make_double2(q[0], q[1]);
+        *reinterpret_cast<double2 *>(w + 2) = make_double2(q[2], q[3]);
       }
     };
     auto issue = [&](int sample, int n) {
       issue_rows_f64<NP>(a.fields, a.P, a.nt, p0, sample, n, raw, vec);
     };
     // integrands of n samples from `sample` on into window rows from w0 on; the
-    // first min(n, kF64Raw) are in flight already
-    auto fill = [&](int sample, int w0, int n) {
+    // first min(n, kF64Raw) are in flight already (`first`: the unit's first rows)
+    auto fill = [&](int sample, int w0, int n, bool first = false) {
       for (int r = 0; r < n; r += kF64Raw) {
         const int m = min(kF64Raw, n - r);
         if (r > 0) issue(sample + r, m);
         cp_async_wait_all();
         __syncthreads();
+        if (first && r == 0) {
+          double q[4];
+          form(0, q);
+          for (int c = 0; c < 4; ++c) {
+            q0[c] = q[c];
+            if (tid < NP) base[4 * pa + c] = q[c];
+          }
+        }
         integrands(w0 + r, m);
         __syncthreads();
       }
@@ -450,7 +475,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
     const int lo = b0 * C - 2;  // sample c0 - 1 of the first block
     const int N = a.nt;
     double yy = 0.0;
-    double f1 = 0.0, f2 = 0.0, f3 = 0.0;  // integrand at the last three samples passed
+    double f1 = 0.0, f2 = 0.0, f3 = 0.0;  // F - F0 at the last three samples passed
     // causal recursion over window rows [r0, R), whose row r holds sample s0 + r;
     // it stops being used at sample N - 1
     auto causal = [&](int r0, int s0) {
@@ -473,11 +498,11 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         }
       }
     };
-    double F0 = 0.0, D0 = 0.0;  // integrand and one-sided derivative at sample 0
+    double e0 = 0.0, D0 = 0.0;  // F - F0 and the one-sided derivative at sample 0
     __syncthreads();  // the previous unit is done with raw and win
     if (b0 > 0) {
       issue(lo - H, H);
-      fill(lo - H, 0, H);  // the samples the causal recursion starts on
+      fill(lo - H, 0, H, true);  // the samples the causal recursion starts on
       for (int r = 0; r < H; ++r) {
         f3 = f2;
         f2 = f1;
@@ -487,15 +512,16 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
       __syncthreads();
     }
     issue(lo, kF64Raw);
-    fill(lo, 0, R);
+    fill(lo, 0, R, b0 == 0);
+    const double Fb = base[pl * 4 + qi];
     if (b0 > 0) {
       causal(0, lo);
     } else {  // rows 0 and 1 lie before the record; y_0 from the reflected series
-      F0 = col[2 * kIntRow];
-      D0 = (-3.0 * F0 + 4.0 * col[3 * kIntRow] - col[4 * kIntRow]) * (kUnscale * inv2h);
+      e0 = col[2 * kIntRow];
+      D0 = (-3.0 * e0 + 4.0 * col[3 * kIntRow] - col[4 * kIntRow]) * inv2h;
       for (int j = H; j >= 1; --j) yy = kRho * (col[(2 + j) * kIntRow] + yy);
-      yy = F0 * ((1.0 + kRho) / (1.0 - kRho)) - yy;
-      f1 = F0;
+      yy = e0 * ((1.0 + kRho) / (1.0 - kRho)) - yy;
+      f1 = e0;
       col[2 * kIntRow] = yy;
       causal(3, lo);
     }
@@ -504,7 +530,7 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
       if (more) issue(b * C - 2 + R, kF64Raw);
       double *const xr = xp + (size_t)(b * C - a.row0) * kSer;
       const int s0 = b * C - 2;  // sample of window row 0
-      double xx = 0.0, c1 = 0.0, c2 = 0.0;  // coefficients one and two samples on
+      double xx = 0.0, c1 = 0.0, c2 = 0.0;  // x, and x one and two samples on
       if (b > 0 && s0 + R < N) {
 #pragma unroll 14
         for (int r = R - 1; r >= C + 2; --r) xx = fma(kRho, xx, col[r * kIntRow]);
@@ -518,7 +544,8 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         for (int r = C - 1; r >= 0; --r) {  // window row r: sample c0 - 1 + r
           xx = fma(kRho, xx, col[r * kIntRow]);
           if (live_b)
-            *reinterpret_cast<double2 *>(xr + r * kSer) = make_double2((c2 - xx) * inv2h, c1);
+            *reinterpret_cast<double2 *>(xr + r * kSer) =
+                make_double2((c2 - xx) * g2h, fma(kGain, c1, Fb));
           c2 = c1;
           c1 = xx;
         }
@@ -528,25 +555,25 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
         if (b == 0) {
           double x1 = 0.0;
           for (int r = H + 3; r >= 3; --r) x1 = fma(kRho, x1, col[r * kIntRow]);
-          pw = D0 - (x1 - kUnscale * F0) * (2.0 * inv2h);
+          pw = D0 - (kGain * x1 - e0) * (2.0 * inv2h);
           for (int i = 0; i < H + 4; ++i) pw *= kRho;  // below rounding from sample H + 4 on
         }
         const double ir = 1.0 / kRho;
         // (used where f1 is sample N - 1)
-        const double DN = (3.0 * f1 - 4.0 * f2 + f3) * (kUnscale * inv2h), FN = kUnscale * f1;
+        const double DN = (3.0 * f1 - 4.0 * f2 + f3) * inv2h, xN = kUngain * f1;
         double cr = 0.0, d2 = 0.0;
         for (int r = R - 1; r >= 0; --r) {
           const int sr = s0 + r;
           if (sr > N - 1) continue;
-          xx = sr == N - 1 ? FN : fma(kRho, xx, col[r * kIntRow]);
+          xx = sr == N - 1 ? xN : fma(kRho, xx, col[r * kIntRow]);
           if (sr == N - 2)
-            cr = DN - (c1 - xx) * (2.0 * inv2h);
+            cr = DN - (c1 - xx) * (2.0 * g2h);
           else if (sr > N - 3 - (H + 4))  // below rounding further on
             cr *= kRho;
           else
             cr = 0.0;
           const int se = sr + 1;  // the sample now complete, in X row r
-          double d = (c2 - xx) * inv2h;
+          double d = (c2 - xx) * g2h;
           if (cr != 0.0) d += cr;
           if (b == 0 && se < H + 4) {
             pw *= ir;
@@ -554,17 +581,19 @@ __global__ void __launch_bounds__(kIntThreads) k_prep_f64_int(PrepArgs<double> a
           }
           if (r < C && live_b && se <= N - 2) {
             double *row = xr + r * kSer;
-            if (se > 0) *reinterpret_cast<double2 *>(row) = make_double2(d, c1);
+            const double v = fma(kGain, c1, Fb);
+            if (se > 0) *reinterpret_cast<double2 *>(row) = make_double2(d, v);
             if (se == 0) {  // sample 0 and the ghost before it
-              *reinterpret_cast<double2 *>(row) = make_double2(D0, c1);
-              *reinterpret_cast<double2 *>(row - kSer) = make_double2(2.0 * D0 - d2, 2.0 * c1 - c2);
+              *reinterpret_cast<double2 *>(row) = make_double2(D0, v);
+              *reinterpret_cast<double2 *>(row - kSer) =
+                  make_double2(2.0 * D0 - d2, fma(kGain, 2.0 * c1 - c2, Fb));
             }
             if (se == N - 2) {  // the last sample, the ghost after it and a zero row
               const int room = a.row0 + a.x_ld - b * C - r;  // rows of X from this one on
-              if (room > 1) *reinterpret_cast<double2 *>(row + kSer) = make_double2(DN, FN);
+              if (room > 1) *reinterpret_cast<double2 *>(row + kSer) = make_double2(DN, f1 + Fb);
               if (room > 2)
                 *reinterpret_cast<double2 *>(row + 2 * kSer) =
-                    make_double2(2.0 * DN - d, 2.0 * FN - c1);
+                    make_double2(2.0 * DN - d, fma(kGain, 2.0 * xN - c1, Fb));
               if (room > 3) *reinterpret_cast<double2 *>(row + 3 * kSer) = make_double2(0.0, 0.0);
             }
           }
@@ -1223,7 +1252,7 @@ cudaError_t launch_prep(const PrepArgs<T> &a0, cudaStream_t s) {
       k_prep_iir_int<<<(unsigned)grid, kIntThreads, smem, s>>>(a, unit);
     } else {
       const size_t smem =
-          ((size_t)kF64Rows * kIntRow + (size_t)kF64Raw * 5 * kIntPanels) * sizeof(T);
+          ((size_t)kF64Rows * kIntRow + (size_t)kF64Raw * 5 * kIntPanels + 4 * kIntPanels) * sizeof(T);
       if ((e = persistent_grid<k_prep_f64_int>(smem, 1.0, n_pg, n_blk, &unit, &grid)) !=
           cudaSuccess)
         return e;

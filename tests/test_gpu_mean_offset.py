@@ -6,8 +6,9 @@ differences in source time that the mean must not spoil.  Compared with the orac
 less each signal's mean.  Bars: the offset's share of a panel's term is about 16
 times the fluctuation's (c_L against c_L' at 20 units and 10 rad per unit of time), a
 window sums 25 panels of one face in the type of the fields with a few roundings a
-panel: 6e-8 x 16 x 25 x 8 = 2e-4 in FP32.  A difference of rounded spline
-coefficients left 6e-4."""
+panel: 6e-8 x 16 x 25 x 8 = 2e-4 in FP32, 1.1e-16 x 3200 = 4e-13 in FP64.  A
+difference of rounded spline coefficients left 6e-4, integrands scaled by a factor
+that is no power of two 1e-12."""
 import numpy as np
 import pytest
 import torch
@@ -41,7 +42,7 @@ def _box(m):
     return np.concatenate(pos), np.concatenate(nrm), np.full(6 * m * m, 1.0 / (m * m))
 
 
-@pytest.mark.parametrize("prec,bar", [("mixed", 2e-4)])
+@pytest.mark.parametrize("prec,bar", [("mixed", 2e-4), ("fp64", 4e-13)])
 @pytest.mark.parametrize("nt", [128, 191, 256, 600, 1000])
 def test_fluctuation_under_a_mean(dev, prec, bar, nt):
     from paper_2312_16263_gb300 import FWH
