@@ -1293,9 +1293,6 @@ fwh_status batch_build(int n, const fwh_handle *hs, double *const *p_out, fwh_ha
   bp.nq = 0;
   for (int i = 0; i < n; ++i) {
     fwh_handle h = hs[i];
-    fwh_status st = plan(h, c, h0->side);
-    if (st != FWH_OK) return fail(h0, st, h->err);
-    CK(h0, cudaStreamSynchronize(h0->side));
     bp.x_ld[i] = batch_x_ld(h, seg, R0);
     if (h->X.bytes < (size_t)h->P * bp.x_ld[i] * kSer * sizeof(T) + kXPad)
       return fail(h0, FWH_ERR_STATE, "series buffer of a batched surface is too small");
@@ -1467,13 +1464,19 @@ extern "C" fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void 
     fwh_status st = prepare_window(h, nt[i]);
     if (st != FWH_OK) return fail(h0, st, h->err);
   }
-  {  // series buffers (the whole record, or a ring of time segments) before the key
-    const FwdConfig c = fwd_config(h0->precision == FWH_FP64, batch_cfg(n, hs, h0));
+  const int cfg = batch_cfg(n, hs, h0);
+  {  // series buffers (the whole record, or a ring of time segments) before the key, and
+     // every call, replayed or not, the plan of the batch's tile shape: a call between
+     // two batches may have left a handle with the plan (window offsets) of its own shape
+    const FwdConfig c = fwd_config(h0->precision == FWH_FP64, cfg);
     const int seg = seg_len_of(h0->precision == FWH_FP64, c);
     const int R = batch_round_segs(h0, c);
-    for (int i = 0; i < n; ++i)
+    for (int i = 0; i < n; ++i) {
       CK(h0, ensure(hs[i]->X, (size_t)hs[i]->P * batch_x_ld(hs[i], seg, R) * kSer *
                                       tsize(h0->precision) + kXPad));
+      const fwh_status st = plan(hs[i], c, s);
+      if (st != FWH_OK) return fail(h0, st, hs[i]->err);
+    }
   }
   std::vector<uintptr_t> key;
   for (int i = 0; i < n; ++i) {
@@ -1488,7 +1491,7 @@ extern "C" fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void 
     key.push_back((uintptr_t)hs[i]->sets.p);
     key.push_back((uintptr_t)hs[i]->imax.p);
   }
-  key.push_back((uintptr_t)(h0->cfg + 1));
+  key.push_back((uintptr_t)cfg);
   key.push_back((uintptr_t)h0->wait_limit);
   key.push_back((uintptr_t)h0->withhold);
   key.push_back((uintptr_t)h0->batch_ring);
