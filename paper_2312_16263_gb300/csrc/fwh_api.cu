@@ -11,6 +11,7 @@
 // R_s_New).  The set's bounding-box diagonal bounds |y1 - y2|, so the bound
 // needs no per-observer data and holds for any observer set.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -57,9 +58,15 @@ struct BatchPlan {
   int form = FWH_BATCH_PIPELINED;  // launch form (fwh_set_batch_options)
 };
 
+uint64_t next_handle_id() {
+  static std::atomic<uint64_t> n{0};
+  return ++n;
+}
+
 }  // namespace
 
 struct fwh_ctx {
+  const uint64_t id = next_handle_id();  // never given twice (an address may be)
   int64_t P = 0, O = 0;
   double mach = 0, aoa = 0, dt = 0, ca = 1, sa = 0;
   int precision = FWH_FP64;
@@ -1480,7 +1487,7 @@ extern "C" fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void 
   }
   std::vector<uintptr_t> key;
   for (int i = 0; i < n; ++i) {
-    key.push_back((uintptr_t)hs[i]);
+    key.push_back((uintptr_t)hs[i]->id);
     key.push_back((uintptr_t)fields[i]);
     key.push_back((uintptr_t)p_out[i]);
     key.push_back((uintptr_t)nt[i]);

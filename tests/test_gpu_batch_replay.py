@@ -2,9 +2,10 @@
 
 A batched call is captured once and replayed for the same arguments.  Between two
 calls a surface may run by itself under another tile shape, which plans its records
-for other windows; every batched call then needs its own plan back.  Against one
-fwh_forward call per surface, to the rounding of the FP64 output sums (1e-12 of the
-largest value)."""
+for other windows; every batched call then needs its own plan back.  And a surface
+that took a closed one's place needs a graph of its own.  Against one fwh_forward
+call per surface, to the rounding of the FP64 output sums (1e-12 of the largest
+value)."""
 import numpy as np
 import pytest
 import torch
@@ -67,3 +68,20 @@ def test_another_tile_shape_between_two_batches(dev, prec, shape, form):
     surfs[0].check()
     for s in surfs:
         s.close()
+
+
+def test_another_surface_in_the_place_of_a_closed_one(dev):
+    """A new surface may get the address and the buffers of one that was closed; it
+    must not get its graph (here: its angle of attack)."""
+    from paper_2312_16263_gb300 import batch_forward
+    fields = _fields("mixed", dev)
+    outs = [torch.empty((5, 300), dtype=torch.float64, device=dev) for _ in range(2)]
+    first = _surface(0, "mixed")
+    for aoa in (0.1, -0.4, 0.3, 0.0):
+        second = _surface(1, "mixed", aoa)
+        batch_forward([first, second], fields, outs)
+        first.check()
+        refs = [first.forward(fields[0]), second.forward(fields[1])]
+        _close(outs, refs)
+        second.close()
+    first.close()
