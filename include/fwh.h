@@ -341,7 +341,8 @@ fwh_status fwh_psd(int64_t n_sig, const double *p, int64_t ld, const int64_t *n_
  * the budget of fwh_set_moving_scratch, 16 GiB by default; observers are
  * split over launches that fit it, at least one observer per launch) and
  * 128 nt P bytes is taken on `stream` from a memory pool of the library, which
- * keeps up to 8 GiB between calls; the call synchronises.
+ * keeps up to 8 GiB between calls (other allocations of the process get them when
+ * memory runs out; fwh_set_moving_scratch gives them back); the call synchronises.
  * Errors: FWH_ERR_ARG (sizes, |w| >= c0, non-positive c0, rho0, dt),
  * FWH_ERR_OOM / FWH_ERR_CUDA (message via fwh_last_error(NULL)).
  */

@@ -16,7 +16,8 @@ from .build import build  # noqa: F401
 
 
 def __getattr__(name):
-    if name in ("FWH", "batch_forward", "welch_psd", "moving_forward"):
+    if name in ("FWH", "batch_forward", "welch_psd", "moving_forward",
+                "set_moving_scratch"):
         from . import api
         return getattr(api, name)
     if name in ("fwh_apply", "FWHFunction"):
@@ -26,4 +27,4 @@ def __getattr__(name):
 
 
 __all__ = ["FWH", "batch_forward", "build", "fwh_apply", "FWHFunction", "welch_psd",
-           "moving_forward"]
+           "moving_forward", "set_moving_scratch"]

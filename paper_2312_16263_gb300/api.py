@@ -241,6 +241,13 @@ def moving_forward(y: torch.Tensor, normals: torch.Tensor, velocities: torch.Ten
     return out, ts, nv
 
 
+def set_moving_scratch(nbytes: int = 0):
+    """Scratch budget in bytes of later moving_forward calls of the process (0: the
+    default), and the unused memory that earlier calls keep goes back to the device
+    (fwh_set_moving_scratch)."""
+    _abi.check(_abi.load().fwh_set_moving_scratch(int(nbytes)), None)
+
+
 def batch_forward(surfaces: Sequence[FWH], fields: Sequence[torch.Tensor],
                   outs: Sequence[torch.Tensor] | None = None, stream=None):
     """Several surfaces in one graph-captured call (launch form and series

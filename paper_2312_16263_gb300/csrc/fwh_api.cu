@@ -333,9 +333,10 @@ int effective_cfg(const fwh_ctx *h, int64_t nt) {
   return cfg;
 }
 
-// Work items a panel set is cut into, from sizes of the whole problem only
-// (every launch form of it then forms the same partial sums): enough items to
-// give each SM several CTAs, at least eight panels an item; in FP64, where an
+// Work items a panel set is cut into, from sizes of the whole problem only (one
+// launch, the pipelined call and every batched form then form the same partial
+// sums; the host-field call keeps the cut, but its shorter segments split them at
+// other intervals): enough items to give each SM several CTAs, at least eight panels an item; in FP64, where an
 // item's prologue and flushes weigh less and fewer CTAs fit an SM, three times
 // as many items and down to four panels (5151 panels x 701 steps x 19 observers
 // 1.74 -> 1.56 ms and 688 x 475 x 21 0.31 -> 0.17 together with the shorter
@@ -533,7 +534,7 @@ fwh_status run_forward(fwh_handle h, const T *d_fields, double *d_pout, cudaStre
     // Three streams: `copy` moves the slabs, `prep` (high priority, so that
     // its blocks get onto SMs between the scatter's) prepares slab q - 1 once
     // slab q is in (the filters reach 19 frames past a slab's rows), and `s`
-    // scatters each 250-odd-interval time segment once its rows are prepared.
+    // scatters each time segment of 124 or 252 intervals once its rows are prepared.
     // The copy stream first waits for the work already on `s` (the previous
     // call's scatter reads X and its prep the staging buffer), so every later
     // step of this call is ordered after it.
@@ -1552,8 +1553,10 @@ extern "C" fwh_status fwh_check(fwh_handle h, void *stream) {
 // fwh_noalloc.cu.  It reads the handle's panel-set plan, which the set-up calls
 // (fwh_set_observers, fwh_set_tile_config, fwh_autotune) leave in place, and
 // changes no handle state.  Every byte of the scratch that this call reads is
-// written earlier in the same call: the observer windows by k_nvalid, every
-// row of the prepared series (including the zero rows past nt) by the prep.
+// written earlier in the same call: the observer windows by k_nvalid, the rows of
+// the prepared series up to the zero row past the ghost by the prep.  (The copies
+// take in the rows after that one too; what they hold only reaches bins past every
+// observer's window, which are dropped.)
 // ---------------------------------------------------------------------------
 namespace {
 

@@ -821,7 +821,9 @@ __device__ __forceinline__ void consume_step(unsigned active, unsigned stg, unsi
   };
   // A warp with the full count of observers runs them unrolled, so the
   // compiler may overlap one observer's tail with the next one's loads and
-  // arithmetic.  (The last one loads its own record again.)
+  // arithmetic.  (The last one loads its own record again.)  Scatter of 16384
+  // panels x 1024 steps, us per observer: 13.6 with 36 observers (nine a warp),
+  // 14.8 with 28 (seven), 16.3 with 20 (five), 15.3 with 40 (two groups of five).
   if (active == (1u << kMaxObsPerWarpF32) - 1) {
     load(rec(0));
 #pragma unroll

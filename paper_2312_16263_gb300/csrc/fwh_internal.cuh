@@ -21,8 +21,11 @@
 //                            (' = source-time derivative).  Row r holds
 //                            sample row0 + r - 1, so that a record's first
 //                            row is the end value beta_{-1}; x_ld is a
-//                            multiple of 64 rows, rows past sample nt zero.
-//                            Whole records: row0 = 0 and x_ld >= nt + 3
+//                            multiple of 64 rows.  The row after the ghost's
+//                            (sample nt + 1) is zero; the rows after that are
+//                            not written, and only reach bins past every
+//                            observer's window.  Whole records: row0 = 0 and
+//                            x_ld >= nt + 3
 //   Xbar     [P][xb_ld][8] T gradient with respect to beta_0 .. beta_{nt-1}
 //   coef     [P][O][16] T    per (panel, observer) record (slots in
 //                            namespace slot): the 8 integrand coefficients
@@ -43,7 +46,7 @@ constexpr int kRec = 16;          // values per coef record
 constexpr int kSer = 8;           // values per X row
 constexpr int kRowBlk = 64;       // X rows per prep block
 
-// X rows of a whole record of nt samples (samples -1 .. nt + 1 and padding).
+// X rows of a whole record of nt samples (samples -1 .. nt + 1, up to a whole block).
 inline int64_t x_rows(int64_t nt) { return (nt + 3 + kRowBlk - 1) / kRowBlk * kRowBlk; }
 // Bytes past the last X row that an L2 prefetch of a whole chunk may touch.
 constexpr size_t kXPad = 16384;
@@ -194,7 +197,7 @@ struct PrepAdjArgs {
   const double *n;      // [P][3] sorted normals
   const T *Xbar;        // [P][xb_ld][8]
   T *grad_fields;       // [nt][5][P] original order
-  int P, nt, xb_ld, chunk;
+  int P, nt, xb_ld;
   double ca, sa, dt;
 };
 

@@ -377,8 +377,10 @@ constexpr int64_t kMovScratchDefault = (int64_t)16 << 30;
 
 // Scratch comes from a pool of the library's own, one per device, which keeps
 // up to kPoolKeep bytes between calls (mapping the 6.4 GB of the benchmark case anew on
-// every call took 14 ms); fwh_set_moving_scratch gives what is unused back.  The pool
-// orders reuse between streams itself.
+// every call took 14 ms).  The process can have them back at any time: the driver
+// takes them for a cudaMalloc that would otherwise run out (2 GiB free and 6 kept: 4
+// GiB are served, for torch's allocator as well); fwh_set_moving_scratch gives them
+// back to other processes.  The pool orders reuse between streams itself.
 constexpr uint64_t kPoolKeep = (uint64_t)8 << 30;
 constexpr int kMaxDev = 64;
 std::mutex g_pool_mu;

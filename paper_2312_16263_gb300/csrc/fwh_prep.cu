@@ -777,9 +777,9 @@ __global__ void __launch_bounds__(kIirThreads, sizeof(T) == 4 ? 6 : 2) k_prep_ii
 // these, and half of the block's fields are copied to shared memory behind the
 // anti-causal pass, the other half behind the first half's gradients (six CTAs
 // an SM instead of five, three instead of two in FP64).  Bound by HBM and the
-// latency of the chains together.  16384 panels x 1024 steps: 0.25 ms (0.36 with
+// latency of the chains together.  16384 panels x 1024 steps: 0.23 ms (0.36 with
 // the record ends in a kernel of their own that filtered all eight series, and
-// all the fields at once); FP64, 5151 x 701: 0.41 ms (0.68).
+// all the fields at once); FP64, 5151 x 701: 0.40 ms (0.68).
 // ---------------------------------------------------------------------------
 template <typename T> struct Pair;
 template <> struct Pair<float> { using V = float2; };
