@@ -28,12 +28,14 @@
 //    the FP64 pipe alone: against long double the result is that of three FP64
 //    steps, to rounding up to tip Mach numbers of 0.9 at 30 frames a revolution,
 //    1e-11 at 18), and the spline of g at tau* goes to a shared-memory tile from
-//    which each warp sums its panels, one FP64 atomic per warp and bin.
-// About 130 FP64 operations per (panel, sample, observer); bound by the FP64 pipe.
-// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 63.0 ms for
+//    which each warp sums its panels, one FP64 atomic per warp and bin.  Delays
+//    and bin times count from the delay at the panel's first frame: that halves
+//    the rounding of the arrivals, which is the error that is left.
+// About 131 FP64 operations per (panel, sample, observer); bound by the FP64 pipe.
+// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 63.2 ms for
 // k_mscatter (135.4 with moments, four columns, divisions in Newton's method
 // and a shuffle sum per bin: about 380 operations), 1.84 ms for k_mseries (5.65
-// with each frame's integrands formed three times), 65.0 ms a call (164).
+// with each frame's integrands formed three times), 65.5 ms a call (164).
 // Scratch: two FP64 columns of nt per (panel, observer) of a launch; the host
 // splits the observers into launches by the scratch budget.
 #include <cuda_runtime.h>
@@ -239,8 +241,10 @@ __global__ void __launch_bounds__(kMTile, 7) k_mscatter(MovArgs a) {
     iq = 1.0 / q;
   }
   // signal g and delay Delta at every frame (Eqs. pT, pL, tau) and the forward
-  // elimination of both; threads past the last panel only join the sums below
-  double g = 0.0, dl = 0.0, zg = 0.0, zd = 0.0;
+  // elimination of both, of Delta less its value dl0 at the first frame (bin times
+  // less dl0 below): a far observer's distance then rounds neither the spline nor the
+  // arrivals.  Threads past the last panel only join the sums below
+  double g = 0.0, dl = 0.0, zg = 0.0, zd = 0.0, dl0 = 0.0;
   for (int i = 0; live && i < N; ++i) {
     const double *rw = a.S + (size_t)i * kMRow * P + pp;
     double row[kMRow];
@@ -283,8 +287,10 @@ __global__ void __launch_bounds__(kMTile, 7) k_mscatter(MovArgs a) {
     const double ip = ipiv[min(i, kPiv - 1)];
     if (i == 0) {
       zg = g;
-      zd = dl;
+      dl0 = dl;
+      dl = 0.0;
     } else {
+      dl -= dl0;
       zg = fma(6.0, g, -zg) * ip;
       zd = fma(6.0, dl, -zd) * ip;
     }
@@ -311,7 +317,7 @@ __global__ void __launch_bounds__(kMTile, 7) k_mscatter(MovArgs a) {
   // observer bins downwards: every thread walks the same j; each warp sums its
   // panels kMBins at a time and adds them with one atomic a bin
   const int nv = a.nv[o];
-  const double ts = a.ts[o], scale = a.dS[pp] * (kInv4Pi / 6.0);
+  const double ts = a.ts[o] - dl0, scale = a.dS[pp] * (kInv4Pi / 6.0);
   double(*tl)[33] = tile[threadIdx.x >> 5];
   double ak = fma((double)k, h, (D[0] + 4.0 * D[1] + D[2]) * (1.0 / 6.0));  // arrival of node k
   for (int j1 = nv; j1 > 0; j1 -= kMBins) {
