@@ -100,6 +100,7 @@ struct fwh_ctx {
   bool err_pending = false;
   // per-nt
   int64_t nt = -1;
+  int64_t nvalid_nt = -1;  // record length of the window in `nvalid`
   std::vector<int> h_nvalid;
   std::vector<double> h_tstart;
   // planner
@@ -232,6 +233,19 @@ int default_cfg(const fwh_ctx *h) {
   return 0;
 }
 
+// Tables of a handle are copied to the device in stream order, from host memory that a
+// replayed graph would read again: not while `s` is captured.
+fwh_status table_copy(fwh_handle h, void *dst, const void *src, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(h, cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone)
+    return fail(h, FWH_ERR_CUDA,
+                "the call copies tables to the device (its first one for this record length or "
+                "tile shape) and cannot be captured; make one such call before the capture");
+  CK(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+  return FWH_OK;
+}
+
 // Observer tiling for a config: the fewest groups that hold all observers,
 // and observers per warp as even as they go over those (37 observers: two
 // groups of 20 and 17, not 36 and 1).
@@ -244,17 +258,20 @@ void obs_tiling(const fwh_ctx *h, const FwdConfig &c, int *obs_per_cta, int *gro
 }
 
 // Panel sets for a config, and the plan kernel's per-(set, observer) shift
-// table and per-record window offsets, enqueued on `s`.
+// table and per-record window offsets, enqueued on `s` with the copies of the set
+// tables (earlier calls on `s` may still be reading the former ones).
 fwh_status plan(fwh_handle h, const FwdConfig &c, cudaStream_t s) {
   const bool fp64 = h->precision == FWH_FP64;
   const int smax = fwd_slack(fp64, c);
   const int sb = c.acc == 5 ? 8 : 4;  // bytes per FP32 window slot (sum, or sum + compensation)
   if (h->plan_win == c.win && h->plan_slack == smax && h->plan_sb == sb) return FWH_OK;
+  h->plan_win = -1;  // until the new one is complete
   h->set_begin = build_sets(h->y, h->P, h->mach, h->dt, smax);
   const size_t bytes = h->set_begin.size() * sizeof(int);
   const int nsets = (int)h->set_begin.size() - 1;
   CK(h, ensure(h->sets, bytes));
-  CK(h, cudaMemcpy(h->sets.p, h->set_begin.data(), bytes, cudaMemcpyHostToDevice));
+  fwh_status st = table_copy(h, h->sets.p, h->set_begin.data(), bytes, s);
+  if (st != FWH_OK) return st;
   {  // work order: sets by descending panel count
     std::vector<int> ord(nsets);
     std::iota(ord.begin(), ord.end(), 0);
@@ -262,7 +279,8 @@ fwh_status plan(fwh_handle h, const FwdConfig &c, cudaStream_t s) {
       return h->set_begin[x + 1] - h->set_begin[x] > h->set_begin[y + 1] - h->set_begin[y];
     });
     CK(h, ensure(h->sord, ord.size() * sizeof(int)));
-    CK(h, cudaMemcpy(h->sord.p, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice));
+    st = table_copy(h, h->sord.p, ord.data(), ord.size() * sizeof(int), s);
+    if (st != FWH_OK) return st;
   }
   CK(h, ensure(h->imax, (size_t)nsets * h->O * sizeof(int)));
   const int *i0 = reinterpret_cast<const int *>(h->i0.p);
@@ -300,11 +318,20 @@ fwh_status prepare_window(fwh_handle h, int64_t nt) {
       h->h_nvalid[o] = (int)nv;
       h->h_tstart[o] = ts;
     }
-    CK(h, ensure(h->nvalid, h->O * sizeof(int)));
-    CK(h, cudaMemcpy(h->nvalid.p, h->h_nvalid.data(), h->O * sizeof(int),
-                     cudaMemcpyHostToDevice));
     h->nt = nt;
   }
+  return FWH_OK;
+}
+
+// The window on the device, for the calls that follow on `s`: the copy is ordered
+// behind the work already on `s`, which may read the window of another record length.
+fwh_status upload_window(fwh_handle h, cudaStream_t s) {
+  if (h->nvalid_nt == h->nt) return FWH_OK;
+  CK(h, ensure(h->nvalid, h->O * sizeof(int)));
+  const fwh_status st =
+      table_copy(h, h->nvalid.p, h->h_nvalid.data(), h->O * sizeof(int), s);
+  if (st != FWH_OK) return st;
+  h->nvalid_nt = h->nt;
   return FWH_OK;
 }
 
@@ -407,6 +434,7 @@ PrepArgs<T> prep_args(const fwh_ctx *h, const T *fields, int64_t nt, T *X, int x
 // must not allocate or copy from the host find it in place.
 fwh_status plan_default(fwh_handle h) {
   const FwdConfig c = fwd_config(h->precision == FWH_FP64, h->cfg >= 0 ? h->cfg : default_cfg(h));
+  CK(h, cudaDeviceSynchronize());  // calls in flight on any stream may read the present plan
   fwh_status st = plan(h, c, 0);
   if (st != FWH_OK) return st;
   CK(h, cudaStreamSynchronize(0));
@@ -911,7 +939,7 @@ fwh_status fwh_set_observers(fwh_handle h, int64_t O, const double *xyz) {
   h->Rmin_loc = h->Rmin;
   h->xobs = x;
   h->O = O;
-  h->nt = -1;         // window depends on the observers
+  h->nt = h->nvalid_nt = -1;  // window depends on the observers
   h->plan_win = -1;   // records were rewritten: window offsets must be re-planned
   h->plan_sb = -1;
   drop_graphs(h);
@@ -942,6 +970,7 @@ fwh_status fwh_set_observer_extremes(fwh_handle h, const double *r_max, const do
                       "r_min <= its smallest)");
   }
   std::vector<double> mx(r_max, r_max + h->O), mn(r_min, r_min + h->O);
+  CK(h, cudaDeviceSynchronize());  // calls in flight on any stream may read the records
   CK(h, cudaMemcpy(h->d_Rmax, mx.data(), h->O * sizeof(double), cudaMemcpyHostToDevice));
   CK(h, cudaMemcpy(h->d_Rmin, mn.data(), h->O * sizeof(double), cudaMemcpyHostToDevice));
   GeomArgs g{};
@@ -965,7 +994,7 @@ fwh_status fwh_set_observer_extremes(fwh_handle h, const double *r_max, const do
                              reinterpret_cast<int *>(h->i0.p), 0));
   h->Rmax = mx;
   h->Rmin = mn;
-  h->nt = -1;
+  h->nt = h->nvalid_nt = -1;
   h->plan_win = -1;
   drop_graphs(h);
   return plan_default(h);
@@ -992,6 +1021,7 @@ fwh_status fwh_forward(fwh_handle h, const void *fields, int64_t nt, double *p_o
   fwh_status st = take_deferred(h);
   if (st != FWH_OK) return st;
   st = prepare_nt(h, nt);
+  if (st == FWH_OK) st = upload_window(h, s);
   if (st != FWH_OK) return st;
   const size_t ts = tsize(h->precision);
   const size_t fbytes = (size_t)nt * 5 * h->P * ts;
@@ -1034,6 +1064,7 @@ fwh_status fwh_backward(fwh_handle h, const void *fields, int64_t nt, const doub
   fwh_status st = take_deferred(h);
   if (st != FWH_OK) return st;
   st = prepare_nt(h, nt);
+  if (st == FWH_OK) st = upload_window(h, s);
   if (st != FWH_OK) return st;
   const size_t ts = tsize(h->precision);
   const size_t fbytes = (size_t)nt * 5 * h->P * ts;
@@ -1085,6 +1116,7 @@ fwh_status fwh_autotune(fwh_handle h, int64_t nt, int *chosen, void *stream) {
   if (h->O < 1) return fail(h, FWH_ERR_STATE, "fwh_set_observers must come first");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   fwh_status st = prepare_nt(h, nt);
+  if (st == FWH_OK) st = upload_window(h, s);
   if (st != FWH_OK) return st;
   const size_t ts = tsize(h->precision);
   Buf f, po;
@@ -1470,6 +1502,7 @@ extern "C" fwh_status fwh_batch_forward(int n, const fwh_handle *hs, const void 
     if (!is_device_ptr(fields[i]) || !is_device_ptr(p_out[i]))
       return fail(h0, FWH_ERR_ARG, "batched forward takes device buffers");
     fwh_status st = prepare_window(h, nt[i]);
+    if (st == FWH_OK) st = upload_window(h, s);
     if (st != FWH_OK) return fail(h0, st, h->err);
   }
   const int cfg = batch_cfg(n, hs, h0);
