@@ -1030,8 +1030,8 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
   PipeState ps;
   unsigned char *wbase = smem_raw;
   unsigned step = 0;
+  int maxo = 0;  // observers of the largest group: the same windows' places for every surface
   if constexpr (PIPE != 0) {
-    int maxo = 0;
     for (int i = 0; i < n_surf; ++i) maxo = max(maxo, args[i].obs_per_cta);
     // (its barrier also orders the item ring's initialisation above)
     wbase = pipe_setup<T, TK, NW>(smem_raw, maxo, nst, bars, &abort_flag, ps);
@@ -1071,7 +1071,9 @@ __device__ __forceinline__ void forward_batch_cta(const BatchParams<T> &P, int *
         const int sf = batch_surface(prefix, n_surf, item);
         const FwdArgs<T> &a = args[sf];
         const Item<T, NW> it(a, item - prefix[sf], w);
-        T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * it.opw * a.wfl;
+        // (not it.opw apart: the other warps may still work on an item of a surface
+        // with another number of observers)
+        T *wwin = reinterpret_cast<T *>(wbase) + (size_t)w * (maxo / NW) * a.wfl;
         if constexpr (sizeof(T) == 4)
           consume_item_f32<TK, NW, ACC == 5>(a, it, ps, step, wwin, st + w * kMaxObsPerWarp, w);
         else
