@@ -32,7 +32,7 @@
 //    and bin times count from the delay at the panel's first frame: that halves
 //    the rounding of the arrivals, which is the error that is left.
 // About 131 FP64 operations per (panel, sample, observer); bound by the FP64 pipe.
-// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 63.2 ms for
+// Spinning sphere of 8192 panels x 2048 frames x 16 observers: 63.6 ms for
 // k_mscatter (135.4 with moments, four columns, divisions in Newton's method
 // and a shuffle sum per bin: about 380 operations), 1.84 ms for k_mseries (5.65
 // with each frame's integrands formed three times), 65.5 ms a call (164).
