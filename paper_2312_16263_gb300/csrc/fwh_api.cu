@@ -363,12 +363,12 @@ int effective_cfg(const fwh_ctx *h, int64_t nt) {
 // Work items a panel set is cut into, from sizes of the whole problem only (one
 // launch, the pipelined call and every batched form then form the same partial
 // sums; the host-field call keeps the cut, but its shorter segments split them at
-// other intervals): enough items to give each SM several CTAs, at least eight panels an item; in FP64, where an
-// item's prologue and flushes weigh less and fewer CTAs fit an SM, three times
-// as many items and down to four panels (5151 panels x 701 steps x 19 observers
-// 1.74 -> 1.56 ms and 688 x 475 x 21 0.31 -> 0.17 together with the shorter
-// segments; four panels an item in mixed precision: 23 -> 30 us at 2048 x 256
-// x 8).
+// other intervals): enough items to give each SM several CTAs, at least eight
+// panels an item; in FP64, where an item's prologue and flushes weigh less and
+// fewer CTAs fit an SM, three times as many items and down to four panels (5151
+// panels x 701 steps x 19 observers 1.74 -> 1.56 ms and 688 x 475 x 21 0.31 -> 0.17
+// together with the shorter segments; four panels an item in mixed precision: 23
+// -> 30 us at 2048 x 256 x 8).
 int set_subs(const fwh_ctx *h, int groups, int n_segs) {
   const bool fp64 = h->precision == FWH_FP64;
   const int64_t nsets = (int64_t)h->set_begin.size() - 1;
